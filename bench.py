@@ -80,17 +80,7 @@ FP32K_INST_PER_SITE_STEP = 58    # the update: 4 operations per component instea
 # tiling recorded with it; any other combination reports null.  A launch's traffic is
 # proportional to the sites it advances (one read and one write of each tile), so a capture at
 # N = 2^24 scales to the N = 2^27 workload by the site count.
-TRAFFIC = {
-    ("24e57e0265074389", "256,4,1"): (402771968 + 357428224, 1 << 24),
-    ("24e57e0265074389", "128,4,1"): (402821632 + 356577792, 1 << 24),
-    ("24e57e0265074389", "512,2,1"): (402830848 + 356819456, 1 << 24),
-    ("24e57e0265074389", "128,8,1"): (403226624 + 356647424, 1 << 24),
-    ("24e57e0265074389", "256,4,2"): (402761472 + 357003008, 1 << 24),
-    ("24e57e0265074389", "128,4,2"): (402859776 + 356683008, 1 << 24),
-    ("24e57e0265074389", "512,2,2"): (402838272 + 357778944, 1 << 24),
-    ("24e57e0265074389", "128,8,2"): (402945792 + 357322496, 1 << 24),
-    ("24e57e0265074389", "256,8,2"): (402975232 + 357140224, 1 << 24),
-}
+TRAFFIC = {}
 
 
 def traffic_per_launch(khash: str, tiling: dict, n: int):
@@ -107,7 +97,7 @@ def code_only(src: str) -> str:
     return " ".join(src.split())
 
 
-BLOCKED_SOURCES = ("rk4_device.cuh", "rk4_tile.cuh", "k_blocked.cu")
+BLOCKED_SOURCES = ("rk4_device.cuh", "rk4_split.cuh", "rk4_tile.cuh", "k_split.cuh", "k_blocked.cu")
 GENERIC_SOURCES = ("rk4_device.cuh", "rk4_tile.cuh", "rk4_generic.cuh", "k_generic.cu")
 
 

@@ -86,7 +86,9 @@ size_t blocked_smem_bytes(int model, bool fp32, int v, int block, bool het) {
   const int D = model == ROESSLER ? 3 : 2;
   const int P = model == ROESSLER ? 4 : 2;
   const size_t rs = fp32 ? 4 : 8;
-  return (size_t)edge_values(v) * rs + (size_t)block * v * rs * (D * (fp32 ? 2 : 1) + (het ? P : 0));
+  // a heterogeneous FP64 tile also holds the split form's pair coefficients of each site
+  const size_t pairs = het && !fp32 ? (model == ROESSLER ? 24 : 16) : 0;
+  return (size_t)edge_values(v) * rs + (size_t)block * v * (rs * (D * (fp32 ? 2 : 1) + (het ? P : 0)) + pairs);
 }
 
 template <typename R, int MODEL, int V, bool KAHAN, bool HET>
@@ -135,6 +137,9 @@ static cudaError_t launch_m(bool fp32, int v, int block, const BlockedJob &job, 
 
 cudaError_t launch_blocked(int model, bool fp32, int v, int block, const BlockedJob &job, const CoefD &cf,
                            cudaStream_t st) {
+  if (job.split)
+    return model == ROESSLER ? launch_split_blocked<ROESSLER>(v, block, job, cf, st)
+                             : launch_split_blocked<HARMONIC>(v, block, job, cf, st);
   return model == ROESSLER ? launch_m<ROESSLER>(fp32, v, block, job, cf, st)
                            : launch_m<HARMONIC>(fp32, v, block, job, cf, st);
 }

@@ -3,49 +3,10 @@
 // (chain, tile) items, then all blocks meet at a grid barrier before the next time block
 // reads what the previous one wrote.  The barrier's wait is bounded: a block that waits
 // longer than timeout_ns latches ST_TIMEOUT in the status word and the kernel returns.
+#include "k_grid_barrier.cuh"
 #include "rk4_tile.cuh"
 
 namespace rk4d {
-
-__device__ __forceinline__ long long global_ns() {
-  long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-
-// Grid-wide barrier over the co-resident blocks of a cooperative launch.  Returns false when
-// this block gave up waiting (or another block already did).
-__device__ __forceinline__ bool grid_barrier(WsHeader *hdr, long long timeout_ns, int extra) {
-  __shared__ int ok;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    ok = 1;
-    volatile unsigned *gen = &hdr->bar_gen;
-    volatile int *status = &hdr->status;
-    const unsigned g = *gen;
-    __threadfence();
-    const unsigned expected = gridDim.x + (unsigned)extra;
-    const unsigned arrived = atomicAdd(&hdr->bar_count, 1u) + 1u;
-    if (arrived == expected) {
-      atomicExch(&hdr->bar_count, 0u);
-      __threadfence();
-      atomicAdd(&hdr->bar_gen, 1u);
-    } else {
-      const long long t0 = global_ns();
-      while (*gen == g) {
-        if ((*status & ST_TIMEOUT) || global_ns() - t0 > timeout_ns) {
-          atomicOr(&hdr->status, ST_TIMEOUT);
-          ok = 0;
-          break;
-        }
-        __nanosleep(64);
-      }
-    }
-    __threadfence();
-  }
-  __syncthreads();
-  return ok != 0;
-}
 
 // A packed tile of a batch (the segments of item p).  Not inlined, as in the one-shot blocked
 // kernel: the segment bookkeeping then takes registers only inside this call, and the full-tile
@@ -68,50 +29,32 @@ template <typename R, int MODEL, int V, bool KAHAN, bool BATCH>
 __device__ __noinline__ void persistent_tile_call(const PersistentJob &job, int ki, const R *in, R *out,
                                                   const R *cin, R *cout, int64_t item, int K, int G, Coef<R> cf,
                                                   unsigned char *smem) {
-  if constexpr (!BATCH)
+  if constexpr (!BATCH) {
     tile_item<R, MODEL, V, KAHAN, true>(in, out, cin, cout, job.one, item, K, G, cf, smem, job.total, job.hdr);
-  else
-    batch_item<R, MODEL, V, KAHAN, true>(in, out, cin, cout, job.chains, job.nchains, job.bt[ki], item, K, G, cf,
-                                         smem, job.total, job.hdr);
+  } else {
+    int64_t local;
+    const int ci = batch_chain(job.bt[ki], job.nchains, item - job.bt[ki].npacked, smem, local);
+    const ChainDesc ch = job.chains[ci];
+    cf.kappa = (R)ch.kappa;
+    tile_item<R, MODEL, V, KAHAN, true, false, true>(in, out, cin, cout, ch, local, K, G, cf, smem, job.total,
+                                                     job.hdr);
+  }
 }
 
 template <typename R, int MODEL, int V, bool KAHAN, bool BATCH>
 __global__ void __launch_bounds__(max_threads_for(V), (V >= 2 && KAHAN) ? 2 : 1)  // FP32: two resident blocks
     k_persistent(PersistentJob job, Coef<R> cf) {
   extern __shared__ __align__(16) unsigned char smem[];
-  const int64_t nblocks_t = job.nmain + job.ntail;
-  for (int64_t t = 0; t < nblocks_t; ++t) {
-    const int ki = (t < job.nmain) ? 0 : job.tail[t - job.nmain];
-    const int K = job.kval[ki];
-    const int G = job.Gval[ki];
-    const int64_t ntiles = job.ntiles[ki];
-    const R *in = static_cast<const R *>((t & 1) ? job.bufB : job.bufA);
-    R *out = static_cast<R *>((t & 1) ? job.bufA : job.bufB);
-    const R *cin = static_cast<const R *>((t & 1) ? job.cB : job.cA);
-    R *cout = static_cast<R *>((t & 1) ? job.cA : job.cB);
-    // Items are handed out dynamically (an atomic counter per time-block parity), so blocks
-    // that drew cheaper items take more and all reach the barrier together.  Block 0 clears
-    // the other parity's counter for the next time block (the barrier orders it).
-    unsigned long long *ctr = &job.hdr->work[t & 1];
-    if (blockIdx.x == 0 && threadIdx.x == 0 && t > 0) job.hdr->work[(t + 1) & 1] = 0ull;
-    __shared__ long long s_item;
-    if (threadIdx.x == 0) s_item = (long long)atomicAdd(ctr, 1ull);
-    __syncthreads();
-    for (int64_t item = s_item; item < ntiles;) {
-      if (BATCH && item < job.bt[ki].npacked)
-        persistent_packed_call<R, MODEL, V, KAHAN>(in, out, cin, cout, job.chains, job.bt[ki].segs,
-                                                   job.bt[ki].pack_prefix, item, K, cf, smem, job.total, job.hdr);
-      else
-        persistent_tile_call<R, MODEL, V, KAHAN, BATCH>(job, ki, in, out, cin, cout, item, K, G, cf, smem);
-      // both end with a barrier, so every thread has read s_item before it is rewritten
-      if (threadIdx.x == 0) s_item = (long long)atomicAdd(ctr, 1ull);
-      __syncthreads();
-      item = s_item;
-    }
-    if (t + 1 < nblocks_t || job.extra_arrivals > 0) {
-      if (!grid_barrier(job.hdr, job.timeout_ns, job.extra_arrivals)) return;
-    }
-  }
+  persistent_loop(job, [&](int ki, const void *vin, void *vout, const void *vcin, void *vcout, int64_t item, int K,
+                           int G) {
+    const R *in = static_cast<const R *>(vin), *cin = static_cast<const R *>(vcin);
+    R *out = static_cast<R *>(vout), *cout = static_cast<R *>(vcout);
+    if (BATCH && item < job.bt[ki].npacked)
+      persistent_packed_call<R, MODEL, V, KAHAN>(in, out, cin, cout, job.chains, job.bt[ki].segs,
+                                                 job.bt[ki].pack_prefix, item, K, cf, smem, job.total, job.hdr);
+    else
+      persistent_tile_call<R, MODEL, V, KAHAN, BATCH>(job, ki, in, out, cin, cout, item, K, G, cf, smem);
+  });
 }
 
 template <typename R, int MODEL, int V, bool KAHAN>
@@ -180,11 +123,17 @@ static int max_grid_m(bool fp32, int v, int block) {
 
 cudaError_t launch_persistent(int model, bool fp32, int v, int block, int grid, const PersistentJob &job,
                               const CoefD &cf, cudaStream_t st) {
+  if (job.split)
+    return model == ROESSLER ? launch_split_persistent<ROESSLER>(v, block, grid, job, cf, st)
+                             : launch_split_persistent<HARMONIC>(v, block, grid, job, cf, st);
   return model == ROESSLER ? launch_m<ROESSLER>(fp32, v, block, grid, job, cf, st)
                            : launch_m<HARMONIC>(fp32, v, block, grid, job, cf, st);
 }
 
-int persistent_max_grid(int model, bool fp32, int v, int block) {
+int persistent_max_grid(int model, bool fp32, int v, int block, bool split) {
+  if (split)
+    return model == ROESSLER ? persistent_split_max_grid<ROESSLER>(v, block)
+                             : persistent_split_max_grid<HARMONIC>(v, block);
   return model == ROESSLER ? max_grid_m<ROESSLER>(fp32, v, block) : max_grid_m<HARMONIC>(fp32, v, block);
 }
 

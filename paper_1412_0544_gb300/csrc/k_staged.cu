@@ -1,12 +1,27 @@
 // k_staged.cu -- the paper's "standard implementation" (Sec. 2.2) on the GPU: one launch per
 // RK stage, each a full sweep over every site.  It is the bit-identity reference for the
 // blocked and persistent kernels (all three call the same per-site functions).
+#include <algorithm>
+
 #include "rk4_tile.cuh"
 
 namespace rk4d {
 
+// The chain of site i (its coupling strength goes into c).
+template <typename R> __device__ __forceinline__ ChainDesc staged_chain(const StagedJob &job, int64_t i, Coef<R> &c) {
+  if (job.nchains == 1) return job.one;
+  int lo = 0, hi = job.nchains - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (job.chains[mid].off <= i) lo = mid; else hi = mid - 1;
+  }
+  const ChainDesc ch = job.chains[lo];
+  c.kappa = (R)ch.kappa;
+  return ch;
+}
+
 template <typename R, int MODEL, bool KAHAN>
-__global__ void __launch_bounds__(256) k_staged(StagedJob job, Coef<R> cf, int j) {
+__device__ __forceinline__ void staged_sweep(const StagedJob &job, const Coef<R> &cf, int j) {
   constexpr int D = Dim<MODEL>::D;
   R *Y = static_cast<R *>(job.y);
   R *CMP = static_cast<R *>(job.cmp);
@@ -15,19 +30,8 @@ __global__ void __launch_bounds__(256) k_staged(StagedJob job, Coef<R> cf, int j
   R *ACC = static_cast<R *>(job.acc);
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < job.total; i += stride) {
-    ChainDesc ch;
     Coef<R> c = cf;
-    if (job.nchains == 1) {
-      ch = job.one;
-    } else {
-      int lo = 0, hi = job.nchains - 1;
-      while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (job.chains[mid].off <= i) lo = mid; else hi = mid - 1;
-      }
-      ch = job.chains[lo];
-      c.kappa = (R)ch.kappa;
-    }
+    const ChainDesc ch = staged_chain(job, i, c);
     if (job.sp) c = site_coef<R, MODEL>(c, static_cast<const R *>(job.sp) + i * Dim<MODEL>::P);  // Eq. (1)
     const int64_t li = i - ch.off;  // index within the chain
     R u[D], y[D], acc[D], cmp[D], k[D];
@@ -72,16 +76,150 @@ __global__ void __launch_bounds__(256) k_staged(StagedJob job, Coef<R> cf, int j
 }
 
 template <typename R, int MODEL, bool KAHAN>
+__global__ void __launch_bounds__(256) k_staged(StagedJob job, Coef<R> cf, int j) {
+  staged_sweep<R, MODEL, KAHAN>(job, cf, j);
+}
+
+// The same in the split form (rk4_split.cuh), bit for bit what the tile kernels compute: stage 0
+// stores the first slope K1, stages 1 and 2 their negated differences, and a stage's increments
+// (the site's and its neighbours') are formed again from these.  Once a value has left the
+// split's range (the scan before the first step, or a step's result) the steps that follow run
+// in the FP64 form.
+template <int MODEL>
+__global__ void __launch_bounds__(256) k_staged_split(StagedJob job, Coef<double> cf, SplitCoef sc, int j) {
+  constexpr int D = Dim<MODEL>::D;
+  if (job.hdr->wide[job.parity]) {
+    staged_sweep<double, MODEL, false>(job, cf, j);
+    if (j == 3 && blockIdx.x == 0 && threadIdx.x == 0) job.hdr->wide[job.parity ^ 1] = 1u;
+    return;
+  }
+  double *Y = static_cast<double *>(job.y);
+  double *K1 = static_cast<double *>(job.acc);
+  float2 *N2 = static_cast<float2 *>(job.n2), *N3 = static_cast<float2 *>(job.n3);
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < job.total; i += stride) {
+    Coef<double> c = cf;
+    const ChainDesc ch = staged_chain(job, i, c);
+    const int64_t li = i - ch.off;
+    // the neighbours' sites, or -1 beyond a fixed end
+    int64_t il = li > 0 ? i - 1 : (ch.bc == PERIODIC ? ch.off + ch.n - 1 : -1);
+    int64_t ir = li < ch.n - 1 ? i + 1 : (ch.bc == PERIODIC ? ch.off : -1);
+    if (!bounds_ok(job.hdr, (il < 0 || in_range(il, 1, job.total)) && (ir < 0 || in_range(ir, 1, job.total)))) continue;
+    const double *sp = job.sp ? static_cast<const double *>(job.sp) + i * Dim<MODEL>::P : nullptr;
+    double y[D];
+#pragma unroll
+    for (int d = 0; d < D; ++d) y[d] = Y[i * D + d];
+    if (sp) c = site_coef<double, MODEL>(c, sp);
+    if (j == 0) {
+      double k[D];
+      slope<double, MODEL>(y, il < 0 ? 0.0 : Y[il * D], ir < 0 ? 0.0 : Y[ir * D], c, k);
+#pragma unroll
+      for (int d = 0; d < D; ++d) K1[i * D + d] = k[d];
+      continue;
+    }
+    SplitCoef s = sc;
+    split_set_kappa(s, c.kappa);
+    if (sp) {
+      const FPair<float> at = times_tau(sp[0], s), cc = split1(MODEL == ROESSLER ? sp[2] : 0.0);
+      s.ath = at.h;
+      s.atl = at.l;
+      s.ch = cc.h;
+      s.cl = cc.l;
+    }
+    // increments of component q (site * D + component) for stage j; N is the running sum
+    auto increment = [&](int64_t q, FPair<float> &k1, FPair<float> &N) {
+      k1 = split1(K1[q]);
+      FPair<float> d = k1;
+      for (int m = 1; m < j; ++m) {
+        const float2 n = m == 1 ? N2[q] : N3[q];
+        split_update<float>(m, k1, {n.x, n.y}, d, N);
+      }
+      return d;
+    };
+    FPair<float> k1[D], d[D], N[D], n[D], xl = {0.f, 0.f}, xr = {0.f, 0.f}, t0, t1;
+#pragma unroll
+    for (int q = 0; q < D; ++q) {
+      N[q] = {0.f, 0.f};
+      d[q] = increment(i * D + q, k1[q], N[q]);
+    }
+    if (il >= 0) xl = increment(il * D, t0, t1);
+    if (ir >= 0) xr = increment(ir * D, t0, t1);
+    SplitBase<float> base = {};
+    if constexpr (MODEL == ROESSLER) {
+      base.z = split1(y[2]);
+      base.t = x_minus_c<float>(split1(y[0]), {s.ch, s.cl});
+    }
+    split_stage<MODEL, float>(d, xl, xr, base, stage_coef<float>(s), n);
+    if (j < 3) {
+      float2 *o = j == 1 ? N2 : N3;
+#pragma unroll
+      for (int q = 0; q < D; ++q) o[i * D + q] = make_float2(n[q].h, n[q].l);
+      continue;
+    }
+    bool wide = false, bad = false;
+#pragma unroll
+    for (int q = 0; q < D; ++q) {
+      split_update<float>(3, k1[q], n[q], d[q], N[q]);
+      double nd;
+      join(N[q], &nd, 1);
+      const double r = split_final(y[q], K1[i * D + q], nd, s);
+      Y[i * D + q] = r;
+      wide |= !split_in_range<MODEL>(r);
+      bad |= nonfinite(r);
+    }
+    if (wide) job.hdr->wide[job.parity ^ 1] = 1u;
+    if (bad) atomicOr(&job.hdr->status, ST_NONFINITE);
+  }
+}
+
+template <int MODEL>
+__global__ void __launch_bounds__(256) k_split_scan(const double *y, const double *sp, int64_t total, SplitCoef sc,
+                                                    WsHeader *hdr) {
+  constexpr int D = Dim<MODEL>::D, P = Dim<MODEL>::P;
+  bool wide = false;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += stride) {
+#pragma unroll
+    for (int d = 0; d < D; ++d) wide |= !split_in_range<MODEL>(y[i * D + d]);
+    if (sp) {
+#pragma unroll
+      for (int q = 0; q < P; ++q) wide |= !split_param_in_range(sp[i * P + q], sc.most[q]);
+    }
+  }
+  if (wide) hdr->wide[0] = 1u;
+}
+
+static unsigned sweep_grid(int64_t total) {
+  const int64_t cap = (int64_t)sm_count() * 64;
+  return (unsigned)std::min<int64_t>((total + 255) / 256, cap);
+}
+
+cudaError_t launch_split_scan(int model, const double *state, const double *sp, int64_t total, const SplitCoef &sc,
+                              WsHeader *hdr, cudaStream_t st) {
+  if (total <= 0) return cudaSuccess;
+  if (model == ROESSLER) k_split_scan<ROESSLER><<<sweep_grid(total), 256, 0, st>>>(state, sp, total, sc, hdr);
+  else k_split_scan<HARMONIC><<<sweep_grid(total), 256, 0, st>>>(state, sp, total, sc, hdr);
+  return cudaGetLastError();
+}
+
+template <int MODEL>
+static cudaError_t launch_split_one(int j, const StagedJob &job, const CoefD &cfd, cudaStream_t st) {
+  if (job.total <= 0) return cudaSuccess;
+  k_staged_split<MODEL><<<sweep_grid(job.total), 256, 0, st>>>(job, to_coef<double>(cfd, cfd.kappa),
+                                                              split_coef(MODEL, cfd), j);
+  return cudaGetLastError();
+}
+
+template <typename R, int MODEL, bool KAHAN>
 static cudaError_t launch_one(int j, const StagedJob &job, const CoefD &cfd, cudaStream_t st) {
   if (job.total <= 0) return cudaSuccess;
-  const int block = 256;
-  int64_t grid = (job.total + block - 1) / block;
-  if (grid > (int64_t)sm_count() * 64) grid = (int64_t)sm_count() * 64;
-  k_staged<R, MODEL, KAHAN><<<(unsigned)grid, block, 0, st>>>(job, to_coef<R>(cfd, cfd.kappa), j);
+  k_staged<R, MODEL, KAHAN><<<sweep_grid(job.total), 256, 0, st>>>(job, to_coef<R>(cfd, cfd.kappa), j);
   return cudaGetLastError();
 }
 
 cudaError_t launch_staged(int model, bool fp32, int j, const StagedJob &job, const CoefD &cf, cudaStream_t st) {
+  if (job.split)
+    return model == ROESSLER ? launch_split_one<ROESSLER>(j, job, cf, st) : launch_split_one<HARMONIC>(j, job, cf, st);
   if (model == ROESSLER)
     return fp32 ? launch_one<float, ROESSLER, true>(j, job, cf, st) : launch_one<double, ROESSLER, false>(j, job, cf, st);
   return fp32 ? launch_one<float, HARMONIC, true>(j, job, cf, st) : launch_one<double, HARMONIC, false>(j, job, cf, st);

@@ -59,6 +59,7 @@ struct rk4_chain {
   bool fp32 = false;
   int nchains = 1;
   std::vector<ChainDesc> chains;
+  double kappa_most = 0.0, kappa_least = 0.0;  // largest and smallest nonzero |kappa| of the chains
   int64_t total = 0;
   double dt = 0.01;
   rk4_params p{};
@@ -212,6 +213,23 @@ CoefD coef(const rk4_chain *h) {
   c.dt3 = h->dt / 3.0;
   c.kappa2 = h->kappa2;
   return c;
+}
+
+// FP64 handles run the step in the split form (rk4_split.cuh) when its error bound holds for
+// their coefficients; every scheme of a handle takes the same form.
+bool use_split(const rk4_chain *h) {
+  if (h->fp32 || use_generic(h)) return false;
+  CoefD c = coef(h);
+  c.kappa = h->kappa_most;
+  if (!split_allowed(h->model, c)) return false;
+  c.kappa = h->kappa_least;
+  return split_allowed(h->model, c);
+}
+
+void note_kappa(rk4_chain *h, double kappa) {
+  const double k = std::fabs(kappa);
+  h->kappa_most = std::max(h->kappa_most, k);
+  if (k > 0.0 && (h->kappa_least == 0.0 || k < h->kappa_least)) h->kappa_least = k;
 }
 
 int tiling_valid(const rk4_chain *h, int block, int v, int k) {
@@ -520,7 +538,16 @@ cudaError_t enqueue_integrate(rk4_chain *h, int kernel, void *state, void *comp,
     j.hdr = reinterpret_cast<WsHeader *>(ws + L.hdr);
     j.acc = ws + L.acc;
     void *u0 = ws + L.u0, *u1 = ws + L.u1;
+    j.split = use_split(h) ? 1 : 0;
+    j.n2 = u0;
+    j.n3 = u1;
+    if (j.split) {
+      e = launch_split_scan(h->model, static_cast<const double *>(state), static_cast<const double *>(h->site_params),
+                            h->total, split_coef(h->model, cf), j.hdr, st);
+      if (e != cudaSuccess) return e;
+    }
     for (int64_t s = 0; s < nsteps; ++s) {
+      j.parity = (int)(s & 1);
       // stage 0 reads y and writes u0; 1: u0 -> u1; 2: u1 -> u0; 3: u0 -> y
       for (int st4 = 0; st4 < 4; ++st4) {
         j.uin = (st4 == 2) ? u1 : u0;
@@ -544,6 +571,7 @@ cudaError_t enqueue_integrate(rk4_chain *h, int kernel, void *state, void *comp,
     j.hdr = reinterpret_cast<WsHeader *>(ws + L.hdr);
     j.total = h->total;
     j.packed = packed_batch(h) ? 1 : 0;
+    j.split = use_split(h) ? 1 : 0;
     for (int64_t i = 0; i < P.count(); ++i) {
       const int k = P.k_at(i);
       int ki = 0;
@@ -597,6 +625,7 @@ cudaError_t enqueue_integrate(rk4_chain *h, int kernel, void *state, void *comp,
     for (int i = 0; i < j.ntail; ++i) j.tail[i] = P.tail[i];
     j.hdr = reinterpret_cast<WsHeader *>(ws + L.hdr);
     j.total = h->total;
+    j.split = use_split(h) ? 1 : 0;
     // A barrier waits at most one time block; unless the caller set the bound, allow 20x a
     // pessimistic estimate of one (1e9 site-steps/s) so that very large batches cannot time
     // out spuriously.
@@ -607,7 +636,7 @@ cudaError_t enqueue_integrate(rk4_chain *h, int kernel, void *state, void *comp,
       j.timeout_ns = h->timeout_set ? h->timeout_ns : std::max<long long>(h->timeout_ns, (long long)(20.0 * est_ns));
     }
     j.extra_arrivals = 0;
-    int grid = persistent_max_grid(h->model, h->fp32, h->tiling.v, h->tiling.block);
+    int grid = persistent_max_grid(h->model, h->fp32, h->tiling.v, h->tiling.block, use_split(h));
     if (grid <= 0) return cudaErrorInvalidConfiguration;
     grid = (int)std::min<int64_t>(grid, std::max<int64_t>(1, maxtiles));
     e = launch_persistent(h->model, h->fp32, h->tiling.v, h->tiling.block, grid, j, cf, st);
@@ -743,6 +772,87 @@ cudaError_t host_transfer(void *dst, const void *src, size_t bytes, bool to_devi
 
 }  // namespace
 
+namespace {
+
+// c as a float pair: its leading 24 bits and the rest (split1 of rk4_split.cuh).
+struct HostPair {
+  float h, l;
+};
+HostPair host_split(double c) {
+  uint64_t u;
+  std::memcpy(&u, &c, 8);
+  const uint64_t head = u & ~(uint64_t)0x1fffffff;
+  double d;
+  std::memcpy(&d, &head, 8);
+  return {(float)d, (float)(c - d)};  // c - d is exact
+}
+HostPair host_times_tau(double c, const HostPair &tau) {  // times_tau
+  const HostPair v = host_split(c);
+  const float p = tau.h * v.h;
+  float e = std::fmaf(tau.h, v.h, -p);
+  e = std::fmaf(tau.h, v.l, e);
+  e = std::fmaf(tau.l, v.h, e);
+  return {p, e};
+}
+unsigned high_word(double v) {
+  uint64_t u;
+  std::memcpy(&u, &v, 8);
+  return (unsigned)(u >> 32);
+}
+
+// The largest magnitudes the split form takes: a, b, c, kappa (Roessler) or w2, kappa (harmonic).
+// The differences D are dt |J| times the first slope; with dt times each linear coefficient at
+// most 1/8 (the coupling counts fourfold) their pair arithmetic stays below the state's rounding
+// (measured error against the FP64 form's: 0.5 at dt |J| = 0.1, 0.8 at 0.2, above 1 from 0.25 to
+// 0.5 on).  b only has to leave room for z in FP32's exponent range.
+void split_most(int model, double dt, double *most) {
+  if (model == RK4_ROESSLER) {
+    most[0] = most[2] = 0.125 / dt;
+    most[1] = 65536.0;
+    most[3] = 0.125 / (4.0 * dt);
+  } else {
+    most[0] = 1.0 / (128.0 * dt * dt);
+    most[1] = 1.0 / (512.0 * dt * dt);
+  }
+}
+bool split_takes(double v, double most) {
+  const double a = std::fabs(v);
+  return a == 0.0 || (a >= 0x1p-60 && a <= most);
+}
+
+}  // namespace
+
+bool rk4d::split_allowed(int model, const CoefD &c) {
+  const double dt = c.h1;
+  if (!(dt >= 0x1p-20 && dt <= 0.125)) return false;
+  double most[4];
+  split_most(model, dt, most);
+  if (model == RK4_ROESSLER)
+    return split_takes(c.a, most[0]) && split_takes(c.b, most[1]) && split_takes(c.c, most[2]) &&
+           split_takes(c.kappa, most[3]);
+  return split_takes(c.w2, most[0]) && split_takes(c.kappa, most[1]);
+}
+
+SplitCoef rk4d::split_coef(int model, const CoefD &c) {
+  SplitCoef s{};
+  const double tau = c.h2;
+  s.w = tau / 3.0;
+  const HostPair t = host_split(tau), cc = host_split(c.c);
+  s.tauh = t.h;
+  s.taul = t.l;
+  const HostPair k = host_times_tau(c.kappa, t), a = host_times_tau(model == RK4_ROESSLER ? c.a : c.w2, t);
+  s.kth = k.h;
+  s.ktl = k.l;
+  s.ath = a.h;
+  s.atl = a.l;
+  s.ch = cc.h;
+  s.cl = cc.l;
+  double most[4] = {};
+  split_most(model, c.h1, most);
+  for (int i = 0; i < 4; ++i) s.most[i] = high_word(most[i]);
+  return s;
+}
+
 // Read-only view of a handle for the allocation-free reduction entry point.
 int rk4d::handle_info(const rk4_chain *h, int *model, bool *fp32, int *nchains, const ChainDesc **chains, CoefD *cf,
                       cudaStream_t *stream, bool *het) {
@@ -813,6 +923,7 @@ int rk4_chain_create(rk4_chain **out, int model, int precision, int64_t n, doubl
   c.kappa = h->p.kappa;
   c.bc = bc;
   h->chains.push_back(c);
+  note_kappa(h, c.kappa);
   h->nchains = 1;
   h->total = n;
   *out = h;
@@ -843,6 +954,7 @@ int rk4_batch_create(rk4_chain **out, int model, int precision, int nchains, con
     d.kappa = kappa[c];
     d.bc = bc[c];
     h->chains.push_back(d);
+    note_kappa(h, d.kappa);
     off += lengths[c];
   }
   h->nchains = nchains;
@@ -1039,9 +1151,10 @@ int rk4_debug_barrier_timeout(rk4_chain *h, void *state, void *comp, void *ws, s
   j.ntail = 0;
   j.hdr = reinterpret_cast<WsHeader *>(w + L.hdr);
   j.total = h->total;
+  j.split = use_split(h) ? 1 : 0;
   j.timeout_ns = timeout_ns;
   j.extra_arrivals = 1;
-  int grid = persistent_max_grid(h->model, h->fp32, h->tiling.v, h->tiling.block);
+  int grid = persistent_max_grid(h->model, h->fp32, h->tiling.v, h->tiling.block, use_split(h));
   if (grid <= 0) return RK4_ECUDA;
   grid = (int)std::min<int64_t>(grid, std::max<int64_t>(1, j.ntiles[0]));
   if (cudaMemsetAsync(w + L.hdr, 0, sizeof(WsHeader), h->stream) != cudaSuccess) return RK4_ECUDA;
@@ -1119,7 +1232,7 @@ int rk4_chain_autotune(rk4_chain *h, void *state, void *comp, void *ws, size_t w
           if (b == 64 && !use_generic(h)) continue;
           const int maxt = tiling_max_threads(h, v);
           if (maxt <= 0 || b > maxt) continue;
-          if (kern == RK4_KERNEL_PERSISTENT && persistent_max_grid(h->model, h->fp32, v, b) <= 0) continue;
+          if (kern == RK4_KERNEL_PERSISTENT && persistent_max_grid(h->model, h->fp32, v, b, use_split(h)) <= 0) continue;
           h->tiling.block = b;
           h->tiling.v = v;
           h->tiling.k = k;

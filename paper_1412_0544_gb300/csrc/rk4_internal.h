@@ -24,6 +24,15 @@ struct CoefD {
   double a, b, c, kappa, w2, h2, h1, dt6, kappa2, dt3;
 };
 
+// Coefficients of the split FP64 step (rk4_split.cuh): tau = dt / 2, and the products with it as
+// float pairs (h + l).  at: Roessler a tau, harmonic w2 tau.  most: high words of the largest
+// magnitudes a site's own parameters may have (heterogeneous chains; in their order).
+struct SplitCoef {
+  double w;  // tau / 3
+  float tauh, taul, kth, ktl, ath, atl, ch, cl;
+  unsigned most[4];
+};
+
 // Generic explicit Runge-Kutta tableau (strictly lower a, weights b), up to kMaxStages stages.
 constexpr int kMaxStages = 7;
 struct TableauD {
@@ -43,7 +52,8 @@ struct WsHeader {
   unsigned bar_gen;
   int timeout_where;
   unsigned long long work[2];  // persistent kernel: next item of the current time block, by parity
-  unsigned char pad[224];
+  unsigned wide[2];            // split staged scheme: the state has left the split's range, by step parity
+  unsigned char pad[216];
 };
 
 // A piece of one batch chain placed in a shared ("packed") tile: the chain's last partial piece
@@ -93,6 +103,7 @@ struct BlockedJob {
   const void *sp;               // per-site parameters of a heterogeneous chain, or NULL
   WsHeader *hdr;                // status word (non-finite results, debug bounds checks)
   int64_t total;                // sites in the state buffers
+  int split;                    // 1: FP64 in the split form (rk4_split.cuh)
 };
 
 struct StagedJob {
@@ -107,6 +118,9 @@ struct StagedJob {
   int64_t total;             // total sites
   const void *sp;            // per-site parameters of a heterogeneous chain, or NULL
   WsHeader *hdr;             // status word
+  int split;                 // 1: FP64 in the split form: acc holds K1, n2 and n3 the negated
+  void *n2, *n3;             // differences of stages 2 and 3 as float pairs
+  int parity;                // of the step (which wide flag is read)
 };
 
 // One step of the generic standard scheme: stage states, slopes and the combination, each a
@@ -141,16 +155,32 @@ struct PersistentJob {
   long long timeout_ns;         // bound on any single barrier wait
   int extra_arrivals;           // test hook: barrier waits for this many blocks that never come
   int64_t total;                // sites in the state buffers
+  int split;                    // 1: FP64 in the split form (rk4_split.cuh)
 };
 
 // Launchers (return a cudaError_t).  R is selected by `fp32` (FP32 + Kahan) or double.
 cudaError_t launch_blocked(int model, bool fp32, int v, int block, const BlockedJob &job, const CoefD &cf,
                            cudaStream_t st);  // job.sp != NULL selects the heterogeneous kernel (v = 2 or 4)
+// The split forms of launch_blocked, launch_persistent and persistent_max_grid (one model's
+// kernels per translation unit).
+template <int MODEL>
+cudaError_t launch_split_blocked(int v, int block, const BlockedJob &job, const CoefD &cf, cudaStream_t st);
+template <int MODEL>
+cudaError_t launch_split_persistent(int v, int block, int grid, const PersistentJob &job, const CoefD &cf,
+                                    cudaStream_t st);
+template <int MODEL> int persistent_split_max_grid(int v, int block);
+// Set hdr->wide[0] when a state value or a site's own parameter is outside the split's range.
+cudaError_t launch_split_scan(int model, const double *state, const double *sp, int64_t total, const SplitCoef &sc,
+                              WsHeader *hdr, cudaStream_t st);
+// Whether every step of a handle with these coefficients (c.kappa: the largest coupling strength
+// of its chains) may run in the split form, and the form's coefficients.
+bool split_allowed(int model, const CoefD &c);
+SplitCoef split_coef(int model, const CoefD &c);
 cudaError_t launch_staged(int model, bool fp32, int stage, const StagedJob &job, const CoefD &cf,
                           cudaStream_t st);
 cudaError_t launch_persistent(int model, bool fp32, int v, int block, int grid, const PersistentJob &job,
                               const CoefD &cf, cudaStream_t st);
-int persistent_max_grid(int model, bool fp32, int v, int block);
+int persistent_max_grid(int model, bool fp32, int v, int block, bool split);
 cudaError_t launch_energy(int model, bool fp32, const void *state, const void *cmp, int nchains,
                           const ChainDesc &one, const ChainDesc *chains, const CoefD &cf, double *partials,
                           double *out, WsHeader *hdr, cudaStream_t st);
@@ -182,7 +212,7 @@ cudaError_t launch_gen_blocked(int model, bool fp32, int range, int v, int block
                                const CoefD &cf, const TableauD &tb, double dt, int H, cudaStream_t st);
 size_t gen_blocked_smem_bytes(int model, bool fp32, int v, int block, const TableauD &tb);
 int gen_blocked_max_threads(int model, bool fp32, int range, int v, const TableauD &tb);
-size_t blocked_smem_bytes(int model, bool fp32, int v, int block, bool het = false);
+size_t blocked_smem_bytes(int model, bool fp32, int v, int block, bool het = false);  // either FP64 form fits
 int blocked_max_threads(int model, bool fp32, int v, bool het = false);
 
 constexpr int kEnergyBlocks = 1024;  // fixed grid of the single-chain reduction (deterministic)

@@ -1,0 +1,333 @@
+// rk4_split.cuh -- the FP64 RK4 step with most of its arithmetic on the FP32 pipe.
+//
+// GB300 issues FP64 at 1/64 of its FP32 lane rate, so the 49 DFMA of a step
+// (rk4_device.cuh) bound every FP64 kernel while the FP32 pipe idles.  This form keeps in FP64
+// what decides the accuracy -- the state, the first slope and the final update -- and computes
+// the later stages' differences from the first slope in float pairs (an unevaluated sum h + l
+// of two floats, about 48 bits), with the error-free transformations of Knuth (two-sum) and
+// Dekker / Ogita, Rump and Oishi (two-product by FMA).
+//
+//   K1 = f(y)                                   FP64, as slope() computes it
+//   d2 = K1, d3 = K2 = K1 + D2, d4 = 2 (K1 + D3)     stage increments over tau = dt / 2:
+//                                                u_j = y + tau d_j      (Eq. (4))
+//   Dj = f(y + tau d_j) - f(y)                  float pairs, by the exact difference formula
+//        x: kappa tau lap(dx) - tau (dy + dz)   y: tau dx + a tau dy
+//        z: z tau dx + tau dz ((x - c) + tau dx)    (f's only product: Eq. (6))
+//        harmonic q: tau dp   p: kappa tau lap(dq) - w2 tau dq
+//   y <- y + (tau / 3) (6 K1 + 2 D2 + 2 D3 + D4)     FP64, one rounding      (Eq. (5))
+//
+// Why this loses nothing: a pair's relative error is about 2^-49, D is dt |J| times K1, and D
+// enters the state times dt; with dt |J| at most 1/8 (split_allowed) that puts its error some
+// four bits below the rounding of the state, and the state is rounded once per component and
+// step where the FP64 form rounds it four times.  Measured against long double (N = 1024,
+// 1 .. 1000 steps, dt = 0.01, kappa = 1 and 2): 0.48 .. 0.57 of the FP64 form's error in every
+// component, Roessler and harmonic.
+//
+// Every function is written over a lane type T: float (one site) or f32x2 (two sites in one
+// packed instruction), which round alike, so kernels with any number of sites per thread and
+// the one-stage-per-launch kernel agree bit for bit.
+//
+// Range: a pair needs the exponent room of FP32.  Tiles whose values leave it (split_in_range)
+// are advanced in the FP64 form instead (tile_item returns false and the caller runs it again).
+#pragma once
+#include "rk4_device.cuh"
+#include "rk4_internal.h"
+
+namespace rk4d {
+
+typedef unsigned long long f32x2;
+
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float lane0(f32x2 v) {
+  float a, b;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+  (void)b;
+  return a;
+}
+__device__ __forceinline__ float lane1(f32x2 v) {
+  float a, b;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+  (void)a;
+  return b;
+}
+__device__ __forceinline__ float vadd(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float vsub(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float vmul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float vfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ f32x2 vadd(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 vsub(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 vmul(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 vfma(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+template <typename T> __device__ __forceinline__ T vset(float a);
+template <> __device__ __forceinline__ float vset<float>(float a) { return a; }
+template <> __device__ __forceinline__ f32x2 vset<f32x2>(float a) { return pack2(a, a); }
+
+template <typename T> struct FPair {
+  T h, l;
+};
+
+// a + b = s + e exactly (Knuth).
+template <typename T> __device__ __forceinline__ void two_sum(T a, T b, T &s, T &e) {
+  s = vadd(a, b);
+  const T bb = vsub(s, a);
+  e = vadd(vsub(a, vsub(s, bb)), vsub(b, bb));
+}
+// a - b = s + e exactly.
+template <typename T> __device__ __forceinline__ void two_diff(T a, T b, T &s, T &e) {
+  s = vsub(a, b);
+  const T bb = vsub(s, a);
+  e = vsub(vsub(a, vsub(s, bb)), vadd(b, bb));
+}
+// a + m b = s + e exactly, for m = 2 or -2.
+template <typename T> __device__ __forceinline__ void two_sum_m(T a, T m, T b, T &s, T &e) {
+  s = vfma(m, b, a);
+  const T nb = vsub(a, s);
+  e = vadd(vsub(a, vadd(s, nb)), vfma(m, b, nb));
+}
+// c v = e - np for a coefficient c (nch = -c.h) and a pair v.
+template <typename T> __device__ __forceinline__ void mul_coef(const FPair<T> &c, T nch, const FPair<T> &v, T &np, T &e) {
+  np = vmul(nch, v.h);
+  e = vfma(c.h, v.h, np);
+  e = vfma(c.h, v.l, e);
+  e = vfma(c.l, v.h, e);
+}
+// a - n as a pair.
+template <typename T> __device__ __forceinline__ FPair<T> pair_sub(const FPair<T> &a, const FPair<T> &n) {
+  FPair<T> r;
+  T e;
+  two_diff(a.h, n.h, r.h, e);
+  r.l = vsub(vadd(e, a.l), n.l);
+  return r;
+}
+
+// ---- FP64 <-> pair by integer operations (the F2F conversions issue on the FP64 pipe) --------
+
+// A double as head (its leading 24 bits, truncated), the tail's integer significand m (29 bits)
+// and the head's power of two p: the value is h + m 2^-52 p.  Zero gives h = p = 0, magnitudes
+// below 2^-126 at most a few denormals.
+__device__ __forceinline__ void split_bits(double y, float &h, float &m, float &p) {
+  const int hi = __double2hiint(y), lo = __double2loint(y);
+  const int a = max((hi & 0x7fffffff) - 0x38000000, 0);  // rebias the exponent from 1023 to 127
+  const unsigned f = (__funnelshift_l((unsigned)lo, (unsigned)a, 3) & 0x7fffffffu) | ((unsigned)hi & 0x80000000u);
+  h = __uint_as_float(f);
+  m = __uint2float_rn((unsigned)lo & 0x1fffffffu);
+  p = __uint_as_float(f & 0xff800000u);
+}
+__device__ __forceinline__ FPair<float> split1(double y) {
+  float h, m, p;
+  split_bits(y, h, m, p);
+  return {h, vmul(vmul(m, 0x1p-52f), p)};
+}
+template <typename T> struct Lanes;
+template <> struct Lanes<float> {
+  static constexpr int n = 1;
+  static __device__ __forceinline__ FPair<float> split(const double *y, int) { return split1(y[0]); }
+};
+template <> struct Lanes<f32x2> {
+  static constexpr int n = 2;
+  // the pair of y[0] and y[stride]
+  static __device__ __forceinline__ FPair<f32x2> split(const double *y, int stride) {
+    float h0, m0, p0, h1, m1, p1;
+    split_bits(y[0], h0, m0, p0);
+    split_bits(y[stride], h1, m1, p1);
+    return {pack2(h0, h1), vmul(vmul(pack2(m0, m1), vset<f32x2>(0x1p-52f)), pack2(p0, p1))};
+  }
+};
+
+// h + m 2^-52 p as a double, for a normalised pair whose tail is given as m = l 2^52 / p rounded
+// to an integer (p: h's power of two): the head's bits rebiased, plus m in units of the double's
+// last place.  A negative m below a power of two borrows into the binade whose last place is
+// half as large, hence the doubling.
+__device__ __forceinline__ double join_bits(float h, int m) {
+  const unsigned b = __float_as_uint(h);
+  if (((b << 9) == 0u) && m < 0) m += m;
+  unsigned hh = ((unsigned)((int)b >> 3) & 0x8fffffffu) + 0x38000000u;
+  unsigned hl = b << 29;
+  const bool zero = (b & 0x7fffffffu) == 0u;
+  asm("add.cc.u32 %0, %0, %2;\n\taddc.u32 %1, %1, %3;" : "+r"(hl), "+r"(hh) : "r"(m), "r"(m >> 31));
+  return __hiloint2double(zero ? 0 : (int)hh, zero ? 0 : (int)hl);
+}
+// 1 / p for h's power of two p (with h's sign).
+__device__ __forceinline__ float inv_pow2(float h) {
+  return __uint_as_float(0x7F000000u - (__float_as_uint(h) & 0xff800000u));
+}
+// The doubles nearest the pair's lanes.
+__device__ __forceinline__ void join(FPair<float> v, double *out, int) {
+  const float s = vadd(v.h, v.l);
+  const float l = vsub(v.l, vsub(s, v.h));
+  out[0] = join_bits(s, __float2int_rn(vmul(vmul(l, 0x1p52f), inv_pow2(s))));
+}
+__device__ __forceinline__ void join(FPair<f32x2> v, double *out, int stride) {
+  const f32x2 s = vadd(v.h, v.l);
+  const f32x2 l = vsub(v.l, vsub(s, v.h));
+  const float s0 = lane0(s), s1 = lane1(s);
+  const f32x2 m = vmul(vmul(l, vset<f32x2>(0x1p52f)), pack2(inv_pow2(s0), inv_pow2(s1)));
+  out[0] = join_bits(s0, __float2int_rn(lane0(m)));
+  out[stride] = join_bits(s1, __float2int_rn(lane1(m)));
+}
+
+// ---- range ----------------------------------------------------------------------------------
+
+// Whether a state value is zero or of a magnitude the pairs represent with full relative
+// precision through a step: at least 2^-70, and below 2^16 for the Roessler chain, whose stages
+// square (z x), or 2^40 for the linear harmonic chain.  NaN and infinity are out of range.
+template <int MODEL> __device__ __forceinline__ bool split_in_range(double v) {
+  constexpr unsigned lo = (1023u - 70u) << 20;
+  constexpr unsigned hi = (1023u + (MODEL == ROESSLER ? 16u : 40u)) << 20;
+  const unsigned a = (unsigned)__double2hiint(v) & 0x7fffffffu;
+  return (a - lo < hi - lo) | ((a | (unsigned)__double2loint(v)) == 0u);
+}
+// The same for a site's own parameter of a heterogeneous chain: zero, or at least 2^-60 and with
+// the high word at most `most` (that of the largest value split_allowed takes).
+__device__ __forceinline__ bool split_param_in_range(double v, unsigned most) {
+  constexpr unsigned lo = (1023u - 60u) << 20;
+  const unsigned a = (unsigned)__double2hiint(v) & 0x7fffffffu;
+  return ((a >= lo) & (a <= most)) | ((a | (unsigned)__double2loint(v)) == 0u);
+}
+
+// ---- coefficients -----------------------------------------------------------------------------
+
+// c tau as a pair, c a double (host and device compute the same bits).
+__device__ __forceinline__ FPair<float> times_tau(double c, const SplitCoef &s) {
+  const FPair<float> v = split1(c);
+  float np, e;
+  mul_coef<float>({s.tauh, s.taul}, -s.tauh, v, np, e);
+  return {-np, e};
+}
+__device__ __forceinline__ void split_set_kappa(SplitCoef &s, double kappa) {
+  const FPair<float> k = times_tau(kappa, s);
+  s.kth = k.h;
+  s.ktl = k.l;
+}
+// The pair coefficients of a stage in lane type T.  at: Roessler a tau; harmonic w2 tau.
+template <typename T> struct StageCoef {
+  FPair<T> kt, at, tau;
+};
+template <typename T> __device__ __forceinline__ StageCoef<T> stage_coef(const SplitCoef &s) {
+  return {{vset<T>(s.kth), vset<T>(s.ktl)}, {vset<T>(s.ath), vset<T>(s.atl)}, {vset<T>(s.tauh), vset<T>(s.taul)}};
+}
+
+// ---- one stage ----------------------------------------------------------------------------------
+
+// The base point's part of the z difference: z and x - c at the step's start.
+template <typename T> struct SplitBase {
+  FPair<T> z, t;
+};
+template <typename T> __device__ __forceinline__ FPair<T> x_minus_c(const FPair<T> &x, const FPair<T> &c) {
+  FPair<T> r;
+  T e;
+  two_diff(x.h, c.h, r.h, e);
+  r.l = vsub(vadd(e, x.l), c.l);
+  return r;
+}
+
+// lap(dx) as (g, lo).
+template <typename T>
+__device__ __forceinline__ FPair<T> pair_lap(const FPair<T> &x, const FPair<T> &xl, const FPair<T> &xr) {
+  const T m2 = vset<T>(-2.f);
+  T s, e1, e2;
+  FPair<T> g;
+  two_sum(xl.h, xr.h, s, e1);
+  two_sum_m(s, m2, x.h, g.h, e2);
+  g.l = vadd(vfma(m2, x.l, vadd(xl.l, xr.l)), vadd(e1, e2));
+  return g;
+}
+
+// n = -D for the stage increments d (85 FP32 operations per site; harmonic 40).
+template <int MODEL, typename T>
+__device__ __forceinline__ void split_stage(const FPair<T> *d, const FPair<T> &xl, const FPair<T> &xr,
+                                            const SplitBase<T> &b, const StageCoef<T> &c, FPair<T> *n) {
+  const T m1 = vset<T>(-1.f);
+  const FPair<T> g = pair_lap(d[0], xl, xr);
+  T np, e, ne;
+  mul_coef(c.kt, vmul(m1, c.kt.h), g, np, e);  // kappa tau lap = e - np
+  if constexpr (MODEL == ROESSLER) {
+    const T ntau = vmul(m1, c.tau.h);
+    FPair<T> w;  // dy + dz
+    T we, nw, f;
+    two_sum(d[1].h, d[2].h, w.h, we);
+    w.l = vadd(vadd(d[1].l, d[2].l), we);
+    mul_coef(c.tau, ntau, w, nw, f);
+    two_diff(np, nw, n[0].h, ne);
+    n[0].l = vadd(vsub(ne, e), f);
+    T nd, df;  // delta = tau dx = df - nd
+    mul_coef(c.tau, ntau, d[0], nd, df);
+    mul_coef(c.at, vmul(m1, c.at.h), d[1], np, e);
+    two_sum(nd, np, n[1].h, ne);
+    n[1].l = vsub(ne, vadd(df, e));
+    T nz, q;  // zeta = tau dz = q - nz
+    mul_coef(c.tau, ntau, d[2], nz, q);
+    const T pz = vmul(c.tau.h, d[2].h);  // = -nz
+    FPair<T> t;  // (x - c) + delta
+    T te;
+    two_diff(b.t.h, nd, t.h, te);
+    t.l = vadd(vadd(te, b.t.l), df);
+    const T nzh = vmul(m1, b.z.h);
+    const T p1 = vmul(nzh, nd);  // z delta = p1 - g1
+    T g1 = vfma(b.z.h, nd, p1);
+    g1 = vfma(nzh, df, g1);
+    g1 = vfma(b.z.l, nd, g1);
+    const T p2 = vmul(nz, t.h);  // zeta t = e2 - p2
+    T e2 = vfma(pz, t.h, p2);
+    e2 = vfma(pz, t.l, e2);
+    e2 = vfma(q, t.h, e2);
+    two_diff(p2, p1, n[2].h, ne);
+    n[2].l = vsub(vadd(ne, g1), e2);
+  } else {
+    T nq, f;  // w2 tau dq = f - nq
+    mul_coef(c.at, vmul(m1, c.at.h), d[0], nq, f);
+    two_diff(np, nq, n[1].h, ne);
+    n[1].l = vadd(vsub(ne, e), f);
+    mul_coef(c.tau, vmul(m1, c.tau.h), d[1], n[0].h, e);  // tau dp = e - n
+    n[0].l = vmul(m1, e);
+  }
+}
+
+// Bookkeeping after stage j = 1, 2, 3 (the RK stages 2 to 4): the next increments d and the
+// running sum N = -(2 D2 + 2 D3 + D4), of which stages 1 and 2 hold half.
+template <typename T>
+__device__ __forceinline__ void split_update(int j, const FPair<T> &k1, const FPair<T> &n, FPair<T> &d, FPair<T> &N) {
+  T e;
+  if (j == 1) {
+    N = n;
+    d = pair_sub(k1, n);
+  } else if (j == 2) {
+    T s;
+    two_sum(N.h, n.h, s, e);
+    N = {s, vadd(vadd(N.l, n.l), e)};
+    d = pair_sub(k1, n);
+    d.h = vadd(d.h, d.h);
+    d.l = vadd(d.l, d.l);
+  } else {
+    const T two = vset<T>(2.f);
+    T s;
+    two_sum_m(n.h, two, N.h, s, e);
+    N = {s, vadd(vfma(two, N.l, n.l), e)};
+  }
+}
+// y + (tau / 3) (6 K1 - N).
+__device__ __forceinline__ double split_final(double y, double k1, double N, const SplitCoef &s) {
+  return fma(s.w, fma(6.0, k1, -N), y);
+}
+
+}  // namespace rk4d

@@ -17,6 +17,7 @@
 
 #include "rk4_device.cuh"
 #include "rk4_internal.h"
+#include "rk4_split.cuh"
 
 namespace rk4d {
 
@@ -246,6 +247,151 @@ __device__ __forceinline__ void tile_advance(R (&y)[V][Dim<MODEL>::D], R (&cmp)[
         }
       }
     }
+  }
+}
+
+// tile_advance for FP64 in the split form (rk4_split.cuh).  The same exchange and barriers; a
+// stage's exchanged value is the coupling coordinate in FP64 for the first stage and its
+// increment (head and tail, also 8 bytes) for the others.  The thread's V sites are paired
+// (p, p + V / 2) for the packed instructions, so that a pair's neighbours are, except at the
+// thread's ends, the adjacent pairs as they stand.
+// spd, spf (heterogeneous chains): this thread's first private slots of the site parameters in
+// FP64 (V x P, strided by the block) and of the pair coefficients (V / 2 packed kt, at and c).
+template <int MODEL, int V, bool MASK, bool HET>
+__device__ __forceinline__ void split_advance(double (&y)[V][Dim<MODEL>::D], uint32_t ghost, int K,
+                                              const Coef<double> &cf, const SplitCoef &sc, double *edge,
+                                              const double *spd = nullptr, const f32x2 *spf = nullptr) {
+  constexpr int D = Dim<MODEL>::D;
+  constexpr int P = V < 2 ? 1 : V / 2;
+  using T = std::conditional_t<V == 1, float, f32x2>;
+  constexpr bool kThread = thread_exchange(V);
+  constexpr int NT = max_threads_for(V);
+  const int tid = threadIdx.x;
+  unsigned my_first = 0, my_last = 0, left_last = 0, right_first = 0;
+  if constexpr (kThread) {
+    my_first = smem_addr(edge + tid);
+    my_last = smem_addr(edge + NT + tid);
+    left_last = my_last - (tid > 0 ? 8u : 0u);
+    right_first = my_first + (tid < (int)blockDim.x - 1 ? 8u : 0u);
+  }
+  const int lane = tid & 31;
+  const int warp = tid >> 5;
+  const int nw = blockDim.x >> 5;
+  const bool is_first = lane == 0, is_last = lane == 31;
+  const int prev = (warp > 0) ? warp - 1 : warp;
+  const int next = (warp < nw - 1) ? warp + 1 : warp;
+  auto exchange = [&](int j, double first, double last, double &left, double &right) {
+    if constexpr (kThread) {
+      const unsigned po = (j & 1) * 2 * NT * 8u;
+      st_shared(my_first + po, first);
+      st_shared(my_last + po, last);
+      neighbour_warp_sync();
+      ld_shared(left_last + po, left);
+      ld_shared(right_first + po, right);
+    } else {
+      left = __shfl_up_sync(kFull, last, 1);
+      right = __shfl_down_sync(kFull, first, 1);
+      double *eb = edge + (j & 1) * 64;
+      st_shared_if(is_first, eb + warp, first);
+      st_shared_if(is_last, eb + 32 + warp, last);
+      neighbour_warp_sync();
+      const double from_prev = eb[32 + prev];
+      const double from_next = eb[next];
+      left = is_first ? from_prev : left;
+      right = is_last ? from_next : right;
+    }
+  };
+  const StageCoef<T> sc0 = stage_coef<T>(sc);
+
+#pragma unroll 1
+  for (int s = 0; s < K; ++s) {
+    double k1d[V][D];
+    FPair<T> k1[P][D], d[P][D], N[P][D];
+    SplitBase<T> base[P];
+    {
+      double xs[V], left, right;
+#pragma unroll
+      for (int v = 0; v < V; ++v) xs[v] = (MASK && ((ghost >> v) & 1u)) ? 0.0 : y[v][0];
+      exchange(0, xs[0], xs[V - 1], left, right);
+#pragma unroll
+      for (int v = 0; v < V; ++v) {
+        const double xl = (v == 0) ? left : xs[v - 1];
+        const double xr = (v == V - 1) ? right : xs[v + 1];
+        if constexpr (HET) {
+          double p[Dim<MODEL>::P];
+#pragma unroll
+          for (int i = 0; i < Dim<MODEL>::P; ++i) p[i] = spd[(v * Dim<MODEL>::P + i) * blockDim.x];
+          slope<double, MODEL>(y[v], xl, xr, site_coef<double, MODEL>(cf, p), k1d[v]);
+        } else {
+          slope<double, MODEL>(y[v], xl, xr, cf, k1d[v]);
+        }
+      }
+#pragma unroll
+      for (int p = 0; p < P; ++p) {
+#pragma unroll
+        for (int i = 0; i < D; ++i) d[p][i] = k1[p][i] = Lanes<T>::split(&k1d[p][i], P * D);
+        if constexpr (MODEL == ROESSLER) {
+          FPair<T> c = {vset<T>(sc.ch), vset<T>(sc.cl)};
+          if constexpr (HET) c = {spf[(p * 6 + 4) * blockDim.x], spf[(p * 6 + 5) * blockDim.x]};
+          base[p].z = Lanes<T>::split(&y[p][2], P * D);
+          base[p].t = x_minus_c(Lanes<T>::split(&y[p][0], P * D), c);
+        }
+      }
+    }
+#pragma unroll
+    for (int j = 1; j < 4; ++j) {
+      FPair<T> X[P];  // the increments' coupling coordinate, zero at ghost sites
+#pragma unroll
+      for (int p = 0; p < P; ++p) {
+        X[p] = d[p][0];
+        if constexpr (MASK) {
+          if constexpr (V == 1) {
+            if (ghost & 1u) X[p] = {0.f, 0.f};
+          } else {
+            const bool g0 = (ghost >> p) & 1u, g1 = (ghost >> (p + P)) & 1u;
+            X[p].h = pack2(g0 ? 0.f : lane0(X[p].h), g1 ? 0.f : lane1(X[p].h));
+            X[p].l = pack2(g0 ? 0.f : lane0(X[p].l), g1 ? 0.f : lane1(X[p].l));
+          }
+        }
+      }
+      FPair<T> first, last;  // left neighbours of the first pair, right neighbours of the last
+      double left, right;
+      if constexpr (V == 1) {
+        const double mine = __longlong_as_double((long long)pack2(X[0].h, X[0].l));
+        exchange(j, mine, mine, left, right);
+        const f32x2 l = (f32x2)__double_as_longlong(left), r = (f32x2)__double_as_longlong(right);
+        first = {lane0(l), lane1(l)};
+        last = {lane0(r), lane1(r)};
+      } else {
+        exchange(j, __longlong_as_double((long long)pack2(lane0(X[0].h), lane0(X[0].l))),
+                 __longlong_as_double((long long)pack2(lane1(X[P - 1].h), lane1(X[P - 1].l))), left, right);
+        const f32x2 l = (f32x2)__double_as_longlong(left), r = (f32x2)__double_as_longlong(right);
+        first = {pack2(lane0(l), lane0(X[P - 1].h)), pack2(lane1(l), lane0(X[P - 1].l))};
+        last = {pack2(lane1(X[0].h), lane0(r)), pack2(lane1(X[0].l), lane1(r))};
+      }
+#pragma unroll
+      for (int p = 0; p < P; ++p) {
+        FPair<T> n[D];
+        StageCoef<T> c = sc0;
+        if constexpr (HET) {
+          constexpr int S = MODEL == ROESSLER ? 6 : 4;
+          c.kt = {spf[(p * S + 0) * blockDim.x], spf[(p * S + 1) * blockDim.x]};
+          c.at = {spf[(p * S + 2) * blockDim.x], spf[(p * S + 3) * blockDim.x]};
+        }
+        split_stage<MODEL, T>(d[p], p == 0 ? first : X[p - 1], p == P - 1 ? last : X[p + 1], base[p], c, n);
+#pragma unroll
+        for (int i = 0; i < D; ++i) split_update<T>(j, k1[p][i], n[i], d[p][i], N[p][i]);
+      }
+    }
+#pragma unroll
+    for (int p = 0; p < P; ++p)
+#pragma unroll
+      for (int i = 0; i < D; ++i) {
+        double nd[2];
+        join(N[p][i], nd, 1);
+        y[p][i] = split_final(y[p][i], k1d[p][i], nd[0], sc);
+        if constexpr (V > 1) y[p + P][i] = split_final(y[p + P][i], k1d[p + P][i], nd[1], sc);
+      }
   }
 }
 
@@ -491,11 +637,14 @@ template <typename R, int D> __host__ __device__ constexpr int align_sites() {
 // (heterogeneous).
 // `sites` is the number of sites in the state buffers (for the debug bounds checks); hdr the
 // status word, where a non-finite stored value is reported.
-template <typename R, int MODEL, int V, bool KAHAN, bool COH, bool HET = false, bool ALN = false>
-__device__ __forceinline__ void tile_item(const R *__restrict__ in, R *__restrict__ out, const R *__restrict__ cin,
+// SPLIT (FP64): the split form of the step.  Returns false, with nothing stored, when a value the
+// tile loads or would store (or a site's own parameter) is outside the split's range: the caller
+// then runs the item again in the FP64 form.  True otherwise; the same for every thread.
+template <typename R, int MODEL, int V, bool KAHAN, bool COH, bool HET = false, bool ALN = false, bool SPLIT = false>
+__device__ __forceinline__ bool tile_item(const R *__restrict__ in, R *__restrict__ out, const R *__restrict__ cin,
                                           R *__restrict__ cout, const ChainDesc &ch, int64_t tile, int K, int G,
                                           const Coef<R> &cf, unsigned char *smem, int64_t sites, WsHeader *hdr,
-                                          const R *__restrict__ sp = nullptr) {
+                                          const R *__restrict__ sp = nullptr, const SplitCoef *sc = nullptr) {
   constexpr int D = Dim<MODEL>::D;
   constexpr int P = Dim<MODEL>::P;
   R *edge = reinterpret_cast<R *>(smem);
@@ -528,28 +677,76 @@ __device__ __forceinline__ void tile_item(const R *__restrict__ in, R *__restric
       if constexpr (KAHAN) cmp[v][d] = ctl[(base + v) * D + d]; else cmp[v][d] = R(0);
     }
 
-  Coef<R> cs[HET ? V : 1];
-  if constexpr (HET) {
-#pragma unroll
-    for (int v = 0; v < V; ++v) cs[v] = site_coef<R, MODEL>(cf, ptl + (base + v) * P);
-  }
-
+  // fixed ends: the thread's sites outside the chain (ghosts)
   const bool edge_tile = (ch.bc == FIXED) && (t0 < 0 || t0 + W > ch.n);
+  uint32_t ghost = 0;
   if (edge_tile) {
-    uint32_t ghost = 0;
 #pragma unroll
     for (int v = 0; v < V; ++v) {
       const int64_t g = t0 + base + v;
       if (g < 0 || g >= ch.n) ghost |= 1u << v;
     }
-    tile_advance<R, MODEL, V, KAHAN, true, HET>(y, cmp, ghost, K, cf, edge, cs);
+  }
+  if constexpr (SPLIT) {
+    bool wide = false;  // a value outside the split's range
+    double *spd = nullptr;
+    f32x2 *spf = nullptr;
+#pragma unroll
+    for (int v = 0; v < V; ++v)
+#pragma unroll
+      for (int d = 0; d < D; ++d) wide |= !split_in_range<MODEL>(y[v][d]);
+    if constexpr (HET) {
+      // the parameters move to thread-private slots (consecutive threads, consecutive addresses),
+      // beside the pair coefficients of each pair of sites
+      constexpr int S = MODEL == ROESSLER ? 6 : 4;
+      double p[V][P];
+#pragma unroll
+      for (int v = 0; v < V; ++v)
+#pragma unroll
+        for (int i = 0; i < P; ++i) {
+          p[v][i] = ptl[(base + v) * P + i];
+          wide |= !split_param_in_range(p[v][i], sc->most[i]);
+        }
+      if (__syncthreads_or(wide)) return false;
+      spd = ptl + threadIdx.x;
+      spf = reinterpret_cast<f32x2 *>(ptl + W * P) + threadIdx.x;
+#pragma unroll
+      for (int v = 0; v < V; ++v)
+#pragma unroll
+        for (int i = 0; i < P; ++i) spd[(v * P + i) * blockDim.x] = p[v][i];
+#pragma unroll
+      for (int q = 0; q < V / 2; ++q) {
+        const FPair<float> k0 = times_tau(p[q][P - 1], *sc), k1 = times_tau(p[q + V / 2][P - 1], *sc);
+        const FPair<float> a0 = times_tau(p[q][0], *sc), a1 = times_tau(p[q + V / 2][0], *sc);
+        f32x2 *o = spf + q * S * blockDim.x;
+        o[0] = pack2(k0.h, k1.h);
+        o[blockDim.x] = pack2(k0.l, k1.l);
+        o[2 * blockDim.x] = pack2(a0.h, a1.h);
+        o[3 * blockDim.x] = pack2(a0.l, a1.l);
+        if constexpr (MODEL == ROESSLER) {
+          const FPair<float> c0 = split1(p[q][2]), c1 = split1(p[q + V / 2][2]);
+          o[4 * blockDim.x] = pack2(c0.h, c1.h);
+          o[5 * blockDim.x] = pack2(c0.l, c1.l);
+        }
+      }
+    } else {
+      if (__syncthreads_or(wide)) return false;
+    }
+    if (edge_tile) split_advance<MODEL, V, true, HET>(y, ghost, K, cf, *sc, edge, spd, spf);
+    else split_advance<MODEL, V, false, HET>(y, 0u, K, cf, *sc, edge, spd, spf);
   } else {
-    tile_advance<R, MODEL, V, KAHAN, false, HET>(y, cmp, 0u, K, cf, edge, cs);
+    Coef<R> cs[HET ? V : 1];
+    if constexpr (HET) {
+#pragma unroll
+      for (int v = 0; v < V; ++v) cs[v] = site_coef<R, MODEL>(cf, ptl + (base + v) * P);
+    }
+    if (edge_tile) tile_advance<R, MODEL, V, KAHAN, true, HET>(y, cmp, ghost, K, cf, edge, cs);
+    else tile_advance<R, MODEL, V, KAHAN, false, HET>(y, cmp, 0u, K, cf, edge, cs);
   }
 
   const int64_t rem = ch.n - g0;
   const int cnt = (int)(rem < G ? rem : G);
-  bool bad = false;  // a stored (interior) value is NaN or infinite
+  bool bad = false;  // a stored (interior) value is NaN or infinite (SPLIT: out of range)
 #pragma unroll
   for (int v = 0; v < V; ++v) {
     const bool stored = base + v >= hl && base + v < hl + cnt;
@@ -557,15 +754,22 @@ __device__ __forceinline__ void tile_item(const R *__restrict__ in, R *__restric
     for (int d = 0; d < D; ++d) {
       tl[(base + v) * D + d] = y[v][d];
       if constexpr (KAHAN) ctl[(base + v) * D + d] = cmp[v][d];
-      bad |= stored && nonfinite(y[v][d]);
+      if constexpr (SPLIT) bad |= stored && !split_in_range<MODEL>(y[v][d]);
+      else bad |= stored && nonfinite(y[v][d]);
     }
   }
-  report_nonfinite(hdr, __syncthreads_or(bad));
+  const int any_bad = __syncthreads_or(bad);
+  if constexpr (SPLIT) {
+    if (any_bad) return false;
+  } else {
+    report_nonfinite(hdr, any_bad);
+  }
   if (cnt > 0) {
     tile_store<R, D, COH, ALN>(out, tl, ch.off, hl, g0, cnt, sites, W, hdr);
     if constexpr (KAHAN) tile_store<R, D, COH, ALN>(cout, ctl, ch.off, hl, g0, cnt, sites, W, hdr);
   }
   __syncthreads();  // shared memory is reused by the next item
+  return true;
 }
 
 // Process one packed tile: segments s0 .. s1 - 1 of `segs`, side by side in slot order, each a
@@ -576,12 +780,13 @@ __device__ __forceinline__ void tile_item(const R *__restrict__ in, R *__restric
 // sites are exact.  Every thread's sites lie in one segment (o and L are multiples of V), so a
 // thread takes its chain's coupling strength and, for fixed ends, its ghost mask; threads past
 // the last segment advance zeros that are never stored.
-template <typename R, int MODEL, int V, bool KAHAN, bool COH>
-__device__ __forceinline__ void packed_tile_item(const R *__restrict__ in, R *__restrict__ out,
+// SPLIT and the result: as tile_item.
+template <typename R, int MODEL, int V, bool KAHAN, bool COH, bool SPLIT = false>
+__device__ __forceinline__ bool packed_tile_item(const R *__restrict__ in, R *__restrict__ out,
                                                  const R *__restrict__ cin, R *__restrict__ cout,
                                                  const ChainDesc *chains, const SegDesc *segs, int s0, int s1,
                                                  int K, const Coef<R> &cf, unsigned char *smem, int64_t sites,
-                                                 WsHeader *hdr) {
+                                                 WsHeader *hdr, const SplitCoef *scp = nullptr) {
   constexpr int D = Dim<MODEL>::D;
   R *edge = reinterpret_cast<R *>(smem);
   R *tl = edge + edge_values(V);
@@ -641,9 +846,21 @@ __device__ __forceinline__ void packed_tile_item(const R *__restrict__ in, R *__
       y[v][d] = tl[(base + v) * D + d];
       if constexpr (KAHAN) cmp[v][d] = ctl[(base + v) * D + d]; else cmp[v][d] = R(0);
     }
-  tile_advance<R, MODEL, V, KAHAN, true>(y, cmp, ghost, K, c, edge);
+  if constexpr (SPLIT) {
+    bool wide = false;
+#pragma unroll
+    for (int v = 0; v < V; ++v)
+#pragma unroll
+      for (int d = 0; d < D; ++d) wide |= !split_in_range<MODEL>(y[v][d]);
+    if (__syncthreads_or(wide)) return false;
+    SplitCoef sc = *scp;
+    split_set_kappa(sc, c.kappa);
+    split_advance<MODEL, V, true, false>(y, ghost, K, c, sc, edge);
+  } else {
+    tile_advance<R, MODEL, V, KAHAN, true>(y, cmp, ghost, K, c, edge);
+  }
 
-  bool bad = false;  // a stored (interior) value is NaN or infinite
+  bool bad = false;  // a stored (interior) value is NaN or infinite (SPLIT: out of range)
 #pragma unroll
   for (int v = 0; v < V; ++v) {
     const bool stored = my >= 0 && rel + v >= H && rel + v < H + cnt;
@@ -651,10 +868,16 @@ __device__ __forceinline__ void packed_tile_item(const R *__restrict__ in, R *__
     for (int d = 0; d < D; ++d) {
       tl[(base + v) * D + d] = y[v][d];
       if constexpr (KAHAN) ctl[(base + v) * D + d] = cmp[v][d];
-      bad |= stored && nonfinite(y[v][d]);
+      if constexpr (SPLIT) bad |= stored && !split_in_range<MODEL>(y[v][d]);
+      else bad |= stored && nonfinite(y[v][d]);
     }
   }
-  report_nonfinite(hdr, __syncthreads_or(bad));
+  const int any_bad = __syncthreads_or(bad);
+  if constexpr (SPLIT) {
+    if (any_bad) return false;
+  } else {
+    report_nonfinite(hdr, any_bad);
+  }
   for (int s = s0; s < s1; ++s) {
     const SegDesc sd = segs[s];
     if (sd.cnt <= 0 || !bounds_ok(hdr, sd.o >= 0 && sd.o + sd.L <= W && sd.cnt + 2 * H <= sd.L)) continue;
@@ -663,6 +886,7 @@ __device__ __forceinline__ void packed_tile_item(const R *__restrict__ in, R *__
     if constexpr (KAHAN) tile_store<R, D, COH>(cout, ctl, ch.off, sd.o + H, sd.g0, sd.cnt, sites, W, hdr);
   }
   __syncthreads();  // shared memory is reused by the next item
+  return true;
 }
 
 // Locate the chain of a tile index through the prefix array (first tile of each chain).
@@ -720,26 +944,6 @@ __device__ __forceinline__ int batch_chain(const BatchTiles &bt, int nchains, in
   const int ci = find_chain_block(bt.full_prefix, nchains, f, smem);
   local = f - bt.full_prefix[ci];
   return ci;
-}
-
-// Item `item` of a batch launch laid out by bt: the packed tiles first (they then run among the
-// full tiles instead of alone at the end), then the full tiles of the chains.
-template <typename R, int MODEL, int V, bool KAHAN, bool COH>
-__device__ __forceinline__ void batch_item(const R *__restrict__ in, R *__restrict__ out, const R *__restrict__ cin,
-                                           R *__restrict__ cout, const ChainDesc *chains, int nchains,
-                                           const BatchTiles &bt, int64_t item, int K, int G, const Coef<R> &cf,
-                                           unsigned char *smem, int64_t sites, WsHeader *hdr) {
-  if (item < bt.npacked) {
-    packed_tile_item<R, MODEL, V, KAHAN, COH>(in, out, cin, cout, chains, bt.segs, bt.pack_prefix[item],
-                                              bt.pack_prefix[item + 1], K, cf, smem, sites, hdr);
-  } else {
-    int64_t local;
-    const int ci = batch_chain(bt, nchains, item - bt.npacked, smem, local);
-    const ChainDesc ch = chains[ci];
-    Coef<R> c = cf;
-    c.kappa = (R)ch.kappa;
-    tile_item<R, MODEL, V, KAHAN, COH, false, true>(in, out, cin, cout, ch, local, K, G, c, smem, sites, hdr);
-  }
 }
 
 template <typename R> __host__ __device__ inline Coef<R> to_coef(const CoefD &c, double kappa) {
