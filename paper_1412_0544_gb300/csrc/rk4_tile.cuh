@@ -257,10 +257,18 @@ __device__ __forceinline__ void tile_advance(R (&y)[V][Dim<MODEL>::D], R (&cmp)[
 // thread's ends, the adjacent pairs as they stand.
 // spd, spf (heterogeneous chains): this thread's first private slots of the site parameters in
 // FP64 (V x P, strided by the block) and of the pair coefficients (V / 2 packed kt, at and c).
-template <int MODEL, int V, bool MASK, bool HET>
+// PARK: what a stage does not need every moment (the state and the first slope in FP64, the
+// slope's pairs, the base values of z) lies in a record of the thread's own in shared memory,
+// rec, of split_record_words() 8-byte words -- an odd number, so that the threads of a warp reach
+// the same word of their records without bank conflicts.
+template <int MODEL, int V> __host__ __device__ constexpr int split_record_words() {
+  return (3 * V * Dim<MODEL>::D + (MODEL == ROESSLER ? 2 * V : 0)) | 1;
+}
+template <int MODEL, int V, bool MASK, bool HET, bool PARK = false>
 __device__ __forceinline__ void split_advance(double (&y)[V][Dim<MODEL>::D], uint32_t ghost, int K,
                                               const Coef<double> &cf, const SplitCoef &sc, double *edge,
-                                              const double *spd = nullptr, const f32x2 *spf = nullptr) {
+                                              const double *spd = nullptr, const f32x2 *spf = nullptr,
+                                              double *rec = nullptr) {
   constexpr int D = Dim<MODEL>::D;
   constexpr int P = V < 2 ? 1 : V / 2;
   using T = std::conditional_t<V == 1, float, f32x2>;
@@ -302,6 +310,16 @@ __device__ __forceinline__ void split_advance(double (&y)[V][Dim<MODEL>::D], uin
     }
   };
   const StageCoef<T> sc0 = stage_coef<T>(sc);
+  static_assert(!PARK || V >= 2, "records hold packed pairs");
+  double *rk = rec + V * D;                                      // first slope, FP64
+  f32x2 *rp = reinterpret_cast<f32x2 *>(rec + 2 * V * D);        // its pairs: h, l of each (p, component)
+  f32x2 *rb = reinterpret_cast<f32x2 *>(rec + 3 * V * D);        // z.h, z.l, t.h, t.l of each p
+  if constexpr (PARK) {
+#pragma unroll
+    for (int v = 0; v < V; ++v)
+#pragma unroll
+      for (int i = 0; i < D; ++i) rec[v * D + i] = y[v][i];
+  }
 
 #pragma unroll 1
   for (int s = 0; s < K; ++s) {
@@ -309,6 +327,12 @@ __device__ __forceinline__ void split_advance(double (&y)[V][Dim<MODEL>::D], uin
     FPair<T> k1[P][D], d[P][D], N[P][D];
     SplitBase<T> base[P];
     {
+      if constexpr (PARK) {
+#pragma unroll
+        for (int v = 0; v < V; ++v)
+#pragma unroll
+          for (int i = 0; i < D; ++i) y[v][i] = rec[v * D + i];
+      }
       double xs[V], left, right;
 #pragma unroll
       for (int v = 0; v < V; ++v) xs[v] = (MASK && ((ghost >> v) & 1u)) ? 0.0 : y[v][0];
@@ -335,6 +359,26 @@ __device__ __forceinline__ void split_advance(double (&y)[V][Dim<MODEL>::D], uin
           if constexpr (HET) c = {spf[(p * 6 + 4) * blockDim.x], spf[(p * 6 + 5) * blockDim.x]};
           base[p].z = Lanes<T>::split(&y[p][2], P * D);
           base[p].t = x_minus_c(Lanes<T>::split(&y[p][0], P * D), c);
+        }
+      }
+      if constexpr (PARK) {
+#pragma unroll
+        for (int v = 0; v < V; ++v)
+#pragma unroll
+          for (int i = 0; i < D; ++i) rk[v * D + i] = k1d[v][i];
+#pragma unroll
+        for (int p = 0; p < P; ++p) {
+#pragma unroll
+          for (int i = 0; i < D; ++i) {
+            rp[(p * D + i) * 2] = k1[p][i].h;
+            rp[(p * D + i) * 2 + 1] = k1[p][i].l;
+          }
+          if constexpr (MODEL == ROESSLER) {
+            rb[p * 4] = base[p].z.h;
+            rb[p * 4 + 1] = base[p].z.l;
+            rb[p * 4 + 2] = base[p].t.h;
+            rb[p * 4 + 3] = base[p].t.l;
+          }
         }
       }
     }
@@ -378,9 +422,16 @@ __device__ __forceinline__ void split_advance(double (&y)[V][Dim<MODEL>::D], uin
           c.kt = {spf[(p * S + 0) * blockDim.x], spf[(p * S + 1) * blockDim.x]};
           c.at = {spf[(p * S + 2) * blockDim.x], spf[(p * S + 3) * blockDim.x]};
         }
+        if constexpr (PARK && MODEL == ROESSLER)
+          base[p] = {{rb[p * 4], rb[p * 4 + 1]}, {rb[p * 4 + 2], rb[p * 4 + 3]}};
         split_stage<MODEL, T>(d[p], p == 0 ? first : X[p - 1], p == P - 1 ? last : X[p + 1], base[p], c, n);
 #pragma unroll
-        for (int i = 0; i < D; ++i) split_update<T>(j, k1[p][i], n[i], d[p][i], N[p][i]);
+        for (int i = 0; i < D; ++i) {
+          if constexpr (PARK) {
+            if (j < 3) k1[p][i] = {rp[(p * D + i) * 2], rp[(p * D + i) * 2 + 1]};
+          }
+          split_update<T>(j, k1[p][i], n[i], d[p][i], N[p][i]);
+        }
       }
     }
 #pragma unroll
@@ -389,9 +440,20 @@ __device__ __forceinline__ void split_advance(double (&y)[V][Dim<MODEL>::D], uin
       for (int i = 0; i < D; ++i) {
         double nd[2];
         join(N[p][i], nd, 1);
-        y[p][i] = split_final(y[p][i], k1d[p][i], nd[0], sc);
-        if constexpr (V > 1) y[p + P][i] = split_final(y[p + P][i], k1d[p + P][i], nd[1], sc);
+        if constexpr (PARK) {
+          rec[p * D + i] = split_final(rec[p * D + i], rk[p * D + i], nd[0], sc);
+          rec[(p + P) * D + i] = split_final(rec[(p + P) * D + i], rk[(p + P) * D + i], nd[1], sc);
+        } else {
+          y[p][i] = split_final(y[p][i], k1d[p][i], nd[0], sc);
+          if constexpr (V > 1) y[p + P][i] = split_final(y[p + P][i], k1d[p + P][i], nd[1], sc);
+        }
       }
+  }
+  if constexpr (PARK) {
+#pragma unroll
+    for (int v = 0; v < V; ++v)
+#pragma unroll
+      for (int i = 0; i < D; ++i) y[v][i] = rec[v * D + i];
   }
 }
 
@@ -639,8 +701,10 @@ template <typename R, int D> __host__ __device__ constexpr int align_sites() {
 // status word, where a non-finite stored value is reported.
 // SPLIT (FP64): the split form of the step.  Returns false, with nothing stored, when a value the
 // tile loads or would store (or a site's own parameter) is outside the split's range: the caller
-// then runs the item again in the FP64 form.  True otherwise; the same for every thread.
-template <typename R, int MODEL, int V, bool KAHAN, bool COH, bool HET = false, bool ALN = false, bool SPLIT = false>
+// then runs the item again in the FP64 form.  True otherwise; the same for every thread.  PARK: the
+// threads' records (split_advance) take the tile's place in shared memory while it is advanced.
+template <typename R, int MODEL, int V, bool KAHAN, bool COH, bool HET = false, bool ALN = false, bool SPLIT = false,
+          bool PARK = false>
 __device__ __forceinline__ bool tile_item(const R *__restrict__ in, R *__restrict__ out, const R *__restrict__ cin,
                                           R *__restrict__ cout, const ChainDesc &ch, int64_t tile, int K, int G,
                                           const Coef<R> &cf, unsigned char *smem, int64_t sites, WsHeader *hdr,
@@ -732,8 +796,11 @@ __device__ __forceinline__ bool tile_item(const R *__restrict__ in, R *__restric
     } else {
       if (__syncthreads_or(wide)) return false;
     }
-    if (edge_tile) split_advance<MODEL, V, true, HET>(y, ghost, K, cf, *sc, edge, spd, spf);
-    else split_advance<MODEL, V, false, HET>(y, 0u, K, cf, *sc, edge, spd, spf);
+    double *rec = nullptr;
+    if constexpr (PARK) rec = tl + threadIdx.x * split_record_words<MODEL, V>();
+    if (edge_tile) split_advance<MODEL, V, true, HET, PARK>(y, ghost, K, cf, *sc, edge, spd, spf, rec);
+    else split_advance<MODEL, V, false, HET, PARK>(y, 0u, K, cf, *sc, edge, spd, spf, rec);
+    if constexpr (PARK) __syncthreads();  // every record is read before the tile is written over them
   } else {
     Coef<R> cs[HET ? V : 1];
     if constexpr (HET) {
@@ -780,8 +847,8 @@ __device__ __forceinline__ bool tile_item(const R *__restrict__ in, R *__restric
 // sites are exact.  Every thread's sites lie in one segment (o and L are multiples of V), so a
 // thread takes its chain's coupling strength and, for fixed ends, its ghost mask; threads past
 // the last segment advance zeros that are never stored.
-// SPLIT and the result: as tile_item.
-template <typename R, int MODEL, int V, bool KAHAN, bool COH, bool SPLIT = false>
+// SPLIT, PARK and the result: as tile_item.
+template <typename R, int MODEL, int V, bool KAHAN, bool COH, bool SPLIT = false, bool PARK = false>
 __device__ __forceinline__ bool packed_tile_item(const R *__restrict__ in, R *__restrict__ out,
                                                  const R *__restrict__ cin, R *__restrict__ cout,
                                                  const ChainDesc *chains, const SegDesc *segs, int s0, int s1,
@@ -855,7 +922,10 @@ __device__ __forceinline__ bool packed_tile_item(const R *__restrict__ in, R *__
     if (__syncthreads_or(wide)) return false;
     SplitCoef sc = *scp;
     split_set_kappa(sc, c.kappa);
-    split_advance<MODEL, V, true, false>(y, ghost, K, c, sc, edge);
+    double *rec = nullptr;
+    if constexpr (PARK) rec = tl + threadIdx.x * split_record_words<MODEL, V>();
+    split_advance<MODEL, V, true, false, PARK>(y, ghost, K, c, sc, edge, nullptr, nullptr, rec);
+    if constexpr (PARK) __syncthreads();
   } else {
     tile_advance<R, MODEL, V, KAHAN, true>(y, cmp, ghost, K, c, edge);
   }
