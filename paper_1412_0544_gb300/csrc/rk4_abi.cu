@@ -125,9 +125,7 @@ int stages(const rk4_chain *h) { return use_generic(h) ? h->tab.s : 4; }
 // earlier stages a needed stage uses.  A stage outside this set (Dormand-Prince 5's seventh,
 // with b_7 = 0) cannot influence y, so the dependency cone of one step spans at most this
 // many stages: the tile halo and the sub-domain reach are sized by it.
-int needed_stages(const rk4_chain *h) {
-  if (!use_generic(h)) return 4;
-  const TableauD &t = h->tab;
+uint32_t needed_mask(const TableauD &t) {
   uint32_t need = 0;
   for (int m = 0; m < t.s; ++m)
     if (t.b[m] != 0.0) need |= 1u << m;
@@ -135,8 +133,13 @@ int needed_stages(const rk4_chain *h) {
     if ((need >> j) & 1u)
       for (int m = 0; m < j; ++m)
         if (t.a[j][m] != 0.0) need |= 1u << m;
+  return need;
+}
+int needed_stages(const rk4_chain *h) {
+  if (!use_generic(h)) return 4;
+  const uint32_t need = needed_mask(h->tab);
   int n = 0;
-  for (int m = 0; m < t.s; ++m) n += (need >> m) & 1u;
+  for (int m = 0; m < h->tab.s; ++m) n += (need >> m) & 1u;
   return n;
 }
 
@@ -218,8 +221,9 @@ CoefD coef(const rk4_chain *h) {
 // FP64 handles run the step in the split form (rk4_split.cuh) when its error bound holds for
 // their coefficients; every scheme of a handle takes the same form.
 bool use_split(const rk4_chain *h) {
-  if (h->fp32 || use_generic(h)) return false;
+  if (h->fp32) return false;
   CoefD c = coef(h);
+  if (use_generic(h) && (use_het(h) || !split_tableau_allowed(h->tab))) return false;
   c.kappa = h->kappa_most;
   if (!split_allowed(h->model, c)) return false;
   c.kappa = h->kappa_least;
@@ -520,7 +524,14 @@ cudaError_t enqueue_integrate(rk4_chain *h, int kernel, void *state, void *comp,
     j.chains = dev_chains(h, ws, L);
     j.total = h->total;
     j.hdr = reinterpret_cast<WsHeader *>(ws + L.hdr);
+    j.split = use_split(h) ? 1 : 0;
+    if (j.split) {
+      e = launch_split_scan(h->model, static_cast<const double *>(state), nullptr, h->total,
+                            split_coef(h->model, cf, true), j.hdr, st);
+      if (e != cudaSuccess) return e;
+    }
     for (int64_t s = 0; s < nsteps; ++s) {
+      j.parity = (int)(s & 1);
       e = launch_gen_staged_step(h->model, h->fp32, coupling_range(h), j, cf, h->tab, h->dt, st);
       if (e != cudaSuccess) return e;
     }
@@ -774,16 +785,17 @@ cudaError_t host_transfer(void *dst, const void *src, size_t bytes, bool to_devi
 
 namespace {
 
-// c as a float pair: its leading 24 bits and the rest (split1 of rk4_split.cuh).
+// c as a float pair: the head rounded to 24 bits (ties away from zero) and the rest (split1 of
+// rk4_split.cuh).
 struct HostPair {
   float h, l;
 };
 HostPair host_split(double c) {
   uint64_t u;
   std::memcpy(&u, &c, 8);
-  const uint64_t head = u & ~(uint64_t)0x1fffffff;
+  u = (u + 0x10000000u) & ~(uint64_t)0x1fffffff;
   double d;
-  std::memcpy(&d, &head, 8);
+  std::memcpy(&d, &u, 8);
   return {(float)d, (float)(c - d)};  // c - d is exact
 }
 HostPair host_times_tau(double c, const HostPair &tau) {  // times_tau
@@ -829,17 +841,74 @@ bool rk4d::split_allowed(int model, const CoefD &c) {
   split_most(model, dt, most);
   if (model == RK4_ROESSLER)
     return split_takes(c.a, most[0]) && split_takes(c.b, most[1]) && split_takes(c.c, most[2]) &&
-           split_takes(c.kappa, most[3]);
-  return split_takes(c.w2, most[0]) && split_takes(c.kappa, most[1]);
+           split_takes(c.kappa, most[3]) && split_takes(c.kappa2, most[3]);
+  return split_takes(c.w2, most[0]) && split_takes(c.kappa, most[1]) && split_takes(c.kappa2, most[1]);
 }
 
-SplitCoef rk4d::split_coef(int model, const CoefD &c) {
+bool rk4d::split_tableau_allowed(const TableauD &t) {
+  // entries within the pairs' range, and rows small enough that the differences' pair errors,
+  // multiplied by them, stay as far below the state's rounding as split_most assumes
+  double b = 0.0;
+  for (int j = 0; j < t.s; ++j) {
+    double row = 0.0, sum = 0.0;
+    for (int m = 0; m < j; ++m) {
+      if (!split_takes(t.a[j][m], 64.0)) return false;
+      sum += t.a[j][m];
+      row += std::fabs(t.a[j][m]);
+    }
+    if (!split_takes(sum, 2.0) || row > 64.0 || !split_takes(t.b[j], 64.0)) return false;
+    b += std::fabs(t.b[j]);
+  }
+  return b <= 8.0;
+}
+
+// a + b as a sum and its exact error.
+double host_two_sum(double a, double b, double *err) {
+  const double s = a + b, bb = s - a;
+  *err += (a - (s - bb)) + (b - bb);
+  return s;
+}
+
+SplitTableau rk4d::split_tableau(const TableauD &t) {
+  SplitTableau r{};
+  r.s = t.s;
+  double b_err = 0.0;  // the weights' sum is r.B + b_err: an error of 2^-54 in it would be a drift
+  for (int j = 0; j < t.s; ++j) {
+    double row = 0.0, row_err = 0.0;
+    for (int m = 0; m < j; ++m) {
+      row = host_two_sum(row, t.a[j][m], &row_err);
+      const HostPair a = host_split(t.a[j][m]);
+      r.ah[j][m] = a.h;
+      r.al[j][m] = a.l;
+      if (t.a[j][m] != 0.0) r.anz[j] |= 1u << m;
+      if (t.a[j][m] != 0.0 && m > 0) r.ma[j][r.na[j]++] = m;
+    }
+    const HostPair c = host_split(row + row_err), b = host_split(t.b[j]);
+    r.ch[j] = c.h;
+    r.cl[j] = c.l;
+    r.bh[j] = b.h;
+    r.bl[j] = b.l;
+    r.B = host_two_sum(r.B, t.b[j], &b_err);
+    if (t.b[j] != 0.0) r.bnz |= 1u << j;
+    if (t.b[j] != 0.0 && j > 0) r.mb[r.nb++] = j;
+  }
+  const double B = r.B + b_err;
+  r.Bl = (float)((r.B - B) + b_err);
+  r.B = B;
+  r.need = needed_mask(t);
+  return r;
+}
+
+SplitCoef rk4d::split_coef(int model, const CoefD &c, bool generic) {
   SplitCoef s{};
-  const double tau = c.h2;
-  s.w = tau / 3.0;
+  const double tau = generic ? c.h1 : c.h2;
+  s.w = generic ? c.h1 : tau / 3.0;
   const HostPair t = host_split(tau), cc = host_split(c.c);
   s.tauh = t.h;
   s.taul = t.l;
+  const HostPair k2 = host_times_tau(c.kappa2, t);
+  s.k2h = k2.h;
+  s.k2l = k2.l;
   const HostPair k = host_times_tau(c.kappa, t), a = host_times_tau(model == RK4_ROESSLER ? c.a : c.w2, t);
   s.kth = k.h;
   s.ktl = k.l;

@@ -118,4 +118,197 @@ __device__ __forceinline__ void gen_combine(const Tableau<R> &tb, const R (*k)[D
   }
 }
 
+// ---- one-stage-per-launch sweeps ----------------------------------------------------------
+
+template <typename R, int D>
+__device__ __forceinline__ void gen_state_sweep(const GenStagedJob &job, const Tableau<R> &tb, int j) {
+  const R *Y = static_cast<const R *>(job.y);
+  const R *K = static_cast<const R *>(job.k);
+  R *U = static_cast<R *>(job.u);
+  const size_t plane = (size_t)job.total * D;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < job.total; i += stride) {
+    R y[D], k[kMaxStages][D], u[D];
+#pragma unroll
+    for (int d = 0; d < D; ++d) y[d] = Y[i * D + d];
+#pragma unroll
+    for (int m = 0; m < kMaxStages; ++m)
+#pragma unroll
+      for (int d = 0; d < D; ++d) k[m][d] = (m < j) ? K[m * plane + i * D + d] : R(0);
+    gen_stage_state<R, D>(j, tb, y, k, u);
+#pragma unroll
+    for (int d = 0; d < D; ++d) U[i * D + d] = u[d];
+  }
+}
+
+template <typename R, int MODEL, int RANGE>
+__device__ __forceinline__ void gen_slope_sweep(const GenStagedJob &job, const Coef<R> &cf, R kappa2, int j) {
+  constexpr int D = Dim<MODEL>::D;
+  const R *src = static_cast<const R *>(j == 0 ? job.y : job.u);
+  R *K = static_cast<R *>(job.k) + (size_t)j * job.total * D;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < job.total; i += stride) {
+    ChainDesc ch;
+    Coef<R> c = cf;
+    if (job.nchains == 1) {
+      ch = job.one;
+    } else {
+      int lo = 0, hi = job.nchains - 1;
+      while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (job.chains[mid].off <= i) lo = mid; else hi = mid - 1;
+      }
+      ch = job.chains[lo];
+      c.kappa = (R)ch.kappa;
+    }
+    const int64_t li = i - ch.off;
+    auto xat = [&](int64_t q) -> R {  // coupling coordinate of chain site q (boundary-resolved)
+      const int64_t g = (ch.bc == PERIODIC) ? ch.off + wrap(q, ch.n) : ((q < 0 || q >= ch.n) ? -1 : ch.off + q);
+      if (g < 0 || !bounds_ok(job.hdr, in_range(g, 1, job.total))) return R(0);
+      return src[g * D];
+    };
+    R u[D], k[D];
+#pragma unroll
+    for (int d = 0; d < D; ++d) u[d] = src[i * D + d];
+    slope_gen<R, MODEL, RANGE>(u, xat(li - 1), xat(li + 1), RANGE == 2 ? xat(li - 2) : R(0),
+                               RANGE == 2 ? xat(li + 2) : R(0), c, kappa2, k);
+#pragma unroll
+    for (int d = 0; d < D; ++d) K[i * D + d] = k[d];
+  }
+}
+
+template <typename R, int D, bool KAHAN>
+__device__ __forceinline__ void gen_combine_sweep(const GenStagedJob &job, const Tableau<R> &tb) {
+  R *Y = static_cast<R *>(job.y);
+  R *CMP = static_cast<R *>(job.cmp);
+  const R *K = static_cast<const R *>(job.k);
+  const size_t plane = (size_t)job.total * D;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < job.total; i += stride) {
+    R y[D], k[kMaxStages][D], cmp[D];
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+      y[d] = Y[i * D + d];
+      cmp[d] = KAHAN ? CMP[i * D + d] : R(0);
+    }
+#pragma unroll
+    for (int m = 0; m < kMaxStages; ++m)
+#pragma unroll
+      for (int d = 0; d < D; ++d) k[m][d] = (m < tb.s) ? K[m * plane + i * D + d] : R(0);
+    gen_combine<R, D, KAHAN>(tb, k, y, cmp);
+    bool bad = false;
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+      Y[i * D + d] = y[d];
+      if constexpr (KAHAN) CMP[i * D + d] = cmp[d];
+      bad |= nonfinite(y[d]);
+    }
+    if (bad && job.hdr) atomicOr(&job.hdr->status, ST_NONFINITE);
+  }
+}
+
+inline int64_t staged_grid(int64_t total) {
+  int64_t g = (total + 255) / 256;
+  const int64_t cap = (int64_t)sm_count() * 64;
+  return g > cap ? cap : (g < 1 ? 1 : g);
+}
+
+// ---- advancing a tile ----------------------------------------------------------------------
+
+// Two values of the working precision as one 8- or 16-byte shared-memory access.
+template <typename R> struct Pair;
+template <> struct Pair<float> { using T = float2; };
+template <> struct Pair<double> { using T = double2; };
+
+// Advance one tile's registers K steps of the generic scheme.  `edge`: gen_edge_values(V)
+// values of shared memory, two parities of [(first, second) coupling coordinate of each thread
+// | (second-last, last) of each thread].  Every stage each thread stores its two pairs (two
+// vector stores) and, after the stage's one barrier, reads its left neighbour's last pair and
+// its right neighbour's first pair (two vector loads, conflict-free): four shared-memory
+// instructions for the range-2 coupling, where shuffles plus warp-edge slots took 12 (FP32) or
+// 16 (FP64).  The two tile ends read a stand-in (their own pair), which only reaches halo sites.
+template <typename R, int MODEL, int V, int RANGE, bool KAHAN, bool MASK, uint64_t SHAPE>
+__device__ __forceinline__ void gen_tile_advance(R (&y)[V][Dim<MODEL>::D], R (&cmp)[V][Dim<MODEL>::D],
+                                                 uint32_t ghost, int K, const Coef<R> &cf, R kappa2,
+                                                 const Tableau<R> &tb, R *edge) {
+  constexpr int D = Dim<MODEL>::D;
+  static_assert(V >= 2, "the generic kernel holds at least two sites per thread");
+  constexpr int NT = kGenEdgeThreads;
+  using R2 = typename Pair<R>::T;
+  const int tid = threadIdx.x;
+  const int lt = tid > 0 ? tid - 1 : tid;                           // left neighbour thread
+  const int rt = tid < (int)blockDim.x - 1 ? tid + 1 : tid;          // right neighbour thread
+  R k[V][kMaxStages][D];
+
+  int parity = 0;  // edge slots alternate strictly from stage to stage (s may be odd)
+#pragma unroll 1
+  for (int s = 0; s < K; ++s) {
+#pragma unroll
+    for (int j = 0; j < kMaxStages; ++j) {
+      if (j >= gen_stages<SHAPE>(tb)) break;
+      if (!gen_stage_needed<SHAPE>(j)) continue;  // a compiled shape's dead stage: nothing reads it
+      R u[V][D];
+      R ext[V + 4];  // ext[2 + v] = x of site v; two neighbours on each side
+      R2 *head = reinterpret_cast<R2 *>(edge) + parity * 2 * NT;  // (first, second) per thread
+      R2 *tail = head + NT;                                         // (second-last, last) per thread
+      parity ^= 1;
+#pragma unroll
+      for (int v = 0; v < V; ++v) {
+        gen_stage_state<R, D, SHAPE>(j, tb, y[v], k[v], u[v]);
+        ext[2 + v] = (MASK && ((ghost >> v) & 1u)) ? R(0) : u[v][0];
+      }
+      R2 hv, tv;
+      hv.x = ext[2];
+      hv.y = ext[3];
+      tv.x = ext[V];
+      tv.y = ext[V + 1];
+      head[tid] = hv;
+      tail[tid] = tv;
+      // each thread reads only its neighbour threads' slots: in FP64 the streaming form waits
+      // for the neighbouring warps only (measured +4.6 % for Dormand-Prince 5); in FP32 the two
+      // named barriers per stage cost 22 %, so it keeps the block-wide one
+      if constexpr (SHAPE != 0 && sizeof(R) == 8) neighbour_warp_sync(); else __syncthreads();
+      {
+        const R2 l = tail[lt];
+        const R2 r = head[rt];
+        ext[0] = l.x;
+        ext[1] = l.y;
+        ext[V + 2] = r.x;
+        ext[V + 3] = r.y;
+      }
+#pragma unroll
+      for (int v = 0; v < V; ++v) {
+        R kv[D];
+        slope_gen<R, MODEL, RANGE>(u[v], ext[1 + v], ext[3 + v], RANGE == 2 ? ext[v] : R(0),
+                                   RANGE == 2 ? ext[4 + v] : R(0), cf, kappa2, kv);
+#pragma unroll
+        for (int d = 0; d < D; ++d) k[v][j][d] = kv[d];
+      }
+    }
+#pragma unroll
+    for (int v = 0; v < V; ++v) gen_combine<R, D, KAHAN, SHAPE>(tb, k[v], y[v], cmp[v]);
+  }
+}
+
+template <typename R>
+inline Tableau<R> to_tableau(const TableauD &t, double dt) {
+  Tableau<R> r{};
+  r.s = t.s;
+  for (int j = 0; j < kMaxStages; ++j) {
+    r.anz[j] = 0;
+    for (int m = 0; m < kMaxStages; ++m) {
+      const double a = (j < t.s && m < j) ? t.a[j][m] : 0.0;
+      r.adt[j][m] = (R)(a * dt);
+      if (a != 0.0) r.anz[j] |= 1u << m;
+    }
+  }
+  r.bnz = 0;
+  for (int m = 0; m < kMaxStages; ++m) {
+    const double b = m < t.s ? t.b[m] : 0.0;
+    r.bdt[m] = (R)(b * dt);
+    if (b != 0.0) r.bnz |= 1u << m;
+  }
+  return r;
+}
+
 }  // namespace rk4d

@@ -24,12 +24,12 @@ struct CoefD {
   double a, b, c, kappa, w2, h2, h1, dt6, kappa2, dt3;
 };
 
-// Coefficients of the split FP64 step (rk4_split.cuh): tau = dt / 2, and the products with it as
-// float pairs (h + l).  at: Roessler a tau, harmonic w2 tau.  most: high words of the largest
+// Coefficients of the split FP64 step (rk4_split.cuh): tau = dt / 2 (generic tableaux: dt), and the
+// products with it as float pairs (h + l).  at: Roessler a tau, harmonic w2 tau.  most: high words of the largest
 // magnitudes a site's own parameters may have (heterogeneous chains; in their order).
 struct SplitCoef {
-  double w;  // tau / 3
-  float tauh, taul, kth, ktl, ath, atl, ch, cl;
+  double w;  // tau / 3 (generic tableaux: dt)
+  float tauh, taul, kth, ktl, k2h, k2l, ath, atl, ch, cl;
   unsigned most[4];
 };
 
@@ -135,6 +135,8 @@ struct GenStagedJob {
   const ChainDesc *chains;
   int64_t total;
   WsHeader *hdr;  // status word
+  int split;      // 1: the split form (k[0]: the first slope; the other k and u: float pairs)
+  int parity;     // of the step (which wide flag is read)
 };
 
 struct PersistentJob {
@@ -175,7 +177,25 @@ cudaError_t launch_split_scan(int model, const double *state, const double *sp, 
 // Whether every step of a handle with these coefficients (c.kappa: the largest coupling strength
 // of its chains) may run in the split form, and the form's coefficients.
 bool split_allowed(int model, const CoefD &c);
-SplitCoef split_coef(int model, const CoefD &c);
+SplitCoef split_coef(int model, const CoefD &c, bool generic = false);
+// The generic scheme in the split form: a tableau's rows and weights for the slope differences,
+// as float pairs; a's nonzero pattern (anz, bnz), and the stages the result needs (need).
+struct SplitTableau {
+  int s;
+  uint32_t need, bnz, anz[kMaxStages];
+  int nb, mb[kMaxStages];                      // the stages m >= 1 of nonzero weight, in order
+  int na[kMaxStages], ma[kMaxStages][kMaxStages];  // and those with a nonzero a_jm
+  double B;                                    // sum of the weights, the first slope's factor,
+  float Bl;                                    // and what its rounding leaves
+  float ch[kMaxStages], cl[kMaxStages];        // row sums, the first slope's factors
+  float ah[kMaxStages][kMaxStages], al[kMaxStages][kMaxStages], bh[kMaxStages], bl[kMaxStages];
+};
+bool split_tableau_allowed(const TableauD &t);  // whether the form takes the tableau
+SplitTableau split_tableau(const TableauD &t);
+cudaError_t launch_gen_split(int model, int range, int sites, const BlockedJob &job, const CoefD &cf,
+                             const TableauD &tb, double dt, int H, cudaStream_t st);  // tiles of `sites` sites
+cudaError_t launch_gen_split_step(int model, int range, const GenStagedJob &job, const CoefD &cf,
+                                  const TableauD &tb, double dt, cudaStream_t st);
 cudaError_t launch_staged(int model, bool fp32, int stage, const StagedJob &job, const CoefD &cf,
                           cudaStream_t st);
 cudaError_t launch_persistent(int model, bool fp32, int v, int block, int grid, const PersistentJob &job,

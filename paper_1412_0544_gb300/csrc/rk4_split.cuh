@@ -29,6 +29,8 @@
 //
 // Range: a pair needs the exponent room of FP32.  Tiles whose values leave it (split_in_range)
 // are advanced in the FP64 form instead (tile_item returns false and the caller runs it again).
+// A tile of NaN alone, what a chain that has blown up consists of, stays: its first slope and so
+// its result are NaN in either form.
 #pragma once
 #include "rk4_device.cuh"
 #include "rk4_internal.h"
@@ -56,7 +58,10 @@ __device__ __forceinline__ float lane1(f32x2 v) {
 }
 __device__ __forceinline__ float vadd(float a, float b) { return __fadd_rn(a, b); }
 __device__ __forceinline__ float vsub(float a, float b) { return __fsub_rn(a, b); }
-__device__ __forceinline__ float vmul(float a, float b) { return __fmul_rn(a, b); }
+// Products as FMAs with a zero addend (a zero product comes out as +0): ptxas was seen to contract
+// a packed mul.rn and a later add.rn into one FMA (CUDA 13.0; the packed and the scalar forms of
+// a normalisation after a product then differed), which an FMA rules out at the same cost.
+__device__ __forceinline__ float vmul(float a, float b) { return __fmaf_rn(a, b, 0.f); }
 __device__ __forceinline__ float vfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ f32x2 vadd(f32x2 a, f32x2 b) {
   f32x2 r;
@@ -70,7 +75,7 @@ __device__ __forceinline__ f32x2 vsub(f32x2 a, f32x2 b) {
 }
 __device__ __forceinline__ f32x2 vmul(f32x2 a, f32x2 b) {
   f32x2 r;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(0ull));
   return r;
 }
 __device__ __forceinline__ f32x2 vfma(f32x2 a, f32x2 b, f32x2 c) {
@@ -111,6 +116,11 @@ template <typename T> __device__ __forceinline__ void mul_coef(const FPair<T> &c
   e = vfma(c.h, v.l, e);
   e = vfma(c.l, v.h, e);
 }
+// The pair with its tail at most half a unit of its head (|h| >= |l| up to the head's cancellation).
+template <typename T> __device__ __forceinline__ FPair<T> pair_norm(const FPair<T> &v) {
+  const T s = vadd(v.h, v.l);
+  return {s, vsub(v.l, vsub(s, v.h))};
+}
 // a - n as a pair.
 template <typename T> __device__ __forceinline__ FPair<T> pair_sub(const FPair<T> &a, const FPair<T> &n) {
   FPair<T> r;
@@ -122,16 +132,20 @@ template <typename T> __device__ __forceinline__ FPair<T> pair_sub(const FPair<T
 
 // ---- FP64 <-> pair by integer operations (the F2F conversions issue on the FP64 pipe) --------
 
-// A double as head (its leading 24 bits, truncated), the tail's integer significand m (29 bits)
-// and the head's power of two p: the value is h + m 2^-52 p.  Zero gives h = p = 0, magnitudes
-// below 2^-126 at most a few denormals.
+// A double as head (rounded to 24 bits, ties away from zero), the tail's integer significand m (28
+// bits and sign) and the power of two p of the double itself: the value is h + m 2^-52 p.  Zero
+// gives h = p = 0, magnitudes below 2^-126 at most a few denormals.  (A truncated head would save
+// four integer operations; its one-signed tails, up to twice as large, doubled the error of the
+// later slopes' differences.)
 __device__ __forceinline__ void split_bits(double y, float &h, float &m, float &p) {
-  const int hi = __double2hiint(y), lo = __double2loint(y);
-  const int a = max((hi & 0x7fffffff) - 0x38000000, 0);  // rebias the exponent from 1023 to 127
-  const unsigned f = (__funnelshift_l((unsigned)lo, (unsigned)a, 3) & 0x7fffffffu) | ((unsigned)hi & 0x80000000u);
-  h = __uint_as_float(f);
-  m = __uint2float_rn((unsigned)lo & 0x1fffffffu);
-  p = __uint_as_float(f & 0xff800000u);
+  const int hi = __double2hiint(y);
+  const unsigned lo = (unsigned)__double2loint(y);
+  const unsigned sign = (unsigned)hi & 0x80000000u;
+  const unsigned a = (unsigned)max((hi & 0x7fffffff) - 0x38000000, 0);  // exponent bias 1023 -> 127
+  const unsigned rl = lo + 0x10000000u, rh = a + (rl < lo ? 1u : 0u);
+  h = __uint_as_float(__funnelshift_l(rl, rh, 3) | sign);
+  m = __int2float_rn((int)(lo << 3) >> 3);
+  p = __uint_as_float(((a << 3) & 0x7f800000u) | sign);
 }
 __device__ __forceinline__ FPair<float> split1(double y) {
   float h, m, p;
@@ -197,6 +211,10 @@ template <int MODEL> __device__ __forceinline__ bool split_in_range(double v) {
   const unsigned a = (unsigned)__double2hiint(v) & 0x7fffffffu;
   return (a - lo < hi - lo) | ((a | (unsigned)__double2loint(v)) == 0u);
 }
+__device__ __forceinline__ bool is_nan(double v) {
+  const unsigned a = (unsigned)__double2hiint(v) & 0x7fffffffu;
+  return a > 0x7ff00000u || (a == 0x7ff00000u && __double2loint(v) != 0);
+}
 // The same for a site's own parameter of a heterogeneous chain: zero, or at least 2^-60 and with
 // the high word at most `most` (that of the largest value split_allowed takes).
 __device__ __forceinline__ bool split_param_in_range(double v, unsigned most) {
@@ -221,10 +239,13 @@ __device__ __forceinline__ void split_set_kappa(SplitCoef &s, double kappa) {
 }
 // The pair coefficients of a stage in lane type T.  at: Roessler a tau; harmonic w2 tau.
 template <typename T> struct StageCoef {
-  FPair<T> kt, at, tau;
+  FPair<T> kt, at, tau, k2;  // k2: kappa2 tau (coupling range 2)
 };
 template <typename T> __device__ __forceinline__ StageCoef<T> stage_coef(const SplitCoef &s) {
-  return {{vset<T>(s.kth), vset<T>(s.ktl)}, {vset<T>(s.ath), vset<T>(s.atl)}, {vset<T>(s.tauh), vset<T>(s.taul)}};
+  return {{vset<T>(s.kth), vset<T>(s.ktl)},
+          {vset<T>(s.ath), vset<T>(s.atl)},
+          {vset<T>(s.tauh), vset<T>(s.taul)},
+          {vset<T>(s.k2h), vset<T>(s.k2l)}};
 }
 
 // ---- one stage ----------------------------------------------------------------------------------
@@ -253,14 +274,23 @@ __device__ __forceinline__ FPair<T> pair_lap(const FPair<T> &x, const FPair<T> &
   return g;
 }
 
-// n = -D for the stage increments d (85 FP32 operations per site; harmonic 40).
-template <int MODEL, typename T>
+// n = -D for the stage increments d (85 FP32 operations per site; harmonic 40; 28 more with
+// second neighbours).
+template <int MODEL, typename T, int RANGE = 1, bool NORM = false>
 __device__ __forceinline__ void split_stage(const FPair<T> *d, const FPair<T> &xl, const FPair<T> &xr,
-                                            const SplitBase<T> &b, const StageCoef<T> &c, FPair<T> *n) {
+                                            const SplitBase<T> &b, const StageCoef<T> &c, FPair<T> *n,
+                                            const FPair<T> &xl2 = {}, const FPair<T> &xr2 = {}) {
   const T m1 = vset<T>(-1.f);
   const FPair<T> g = pair_lap(d[0], xl, xr);
   T np, e, ne;
   mul_coef(c.kt, vmul(m1, c.kt.h), g, np, e);  // kappa tau lap = e - np
+  if constexpr (RANGE == 2) {
+    T np2, e2, s;
+    mul_coef(c.k2, vmul(m1, c.k2.h), pair_lap(d[0], xl2, xr2), np2, e2);
+    two_sum(np, np2, s, ne);
+    np = s;
+    e = vsub(vadd(e, e2), ne);
+  }
   if constexpr (MODEL == ROESSLER) {
     const T ntau = vmul(m1, c.tau.h);
     FPair<T> w;  // dy + dz
@@ -277,11 +307,18 @@ __device__ __forceinline__ void split_stage(const FPair<T> *d, const FPair<T> &x
     n[1].l = vsub(ne, vadd(df, e));
     T nz, q;  // zeta = tau dz = q - nz
     mul_coef(c.tau, ntau, d[2], nz, q);
-    const T pz = vmul(c.tau.h, d[2].h);  // = -nz
+    T pz = vmul(c.tau.h, d[2].h);  // = -nz
+    if constexpr (NORM) {
+      const FPair<T> zn = pair_norm(FPair<T>{pz, q});
+      pz = zn.h;
+      q = zn.l;
+      nz = vmul(m1, pz);
+    }
     FPair<T> t;  // (x - c) + delta
     T te;
     two_diff(b.t.h, nd, t.h, te);
     t.l = vadd(vadd(te, b.t.l), df);
+    if constexpr (NORM) t = pair_norm(t);
     const T nzh = vmul(m1, b.z.h);
     const T p1 = vmul(nzh, nd);  // z delta = p1 - g1
     T g1 = vfma(b.z.h, nd, p1);
@@ -324,6 +361,29 @@ __device__ __forceinline__ void split_update(int j, const FPair<T> &k1, const FP
     two_sum_m(n.h, two, N.h, s, e);
     N = {s, vadd(vfma(two, N.l, n.l), e)};
   }
+}
+// a + c v and a - c v for a coefficient pair c.
+template <typename T> __device__ __forceinline__ FPair<T> pair_fma(const FPair<T> &c, T nch, const FPair<T> &v, const FPair<T> &a) {
+  T np, e, ne;
+  FPair<T> r;
+  mul_coef(c, nch, v, np, e);
+  two_diff(a.h, np, r.h, ne);
+  r.l = vadd(vadd(a.l, e), ne);
+  return r;
+}
+template <typename T> __device__ __forceinline__ FPair<T> pair_fnma(const FPair<T> &c, T nch, const FPair<T> &v, const FPair<T> &a) {
+  T np, e, ne;
+  FPair<T> r;
+  mul_coef(c, nch, v, np, e);
+  two_sum(a.h, np, r.h, ne);
+  r.l = vadd(vsub(a.l, e), ne);
+  return r;
+}
+// c v.
+template <typename T> __device__ __forceinline__ FPair<T> pair_mul(const FPair<T> &c, T nch, const FPair<T> &v) {
+  T np, e;
+  mul_coef(c, nch, v, np, e);
+  return {vmul(c.h, v.h), e};
 }
 // y + (tau / 3) (6 K1 - N).
 __device__ __forceinline__ double split_final(double y, double k1, double N, const SplitCoef &s) {

@@ -751,8 +751,17 @@ __device__ __forceinline__ bool tile_item(const R *__restrict__ in, R *__restric
       if (g < 0 || g >= ch.n) ghost |= 1u << v;
     }
   }
+  bool nan_tile = false;  // SPLIT: every value is NaN already (a chain that has blown up), and stays so
   if constexpr (SPLIT) {
-    bool wide = false;  // a value outside the split's range
+    bool wide = false, live = false;  // a value outside the split's range; one that is not NaN
+    auto values_live = [&]() {
+      bool l = false;
+#pragma unroll
+      for (int v = 0; v < V; ++v)
+#pragma unroll
+        for (int d = 0; d < D; ++d) l |= !is_nan(y[v][d]) && !((ghost >> v) & 1u);
+      return l;
+    };
     double *spd = nullptr;
     f32x2 *spf = nullptr;
 #pragma unroll
@@ -769,9 +778,12 @@ __device__ __forceinline__ bool tile_item(const R *__restrict__ in, R *__restric
 #pragma unroll
         for (int i = 0; i < P; ++i) {
           p[v][i] = ptl[(base + v) * P + i];
-          wide |= !split_param_in_range(p[v][i], sc->most[i]);
+          const bool out = !split_param_in_range(p[v][i], sc->most[i]);
+          wide |= out;
+          live |= out;
         }
-      if (__syncthreads_or(wide)) return false;
+      nan_tile = __syncthreads_or(wide);
+      if (nan_tile && __syncthreads_or(live || values_live())) return false;
       spd = ptl + threadIdx.x;
       spf = reinterpret_cast<f32x2 *>(ptl + W * P) + threadIdx.x;
 #pragma unroll
@@ -794,7 +806,8 @@ __device__ __forceinline__ bool tile_item(const R *__restrict__ in, R *__restric
         }
       }
     } else {
-      if (__syncthreads_or(wide)) return false;
+      nan_tile = __syncthreads_or(wide);
+      if (nan_tile && __syncthreads_or(live || values_live())) return false;
     }
     double *rec = nullptr;
     if constexpr (PARK) rec = tl + threadIdx.x * split_record_words<MODEL, V>();
@@ -827,7 +840,8 @@ __device__ __forceinline__ bool tile_item(const R *__restrict__ in, R *__restric
   }
   const int any_bad = __syncthreads_or(bad);
   if constexpr (SPLIT) {
-    if (any_bad) return false;
+    if (any_bad && !nan_tile) return false;
+    report_nonfinite(hdr, nan_tile);
   } else {
     report_nonfinite(hdr, any_bad);
   }
@@ -913,13 +927,22 @@ __device__ __forceinline__ bool packed_tile_item(const R *__restrict__ in, R *__
       y[v][d] = tl[(base + v) * D + d];
       if constexpr (KAHAN) cmp[v][d] = ctl[(base + v) * D + d]; else cmp[v][d] = R(0);
     }
+  bool nan_tile = false;  // as in tile_item
   if constexpr (SPLIT) {
     bool wide = false;
 #pragma unroll
     for (int v = 0; v < V; ++v)
 #pragma unroll
       for (int d = 0; d < D; ++d) wide |= !split_in_range<MODEL>(y[v][d]);
-    if (__syncthreads_or(wide)) return false;
+    nan_tile = __syncthreads_or(wide);
+    if (nan_tile) {
+      bool live = false;
+#pragma unroll
+      for (int v = 0; v < V; ++v)
+#pragma unroll
+        for (int d = 0; d < D; ++d) live |= my >= 0 && !is_nan(y[v][d]) && !((ghost >> v) & 1u);
+      if (__syncthreads_or(live)) return false;
+    }
     SplitCoef sc = *scp;
     split_set_kappa(sc, c.kappa);
     double *rec = nullptr;
@@ -944,7 +967,8 @@ __device__ __forceinline__ bool packed_tile_item(const R *__restrict__ in, R *__
   }
   const int any_bad = __syncthreads_or(bad);
   if constexpr (SPLIT) {
-    if (any_bad) return false;
+    if (any_bad && !nan_tile) return false;
+    report_nonfinite(hdr, nan_tile);
   } else {
     report_nonfinite(hdr, any_bad);
   }

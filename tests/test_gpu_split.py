@@ -157,3 +157,117 @@ def test_more_accurate_than_the_fp64_form(gh, model):
             theirs = float(np.sqrt(np.sum((plain[d] - exact[d]) ** 2)))
             print(f"model {model} component {d} after {count} steps: {ours / theirs:.2f} of the FP64 form's error")
             assert ours <= theirs
+
+
+# ---- generic tableaux ---------------------------------------------------------------------------
+
+import oracle_pins as P  # noqa: E402
+
+
+def gen_run(y0, A, b, *, model=ROE, bc=PER, nsteps=10, kappa2=0.0, kernel=BLOCKED, tiling=None, dt=0.01):
+    import torch
+    import paper_1412_0544_gb300 as rk
+    h = rk.rk4_chain_create(model, rk.RK4_FP64, y0.shape[0], dt, bc, dict(kappa=1.1, omega0=0.9))
+    try:
+        rk.rk4_chain_set_tableau(h, A, b)
+        rk.rk4_chain_set_coupling2(h, kappa2)
+        rk.rk4_chain_set_kernel(h, kernel)
+        if tiling:
+            rk.rk4_chain_set_tiling(h, *tiling)
+        st = torch.from_numpy(np.ascontiguousarray(y0)).cuda()
+        ws = torch.empty(rk.rk4_chain_workspace_bytes(h), dtype=torch.uint8, device="cuda")
+        rk.rk4_chain_integrate(h, st, None, ws, nsteps)
+        assert rk.rk4_chain_status(h, ws) == rk.RK4_OK
+        return st.cpu().numpy()
+    finally:
+        rk.rk4_chain_destroy(h)
+
+
+GEN = [(STAGED, None), (BLOCKED, (64, 2, 1)), (BLOCKED, (256, 2, 4)), (BLOCKED, (128, 4, 3)), (BLOCKED, (256, 4, 8))]
+
+
+@pytest.mark.parametrize("kernel,tiling", GEN)
+@pytest.mark.parametrize("kappa2", [0.0, 0.6])
+def test_generic_pulse_and_wide_values(kernel, tiling, kappa2):
+    """The generic scheme's tiles outside the pairs' range, and the sites a pulse has not reached."""
+    A, b, _ = P.TABLEAUX["dopri5"]
+    n, site, steps = 3001, 1500, 9
+    y0 = np.zeros((n, 2))
+    y0[site] = (1.0, 0.25)
+    prm = oracle.params(kappa=1.1, omega0=0.9, kappa2=kappa2)
+    ref = oracle.rk_integrate(y0, A, b, HAR, FIX, 0.01, steps, prm)
+    got = gen_run(y0, A, b, model=HAR, bc=FIX, nsteps=steps, kappa2=kappa2, kernel=kernel, tiling=tiling)
+    reach = 6 * (2 if kappa2 else 1) * steps
+    assert np.all(got[np.abs(np.arange(n) - site) > reach] == 0.0)
+    assert cf.rel_inf(got, ref) <= 1e-12
+    y0 = ci.uniform_state(n, 3, seed=1110)
+    for i, v in ((0, 1e-200), (700, 3e5), (1100, 1e-90), (n - 1, 7e4)):
+        y0[i, 1] = v
+    ref = oracle.rk_integrate(y0, A, b, ROE, PER, 0.01, 1, prm)
+    got = gen_run(y0, A, b, nsteps=1, kappa2=kappa2, kernel=kernel, tiling=tiling)
+    assert cf.rel_inf(got, ref) <= 1e-12
+
+
+@pytest.mark.parametrize("name", ["dopri5", "rk4"])
+def test_generic_more_accurate_than_the_fp64_form(name):
+    """Against long double, runs of 20 and 100 steps are no further off than the FP64 form the split
+    form replaces (k_m summed with their weights, one addition to the state): both round the
+    state once per step, so the ratio is 1 up to the sampling of 60000 values (0.4 %) and the other
+    roundings of either side (after a single Dormand-Prince step from a random state the split
+    form's are 5 % of the total, against long double; later steps damp them)."""
+    A, b, _ = P.TABLEAUX["dopri5"] if name == "dopri5" else (oracle.RK4_A, oracle.RK4_B, 4)
+    A, b = np.asarray(A, dtype=float), np.asarray(b, dtype=float)
+    y0 = ci.uniform_state(20000, 3, seed=1111)
+
+    def steps(dtype, count):
+        dt, kap, k2, a, c = (dtype(np.float64(v)) for v in (0.01, 1.1, 0.5, 0.2, 9.0))
+        y = [y0[:, d].astype(dtype) for d in range(3)]
+
+        def f(u):
+            lap = np.roll(u[0], 1) - 2 * u[0] + np.roll(u[0], -1)
+            lap2 = np.roll(u[0], 2) - 2 * u[0] + np.roll(u[0], -2)
+            return [kap * lap + (k2 * lap2 - (u[1] + u[2])), u[0] + a * u[1], 1 + u[2] * (u[0] - c)]
+
+        for _ in range(count):
+            ks = []
+            for j in range(len(b)):
+                u = [v.copy() for v in y]
+                for m in range(j):
+                    if A[j, m]:
+                        u = [v + (dtype(A[j, m]) * dt) * k for v, k in zip(u, ks[m])]
+                ks.append(f(u))
+            y = [v + sum((dtype(b[m]) * dt) * ks[m][d] for m in range(len(b)) if b[m]) for d, v in enumerate(y)]
+        return y
+
+    for count in (20, 100):
+        exact, plain = steps(np.longdouble, count), steps(np.float64, count)
+        got = gen_run(y0, A, b, nsteps=count, kappa2=0.5, tiling=(128, 2, 2))
+        ours = np.sqrt(sum(float(np.sum((got[:, d] - exact[d]) ** 2)) for d in range(3)))
+        theirs = np.sqrt(sum(float(np.sum((plain[d] - exact[d]) ** 2)) for d in range(3)))
+        print(f"{name} after {count} steps: {ours / theirs:.3f} of the FP64 form's error")
+        assert ours <= 1.02 * theirs
+
+
+@pytest.mark.parametrize("bc", [PER, FIX])
+def test_nan_spreads_as_in_the_fp64_form(gh, bc):
+    """One NaN site: after m steps exactly the sites within 4 m of it are NaN; a chain that is all
+    NaN stays so and reports it."""
+    import torch
+    import paper_1412_0544_gb300 as rk
+    n, site = 6007, 2900
+    for start, steps in ((site, 3), (None, 7)):
+        y0 = ci.uniform_state(n, 3, seed=1120)
+        y0[slice(None) if start is None else start] = np.nan
+        for kernel, tiling in SCHEMES:
+            h = rk.rk4_chain_create(ROE, rk.RK4_FP64, n, 0.01, bc)
+            rk.rk4_chain_set_kernel(h, kernel)
+            if tiling:
+                rk.rk4_chain_set_tiling(h, *tiling)
+            st = torch.from_numpy(y0.copy()).cuda()
+            ws = torch.empty(rk.rk4_chain_workspace_bytes(h), dtype=torch.uint8, device="cuda")
+            rk.rk4_chain_integrate(h, st, None, ws, steps)
+            assert rk.rk4_chain_status(h, ws) == rk.RK4_ENONFINITE
+            rk.rk4_chain_destroy(h)
+            nan = np.isnan(st.cpu().numpy()).any(axis=1)
+            want = np.ones(n, bool) if start is None else np.abs(np.arange(n) - site) <= 4 * steps
+            assert np.array_equal(nan, want), (kernel, tiling, start)
