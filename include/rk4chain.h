@@ -138,7 +138,9 @@ int rk4_chain_set_kernel(rk4_chain *h, int kernel);
 /* The scheme the handle will run (AUTO resolved).  Errors: RK4_EINVAL. */
 int rk4_chain_get_kernel(const rk4_chain *h, int *kernel);
 
-/* Sets the tiling (block, v, k; G is computed).  block = 0 restores the automatic choice.
+/* Sets the tiling (block, v, k; G is computed).  block = 0 restores the automatic choice, which
+ * each integration makes from the sites and its steps (from the sites alone for a batch);
+ * rk4_chain_get_tiling then reports its seed.
  * The largest block depends on the kernel the handle runs (its register budget): 1024
  * threads for v = 1, 512 for v = 2 and 4, 256 for v = 8, the generic scheme and the
  * heterogeneous FP32 Roessler chain with v = 4.  Errors: RK4_EINVAL when block, v or k is out
@@ -196,10 +198,10 @@ int rk4_chain_step(rk4_chain *h, void *state, void *comp, void *ws, size_t ws_by
  * NULL it receives t0 + n dt, n being the steps taken through this handle so far (no
  * repeated addition).  Launch sequences of the same shape are replayed from a cached CUDA
  * graph.  The blocked scheme makes launches of k steps (the tiling's k) into a ping-pong copy
- * in ws and must end in `state` after an even number of launches: an odd count is evened by
- * splitting one launch in two (nsteps = k runs as two launches of k / 2), so calls of an
- * even multiple of k steps run at the tiling's full k.  Errors: RK4_EINVAL, RK4_ENOMEM_WS,
- * RK4_ECUDA. */
+ * in ws and must end in `state` after an even number of launches: a chain's steps are divided
+ * evenly over the smallest even number of launches of at most k steps (nsteps = k runs as two
+ * launches of k / 2), so calls of an even multiple of k steps run at the tiling's full k.
+ * Errors: RK4_EINVAL, RK4_ENOMEM_WS, RK4_ECUDA. */
 int rk4_chain_integrate(rk4_chain *h, void *state, void *comp, void *ws, size_t ws_bytes,
                         int64_t nsteps, double *t);
 

@@ -193,6 +193,8 @@ static uint64_t compiled_shape(const TableauD &t, int v) {
   return (sh == kShapeDopri5 || sh == kShapeRK4) ? sh : 0;
 }
 
+bool gen_compiled(const TableauD &t) { return compiled_shape(t, 4) != 0; }
+
 template <typename R, int MODEL, int V, int RANGE, bool KAHAN, uint64_t SHAPE>
 static int gen_max_threads_s() {
   cudaFuncAttributes a;

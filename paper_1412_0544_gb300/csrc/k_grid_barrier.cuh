@@ -49,9 +49,12 @@ __device__ __forceinline__ bool grid_barrier(WsHeader *hdr, long long timeout_ns
 // are gone, then all meet at the grid barrier.  item_fn(ki, in, out, cin, cout, item, K, G)
 // processes one item and ends with a barrier of the block.
 template <typename F> __device__ __forceinline__ void persistent_loop(const PersistentJob &job, F &&item_fn) {
-  const int64_t nblocks_t = job.nmain + job.ntail;
+  int64_t nblocks_t = job.cnt[0];
+  for (int i = 1; i < job.nk; ++i) nblocks_t += job.cnt[i];
+  int ki = 0;
+  int64_t ki_end = job.cnt[0];  // the time block at which the next kval begins
   for (int64_t t = 0; t < nblocks_t; ++t) {
-    const int ki = (t < job.nmain) ? 0 : job.tail[t - job.nmain];
+    while (t >= ki_end) ki_end += job.cnt[++ki];
     const int K = job.kval[ki];
     const int G = job.Gval[ki];
     const int64_t ntiles = job.ntiles[ki];

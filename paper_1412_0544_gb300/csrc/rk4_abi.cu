@@ -41,15 +41,26 @@ struct WsLayout {
   size_t hdr, partials, result, chains, prefix, tiles, state, comp, u0, u1, acc, total;
 };
 
-// One launch plan: the k of every launch (or time block) and whether the result needs copying
-// back from the workspace because the count of ping-pong swaps is odd.
+// One launch plan: cnt[i] launches (or time blocks) of kval[i] steps, one i after the other, and
+// whether the result needs copying back from the workspace because their number is odd.
 struct Plan {
-  int64_t nmain = 0;            // launches with kval[0]
-  std::vector<int> tail;        // indices into kval
-  std::vector<int> kval;        // distinct k values, kval[0] = the main k
+  std::vector<int> kval;
+  std::vector<int64_t> cnt;
   bool copy_back = false;
-  int64_t count() const { return nmain + (int64_t)tail.size(); }
-  int k_at(int64_t i) const { return kval[i < nmain ? 0 : tail[i - nmain]]; }
+  void add(int k, int64_t times = 1) {
+    for (size_t i = 0; i < kval.size(); ++i)
+      if (kval[i] == k) {
+        cnt[i] += times;
+        return;
+      }
+    kval.push_back(k);
+    cnt.push_back(times);
+  }
+  int64_t count() const {
+    int64_t s = 0;
+    for (int64_t c : cnt) s += c;
+    return s;
+  }
 };
 
 }  // namespace
@@ -68,6 +79,10 @@ struct rk4_chain {
   int kernel = RK4_KERNEL_AUTO;
   bool tiling_auto = true;
   rk4_tiling tiling{};
+  rk4_tiling run{};  // what the current integration runs with (run_tiling), and its automatic choice
+  rk4_tiling auto_tiling{};
+  int64_t auto_steps = -1;
+  unsigned auto_version = 0;
   double t0 = 0.0;
   int64_t nstep = 0;
   bool graphs = true;
@@ -260,10 +275,10 @@ int tiling_max_threads(const rk4_chain *h, int v) {
 }
 
 void default_tiling(rk4_chain *h) {
-  // Seed choice from the register and shared-memory budget (the paper suggests sizing the
-  // cluster from the cache; here a tile should fill a block's registers): FP64 is bound by
-  // the FP64 pipe, so k = 1 keeps the redundant halo work minimal; FP32 is bandwidth-bound
-  // at k = 1, so several steps per launch pay off.
+  // The seed of the automatic choice, from the register and shared-memory budget (the paper
+  // suggests sizing the cluster from the cache; here a tile should fill a block's registers):
+  // what a handle runs with whose form has no measured costs (run_tiling), FP64 on the FP64 pipe
+  // alone, where k = 1 keeps the redundant halo work minimal.
   if (use_generic(h)) {
     h->tiling.block = 128;
     h->tiling.v = 2;
@@ -278,6 +293,7 @@ void default_tiling(rk4_chain *h) {
     h->tiling.k = h->fp32 ? 4 : 1;
   }
   h->tiling.G = tile_interior(h, h->tiling.block * h->tiling.v, h->tiling.k);
+  h->tiling_auto = true;
 }
 
 int64_t tiles_for(const rk4_chain *h, int G) {
@@ -310,36 +326,169 @@ int tile_interior(const rk4_chain *h, int W, int k) {
 }
 
 
-Plan make_plan(int64_t nsteps, int K) {
+// A chain: nsteps in an even number of launches of at most K steps (the state then ends where it
+// began), as few as possible and as equal as possible: a launch of k steps recomputes 2 H sites
+// per tile and step, H in proportion to k, so for a given number of launches equal ones waste
+// least (50 steps at K = 16: 13 + 13 + 12 + 12 instead of 16 + 16 + 16 + 2).
+Plan balanced_plan(int64_t nsteps, int K) {
+  int64_t L = (nsteps + K - 1) / K;
+  if (L % 2 == 1 && L < nsteps) ++L;
   Plan P;
-  P.kval.push_back(K);
+  P.copy_back = L % 2 == 1;
+  const int64_t base = nsteps / L, more = nsteps % L;
+  if (more > 0) P.add((int)base + 1, more);
+  P.add((int)base, L - more);
+  return P;
+}
+
+// A batch whose tiling the caller chose: K as often as it goes, then what is left, split in two
+// where that makes the number of launches even.
+Plan batch_plan(int64_t nsteps, int K) {
+  Plan P;
   const int64_t q = nsteps / K;
   const int r = (int)(nsteps % K);
-  auto kidx = [&](int k) {
-    for (size_t i = 0; i < P.kval.size(); ++i)
-      if (P.kval[i] == k) return (int)i;
-    P.kval.push_back(k);
-    return (int)P.kval.size() - 1;
-  };
-  P.nmain = q;
-  if (r > 0) P.tail.push_back(kidx(r));
-  if (P.count() % 2 == 1) {
-    if (r >= 2) {
-      P.tail.clear();
-      P.tail.push_back(kidx(r / 2));
-      P.tail.push_back(kidx(r - r / 2));
-    } else if (K >= 2 && q >= 1) {
-      P.nmain = q - 1;
-      std::vector<int> t;
-      t.push_back(kidx(K / 2));
-      t.push_back(kidx(K - K / 2));
-      for (int x : P.tail) t.push_back(x);
-      P.tail = t;
-    } else {
-      P.copy_back = true;
-    }
+  P.kval.push_back(K);
+  P.cnt.push_back(q);
+  if ((q + (r > 0 ? 1 : 0)) % 2 == 0) {
+    if (r > 0) P.add(r);
+  } else if (r >= 2) {
+    P.add(r / 2);
+    P.add(r - r / 2);
+  } else if (K >= 2 && q >= 1) {
+    P.cnt[0] = q - 1;
+    P.add(K / 2);
+    P.add(K - K / 2);
+    if (r > 0) P.add(r);
+  } else {
+    if (r > 0) P.add(r);
+    P.copy_back = true;
   }
   return P;
+}
+
+// A batch under the automatic tiling: the kval of every plan are the same (K and powers of two
+// below it), so that the batch's tables hold for any number of steps: no rebuild from one call
+// to the next, and a launch sequence captured by the caller stays good after calls of other
+// lengths.
+Plan batch_auto_plan(int64_t nsteps, int K) {
+  Plan P;
+  for (int k = K, i = 0; k >= 1 && i < kMaxDistinctK; k = k == 16 ? 4 : k / 2, ++i) {
+    P.add(k, nsteps / k);
+    nsteps %= k;
+  }
+  if (P.count() % 2 == 0) return P;
+  for (int i = (int)P.kval.size() - 2; i >= 0; --i)  // 16 -> 4 x 4, 8 -> 2 x 4, 4 -> 2 x 2, 2 -> 2 x 1
+    if (P.cnt[i] > 0) {
+      --P.cnt[i];
+      P.cnt[i + 1] += P.kval[i] / P.kval[i + 1];
+      return P;
+    }
+  P.copy_back = true;
+  return P;
+}
+
+Plan make_plan(const rk4_chain *h, int64_t nsteps, int K) {
+  if (h->nchains == 1) return balanced_plan(nsteps, K);
+  return h->tiling_auto ? batch_auto_plan(nsteps, K) : batch_plan(nsteps, K);
+}
+
+// What a launch costs, fitted on a GB300 (152 SMs, 2070 MHz) in us: A + max(B k, w (C + D k)) for k
+// steps when every SM gets w tiles.  A is the launch and the tile's way in and out, B a step's
+// latency when a tile has an SM to itself (1000 sites, k = 1 .. 16), C + D k the SM's time per tile
+// when it is full (2^22 sites).  Roessler; the harmonic chain's costs are in nearly the same
+// proportions.  The stages a generic step needs scale B and D (six: Dormand-Prince 5).
+struct TileCost {
+  int block, v;
+  float A, B, C, D;
+};
+const TileCost kCostFp64[] = {{64, 1, 2.7f, 1.20f, 0.47f, 0.307f}, {128, 1, 2.9f, 1.22f, 0.43f, 0.522f},
+                              {256, 1, 3.0f, 1.65f, 0.40f, 1.03f}, {512, 1, 3.4f, 2.64f, 1.25f, 2.10f},
+                              {256, 2, 3.6f, 2.84f, 1.40f, 2.11f}, {128, 4, 4.7f, 3.24f, 1.00f, 1.99f},
+                              {256, 4, 5.6f, 5.35f, 2.00f, 4.13f}};
+const TileCost kCostFp32[] = {{256, 1, 4.1f, 0.33f, 0.52f, 0.098f}, {128, 2, 4.9f, 0.32f, 0.50f, 0.060f},
+                              {256, 2, 5.2f, 0.37f, 1.20f, 0.122f}, {128, 4, 7.0f, 0.31f, 0.95f, 0.093f},
+                              {256, 4, 7.9f, 0.35f, 2.00f, 0.190f}, {512, 4, 7.5f, 0.62f, 4.60f, 0.390f}};
+const TileCost kCostHet64[] = {{64, 2, 5.8f, 1.78f, 0.95f, 0.54f}, {128, 2, 5.7f, 1.93f, 0.95f, 0.975f},
+                               {256, 2, 6.2f, 2.87f, 2.00f, 2.12f}};
+const TileCost kCostHet32[] = {{128, 2, 7.0f, 0.31f, 0.80f, 0.054f}, {256, 2, 7.3f, 0.37f, 1.75f, 0.115f},
+                               {128, 4, 10.5f, 0.29f, 1.60f, 0.080f}, {256, 4, 11.6f, 0.36f, 3.20f, 0.190f}};
+const TileCost kCostGen64[] = {{64, 2, 4.0f, 4.48f, 0.57f, 1.37f}, {128, 2, 3.8f, 4.75f, 0.55f, 2.10f},
+                               {256, 2, 4.2f, 6.70f, 1.10f, 5.10f}};
+const TileCost kCostGen32[] = {{128, 2, 5.3f, 0.80f, 0.55f, 0.27f}, {256, 2, 5.7f, 0.95f, 1.30f, 0.64f}};
+const TileCost kCostGen32Shape[] = {{128, 4, 7.0f, 0.47f, 0.65f, 0.28f}, {256, 4, 7.9f, 0.68f, 1.50f, 0.60f},
+                                    {512, 4, 7.5f, 1.32f, 3.80f, 1.20f}};
+
+// Tiles of a launch of k steps at block x v, in units of whole tiles (from at most 512 of a
+// batch's chains).
+double tiles_estimate(const rk4_chain *h, int W, int v, int k) {
+  const int H = halo(h, k), G = tile_interior(h, W, k);
+  const int64_t step = std::max<int64_t>(1, h->nchains / 512);
+  double slots = 0.0;
+  int64_t seen = 0, sites = 0;
+  for (int64_t c = 0; c < h->nchains; c += step, ++seen) {
+    const int64_t n = h->chains[c].n, full = n / G, rem = n % G;
+    sites += n;
+    slots += (double)full * W;
+    if (rem > 0) slots += packed_batch(h) ? (double)((rem + 2 * H + v - 1) / v * v) : (double)W;
+  }
+  return slots / W * ((double)h->total / (double)sites);
+}
+
+// The tiling an integration of nsteps runs with.  One that was set or tuned is taken as it is.
+// The automatic choice (whose seed rk4_chain_get_tiling reports) depends on the sites and the
+// steps: a short chain needs small tiles to reach every SM and many steps per launch to pay for
+// the launch, a long one wide tiles.  Measured against the seed, us per step: FP64 1000 sites 10.7
+// -> 1.6 (128 x 1, k = 8), 65537 sites 10.7 -> 3.2 (512 x 1, k = 8), 2^22 sites 164 -> 126 (256 x 4,
+// k = 8); FP32 65537 sites 2.6 -> 0.8 (128 x 2, k = 16), 2^22 sites 18.2 -> 10.0 (256 x 4, k = 16).
+// The FP64 form (coefficients outside split_allowed) keeps the seed.
+rk4_tiling run_tiling(rk4_chain *h, int64_t nsteps) {
+  if (!h->tiling_auto) return h->tiling;
+  if (h->nchains > 1) nsteps = 1024;  // a batch's tables must not depend on the steps
+  if (h->auto_steps == nsteps && h->auto_version == h->config_version) return h->auto_tiling;
+  const TileCost *cost = nullptr;
+  int n = 0;
+  float stages = 1.f;
+#define RK4_COST(T) (cost = T, n = (int)(sizeof(T) / sizeof(T[0])))
+  if (use_generic(h)) {
+    stages = (float)needed_stages(h) / 6.f;
+    if (!h->fp32 && use_split(h)) RK4_COST(kCostGen64);
+    else if (h->fp32 && gen_compiled(h->tab)) RK4_COST(kCostGen32Shape);
+    else if (h->fp32) RK4_COST(kCostGen32);
+  } else if (use_het(h)) {
+    if (h->fp32) RK4_COST(kCostHet32);
+    else if (use_split(h)) RK4_COST(kCostHet64);
+  } else if (h->fp32) {
+    RK4_COST(kCostFp32);
+  } else if (use_split(h)) {
+    RK4_COST(kCostFp64);
+  }
+#undef RK4_COST
+  rk4_tiling best = h->tiling;
+  double best_us = 1e300;
+  const double sms = sm_count();
+  for (int c = 0; c < n; ++c) {
+    int last = 0;
+    if (cost[c].block > tiling_max_threads(h, cost[c].v)) continue;
+    for (int kmax : {1, 2, 3, 4, 5, 6, 8, 10, 12, 16}) {
+      if (h->nchains > 1 && (kmax & (kmax - 1)) != 0) continue;
+      const Plan P = make_plan(h, nsteps, kmax);
+      const int k = P.kval[0], W = cost[c].block * cost[c].v;
+      if (k == last || !tiling_valid(h, cost[c].block, cost[c].v, k)) continue;
+      last = k;
+      double w = tiles_estimate(h, W, cost[c].v, k) / sms;
+      w = w <= 4.0 ? std::ceil(w) : w + 0.5;  // few tiles: the busiest SM decides
+      const double us = (double)P.count() *
+                        (cost[c].A + std::max((double)cost[c].B * stages * k, w * (cost[c].C + cost[c].D * stages * k)));
+      if (us < best_us) {
+        best_us = us;
+        best = {cost[c].block, cost[c].v, k, tile_interior(h, W, k)};
+      }
+    }
+  }
+  h->auto_steps = nsteps;
+  h->auto_version = h->config_version;
+  h->auto_tiling = best;
+  return best;
 }
 
 cudaError_t ensure_pinned(rk4_chain *h) {
@@ -389,10 +538,11 @@ BatchTiles dev_ktables(const rk4_chain *h, const char *ws, const WsLayout &L, in
   return bt;
 }
 
-// Fill the tile tables of the first nslots k slots on the device (after upload_tables).
-cudaError_t fill_tile_tables(const rk4_chain *h, char *ws, const WsLayout &L, int nslots, cudaStream_t st) {
+// Fill the tile tables of the k slots that a plan uses on the device (after upload_tables).
+cudaError_t fill_tile_tables(const rk4_chain *h, char *ws, const WsLayout &L, const Plan &P, cudaStream_t st) {
   if (h->nchains == 1) return cudaSuccess;
-  for (int i = 0; i < nslots; ++i) {
+  for (int i = 0; i < (int)P.kval.size(); ++i) {
+    if (P.cnt[i] == 0) continue;
     const BatchTiles bt = dev_ktables(h, ws, L, i);
     if (!bt.tile_chain) continue;
     const cudaError_t e =
@@ -467,7 +617,7 @@ int64_t pack_segments(const rk4_chain *h, int G, int H, int W, int v, int32_t *p
 cudaError_t prepare_tables(rk4_chain *h, const std::vector<int> &kval, int W) {
   if (h->nchains == 1) return cudaSuccess;
   const int packed = packed_batch(h) ? 1 : 0;
-  if (h->tables_k == kval && h->tables_W == W && h->tables_v == h->tiling.v && h->tables_halo == halo(h, 1) &&
+  if (h->tables_k == kval && h->tables_W == W && h->tables_v == h->run.v && h->tables_halo == halo(h, 1) &&
       h->tables_packed == packed)
     return cudaSuccess;
   cudaError_t e = cudaStreamSynchronize(h->stream);
@@ -483,11 +633,11 @@ cudaError_t prepare_tables(rk4_chain *h, const std::vector<int> &kval, int W) {
     }
     t.prefix[h->nchains] = (int32_t)acc;
     h->nfull[i] = acc;
-    h->npacked[i] = packed ? pack_segments(h, G, H, W, h->tiling.v, t.pack_prefix, t.segs) : 0;
+    h->npacked[i] = packed ? pack_segments(h, G, H, W, h->run.v, t.pack_prefix, t.segs) : 0;
   }
   h->tables_k = kval;
   h->tables_W = W;
-  h->tables_v = h->tiling.v;
+  h->tables_v = h->run.v;
   h->tables_halo = halo(h, 1);
   h->tables_packed = packed;
   return cudaSuccess;
@@ -506,7 +656,7 @@ const ChainDesc *dev_chains(const rk4_chain *h, char *ws, const WsLayout &L) {
 cudaError_t enqueue_integrate(rk4_chain *h, int kernel, void *state, void *comp, char *ws, const WsLayout &L,
                               const Plan &P, int64_t nsteps, cudaStream_t st) {
   const CoefD cf = coef(h);
-  const int W = h->tiling.block * h->tiling.v;
+  const int W = h->run.block * h->run.v;
   // a fresh status word (and barrier counters) for every integration
   cudaError_t e = cudaMemsetAsync(ws + L.hdr, 0, sizeof(WsHeader), st);
   if (e != cudaSuccess) return e;
@@ -571,7 +721,7 @@ cudaError_t enqueue_integrate(rk4_chain *h, int kernel, void *state, void *comp,
   }
   void *wsS = ws + L.state;
   void *wsC = h->fp32 ? (void *)(ws + L.comp) : nullptr;
-  e = fill_tile_tables(h, ws, L, (int)P.kval.size(), st);
+  e = fill_tile_tables(h, ws, L, P, st);
   if (e != cudaSuccess) return e;
   if (kernel == RK4_KERNEL_BLOCKED) {
     BlockedJob j{};
@@ -583,10 +733,11 @@ cudaError_t enqueue_integrate(rk4_chain *h, int kernel, void *state, void *comp,
     j.total = h->total;
     j.packed = packed_batch(h) ? 1 : 0;
     j.split = use_split(h) ? 1 : 0;
-    for (int64_t i = 0; i < P.count(); ++i) {
-      const int k = P.k_at(i);
-      int ki = 0;
-      while (P.kval[ki] != k) ++ki;
+    int ki = 0;
+    int64_t left = P.cnt[0];
+    for (int64_t i = 0; i < P.count(); ++i, --left) {
+      while (left == 0) left = P.cnt[++ki];
+      const int k = P.kval[ki];
       j.K = k;
       j.G = tile_interior(h, W, k);
       if (h->nchains > 1) {
@@ -603,10 +754,10 @@ cudaError_t enqueue_integrate(rk4_chain *h, int kernel, void *state, void *comp,
       j.cin = even ? comp : wsC;
       j.cout = even ? wsC : comp;
       if (use_generic(h))
-        e = launch_gen_blocked(h->model, h->fp32, coupling_range(h), h->tiling.v, h->tiling.block, j, cf, h->tab,
+        e = launch_gen_blocked(h->model, h->fp32, coupling_range(h), h->run.v, h->run.block, j, cf, h->tab,
                                h->dt, halo(h, k), st);
       else
-        e = launch_blocked(h->model, h->fp32, h->tiling.v, h->tiling.block, j, cf, st);
+        e = launch_blocked(h->model, h->fp32, h->run.v, h->run.block, j, cf, st);
       if (e != cudaSuccess) return e;
     }
   } else {  // persistent
@@ -622,6 +773,7 @@ cudaError_t enqueue_integrate(rk4_chain *h, int kernel, void *state, void *comp,
     int64_t maxtiles = 0;
     for (int i = 0; i < j.nk; ++i) {
       j.kval[i] = P.kval[i];
+      j.cnt[i] = P.cnt[i];
       j.Gval[i] = tile_interior(h, W, P.kval[i]);
       if (h->nchains > 1) {
         j.bt[i] = dev_ktables(h, ws, L, i);
@@ -629,11 +781,8 @@ cudaError_t enqueue_integrate(rk4_chain *h, int kernel, void *state, void *comp,
       } else {
         j.ntiles[i] = tiles_for(h, j.Gval[i]);
       }
-      maxtiles = std::max(maxtiles, j.ntiles[i]);
+      if (P.cnt[i] > 0) maxtiles = std::max(maxtiles, j.ntiles[i]);
     }
-    j.nmain = P.nmain;
-    j.ntail = (int)P.tail.size();
-    for (int i = 0; i < j.ntail; ++i) j.tail[i] = P.tail[i];
     j.hdr = reinterpret_cast<WsHeader *>(ws + L.hdr);
     j.total = h->total;
     j.split = use_split(h) ? 1 : 0;
@@ -647,10 +796,10 @@ cudaError_t enqueue_integrate(rk4_chain *h, int kernel, void *state, void *comp,
       j.timeout_ns = h->timeout_set ? h->timeout_ns : std::max<long long>(h->timeout_ns, (long long)(20.0 * est_ns));
     }
     j.extra_arrivals = 0;
-    int grid = persistent_max_grid(h->model, h->fp32, h->tiling.v, h->tiling.block, use_split(h));
+    int grid = persistent_max_grid(h->model, h->fp32, h->run.v, h->run.block, use_split(h));
     if (grid <= 0) return cudaErrorInvalidConfiguration;
     grid = (int)std::min<int64_t>(grid, std::max<int64_t>(1, maxtiles));
-    e = launch_persistent(h->model, h->fp32, h->tiling.v, h->tiling.block, grid, j, cf, st);
+    e = launch_persistent(h->model, h->fp32, h->run.v, h->run.block, grid, j, cf, st);
     if (e != cudaSuccess) return e;
   }
   if (P.copy_back) {
@@ -681,14 +830,14 @@ int integrate_impl(rk4_chain *h, void *state, void *comp, void *ws, size_t ws_by
   if (ws_bytes < L.total) return RK4_ENOMEM_WS;
   if (nsteps == 0) return RK4_OK;
   if (ensure_pinned(h) != cudaSuccess) return RK4_ECUDA;
-  const int K = (kernel == RK4_KERNEL_STAGED) ? 1 : h->tiling.k;
-  const Plan P = make_plan(nsteps, kernel == RK4_KERNEL_STAGED ? 1 : K);
+  h->run = run_tiling(h, nsteps);
+  const Plan P = make_plan(h, nsteps, kernel == RK4_KERNEL_STAGED ? 1 : h->run.k);
   if (kernel != RK4_KERNEL_STAGED) {
     // tile counts must fit a 1-D grid and the int32 prefix tables
     const int kmax = *std::max_element(P.kval.begin(), P.kval.end());
-    if (tiles_for(h, tile_interior(h, h->tiling.block * h->tiling.v, kmax)) > 0x7fffffffLL) return RK4_EUNSUPPORTED;
+    if (tiles_for(h, tile_interior(h, h->run.block * h->run.v, kmax)) > 0x7fffffffLL) return RK4_EUNSUPPORTED;
   }
-  if (prepare_tables(h, P.kval, h->tiling.block * h->tiling.v) != cudaSuccess) return RK4_ECUDA;
+  if (prepare_tables(h, P.kval, h->run.block * h->run.v) != cudaSuccess) return RK4_ECUDA;
   char *w = static_cast<char *>(ws);
 
   const bool use_graph = h->graphs && (kernel != RK4_KERNEL_BLOCKED || P.count() > 1);
@@ -702,9 +851,9 @@ int integrate_impl(rk4_chain *h, void *state, void *comp, void *ws, size_t ws_by
   key.comp = comp;
   key.ws = ws;
   key.nsteps = nsteps;
-  key.block = h->tiling.block;
-  key.v = h->tiling.v;
-  key.k = h->tiling.k;
+  key.block = h->run.block;
+  key.v = h->run.v;
+  key.k = h->run.k;
   key.timeout = h->timeout_ns;
   key.sp = h->site_params;
   key.generic = use_generic(h) ? 1 + (int)h->gen_version : 0;
@@ -954,8 +1103,9 @@ int rk4d::prepare_integrate(rk4_chain *h, int64_t nsteps) {
   if (!h || nsteps < 1) return RK4_EINVAL;
   if (ensure_pinned(h) != cudaSuccess) return RK4_ECUDA;
   const int kernel = effective_kernel(h);
-  const Plan P = make_plan(nsteps, kernel == RK4_KERNEL_STAGED ? 1 : h->tiling.k);
-  return prepare_tables(h, P.kval, h->tiling.block * h->tiling.v) == cudaSuccess ? RK4_OK : RK4_ECUDA;
+  h->run = run_tiling(h, nsteps);
+  const Plan P = make_plan(h, nsteps, kernel == RK4_KERNEL_STAGED ? 1 : h->run.k);
+  return prepare_tables(h, P.kval, h->run.block * h->run.v) == cudaSuccess ? RK4_OK : RK4_ECUDA;
 }
 
 int rk4d::scheme_reach(const rk4_chain *h, int *s, int *range) {
@@ -1057,7 +1207,6 @@ int rk4_chain_set_tiling(rk4_chain *h, int block, int v, int k) {
   if (!h) return RK4_EINVAL;
   h->config_version++;
   if (block == 0) {
-    h->tiling_auto = true;
     default_tiling(h);
     return RK4_OK;
   }
@@ -1192,12 +1341,14 @@ int rk4_debug_barrier_timeout(rk4_chain *h, void *state, void *comp, void *ws, s
   const WsLayout L = layout(h, RK4_KERNEL_PERSISTENT);
   if (ws_bytes < L.total) return RK4_ENOMEM_WS;
   if (ensure_pinned(h) != cudaSuccess) return RK4_ECUDA;
-  const Plan P = make_plan(h->tiling.k, h->tiling.k);  // one time block
+  h->run = h->tiling;
   const int W = h->tiling.block * h->tiling.v;
+  Plan P;  // one time block
+  P.add(h->tiling.k);
   if (prepare_tables(h, P.kval, W) != cudaSuccess) return RK4_ECUDA;
   char *w = static_cast<char *>(ws);
   if (upload_tables(h, w, L, h->stream) != cudaSuccess) return RK4_ECUDA;
-  if (fill_tile_tables(h, w, L, 1, h->stream) != cudaSuccess) return RK4_ECUDA;
+  if (fill_tile_tables(h, w, L, P, h->stream) != cudaSuccess) return RK4_ECUDA;
   PersistentJob j{};
   j.bufA = state;
   j.bufB = w + L.state;
@@ -1216,8 +1367,7 @@ int rk4_debug_barrier_timeout(rk4_chain *h, void *state, void *comp, void *ws, s
   } else {
     j.ntiles[0] = tiles_for(h, j.Gval[0]);
   }
-  j.nmain = 1;
-  j.ntail = 0;
+  j.cnt[0] = 1;
   j.hdr = reinterpret_cast<WsHeader *>(w + L.hdr);
   j.total = h->total;
   j.split = use_split(h) ? 1 : 0;
@@ -1259,6 +1409,8 @@ int rk4_chain_autotune(rk4_chain *h, void *state, void *comp, void *ws, size_t w
   const bool try_staged = on_auto && ws_bytes >= layout(h, RK4_KERNEL_STAGED).total;
   if (kernels.empty() && !try_staged) return RK4_ENOMEM_WS;
   const rk4_tiling saved = h->tiling;
+  const bool saved_auto = h->tiling_auto;
+  h->tiling_auto = false;  // the candidates run as they are
   const int saved_tuned = h->tuned_kernel;
   int best_kernel = 0;
   const bool saved_graphs = h->graphs;
@@ -1266,6 +1418,7 @@ int rk4_chain_autotune(rk4_chain *h, void *state, void *comp, void *ws, size_t w
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) {
     h->graphs = saved_graphs;
+    h->tiling_auto = saved_auto;
     return RK4_ECUDA;
   }
   // Per-step time of an integration of `steps` after a warm-up of `warm`, or a negative value
@@ -1329,13 +1482,14 @@ int rk4_chain_autotune(rk4_chain *h, void *state, void *comp, void *ws, size_t w
   h->graphs = saved_graphs;
   if (rc != RK4_OK || best_ms >= 1e30f) {
     h->tiling = saved;
+    h->tiling_auto = saved_auto;
     h->tuned_kernel = saved_tuned;
     return rc != RK4_OK ? rc : RK4_ECUDA;
   }
   h->tuned_kernel = on_auto ? best_kernel : 0;
   h->config_version++;
   h->tiling = have_tiling ? best_t : saved;
-  h->tiling_auto = !have_tiling && h->tiling_auto;
+  h->tiling_auto = !have_tiling && saved_auto;
   if (best) *best = h->tiling;
   return RK4_OK;
 }

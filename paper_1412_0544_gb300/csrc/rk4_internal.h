@@ -150,9 +150,7 @@ struct PersistentJob {
   int kval[4];                  // steps per time block
   int Gval[4];                  // interior sites per tile for each k
   int64_t ntiles[4];            // tiles per time block for each k
-  int64_t nmain;                // leading time blocks that use kval[0]
-  int ntail;                    // trailing time blocks (0..3)
-  int tail[3];                  // their indices into kval
+  int64_t cnt[4];               // time blocks of kval[0], then of kval[1], ...
   WsHeader *hdr;                // status word and barrier counters (zeroed before launch)
   long long timeout_ns;         // bound on any single barrier wait
   int extra_arrivals;           // test hook: barrier waits for this many blocks that never come
@@ -232,6 +230,7 @@ cudaError_t launch_gen_blocked(int model, bool fp32, int range, int v, int block
                                const CoefD &cf, const TableauD &tb, double dt, int H, cudaStream_t st);
 size_t gen_blocked_smem_bytes(int model, bool fp32, int v, int block, const TableauD &tb);
 int gen_blocked_max_threads(int model, bool fp32, int range, int v, const TableauD &tb);
+bool gen_compiled(const TableauD &tb);  // whether FP32 tile kernels are compiled for the tableau's shape
 size_t blocked_smem_bytes(int model, bool fp32, int v, int block, bool het = false);  // either FP64 form fits
 int blocked_max_threads(int model, bool fp32, int v, bool het = false);
 
