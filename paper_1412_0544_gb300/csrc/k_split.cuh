@@ -3,10 +3,10 @@
 // (k_split_roessler.cu, k_split_harmonic.cu), so that they compile side by side.
 //
 // What bounds it: 13 FP64 instructions per site-step (Roessler: 7 for the first slope, 6 for the
-// update; harmonic 8) at 0.627 T/s allow 4.8e10 site-steps/s; beside them about 300 FP32
+// update; harmonic 8) at 0.6 T/s allow 4.6e10 site-steps/s; beside them about 300 FP32
 // operations (packed two sites per instruction, 40 T lane-operations/s) and 110 integer ones.
-// Measured at N = 2^24 against the FP64 form (49 instructions, 1.23e10 site-steps/s): 3.45e10 at
-// 256 x 4 x 8, 3.33e10 at 128 x 2 x 4; harmonic 5.8e10 against 1.90e10.
+// Measured at N = 2^24 against the FP64 form (49 instructions, 1.23e10 site-steps/s): 3.64e10 at
+// 256 x 4 x 4, 3.32e10 at 128 x 2 x 4; harmonic 6.4e10 (128 x 4 x 4) against 1.90e10.
 #pragma once
 #include "k_grid_barrier.cuh"
 #include "rk4_tile.cuh"

@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(256) k_staged_split(StagedJob job, Coef<double
       split_update<float>(3, k1[q], n[q], d[q], N[q]);
       double nd;
       join(N[q], &nd, 1);
-      const double r = split_final(y[q], K1[i * D + q], nd, s);
+      const double r = split_final(y[q], K1[i * D + q], nd, 6.0, s.w);
       Y[i * D + q] = r;
       wide |= !split_in_range<MODEL>(r);
       bad |= nonfinite(r);

@@ -386,8 +386,8 @@ template <typename T> __device__ __forceinline__ FPair<T> pair_mul(const FPair<T
   return {vmul(c.h, v.h), e};
 }
 // y + (tau / 3) (6 K1 - N).
-__device__ __forceinline__ double split_final(double y, double k1, double N, const SplitCoef &s) {
-  return fma(s.w, fma(6.0, k1, -N), y);
+__device__ __forceinline__ double split_final(double y, double k1, double N, double six, double w) {
+  return fma(w, fma(six, k1, -N), y);
 }
 
 }  // namespace rk4d

@@ -261,10 +261,44 @@ __device__ __forceinline__ void tile_advance(R (&y)[V][Dim<MODEL>::D], R (&cmp)[
 // slope's pairs, the base values of z) lies in a record of the thread's own in shared memory,
 // rec, of split_record_words() 8-byte words -- an odd number, so that the threads of a warp reach
 // the same word of their records without bank conflicts.
+// KREG: the coupling strength is a value of the thread's own (cf.kappa; packed tiles).
 template <int MODEL, int V> __host__ __device__ constexpr int split_record_words() {
   return (3 * V * Dim<MODEL>::D + (MODEL == ROESSLER ? 2 * V : 0)) | 1;
 }
-template <int MODEL, int V, bool MASK, bool HET, bool PARK = false>
+// The FP64 constants of a split step, eight doubles for each warp in shared memory, which a step
+// loads into registers: {1, -2, kappa, a | w2, c | -0, b, 6, tau / 3}.  A DFMA whose operands are
+// three different registers was measured to issue every 16 cycles per SM and one with two (the third
+// a constant or an immediate), or a DADD, every 19 (0.595 and 0.501 T/s, 4 to 32 warps per SM, any
+// number of independent chains).  Left to itself the compiler feeds the constants from the
+// constant bank, and 11 of the step's 13 instructions are of the slow kind.  Not with one site per
+// thread, the form of short chains, which waits for latencies and not for the pipe (1000 sites,
+// 128 x 1 x 8: 1.57 us per step without, 1.64 with).  N = 2^24, site-steps/s,
+// before -> after: 256 x 4 x 8 3.41e10 -> 3.57e10, 256 x 4 x 4 3.42e10 -> 3.64e10, harmonic 128 x 4 x 4
+// 5.74e10 -> 6.43e10.
+__device__ __forceinline__ double *fp64_const_slot() {
+  __shared__ __align__(16) double s[32][8];
+  return s[threadIdx.x >> 5];
+}
+template <int MODEL>
+__device__ __forceinline__ void fp64_const_store(const Coef<double> &cf, double w) {
+  double *s = fp64_const_slot();
+  if ((threadIdx.x & 31) == 0) {
+    s[0] = 1.0;
+    s[1] = -2.0;
+    s[2] = cf.kappa;
+    s[3] = MODEL == ROESSLER ? cf.a : cf.w2;
+    s[4] = MODEL == ROESSLER ? cf.c : -0.0;
+    s[5] = cf.b;
+    s[6] = 6.0;
+    s[7] = w;
+  }
+  __syncwarp();
+}
+__device__ __forceinline__ void ld_shared2(unsigned a, double &u, double &v) {
+  asm volatile("ld.shared.v2.f64 {%0, %1}, [%2];" : "=d"(u), "=d"(v) : "r"(a) : "memory");
+}
+
+template <int MODEL, int V, bool MASK, bool HET, bool PARK = false, bool KREG = false>
 __device__ __forceinline__ void split_advance(double (&y)[V][Dim<MODEL>::D], uint32_t ghost, int K,
                                               const Coef<double> &cf, const SplitCoef &sc, double *edge,
                                               const double *spd = nullptr, const f32x2 *spf = nullptr,
@@ -310,6 +344,12 @@ __device__ __forceinline__ void split_advance(double (&y)[V][Dim<MODEL>::D], uin
     }
   };
   const StageCoef<T> sc0 = stage_coef<T>(sc);
+  constexpr bool kConst = V > 1;
+  unsigned fc = 0;
+  if constexpr (kConst) {
+    fp64_const_store<MODEL>(cf, sc.w);
+    fc = smem_addr(fp64_const_slot());
+  }
   static_assert(!PARK || V >= 2, "records hold packed pairs");
   double *rk = rec + V * D;                                      // first slope, FP64
   f32x2 *rp = reinterpret_cast<f32x2 *>(rec + 2 * V * D);        // its pairs: h, l of each (p, component)
@@ -337,17 +377,35 @@ __device__ __forceinline__ void split_advance(double (&y)[V][Dim<MODEL>::D], uin
 #pragma unroll
       for (int v = 0; v < V; ++v) xs[v] = (MASK && ((ghost >> v) & 1u)) ? 0.0 : y[v][0];
       exchange(0, xs[0], xs[V - 1], left, right);
+      double one = cf.one, m2 = -2.0, kap = cf.kappa, p0 = MODEL == ROESSLER ? cf.a : cf.w2;
+      double p1 = MODEL == ROESSLER ? cf.c : -0.0, p2 = cf.b;
+      if constexpr (kConst) {
+        ld_shared2(fc, one, m2);
+        ld_shared2(fc + 16, kap, p0);
+        ld_shared2(fc + 32, p1, p2);
+        if constexpr (KREG) kap = cf.kappa;
+      }
 #pragma unroll
       for (int v = 0; v < V; ++v) {
         const double xl = (v == 0) ? left : xs[v - 1];
         const double xr = (v == V - 1) ? right : xs[v + 1];
         if constexpr (HET) {
-          double p[Dim<MODEL>::P];
-#pragma unroll
-          for (int i = 0; i < Dim<MODEL>::P; ++i) p[i] = spd[(v * Dim<MODEL>::P + i) * blockDim.x];
-          slope<double, MODEL>(y[v], xl, xr, site_coef<double, MODEL>(cf, p), k1d[v]);
+          const double *q = spd + v * Dim<MODEL>::P * blockDim.x;
+          p0 = q[0];
+          if constexpr (MODEL == ROESSLER) {
+            p2 = q[blockDim.x];
+            p1 = q[2 * blockDim.x];
+          }
+          kap = q[(Dim<MODEL>::P - 1) * blockDim.x];
+        }
+        const double lap = fma(m2, y[v][0], fma(xl, one, xr));  // as slope() computes it
+        if constexpr (MODEL == ROESSLER) {
+          k1d[v][0] = fma(kap, lap, -fma(y[v][1], one, y[v][2]));
+          k1d[v][1] = fma(p0, y[v][1], y[v][0]);
+          k1d[v][2] = fma(y[v][2], y[v][0], fma(-p1, y[v][2], p2));
         } else {
-          slope<double, MODEL>(y[v], xl, xr, cf, k1d[v]);
+          k1d[v][0] = y[v][1];
+          k1d[v][1] = fma(kap, lap, -fma(p0, y[v][0], p1));  // p1 = -0: the rounded product
         }
       }
 #pragma unroll
@@ -434,6 +492,8 @@ __device__ __forceinline__ void split_advance(double (&y)[V][Dim<MODEL>::D], uin
         }
       }
     }
+    double six = 6.0, w = sc.w;
+    if constexpr (kConst) ld_shared2(fc + 48, six, w);
 #pragma unroll
     for (int p = 0; p < P; ++p)
 #pragma unroll
@@ -441,11 +501,11 @@ __device__ __forceinline__ void split_advance(double (&y)[V][Dim<MODEL>::D], uin
         double nd[2];
         join(N[p][i], nd, 1);
         if constexpr (PARK) {
-          rec[p * D + i] = split_final(rec[p * D + i], rk[p * D + i], nd[0], sc);
-          rec[(p + P) * D + i] = split_final(rec[(p + P) * D + i], rk[(p + P) * D + i], nd[1], sc);
+          rec[p * D + i] = split_final(rec[p * D + i], rk[p * D + i], nd[0], six, w);
+          rec[(p + P) * D + i] = split_final(rec[(p + P) * D + i], rk[(p + P) * D + i], nd[1], six, w);
         } else {
-          y[p][i] = split_final(y[p][i], k1d[p][i], nd[0], sc);
-          if constexpr (V > 1) y[p + P][i] = split_final(y[p + P][i], k1d[p + P][i], nd[1], sc);
+          y[p][i] = split_final(y[p][i], k1d[p][i], nd[0], six, w);
+          if constexpr (V > 1) y[p + P][i] = split_final(y[p + P][i], k1d[p + P][i], nd[1], six, w);
         }
       }
   }
@@ -947,7 +1007,7 @@ __device__ __forceinline__ bool packed_tile_item(const R *__restrict__ in, R *__
     split_set_kappa(sc, c.kappa);
     double *rec = nullptr;
     if constexpr (PARK) rec = tl + threadIdx.x * split_record_words<MODEL, V>();
-    split_advance<MODEL, V, true, false, PARK>(y, ghost, K, c, sc, edge, nullptr, nullptr, rec);
+    split_advance<MODEL, V, true, false, PARK, true>(y, ghost, K, c, sc, edge, nullptr, nullptr, rec);
     if constexpr (PARK) __syncthreads();
   } else {
     tile_advance<R, MODEL, V, KAHAN, true>(y, cmp, ghost, K, c, edge);
