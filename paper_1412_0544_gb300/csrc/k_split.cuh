@@ -5,33 +5,60 @@
 // What bounds it: 13 FP64 instructions per site-step (Roessler: 7 for the first slope, 6 for the
 // update; harmonic 8) at 0.6 T/s allow 4.6e10 site-steps/s; beside them about 300 FP32
 // operations (packed two sites per instruction, 40 T lane-operations/s) and 110 integer ones.
-// Measured at N = 2^24 against the FP64 form (49 instructions, 1.23e10 site-steps/s): 3.64e10 at
-// 256 x 4 x 4, 3.32e10 at 128 x 2 x 4; harmonic 6.4e10 (128 x 4 x 4) against 1.90e10.
+// Measured at N = 2^24 against the FP64 form (49 instructions, 1.23e10 site-steps/s): 3.68e10 at
+// 256 x 2 x 4 and 128 x 4 x 4; harmonic 6.4e10 (128 x 4 x 4) against 1.90e10.
 #pragma once
 #include "k_grid_barrier.cuh"
 #include "rk4_tile.cuh"
 
 namespace rk4d {
 
-// Largest block an instantiation is compiled for.  With four sites per thread blocks of up to 256
-// threads have an instantiation of their own, which may use more registers than the one for 512.
-__host__ __device__ constexpr int split_small_block(int v) { return v == 4 ? 256 : max_threads_for(v); }
-// Whether an instantiation parks (split_advance): with four sites per thread the Roessler step
-// holds 241 registers, one block of 256 threads per SM (FP64 pipe 39 % busy); parked it fits 128
-// and two blocks (76 %): N = 2^24, 256 x 4, k = 2: 2.3e10 -> 3.2e10 site-steps/s, k = 8 3.45e10.
-// With two sites (114 registers instead of 128) it measured 2 % slower at 128 threads, and the
-// harmonic step, which fits 126 registers as it is, 3 % slower.  Heterogeneous tiles already hold
-// their parameters in shared memory.
-__host__ __device__ constexpr bool split_parks(int model, int v, int nt, bool het) {
-  return model == ROESSLER && !het && v == 4 && nt <= 256;
+// Sites per thread of the kernel that runs tiles of block x v sites.  The Roessler step takes two (a
+// packed pair) for whatever v > 1, parked in 64 registers (split_advance), so that an SM holds 32
+// warps: N = 2^24, 256 x 2 x 4, 3.10e10 site-steps/s unparked (128 registers, 16 warps) -> 3.68e10;
+// 128 x 4 x 4 with four per thread (parked, 126 registers) 3.52e10 -> 3.68e10.  Tiles of 1024 sites,
+// of which an SM holds two either way, keep four: 256 x 4 x 1 2.71e10 against 2.51e10, x 2 3.27e10
+// against 3.25e10, x 8 3.57e10 against 3.54e10.  One site per thread (nothing to pack, 64 registers as
+// it is) keeps a step shortest where tiles are few.  The harmonic step (98 to 128 registers, only state
+// and slope to park) was faster with the tiling's own v: 128 x 4 x 4 6.43e10 against 6.09e10.
+// Heterogeneous tiles hold their parameters in shared memory and have no room for records; two
+// sites per thread there too, up to 512 threads (N = 2^22: 256 x 4 x 2 1.79e10 -> 1.99e10, 128 x 4 x 4
+// 2.70e10 -> 2.97e10).
+__host__ __device__ constexpr int split_lanes(int model, int v, int block, bool het) {
+  if (model != ROESSLER || v == 1) return v;
+  if (het) return block * v > 1024 ? v : 2;
+  return v >= 4 && block * v == 1024 ? 4 : 2;
 }
-__host__ __device__ constexpr int split_min_blocks(int model, int v, int nt, bool het) {
-  return split_parks(model, v, nt, het) ? 2 : 0;
+__host__ __device__ constexpr bool split_parks(int model, int v, bool het) {
+  return model == ROESSLER && v >= 2 && !het;
 }
-template <int MODEL, int V, bool HET, int NT> static size_t split_smem_bytes(int block) {
+// Largest block and resident blocks of an instantiation.
+__host__ __device__ constexpr int split_max_threads(int model, int v, bool het) {
+  return split_parks(model, v, het) ? (v == 2 ? 1024 : 256) : max_threads_for(v);
+}
+__host__ __device__ constexpr int split_min_blocks(int model, int v, bool het) {
+  return split_parks(model, v, het) && v == 4 ? 2 : 0;
+}
+template <int MODEL, int V, bool HET> static size_t split_smem_bytes(int block) {
   const size_t plain = blocked_smem_bytes(MODEL, false, V, block, HET);
   const size_t parked = sizeof(double) * ((size_t)edge_values(V) + (size_t)block * split_record_words<MODEL, V>());
-  return split_parks(MODEL, V, NT, HET) ? std::max(plain, parked) : plain;
+  return split_parks(MODEL, V, HET) ? std::max(plain, parked) : plain;
+}
+// fn(V, NT, threads) with V and NT compile-time, for tiles of block x v sites.
+template <int MODEL, bool HET, typename R, typename F> static R split_dispatch(int v, int block, R none, F &&fn) {
+  const int lanes = split_lanes(MODEL, v, block, HET), threads = block * v / lanes;
+  auto with = [&](auto vc) -> R {
+    return fn(vc, std::integral_constant<int, split_max_threads(MODEL, decltype(vc)::value, HET)>(), threads);
+  };
+  if constexpr (!HET) {
+    if (lanes == 1) return with(std::integral_constant<int, 1>());
+  }
+  if (lanes == 2) return with(std::integral_constant<int, 2>());
+  if (lanes == 4) return with(std::integral_constant<int, 4>());
+  if constexpr (MODEL == HARMONIC && !HET) {
+    if (lanes == 8) return with(std::integral_constant<int, 8>());
+  }
+  return none;
 }
 
 // An item outside the split's range, in the FP64 form.  Not inlined: it is rare, and its
@@ -64,8 +91,8 @@ __device__ __noinline__ void split_packed_call(const double *in, double *out, co
 
 // The split form of k_blocked: one block per item, a packed batch's packed tiles first.
 template <int MODEL, int V, bool HET, bool PACKED, int NT>
-__global__ void __launch_bounds__(NT, split_min_blocks(MODEL, V, NT, HET)) k_split(BlockedJob job, Coef<double> cf, SplitCoef sc) {
-  constexpr bool PARK = split_parks(MODEL, V, NT, HET);
+__global__ void __launch_bounds__(NT, split_min_blocks(MODEL, V, HET)) k_split(BlockedJob job, Coef<double> cf, SplitCoef sc) {
+  constexpr bool PARK = split_parks(MODEL, V, HET);
   extern __shared__ __align__(16) unsigned char smem[];
   const double *in = static_cast<const double *>(job.in);
   double *out = static_cast<double *>(job.out);
@@ -116,9 +143,8 @@ __device__ __noinline__ void persistent_split_call(const PersistentJob &job, int
 
 // The split form of k_persistent.
 template <int MODEL, int V, bool BATCH, int NT>
-__global__ void __launch_bounds__(NT, split_min_blocks(MODEL, V, NT, false))
-    k_persistent_split(PersistentJob job, Coef<double> cf, SplitCoef sc) {
-  constexpr bool PARK = split_parks(MODEL, V, NT, false);
+__global__ void __launch_bounds__(NT, split_min_blocks(MODEL, V, false)) k_persistent_split(PersistentJob job, Coef<double> cf, SplitCoef sc) {
+  constexpr bool PARK = split_parks(MODEL, V, false);
   extern __shared__ __align__(16) unsigned char smem[];
   persistent_loop(job, [&](int ki, const void *in, void *out, const void *, void *, int64_t item, int K, int G) {
     const double *i = static_cast<const double *>(in);
@@ -136,42 +162,24 @@ static cudaError_t launch_split_k(int block, int64_t grid, const BlockedJob &job
   static PerDevice attr;
   const cudaError_t e = set_smem_limit_once(k_split<MODEL, V, HET, PACKED, NT>, 200 * 1024, attr);
   if (e != cudaSuccess) return e;
-  const size_t smem = split_smem_bytes<MODEL, V, HET, NT>(block);
+  const size_t smem = split_smem_bytes<MODEL, V, HET>(block);
   if (grid > 0)
     k_split<MODEL, V, HET, PACKED, NT><<<(unsigned)grid, block, smem, st>>>(job, to_coef<double>(cfd, cfd.kappa),
                                                                           split_coef(MODEL, cfd));
   return cudaGetLastError();
 }
-template <int MODEL, int V, bool HET>
-static cudaError_t launch_split_v(int block, const BlockedJob &job, const CoefD &cf, cudaStream_t st) {
-  constexpr int S = split_small_block(V), B = max_threads_for(V);
-  if constexpr (!HET) {
-    if (job.nchains > 1 && job.packed) {
-      const int64_t grid = job.ntiles + job.bt.npacked;
-      return block <= S ? launch_split_k<MODEL, V, false, true, S>(block, grid, job, cf, st)
-                        : launch_split_k<MODEL, V, false, true, B>(block, grid, job, cf, st);
-    }
-  }
-  return block <= S ? launch_split_k<MODEL, V, HET, false, S>(block, job.ntiles, job, cf, st)
-                    : launch_split_k<MODEL, V, HET, false, B>(block, job.ntiles, job, cf, st);
-}
-
 template <int MODEL>
 cudaError_t launch_split_blocked(int v, int block, const BlockedJob &job, const CoefD &cf, cudaStream_t st) {
-  if (job.sp) {
-    switch (v) {
-      case 2: return launch_split_v<MODEL, 2, true>(block, job, cf, st);
-      case 4: return launch_split_v<MODEL, 4, true>(block, job, cf, st);
-      default: return cudaErrorInvalidValue;
-    }
-  }
-  switch (v) {
-    case 1: return launch_split_v<MODEL, 1, false>(block, job, cf, st);
-    case 2: return launch_split_v<MODEL, 2, false>(block, job, cf, st);
-    case 4: return launch_split_v<MODEL, 4, false>(block, job, cf, st);
-    case 8: return launch_split_v<MODEL, 8, false>(block, job, cf, st);
-    default: return cudaErrorInvalidValue;
-  }
+  if (job.sp)
+    return split_dispatch<MODEL, true>(v, block, cudaErrorInvalidValue, [&](auto vc, auto nt, int threads) {
+      return launch_split_k<MODEL, decltype(vc)::value, true, false, decltype(nt)::value>(threads, job.ntiles, job, cf, st);
+    });
+  return split_dispatch<MODEL, false>(v, block, cudaErrorInvalidValue, [&](auto vc, auto nt, int threads) {
+    constexpr int V = decltype(vc)::value, NT = decltype(nt)::value;
+    if (job.nchains > 1 && job.packed)
+      return launch_split_k<MODEL, V, false, true, NT>(threads, job.ntiles + job.bt.npacked, job, cf, st);
+    return launch_split_k<MODEL, V, false, false, NT>(threads, job.ntiles, job, cf, st);
+  });
 }
 
 template <int MODEL, int V, int NT>
@@ -180,7 +188,7 @@ static int persistent_split_grid_k(int block) {
   if (set_smem_limit_once(k_persistent_split<MODEL, V, false, NT>, 200 * 1024, attr) != cudaSuccess ||
       set_smem_limit_once(k_persistent_split<MODEL, V, true, NT>, 200 * 1024, attr_b) != cudaSuccess)
     return 0;
-  const size_t smem = split_smem_bytes<MODEL, V, false, NT>(block);
+  const size_t smem = split_smem_bytes<MODEL, V, false>(block);
   int a = 0, b = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_persistent_split<MODEL, V, false, NT>, block, smem) !=
           cudaSuccess ||
@@ -196,7 +204,7 @@ static cudaError_t launch_persistent_split_k(int block, int grid, const Persiste
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid);
   cfg.blockDim = dim3((unsigned)block);
-  cfg.dynamicSmemBytes = split_smem_bytes<MODEL, V, false, NT>(block);
+  cfg.dynamicSmemBytes = split_smem_bytes<MODEL, V, false>(block);
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeCooperative;
@@ -209,27 +217,17 @@ static cudaError_t launch_persistent_split_k(int block, int grid, const Persiste
   return cudaLaunchKernelEx(&cfg, k_persistent_split<MODEL, V, false, NT>, job, cf, sc);
 }
 
-#define RK4_SPLIT_V(FN, ...)                                                                             \
-  switch (v) {                                                                                           \
-    case 1: return FN<MODEL, 1, max_threads_for(1)>(__VA_ARGS__);                                        \
-    case 2: return FN<MODEL, 2, max_threads_for(2)>(__VA_ARGS__);                                        \
-    case 4:                                                                                              \
-      return block <= split_small_block(4) ? FN<MODEL, 4, split_small_block(4)>(__VA_ARGS__)             \
-                                           : FN<MODEL, 4, max_threads_for(4)>(__VA_ARGS__);              \
-    case 8: return FN<MODEL, 8, max_threads_for(8)>(__VA_ARGS__);                                        \
-    default: break;                                                                                      \
-  }
-
 template <int MODEL>
 cudaError_t launch_split_persistent(int v, int block, int grid, const PersistentJob &job, const CoefD &cf,
                                     cudaStream_t st) {
-  RK4_SPLIT_V(launch_persistent_split_k, block, grid, job, cf, st)
-  return cudaErrorInvalidValue;
+  return split_dispatch<MODEL, false>(v, block, cudaErrorInvalidValue, [&](auto vc, auto nt, int threads) {
+    return launch_persistent_split_k<MODEL, decltype(vc)::value, decltype(nt)::value>(threads, grid, job, cf, st);
+  });
 }
 template <int MODEL> int persistent_split_max_grid(int v, int block) {
-  RK4_SPLIT_V(persistent_split_grid_k, block)
-  return 0;
+  return split_dispatch<MODEL, false>(v, block, 0, [&](auto vc, auto nt, int threads) {
+    return persistent_split_grid_k<MODEL, decltype(vc)::value, decltype(nt)::value>(threads);
+  });
 }
-#undef RK4_SPLIT_V
 
 }  // namespace rk4d
