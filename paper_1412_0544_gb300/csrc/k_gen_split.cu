@@ -44,6 +44,7 @@ __device__ __noinline__ void gen_wide_tile(const BlockedJob &job, ChainDesc ch, 
   double *edge = reinterpret_cast<double *>(smem);
   double *tl = edge + gen_edge_values(V);
   tile_load<double, D, false>(tl, static_cast<const double *>(job.in), ch.off, ch.n, ch.bc, t0, W, job.total, job.hdr);
+  tile_load_wait();
   __syncthreads();
   double y[V][D], cmp[V][D];
   const int base = threadIdx.x * V;
@@ -222,6 +223,7 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 2 : 1) k_gen_split(BlockedJob 
   double *tl = reinterpret_cast<double *>(ex + 2 * blockDim.x);  // the tile, then the records in its place
   f32x2 *rec = reinterpret_cast<f32x2 *>(tl) + threadIdx.x * gen_record_words(st.s, D, PARK);
   tile_load<double, D, false>(tl, static_cast<const double *>(job.in), ch.off, ch.n, ch.bc, t0, W, job.total, job.hdr);
+  tile_load_wait();
   __syncthreads();
   double y[2][D];
   const int base = threadIdx.x * 2;

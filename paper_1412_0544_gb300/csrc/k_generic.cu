@@ -90,8 +90,8 @@ __global__ void __launch_bounds__(GenBounds<R, V, SHAPE>::threads) k_gen_blocked
     Coef<R> c;
     locate(it, ch, tile, c);
     const int64_t t0 = tile * (int64_t)G - H;
-    tile_load_async<R, D>(buf, in, ch.off, ch.n, ch.bc, t0, W, job.total, job.hdr);
-    if constexpr (KAHAN) tile_load_async<R, D>(buf + W * D, cin, ch.off, ch.n, ch.bc, t0, W, job.total, job.hdr);
+    tile_load<R, D, false>(buf, in, ch.off, ch.n, ch.bc, t0, W, job.total, job.hdr);
+    if constexpr (KAHAN) tile_load<R, D, false>(buf + W * D, cin, ch.off, ch.n, ch.bc, t0, W, job.total, job.hdr);
     cp_async_commit();
   };
 

@@ -523,7 +523,7 @@ template <bool COH, typename T> __device__ __forceinline__ T gld(const T *p) {
   if constexpr (COH) return __ldcg(p); else return __ldg(p);
 }
 
-// Block-cooperative copies of `count` values between global and shared memory, two forms.
+// Block-cooperative copies of `count` values between global and shared memory.
 //
 // copy_in_vec / copy_out_vec access global memory by 16-byte vectors wherever whole vectors
 // lie inside the range, whatever the range's alignment: when the shared-memory side sits at the
@@ -534,22 +534,8 @@ template <bool COH, typename T> __device__ __forceinline__ T gld(const T *p) {
 // chains start anywhere, so single loads of misaligned windows sat on its critical path
 // (measured 8 % faster with vectors).
 //
-// copy_in / copy_out move whole 16-byte vectors when both sides are aligned and the size is a
-// multiple of 16 bytes (every tile of a single chain), single values otherwise.  In the one-shot
-// tile kernels, whose loads overlap other blocks' arithmetic, this shorter code measured faster
-// for single chains (4 %) and for batches alike (4 %, against copy_in_vec on the same batch).
-template <bool COH, typename R>
-__device__ __forceinline__ void copy_in(R *dst, const R *__restrict__ src, int count) {
-  if ((reinterpret_cast<uintptr_t>(src) & 15u) == 0 && (reinterpret_cast<uintptr_t>(dst) & 15u) == 0 &&
-      ((count * (int)sizeof(R)) & 15) == 0) {
-    const int nv = count * (int)sizeof(R) / 16;
-    const int4 *s4 = reinterpret_cast<const int4 *>(src);
-    int4 *d4 = reinterpret_cast<int4 *>(dst);
-    for (int e = threadIdx.x; e < nv; e += blockDim.x) d4[e] = gld<COH>(s4 + e);
-  } else {
-    for (int e = threadIdx.x; e < count; e += blockDim.x) dst[e] = gld<COH>(src + e);
-  }
-}
+// copy_out moves whole 16-byte vectors when both sides are aligned and the size is a
+// multiple of 16 bytes (every tile of a single chain), single values otherwise.
 template <typename R>
 __device__ __forceinline__ void copy_out(R *__restrict__ dst, const R *src, int count) {
   if ((reinterpret_cast<uintptr_t>(dst) & 15u) == 0 && (reinterpret_cast<uintptr_t>(src) & 15u) == 0 &&
@@ -650,22 +636,33 @@ template <int N> __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-// copy_in's asynchronous form: 16-byte copies where both sides share their offset within a
-// 16-byte line, single values otherwise; nothing outside the range is read.
-template <typename R>
+// Copy into shared memory without waiting (tile_load_wait): 16-byte copies where both sides share
+// their offset within a 16-byte line, single values otherwise; nothing outside the range is read.
+// COH: nothing may come from L1, which copies of less than 16 bytes go through, so those values are
+// loaded (and waited for) here.
+template <bool COH, typename R>
 __device__ __forceinline__ void copy_in_async(R *dst, const R *__restrict__ src, int count) {
   constexpr int kPer = 16 / (int)sizeof(R);
   const unsigned ms = (unsigned)(reinterpret_cast<uintptr_t>(src) & 15u);
   if (ms != (unsigned)(reinterpret_cast<uintptr_t>(dst) & 15u)) {
-    for (int e = threadIdx.x; e < count; e += blockDim.x) cp_async(dst + e, src + e, (int)sizeof(R));
+    if constexpr (COH) {
+      copy_in_vec<COH>(dst, src, count);
+    } else {
+      for (int e = threadIdx.x; e < count; e += blockDim.x) cp_async(dst + e, src + e, (int)sizeof(R));
+    }
     return;
   }
+  auto one = [&](int e) {
+    if constexpr (COH) dst[e] = gld<COH>(src + e); else cp_async(dst + e, src + e, (int)sizeof(R));
+  };
   int head = (int)(((16u - ms) & 15u) / sizeof(R));
   if (head > count) head = count;
   const int nv = (count - head) / kPer;
-  for (int e = threadIdx.x; e < head; e += blockDim.x) cp_async(dst + e, src + e, (int)sizeof(R));
   for (int e = threadIdx.x; e < nv; e += blockDim.x) cp_async(dst + head + e * kPer, src + head + e * kPer, 16);
-  for (int e = head + nv * kPer + threadIdx.x; e < count; e += blockDim.x) cp_async(dst + e, src + e, (int)sizeof(R));
+  if (head > 0)
+    for (int e = threadIdx.x; e < head; e += blockDim.x) one(e);
+  if (head + nv * kPer < count)
+    for (int e = head + nv * kPer + threadIdx.x; e < count; e += blockDim.x) one(e);
 }
 
 // Copy the W sites starting at chain index t0 (may be negative or run past the end) of the
@@ -673,14 +670,19 @@ __device__ __forceinline__ void copy_in_async(R *dst, const R *__restrict__ src,
 // chain.  A tile that crosses a chain end is copied as a few contiguous segments (one index
 // wrap per segment, not per element): at most 2 for chains longer than the tile, N / W + 2
 // for shorter periodic chains.
+// The copies are asynchronous: tile_load_wait (or a commit and a later wait) before the barrier that
+// precedes their use.  Loads into registers and on to shared memory, three 16-byte vectors per
+// thread and array one after the other, took a block 9700 cycles a tile beside 5000 of arithmetic
+// (FP32, 256 x 4 x 4, four resident blocks), with these 5100; N = 2^24, site-steps/s before -> after:
+// FP32 256 x 4 x 4 2.77e11 -> 3.56e11, x 8 4.04e11 -> 4.31e11, x 16 4.53e11 -> 4.55e11, persistent x 8
+// 3.65e11 -> 3.94e11; FP64 256 x 4 x 1 2.71e10 -> 3.07e10, x 2 3.27e10 -> 3.43e10.
 template <typename R, int D, bool COH>
 __device__ __forceinline__ void tile_load(R *tile, const R *__restrict__ src, int64_t off, int64_t n, int bc,
                                           int64_t t0, int W, int64_t sites, WsHeader *hdr) {
   const int total = W * D;
   if (t0 >= 0 && t0 + W <= n) {
     if (!bounds_ok(hdr, in_range(off + t0, W, sites))) return;
-    if constexpr (COH) copy_in_vec<COH>(tile, src + (off + t0) * D, total);  // the persistent kernel
-    else copy_in<COH>(tile, src + (off + t0) * D, total);
+    copy_in_async<COH>(tile, src + (off + t0) * D, total);
     return;
   }
   int covered = 0;  // block-uniform loop over contiguous segments
@@ -705,7 +707,7 @@ __device__ __forceinline__ void tile_load(R *tile, const R *__restrict__ src, in
     const int cnt = len * D;
     if (seg && !bounds_ok(hdr, in_range(seg - src, cnt, sites * D))) seg = nullptr;
     if (seg) {
-      for (int e = threadIdx.x; e < cnt; e += blockDim.x) dst[e] = gld<COH>(seg + e);
+      copy_in_async<COH>(dst, seg, cnt);
     } else {
       for (int e = threadIdx.x; e < cnt; e += blockDim.x) dst[e] = R(0);
     }
@@ -713,18 +715,9 @@ __device__ __forceinline__ void tile_load(R *tile, const R *__restrict__ src, in
   }
 }
 
-// tile_load for a tile kernel that prefetches its next tile: a window inside the chain is
-// copied asynchronously (the caller commits and later waits); a window that crosses a chain
-// end (wrapped or zero-filled segments, a few tiles per chain) is copied synchronously.
-template <typename R, int D>
-__device__ __forceinline__ void tile_load_async(R *tile, const R *__restrict__ src, int64_t off, int64_t n, int bc,
-                                                int64_t t0, int W, int64_t sites, WsHeader *hdr) {
-  if (t0 >= 0 && t0 + W <= n) {
-    if (!bounds_ok(hdr, in_range(off + t0, W, sites))) return;
-    copy_in_async(tile, src + (off + t0) * D, W * D);
-    return;
-  }
-  tile_load<R, D, false>(tile, src, off, n, bc, t0, W, sites, hdr);
+__device__ __forceinline__ void tile_load_wait() {
+  cp_async_commit();
+  cp_async_wait<0>();
 }
 
 // Store `cnt` sites of the tile starting at tile-local site `first` to chain index g0 (VEC:
@@ -789,6 +782,7 @@ __device__ __forceinline__ bool tile_item(const R *__restrict__ in, R *__restric
   tile_load<R, D, COH>(tl, in, ch.off, ch.n, ch.bc, t0, W, sites, hdr);
   if constexpr (KAHAN) tile_load<R, D, COH>(ctl, cin, ch.off, ch.n, ch.bc, t0, W, sites, hdr);
   if constexpr (HET) tile_load<R, P, COH>(ptl, sp, ch.off, ch.n, ch.bc, t0, W, sites, hdr);
+  tile_load_wait();
   __syncthreads();
 
   R y[V][D], cmp[V][D];
@@ -948,6 +942,7 @@ __device__ __forceinline__ bool packed_tile_item(const R *__restrict__ in, R *__
     tl[e] = R(0);
     if constexpr (KAHAN) ctl[e] = R(0);
   }
+  tile_load_wait();
   __syncthreads();
 
   // this thread's segment: the last one starting at or before its first slot
