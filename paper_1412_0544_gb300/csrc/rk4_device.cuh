@@ -124,11 +124,17 @@ __device__ __forceinline__ void stage_update(int j, const R *k, R *y, R *u, R *a
 
 // ---- Packed FP32: two sites per instruction --------------------------------------------
 // GB300 issues FP32 add, multiply and FMA on register pairs (f32x2): one instruction performs
-// the same round-to-nearest operation on both halves, at the FMA pipe's per-lane rate, with
-// half the issue slots.  The FP32 kernels are issue-bound, so the tile kernels advance two
-// adjacent sites (the .x and .y halves) with these forms.  Each half gets exactly the
-// operation the scalar functions above perform, and negation flips the sign bits (exact,
-// signed zeros included), so packed and scalar kernels stay bit-identical.
+// the same round-to-nearest operation on both halves, 64 lane-operations in the two cycles it
+// occupies the scheduler; every other instruction takes one of those cycles away.  The tile kernels
+// therefore advance two sites with these forms and none in between that only flips signs (the packed
+// forms cannot negate an operand): they hold the Roessler sites as X = -x, Y = -y, z, and m = minus the
+// compensation of what they hold, with which every term of Eqs. (6) and (7) and of the Kahan
+// update comes out with the sign it needs.  Rounding is symmetric, so each half still gets the
+// value the scalar functions above compute, and packed and scalar kernels stay bit-identical.  Of 197
+// instructions per warp and step (256 x 4, 116 of them packed arithmetic) 28 had only flipped signs:
+// N = 2^24, site-steps/s before -> after: 256 x 4 x 16 4.55e11 -> 4.68e11, 512 x 4 x 16 4.75e11 -> 4.91e11,
+// harmonic 256 x 8 x 16 7.28e11, Roessler 256 x 8 x 16 5.13e11 (two instructions per step and site that
+// are not arithmetic, half of what four sites per thread have).
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
   float2 d;
   asm("{\n\t.reg .b64 ra, rb, rc, rd;\n\tmov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\t"
@@ -161,39 +167,44 @@ __device__ __forceinline__ float2 mul2(float2 a, float2 b) {
       : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
   return d;
 }
-__device__ __forceinline__ float2 neg2(float2 a) {
-  return make_float2(__uint_as_float(__float_as_uint(a.x) ^ 0x80000000u),
-                     __uint_as_float(__float_as_uint(a.y) ^ 0x80000000u));
-}
 __device__ __forceinline__ float2 splat(float a) { return make_float2(a, a); }
 
-// The coefficients as pairs: both halves from one chain, or from two sites (heterogeneous).
+// The coefficients as pairs, both halves from one chain, or from two sites (heterogeneous); c and
+// w2 negated.
 struct Coef2 {
-  float2 a, b, c, kappa, w2, h2, h1, dt6;
+  float2 a, b, nc, kappa, nw2, h2, h1, dt6;
 };
 __device__ __forceinline__ Coef2 pair_coef(const Coef<float> &p, const Coef<float> &q) {
-  return {make_float2(p.a, q.a),         make_float2(p.b, q.b),   make_float2(p.c, q.c),
-          make_float2(p.kappa, q.kappa), make_float2(p.w2, q.w2), make_float2(p.h2, q.h2),
+  return {make_float2(p.a, q.a),         make_float2(p.b, q.b),     make_float2(-p.c, -q.c),
+          make_float2(p.kappa, q.kappa), make_float2(-p.w2, -q.w2), make_float2(p.h2, q.h2),
           make_float2(p.h1, q.h1),       make_float2(p.dt6, q.dt6)};
 }
+// A site's coordinate d and its compensation as the packed forms hold them, and back.  Back by 0 - v,
+// not by a sign flip: a sum that cancels is +0 in whichever sign it was held.
+template <int MODEL> __device__ __forceinline__ void hold(int d, float &y, float &cmp) {
+  if (MODEL == ROESSLER && d < 2) y = -y; else cmp = -cmp;
+}
+template <int MODEL> __device__ __forceinline__ void unhold(int d, float &y, float &cmp) {
+  if (MODEL == ROESSLER && d < 2) y = __fsub_rn(0.f, y); else cmp = __fsub_rn(0.f, cmp);
+}
 
-// slope() on two sites.
+// slope() on two sites, of and for the coordinates as they are held.
 template <int MODEL>
 __device__ __forceinline__ void slope2(const float2 *u, float2 xl, float2 xr, const Coef2 &cf, float2 *k) {
   const float2 lap = fma2(splat(-2.f), u[0], add2(xl, xr));
   if constexpr (MODEL == ROESSLER) {
-    k[0] = fma2(cf.kappa, lap, neg2(add2(u[1], u[2])));
-    k[1] = fma2(cf.a, u[1], u[0]);
-    k[2] = fma2(u[2], sub2(u[0], cf.c), cf.b);
+    k[0] = fma2(cf.kappa, lap, sub2(u[2], u[1]));             // X' = kappa lap(X) + (y + z)
+    k[1] = fma2(cf.a, u[1], u[0]);                            // Y' = a Y + X
+    k[2] = fma2(u[2], sub2(cf.nc, u[0]), cf.b);               // z' = z (-c - X) + b
   } else {
     k[0] = u[1];
-    k[1] = fma2(cf.kappa, lap, neg2(mul2(cf.w2, u[0])));
+    k[1] = fma2(cf.kappa, lap, mul2(cf.nw2, u[0]));
   }
 }
 
-// stage_update() on two sites (FP32 with the Kahan update).
+// stage_update() on two sites (FP32 with the Kahan update; m = minus the compensation).
 template <int D>
-__device__ __forceinline__ void stage_update2(int j, const float2 *k, float2 *y, float2 *u, float2 *acc, float2 *cmp,
+__device__ __forceinline__ void stage_update2(int j, const float2 *k, float2 *y, float2 *u, float2 *acc, float2 *m,
                                               const Coef2 &cf) {
 #pragma unroll
   for (int d = 0; d < D; ++d) {
@@ -208,9 +219,9 @@ __device__ __forceinline__ void stage_update2(int j, const float2 *k, float2 *y,
       u[d] = fma2(cf.h1, k[d], y[d]);
     } else {
       const float2 s4 = add2(acc[d], k[d]);
-      const float2 s = fma2(cf.dt6, s4, neg2(cmp[d]));
+      const float2 s = fma2(cf.dt6, s4, m[d]);
       const float2 t = add2(y[d], s);
-      cmp[d] = sub2(sub2(t, y[d]), s);
+      m[d] = sub2(s, sub2(t, y[d]));
       y[d] = t;
     }
   }

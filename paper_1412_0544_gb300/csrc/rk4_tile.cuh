@@ -173,6 +173,13 @@ __device__ __forceinline__ void tile_advance(R (&y)[V][Dim<MODEL>::D], R (&cmp)[
   R u[V][D], acc[V][D];
   // FP32-Kahan tiles with an even number of sites per thread run on packed instructions
   constexpr bool kPacked = std::is_same<R, float>::value && KAHAN && (V % 2 == 0);
+  constexpr int P = V / 2;
+  if constexpr (kPacked) {
+#pragma unroll
+    for (int v = 0; v < V; ++v)
+#pragma unroll
+      for (int d = 0; d < D; ++d) hold<MODEL>(d, y[v][d], cmp[v][d]);
+  }
 
 #pragma unroll 2  // halves the loop-carried register moves (measured +4 % in FP32)
   for (int s = 0; s < K; ++s) {
@@ -205,32 +212,35 @@ __device__ __forceinline__ void tile_advance(R (&y)[V][Dim<MODEL>::D], R (&cmp)[
         right = is_last ? from_next : right;
       }
       if constexpr (kPacked) {
-        // sites v and v + 1 in the two halves of packed FP32 instructions
+        // sites p and p + V / 2 in the two halves of packed FP32 instructions: a pair's neighbours
+        // are, except at the thread's ends, the adjacent pairs as they stand
+        float2 X[P];
 #pragma unroll
-        for (int v = 0; v < V; v += 2) {
-          const float2 xl = make_float2((v == 0) ? left : xs[v - 1], xs[v]);
-          const float2 xr = make_float2(xs[v + 1], (v + 2 == V) ? right : xs[v + 2]);
+        for (int p = 0; p < P; ++p) X[p] = make_float2(xs[p], xs[p + P]);
+        const float2 first = make_float2(left, xs[P - 1]), last = make_float2(xs[P], right);
+#pragma unroll
+        for (int p = 0; p < P; ++p) {
           float2 yy[D], uu[D], ac[D], cm[D], k[D];
 #pragma unroll
           for (int d = 0; d < D; ++d) {
-            yy[d] = make_float2(y[v][d], y[v + 1][d]);
-            uu[d] = (j == 0) ? yy[d] : make_float2(u[v][d], u[v + 1][d]);
-            ac[d] = make_float2(acc[v][d], acc[v + 1][d]);
-            cm[d] = make_float2(cmp[v][d], cmp[v + 1][d]);
+            yy[d] = make_float2(y[p][d], y[p + P][d]);
+            uu[d] = (j == 0) ? yy[d] : make_float2(u[p][d], u[p + P][d]);
+            ac[d] = make_float2(acc[p][d], acc[p + P][d]);
+            cm[d] = make_float2(cmp[p][d], cmp[p + P][d]);
           }
-          const Coef2 c2 = HET ? pair_coef(cs[v], cs[v + 1]) : pair_coef(cf, cf);
-          slope2<MODEL>(uu, xl, xr, c2, k);
+          const Coef2 c2 = HET ? pair_coef(cs[p], cs[p + P]) : pair_coef(cf, cf);
+          slope2<MODEL>(uu, p == 0 ? first : X[p - 1], p == P - 1 ? last : X[p + 1], c2, k);
           stage_update2<D>(j, k, yy, uu, ac, cm, c2);
 #pragma unroll
           for (int d = 0; d < D; ++d) {
-            y[v][d] = yy[d].x;
-            y[v + 1][d] = yy[d].y;
-            u[v][d] = uu[d].x;
-            u[v + 1][d] = uu[d].y;
-            acc[v][d] = ac[d].x;
-            acc[v + 1][d] = ac[d].y;
-            cmp[v][d] = cm[d].x;
-            cmp[v + 1][d] = cm[d].y;
+            y[p][d] = yy[d].x;
+            y[p + P][d] = yy[d].y;
+            u[p][d] = uu[d].x;
+            u[p + P][d] = uu[d].y;
+            acc[p][d] = ac[d].x;
+            acc[p + P][d] = ac[d].y;
+            cmp[p][d] = cm[d].x;
+            cmp[p + P][d] = cm[d].y;
           }
         }
       } else {
@@ -247,6 +257,12 @@ __device__ __forceinline__ void tile_advance(R (&y)[V][Dim<MODEL>::D], R (&cmp)[
         }
       }
     }
+  }
+  if constexpr (kPacked) {
+#pragma unroll
+    for (int v = 0; v < V; ++v)
+#pragma unroll
+      for (int d = 0; d < D; ++d) unhold<MODEL>(d, y[v][d], cmp[v][d]);
   }
 }
 
