@@ -79,10 +79,13 @@ struct rk4_chain {
   int kernel = RK4_KERNEL_AUTO;
   bool tiling_auto = true;
   rk4_tiling tiling{};
-  rk4_tiling run{};  // what the current integration runs with (run_tiling), and its automatic choice
-  rk4_tiling auto_tiling{};
-  int64_t auto_steps = -1;
-  unsigned auto_version = 0;
+  rk4_tiling run{};  // what the current integration runs with (run_tiling)
+  // its last few automatic choices, by the number of steps, under one configuration
+  struct {
+    int64_t steps = -1;
+    rk4_tiling tiling{};
+  } automatic[8];
+  unsigned auto_next = 0, auto_version = 0;
   double t0 = 0.0;
   int64_t nstep = 0;
   bool graphs = true;
@@ -392,28 +395,32 @@ Plan make_plan(const rk4_chain *h, int64_t nsteps, int K) {
   return h->tiling_auto ? batch_auto_plan(nsteps, K) : batch_plan(nsteps, K);
 }
 
-// What a launch costs, fitted on a GB300 (152 SMs, 2070 MHz) in us: A + max(B k, w (C + D k)) for k
+// What a launch costs, fitted on a GB300 (152 SMs, 2070 MHz) in us: A + hypot(B k, w (C + D k)) for k
 // steps when every SM gets w tiles.  A is the launch and the tile's way in and out, B a step's
 // latency when a tile has an SM to itself (1000 sites, k = 1 .. 16), C + D k the SM's time per tile
 // when it is full (2^22 sites).  Roessler; the harmonic chain's costs are in nearly the same
-// proportions.  The stages a generic step needs scale B and D (six: Dormand-Prince 5).
+// proportions, except that its 128 x 4 runs ahead of 256 x 2 (2.4 and 3.0 ns per site and SM at
+// k = 4; the same kernel in the Roessler chain, so only the former is listed).  The stages a generic
+// step needs scale B and D (six: Dormand-Prince 5).
 struct TileCost {
   int block, v;
   float A, B, C, D;
 };
-const TileCost kCostFp64[] = {{64, 1, 2.7f, 1.20f, 0.47f, 0.307f}, {128, 1, 2.9f, 1.22f, 0.43f, 0.522f},
-                              {256, 1, 3.0f, 1.65f, 0.40f, 1.03f}, {512, 1, 3.4f, 2.64f, 1.25f, 2.10f},
-                              {256, 2, 3.6f, 2.84f, 1.40f, 2.11f}, {128, 4, 4.7f, 3.24f, 1.00f, 1.99f},
-                              {256, 4, 5.6f, 5.35f, 2.00f, 4.13f}};
-const TileCost kCostFp32[] = {{256, 1, 4.1f, 0.33f, 0.52f, 0.098f}, {128, 2, 4.9f, 0.32f, 0.50f, 0.060f},
-                              {256, 2, 5.2f, 0.37f, 1.20f, 0.122f}, {128, 4, 7.0f, 0.31f, 0.95f, 0.093f},
-                              {256, 4, 7.9f, 0.35f, 2.00f, 0.190f}, {512, 4, 7.5f, 0.62f, 4.60f, 0.390f}};
-const TileCost kCostHet64[] = {{64, 2, 5.8f, 1.78f, 0.95f, 0.54f}, {128, 2, 5.7f, 1.93f, 0.95f, 0.975f},
-                               {256, 2, 6.2f, 2.87f, 2.00f, 2.12f}};
-const TileCost kCostHet32[] = {{128, 2, 7.0f, 0.31f, 0.80f, 0.054f}, {256, 2, 7.3f, 0.37f, 1.75f, 0.115f},
-                               {128, 4, 10.5f, 0.29f, 1.60f, 0.080f}, {256, 4, 11.6f, 0.36f, 3.20f, 0.190f}};
-const TileCost kCostGen64[] = {{64, 2, 4.0f, 4.48f, 0.57f, 1.37f}, {128, 2, 3.8f, 4.75f, 0.55f, 2.10f},
-                               {256, 2, 4.2f, 6.70f, 1.10f, 5.10f}};
+const TileCost kCostFp64[] = {{64, 1, 2.2f, 1.26f, 0.34f, 0.336f}, {128, 1, 2.2f, 1.28f, 0.33f, 0.523f},
+                              {256, 1, 2.4f, 1.70f, 0.21f, 1.024f}, {512, 1, 3.0f, 2.69f, 0.80f, 2.133f},
+                              {128, 2, 2.4f, 2.22f, 0.43f, 0.975f}, {128, 4, 2.8f, 3.01f, 0.51f, 1.875f},
+                              {256, 4, 3.8f, 5.08f, 1.35f, 4.000f}};
+const TileCost kCostFp32[] = {{256, 1, 3.2f, 0.33f, 0.51f, 0.102f}, {128, 2, 3.0f, 0.28f, 0.28f, 0.074f},
+                              {256, 2, 3.3f, 0.38f, 0.58f, 0.154f}, {128, 4, 3.1f, 0.30f, 0.33f, 0.127f},
+                              {256, 4, 3.9f, 0.39f, 0.74f, 0.254f}, {512, 4, 5.5f, 0.61f, 2.10f, 0.500f},
+                              {128, 8, 4.2f, 0.35f, 0.75f, 0.246f}, {256, 8, 5.3f, 0.56f, 2.33f, 0.465f}};
+const TileCost kCostHet64[] = {{64, 2, 3.4f, 1.91f, 0.46f, 0.605f}, {128, 2, 3.5f, 1.96f, 0.39f, 0.975f},
+                               {256, 2, 4.2f, 2.75f, 1.53f, 2.110f}};
+const TileCost kCostHet32[] = {{64, 2, 3.8f, 0.30f, 0.23f, 0.036f}, {128, 2, 3.8f, 0.30f, 0.41f, 0.080f},
+                               {256, 2, 4.1f, 0.39f, 0.87f, 0.169f}, {128, 4, 3.9f, 0.31f, 0.55f, 0.135f},
+                               {256, 4, 5.2f, 0.39f, 1.25f, 0.276f}};
+const TileCost kCostGen64[] = {{64, 2, 2.8f, 4.50f, 0.25f, 1.51f}, {128, 2, 2.9f, 4.57f, 0.42f, 2.12f},
+                               {256, 2, 3.2f, 6.67f, 0.80f, 5.13f}};
 const TileCost kCostGen32[] = {{128, 2, 5.3f, 0.80f, 0.55f, 0.27f}, {256, 2, 5.7f, 0.95f, 1.30f, 0.64f}};
 const TileCost kCostGen32Shape[] = {{128, 4, 7.0f, 0.47f, 0.65f, 0.28f}, {256, 4, 7.9f, 0.68f, 1.50f, 0.60f},
                                     {512, 4, 7.5f, 1.32f, 3.80f, 1.20f}};
@@ -437,14 +444,21 @@ double tiles_estimate(const rk4_chain *h, int W, int v, int k) {
 // The tiling an integration of nsteps runs with.  One that was set or tuned is taken as it is.
 // The automatic choice (whose seed rk4_chain_get_tiling reports) depends on the sites and the
 // steps: a short chain needs small tiles to reach every SM and many steps per launch to pay for
-// the launch, a long one wide tiles.  Measured against the seed, us per step: FP64 1000 sites 10.7
-// -> 1.6 (128 x 1, k = 8), 65537 sites 10.7 -> 3.2 (512 x 1, k = 8), 2^22 sites 164 -> 126 (256 x 4,
-// k = 8); FP32 65537 sites 2.6 -> 0.8 (128 x 2, k = 16), 2^22 sites 18.2 -> 10.0 (256 x 4, k = 16).
+// the launch, a long one wide tiles.  Measured against the seed, us per step: FP64 1000 sites 8.9
+// -> 1.6 (128 x 1, k = 8), 65537 sites 8.9 -> 2.9 (512 x 1, k = 11), 2^22 sites 144 -> 115 (128 x 4,
+// k = 4); FP32 65537 sites 2.3 -> 0.5 (128 x 4, k = 16), 2^22 sites 12.7 -> 8.9 (256 x 8, k = 16).  Over
+// 300 .. 2^24 sites of both models and precisions the choice is within 3 % of the best tiling in the
+// median, 10 % at worst.
 // The FP64 form (coefficients outside split_allowed) keeps the seed.
 rk4_tiling run_tiling(rk4_chain *h, int64_t nsteps) {
   if (!h->tiling_auto) return h->tiling;
   if (h->nchains > 1) nsteps = 1024;  // a batch's tables must not depend on the steps
-  if (h->auto_steps == nsteps && h->auto_version == h->config_version) return h->auto_tiling;
+  if (h->auto_version != h->config_version) {
+    for (auto &a : h->automatic) a.steps = -1;
+    h->auto_version = h->config_version;
+  }
+  for (const auto &a : h->automatic)
+    if (a.steps == nsteps) return a.tiling;
   const TileCost *cost = nullptr;
   int n = 0;
   float stages = 1.f;
@@ -475,19 +489,24 @@ rk4_tiling run_tiling(rk4_chain *h, int64_t nsteps) {
       const int k = P.kval[0], W = cost[c].block * cost[c].v;
       if (k == last || !tiling_valid(h, cost[c].block, cost[c].v, k)) continue;
       last = k;
-      double w = tiles_estimate(h, W, cost[c].v, k) / sms;
-      w = w <= 4.0 ? std::ceil(w) : w + 0.5;  // few tiles: the busiest SM decides
-      const double us = (double)P.count() *
-                        (cost[c].A + std::max((double)cost[c].B * stages * k, w * (cost[c].C + cost[c].D * stages * k)));
+      double us = 0.0;
+      for (size_t i = 0; i < P.kval.size(); ++i) {
+        if (P.cnt[i] == 0) continue;
+        const int ki = P.kval[i];
+        double w = tiles_estimate(h, W, cost[c].v, ki) / sms;
+        w = w <= 4.0 ? std::ceil(w) : w + 0.5;  // few tiles: the busiest SM decides
+        us += (double)P.cnt[i] *
+              (cost[c].A + std::hypot(cost[c].B * stages * ki, w * (cost[c].C + cost[c].D * stages * ki)));
+      }
       if (us < best_us) {
         best_us = us;
         best = {cost[c].block, cost[c].v, k, tile_interior(h, W, k)};
       }
     }
   }
-  h->auto_steps = nsteps;
-  h->auto_version = h->config_version;
-  h->auto_tiling = best;
+  auto &a = h->automatic[h->auto_next++ % 8];
+  a.steps = nsteps;
+  a.tiling = best;
   return best;
 }
 
