@@ -86,6 +86,7 @@ struct rk4_chain {
     rk4_tiling tiling{};
   } automatic[8];
   unsigned auto_next = 0, auto_version = 0;
+  int one_way = 0;  // swap_one_way: 1 state -> workspace, 2 workspace -> state, in one launch
   double t0 = 0.0;
   int64_t nstep = 0;
   bool graphs = true;
@@ -391,6 +392,13 @@ Plan batch_auto_plan(int64_t nsteps, int K) {
 }
 
 Plan make_plan(const rk4_chain *h, int64_t nsteps, int K) {
+  if (h->one_way) {  // with the kval batch_plan has for the same steps, so that the tables serve both
+    Plan P = batch_plan(K, K);
+    P.cnt.assign(P.cnt.size(), 0);
+    P.cnt[0] = 1;
+    P.copy_back = false;
+    return P;
+  }
   if (h->nchains == 1) return balanced_plan(nsteps, K);
   return h->tiling_auto ? batch_auto_plan(nsteps, K) : batch_plan(nsteps, K);
 }
@@ -767,7 +775,7 @@ cudaError_t enqueue_integrate(rk4_chain *h, int kernel, void *state, void *comp,
       } else {
         j.ntiles = tiles_for(h, j.G);
       }
-      const bool even = (i % 2) == 0;
+      const bool even = (i % 2) == 0 && h->one_way != 2;
       j.in = even ? state : wsS;
       j.out = even ? wsS : state;
       j.cin = even ? comp : wsC;
@@ -1116,6 +1124,22 @@ bool rk4d::swap_graphs(rk4_chain *h, bool on) {
   const bool old = h->graphs;
   h->graphs = on;
   return old;
+}
+
+int rk4d::swap_one_way(rk4_chain *h, int way) {
+  const int old = h->one_way;
+  h->one_way = way;
+  return old;
+}
+
+bool rk4d::one_way_allowed(const rk4_chain *h, int64_t nsteps) {
+  return h->nchains > 1 && !h->tiling_auto && effective_kernel(h) == RK4_KERNEL_BLOCKED && h->tiling.k == nsteps;
+}
+
+void rk4d::state_copy(const rk4_chain *h, void *ws, void **state, void **comp) {
+  const WsLayout L = layout(h, RK4_KERNEL_BLOCKED);
+  *state = static_cast<char *>(ws) + L.state;
+  *comp = h->fp32 ? static_cast<char *>(ws) + L.comp : nullptr;
 }
 
 int rk4d::prepare_integrate(rk4_chain *h, int64_t nsteps) {

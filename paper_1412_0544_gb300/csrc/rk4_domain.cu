@@ -52,6 +52,7 @@ struct rk4_domain {
 namespace {
 
 constexpr size_t kAlign = 256;
+constexpr int64_t kWideTileSites = (int64_t)1 << 20;  // from here on 2048-site tiles: see rk4_domain_create
 size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
 bool any_ghost(const rk4_domain *d) { return d->bc == RK4_PERIODIC || d->nparts > 1; }
@@ -210,13 +211,16 @@ int rk4_domain_create(rk4_domain **out, int model, int precision, int64_t n, dou
     return rc;
   }
   // few long parts: one blocked launch over all of them is the natural scheme.  FP32 runs
-  // several steps per launch (bandwidth-bound at k = 1): an exchange period of P steps runs as
-  // two launches of P / 2 steps (an integration ends in the caller's buffer after an even
-  // number of launches), so that is the default k
+  // several steps per launch (bandwidth-bound at k = 1): an exchange period of up to 16 steps is one
+  // launch (run_period), a longer one several of at most 16.  Eight sites per thread where the
+  // parts fill the chip with such tiles (2^24 sites, k = 16: 5.16e11 site-steps/s against 4.66e11 with
+  // four, 256 x 4 x 8 4.38e11).
   rk4_chain_set_kernel(d->h, RK4_KERNEL_BLOCKED);
   if (d->fp32 && ghosts) {
-    const int k = (int)std::min<int64_t>(16, std::max<int64_t>(1, ghost / 8));
-    rk4_chain_set_tiling(d->h, 256, 4, k);  // keeps the default if this shape is not valid
+    const int k = (int)std::min<int64_t>(16, std::max<int64_t>(1, ghost / 4));
+    // keeps what it has if a shape is not valid
+    if (n < kWideTileSites || k < 8 || rk4_chain_set_tiling(d->h, 256, 8, k) != RK4_OK)
+      rk4_chain_set_tiling(d->h, 256, 4, k);
   }
   *out = d;
   return RK4_OK;
@@ -286,7 +290,40 @@ int rk4_domain_exchange(rk4_domain *d, void *state, void *comp) {
 
 namespace {
 
-constexpr int64_t kGraphPeriods = 8;  // exchange periods per captured graph
+constexpr int64_t kGraphPeriods = 8;  // exchange periods per captured graph (even: see run_periods)
+
+// nper whole exchange periods.  Where a period is one launch (one_way_allowed) they go in pairs, one
+// from the caller's buffers into the workspace's copy and one back, instead of two launches of half the
+// steps each: 2^24 sites in 4 parts, FP32, ghost 64, 695 us per period of 16 steps (256 x 4 x 8) -> 594
+// (256 x 8 x 16).
+int run_periods(rk4_domain *d, void *state, void *comp, char *w, const DomLayout &L, int64_t period, int64_t nper,
+                cudaStream_t st) {
+  const GhostPair *pairs = reinterpret_cast<const GhostPair *>(w + L.pairs);
+  auto run = [&](void *s, void *c, int way) -> int {
+    if (launch_ghost_copy(s, c, pairs, (int)d->pairs.size(), d->ghost, d->D * (int)d->es, st) != cudaSuccess)
+      return RK4_ECUDA;
+    const int old = swap_one_way(d->h, way);
+    const int rc = rk4_chain_integrate(d->h, state, comp, w, L.batch, period, nullptr);
+    swap_one_way(d->h, old);
+    return rc;
+  };
+  void *s2 = nullptr, *c2 = nullptr;
+  const bool pair = one_way_allowed(d->h, period);
+  if (pair) state_copy(d->h, w, &s2, &c2);
+  for (int64_t p = 0; p < nper;) {
+    int rc;
+    if (pair && p + 1 < nper) {
+      rc = run(state, comp, 1);
+      if (rc == RK4_OK) rc = run(s2, c2, 2);
+      p += 2;
+    } else {
+      rc = run(state, comp, 0);
+      ++p;
+    }
+    if (rc != RK4_OK) return rc;
+  }
+  return RK4_OK;
+}
 
 // A chunk of nper whole exchange periods as one CUDA graph, replayed `reps` times: captured on
 // first use and reused while the buffers, the chunk and the parts' configuration stay the same
@@ -312,14 +349,7 @@ int run_periods_graph(rk4_domain *d, void *state, void *comp, char *w, const Dom
     double t0 = 0.0;
     int64_t n0 = 0;
     rk4_chain_get_clock(d->h, &t0, &n0);
-    const GhostPair *pairs = reinterpret_cast<const GhostPair *>(w + L.pairs);
-    for (int64_t p = 0; p < nper && rc == RK4_OK; ++p) {
-      if (launch_ghost_copy(state, comp, pairs, (int)d->pairs.size(), d->ghost, d->D * (int)d->es, d->cap) !=
-          cudaSuccess)
-        rc = RK4_ECUDA;
-      else
-        rc = rk4_chain_integrate(d->h, state, comp, w, L.batch, period, nullptr);
-    }
+    rc = run_periods(d, state, comp, w, L, period, nper, d->cap);
     swap_graphs(d->h, old_graphs);
     swap_stream(d->h, old_stream);
     rk4_chain_set_clock(d->h, t0, n0);
@@ -377,12 +407,16 @@ int rk4_domain_integrate(rk4_domain *d, void *state, void *comp, void *ws, size_
     if (rc != RK4_OK) return rc;
     done = reps * kGraphPeriods * period;
   }
-  for (; done < nsteps;) {
-    const int64_t m = std::min(period, nsteps - done);
-    if (exchange_kernel(d, state, comp, w, L) != cudaSuccess) return RK4_ECUDA;
-    const int rc = rk4_chain_integrate(d->h, state, comp, ws, L.batch, m, nullptr);
+  if (any_ghost(d) && nsteps - done >= period) {
+    const int64_t nper = (nsteps - done) / period;
+    const int rc = run_periods(d, state, comp, w, L, period, nper, d->stream);
     if (rc != RK4_OK) return rc;
-    done += m;
+    done += nper * period;
+  }
+  if (done < nsteps) {  // the rest, less than a period (or all steps, without ghost zones)
+    if (exchange_kernel(d, state, comp, w, L) != cudaSuccess) return RK4_ECUDA;
+    const int rc = rk4_chain_integrate(d->h, state, comp, ws, L.batch, nsteps - done, nullptr);
+    if (rc != RK4_OK) return rc;
   }
   d->nstep += nsteps;
   if (t) *t = (double)d->nstep * d->dt;

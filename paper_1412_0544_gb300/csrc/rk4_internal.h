@@ -300,5 +300,11 @@ unsigned config_version(const rk4_chain *h);
 cudaStream_t swap_stream(rk4_chain *h, cudaStream_t st);
 bool swap_graphs(rk4_chain *h, bool on);
 int prepare_integrate(rk4_chain *h, int64_t nsteps);
+// One-way integrations of a batch: with way 1 an integration of tiling.k steps is one blocked launch
+// from the caller's buffers into the workspace's copy of the state (state_copy), with way 2 one
+// from there back; with 0 (the default) it starts and ends in the caller's buffers.  Returns the old way.
+int swap_one_way(rk4_chain *h, int way);
+bool one_way_allowed(const rk4_chain *h, int64_t nsteps);
+void state_copy(const rk4_chain *h, void *ws, void **state, void **comp);
 
 }  // namespace rk4d
