@@ -9,8 +9,9 @@ chain configuration; the state and its ping-pong copy are far larger than the 12
 flush is needed between steps.
 
 Printed: one JSON line (rank 0).  `value` = site-steps/s over all ranks; `roofline` refers to
-the blocked FP64 kernel, which is bound by the FP64 pipe (49 FP64 instructions per site-step
-against the measured FP64 FMA rate of this GPU); `e2e` measures the same through
+the blocked FP64 kernel, which is bound by the FP64 pipe (13 FP64 instructions per site-step, the
+first slope and the update, against the measured FP64 FMA rate of this GPU; the later stages'
+differences run as float pairs on the FP32 pipe); `e2e` measures the same through
 rk4_chain_integrate_host from pinned host memory; `cpu_baseline` is the serial C oracle on the
 host.  Extra keys report the periodic N = 2^24 chain, the FP32-Kahan path, batches of uneven
 chains and the widened schemes.
@@ -50,8 +51,9 @@ HBM_GBS_FALLBACK = 6800.0
 # and clocks; the constants below, from an earlier probe run on a GB300 at 2070 MHz, are the
 # fallback when the probe cannot run).  The classical RK4 Roessler step issues 49 DFMA per
 # site-step in FP64 (4 x 7 slope, whose two additions are issued as exact FMAs a*1+b, 9 stage
-# states, 12 update), so the roof is the DFMA rate.  FP32: the larger of the scalar and packed
-# (f32x2) FMA lane rates.
+# states, 12 update) in its FP64 form and 13 (7 first slope, 6 update) in the split form that the
+# kernels run (the dopri5 scheme 16: 10 and 6), whose other operations are FP32; the roof is the DFMA
+# rate either way.  FP32: the larger of the scalar and packed (f32x2) FMA lane rates.
 FP64_INST_PEAK = 0.6272e12
 FP32_INST_PEAK = 40.12e12
 PEAK_SOURCE = "fallback constants from an earlier pipe_probe run"
@@ -73,14 +75,16 @@ def probe_peaks():
         return {"error": str(e)[:200]}
 
 
-FP64_INST_PER_SITE_STEP = 49     # DFMA (the slope's 8 additions issued as a * 1 + b)
+FP64_INST_PER_SITE_STEP = 49     # DFMA of the FP64 form (the slope's 8 additions issued as a * 1 + b)
+SPLIT_FP64_INST = 13             # DFMA of the split form: first slope 7, update 6
+SPLIT_FP64_INST_GENERIC = 16     # the same with second neighbours: first slope 10, update 6
 FP32K_INST_PER_SITE_STEP = 58    # the update: 4 operations per component instead of 1 FMA
 # DRAM traffic (read + write bytes) per launch of the FP64 blocked kernel from one ncu capture,
 # with the chain length it was taken at: valid only for the kernel code (kernel_hash) and the
 # tiling recorded with it; any other combination reports null.  A launch's traffic is
 # proportional to the sites it advances (one read and one write of each tile), so a capture at
 # N = 2^24 scales to the N = 2^27 workload by the site count.
-TRAFFIC = {}
+TRAFFIC = {("25a07e6ca685f2eb", "128,4,4"): (403031808 + 354918144, 1 << 24)}
 
 
 def traffic_per_launch(khash: str, tiling: dict, n: int):
@@ -333,7 +337,7 @@ def periodic_fp64_extra(rk, torch, stream, n=N_SITES, nsteps=NSTEPS):
         sps = n * nsteps / el
         return {"value": sps, "unit": "site-steps/s", "N": n, "steps": nsteps, "boundary": "periodic",
                 "tiling": tiling, "effective_state_GBs": sps * 2 * D * 8 / 1e9,
-                "fp64_pipe_frac_of_measured": sps * FP64_INST_PER_SITE_STEP / FP64_INST_PEAK}
+                "fp64_pipe_frac_of_measured": sps * SPLIT_FP64_INST / FP64_INST_PEAK}
     finally:
         rk.rk4_chain_destroy(h)
 
@@ -545,13 +549,13 @@ def variant_extra(rk, torch, stream, precision, *, generic=False, het=False, n=N
         if generic:
             rk.rk4_chain_set_tableau(h, DOPRI5_A, DOPRI5_B)
             rk.rk4_chain_set_coupling2(h, 0.5)
-            ops = generic_fp_ops(DOPRI5_A, DOPRI5_B, D, 10, fp32)
+            ops = generic_fp_ops(DOPRI5_A, DOPRI5_B, D, 10, True) if fp32 else SPLIT_FP64_INST_GENERIC
         if het:
             u = ci.uniform01(SEED, 9, 0, 4 * n).reshape(n, 4)
             sp = torch.from_numpy(np.stack([0.15 + 0.1 * u[:, 0], 0.8 + 0.4 * u[:, 1], 8.0 + 2.0 * u[:, 2],
                                             0.5 + 1.5 * u[:, 3]], axis=1)).to(dtype).cuda()
             rk.rk4_chain_set_site_params(h, sp)
-            ops = FP32K_INST_PER_SITE_STEP if fp32 else FP64_INST_PER_SITE_STEP
+            ops = FP32K_INST_PER_SITE_STEP if fp32 else SPLIT_FP64_INST
         st = torch.empty((n, D), dtype=dtype, device="cuda")
         rk.rk4_fill_uniform(st, n * D, SEED, 0, precision, stream)
         cp = torch.zeros_like(st) if fp32 else None
@@ -580,8 +584,10 @@ def domain_extra(rk, torch, stream, precision, nparts=4, ghost=32, n=N_SITES, ns
     h = rk.rk4_chain_create(rk.RK4_ROESSLER, precision, n, DT, rk.RK4_PERIODIC, None, stream)
     try:
         tiling = rk.rk4_chain_get_tiling(rk.rk4_domain_chain(d))
-        # the undivided chain with the same launch shape (k steps per launch)
-        rk.rk4_chain_set_tiling(h, tiling["block"], tiling["v"], tiling["k"])
+        # the undivided chain with the same launch shape (k steps per launch); an FP64 domain has none
+        # set, and both choose by their sites
+        if fp32:
+            rk.rk4_chain_set_tiling(h, tiling["block"], tiling["v"], tiling["k"])
         cst = torch.empty((n, D), dtype=dtype, device="cuda")
         rk.rk4_fill_uniform(cst, n * D, SEED, 0, precision, stream)
         ccp = torch.zeros_like(cst) if fp32 else None
@@ -778,31 +784,21 @@ def main():
     el_k = time_integrate(rk, h, st, None, ws, nsteps, reps, torch)
     launch_s = el_k / (reps * plan_launches)
     sps_k = n * nsteps * reps / el_k
-    achieved_inst = sps_k * FP64_INST_PER_SITE_STEP / 1e9  # G FP64 instructions/s
+    achieved_inst = sps_k * SPLIT_FP64_INST / 1e9  # G FP64 instructions/s
     khash = kernel_hash()
     traffic = traffic_per_launch(khash, tiling, n)
     roofline = {"bound": "alu", "achieved": achieved_inst, "peak": FP64_INST_PEAK / 1e9,
                 "unit": "G FP64 inst/s", "frac": achieved_inst * 1e9 / FP64_INST_PEAK,
-                "traffic": traffic, "kernel": "k_blocked<double, Roessler>",
-                "per_unit": "49 FP64 instructions per interior site-step",
+                "traffic": traffic, "kernel": "k_split<Roessler>",
+                "per_unit": "13 FP64 instructions per interior site-step (first slope 7, update 6)",
+                # what the FP64 form's 49 instructions allow at most, and the rate against that
+                "fp64_form_roof_site_steps": FP64_INST_PEAK / FP64_INST_PER_SITE_STEP,
+                "against_fp64_form_roof": sps_k * FP64_INST_PER_SITE_STEP / FP64_INST_PEAK,
                 "launch_ms": launch_s * 1e3,
-                "peak_source": PEAK_SOURCE + " (DFMA issue rate; all 49 operations of the step can issue "
-                                             "as DFMA)",
+                "peak_source": PEAK_SOURCE + " (DFMA issue rate)",
                 "hbm_frac_effective_state": sps_k * 2 * D * 8 / 1e9 / hbm_peak,
                 # DRAM bandwidth the kernel draws: ncu's bytes per launch over this run's launch time
                 "dram_GBs": traffic / launch_s / 1e9 if traffic else None}
-    if probe and "rk4_fp64_regs_inst_per_s" in probe:
-        # the same RK4 instruction stream on register-resident sites (no loads, exchange or
-        # barriers): the most this instruction mix reaches on the FP64 pipe
-        arith_rate = float(probe["rk4_fp64_regs_inst_per_s"])
-        roofline["arithmetic_only_rate"] = arith_rate / 1e9
-        roofline["frac_of_arithmetic_only"] = achieved_inst * 1e9 / arith_rate
-    if probe and "rk4_fp64_regs_smem_roundtrip_inst_per_s" in probe:
-        # the same stream with a tile kernel's per-stage shared-memory exchange and barrier
-        xrate = float(probe["rk4_fp64_regs_smem_roundtrip_inst_per_s"])
-        roofline["arithmetic_with_exchange_rate"] = xrate / 1e9
-        roofline["frac_of_arithmetic_with_exchange"] = achieved_inst * 1e9 / xrate
-
     # --- end to end through the C ABI with host buffers ------------------------------
     host = torch.empty((n, D), dtype=torch.float64).pin_memory()
     host.copy_(st.cpu())

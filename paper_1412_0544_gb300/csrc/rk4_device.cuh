@@ -1,7 +1,8 @@
 // rk4_device.cuh -- the per-site arithmetic every GPU scheme shares.
 //
-// All kernels (staged, blocked, persistent) call these functions and nothing else for the
-// integrator's floating-point work, so each site runs the same operations in the same order
+// All kernels (staged, blocked, persistent) call these functions, or in FP64 those of the split form
+// (rk4_split.cuh; the forms below are what it falls back on outside its range), and nothing else for
+// the integrator's floating-point work, so each site runs the same operations in the same order
 // with the same rounding, whatever the tiling: the blocked and persistent kernels are
 // bit-identical to the one-stage-per-launch kernel.  Every operation is an explicit
 // round-to-nearest intrinsic, so the compiler cannot contract or reorder differently in
