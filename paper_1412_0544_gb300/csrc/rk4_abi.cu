@@ -31,9 +31,14 @@ struct GraphKey {
   long long timeout = 0;
   const void *sp = nullptr;
   int generic = 0;
+  // the plan's launches: a batch's tables are laid out by kval and its tile counts are baked into the
+  // graph, and the automatic and a set tiling of the same block, v and k make different plans
+  std::vector<int> kval;
+  std::vector<int64_t> cnt;
   bool operator==(const GraphKey &o) const {
     return kernel == o.kernel && state == o.state && comp == o.comp && ws == o.ws && nsteps == o.nsteps &&
-           block == o.block && v == o.v && k == o.k && timeout == o.timeout && sp == o.sp && generic == o.generic;
+           block == o.block && v == o.v && k == o.k && timeout == o.timeout && sp == o.sp && generic == o.generic &&
+           kval == o.kval && cnt == o.cnt;
   }
 };
 
@@ -884,6 +889,8 @@ int integrate_impl(rk4_chain *h, void *state, void *comp, void *ws, size_t ws_by
   key.timeout = h->timeout_ns;
   key.sp = h->site_params;
   key.generic = use_generic(h) ? 1 + (int)h->gen_version : 0;
+  key.kval = P.kval;
+  key.cnt = P.cnt;
   if (!(h->gexec && key == h->gkey)) {
     if (h->gexec) {
       cudaGraphExecDestroy(h->gexec);
