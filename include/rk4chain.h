@@ -82,8 +82,8 @@ enum rk4_bc { RK4_PERIODIC = 0, RK4_FIXED = 1 };
  *   every block of k steps, separated by a bounded-wait grid barrier.
  * Every scheme performs the same floating-point operations per site, so all give
  * bit-identical results.  FP64 steps run their later stages' differences in pairs of floats; a
- * tile with a value that those do not hold (below 2^-70, or from 2^16 on, harmonic 2^40) is advanced in
- * FP64 alone, and results then agree to rounding between tilings. */
+ * tile with a value that those are not good for (below 2^-70; Roessler dt |x - c| > 1/4, dt |y| or dt |z| > 0.3;
+ * harmonic 2^40) is advanced in FP64 alone, and results then agree to rounding between tilings. */
 enum rk4_kernel { RK4_KERNEL_AUTO = 0, RK4_KERNEL_STAGED = 1, RK4_KERNEL_BLOCKED = 2, RK4_KERNEL_PERSISTENT = 3 };
 
 /* Model parameters.  Defaults (rk4_params_default): a = 0.2, b = 1, c = 9 (Sec. 3.1),

@@ -237,7 +237,7 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 2 : 1) k_gen_split(BlockedJob 
 #pragma unroll
     for (int d = 0; d < D; ++d) {
       y[v][d] = tl[(base + v) * D + d];
-      wide |= !split_in_range<MODEL>(y[v][d]);
+      wide |= !split_in_range<MODEL>(y[v][d], d, cf.c, sc);
       live |= !is_nan(y[v][d]) && !((ghost >> v) & 1u);
     }
   }
@@ -257,7 +257,7 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 2 : 1) k_gen_split(BlockedJob 
 #pragma unroll
     for (int d = 0; d < D; ++d) {
       tl[(base + v) * D + d] = y[v][d];
-      wide |= base + v >= H && base + v < H + cnt && !split_in_range<MODEL>(y[v][d]);
+      wide |= base + v >= H && base + v < H + cnt && !split_in_range<MODEL>(y[v][d], d, cf.c, sc);
     }
   if (__syncthreads_or(wide) && !nan_tile) {
     gen_wide_tile<MODEL, RANGE>(job, ch, t0, H, cf, kappa2, tb, smem);
@@ -408,7 +408,7 @@ __global__ void __launch_bounds__(256) k_gen_split_combine(GenStagedJob job, Spl
     join(N, &nd, 1);
     const double r = fma(sc.w, fma(st.B, K[i], -nd), Y[i]);
     Y[i] = r;
-    wide |= !split_in_range<MODEL>(r);
+    wide |= !split_in_range<MODEL>(r, (int)(i % D), sc.c, sc);
     bad |= nonfinite(r);
   }
   if (wide) job.hdr->wide[job.parity ^ 1] = 1u;

@@ -164,7 +164,7 @@ __global__ void __launch_bounds__(256) k_staged_split(StagedJob job, Coef<double
       join(N[q], &nd, 1);
       const double r = split_final(y[q], K1[i * D + q], nd, 6.0, s.w);
       Y[i * D + q] = r;
-      wide |= !split_in_range<MODEL>(r);
+      wide |= !split_in_range<MODEL>(r, q, c.c, s);
       bad |= nonfinite(r);
     }
     if (wide) job.hdr->wide[job.parity ^ 1] = 1u;
@@ -180,7 +180,8 @@ __global__ void __launch_bounds__(256) k_split_scan(const double *y, const doubl
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += stride) {
 #pragma unroll
-    for (int d = 0; d < D; ++d) wide |= !split_in_range<MODEL>(y[i * D + d]);
+    for (int d = 0; d < D; ++d)
+      wide |= !split_in_range<MODEL>(y[i * D + d], d, MODEL == ROESSLER && sp ? sp[i * P + 2] : sc.c, sc);
     if (sp) {
 #pragma unroll
       for (int q = 0; q < P; ++q) wide |= !split_param_in_range(sp[i * P + q], sc.most[q]);

@@ -996,20 +996,25 @@ unsigned high_word(double v) {
 }
 
 // The largest magnitudes the split form takes: a, b, c, kappa (Roessler) or w2, kappa (harmonic).
-// The differences D are dt |J| times the first slope; with dt times each linear coefficient at
-// most 1/8 (the coupling counts fourfold) their pair arithmetic stays below the state's rounding
-// (measured error against the FP64 form's: 0.5 at dt |J| = 0.1, 0.8 at 0.2, above 1 from 0.25 to
-// 0.5 on).  b only has to leave room for z in FP32's exponent range.
+// The differences D are dt |J| times the first slope; with dt times each coefficient at most 1/8 (the
+// coupling counts fourfold) and the state within split_in_range their pair arithmetic stays below the
+// state's rounding (rk4_split.cuh has the errors).
 void split_most(int model, double dt, double *most) {
   if (model == RK4_ROESSLER) {
     most[0] = most[2] = 0.125 / dt;
-    most[1] = 65536.0;
+    most[1] = 0.125 / dt;
     most[3] = 0.125 / (4.0 * dt);
   } else {
     most[0] = 1.0 / (128.0 * dt * dt);
     most[1] = 1.0 / (512.0 * dt * dt);
   }
 }
+// The largest |x - c| and |y|, |z| of a Roessler state (split_in_range).  One step of uniform states, dt =
+// 0.01, a, c and kappa at their limits, error of z in units of the FP64 form's: 0.86 with these, 1.1
+// with dt |x - c| up to 0.3, 1.6 with 0.4; the attractor reaches dt |x - c| = 0.21, dt z = 0.24 for c = 9 and
+// 0.29, 0.49 for c at its limit.
+constexpr double kSplitFar = 0.25, kSplitBig = 0.3;
+constexpr double kSplitMostDt[] = {1.0 / 16, 1.0 / 8};  // Roessler (1.05 .. 1.3 from 1/12 on), harmonic
 bool split_takes(double v, double most) {
   const double a = std::fabs(v);
   return a == 0.0 || (a >= 0x1p-60 && a <= most);
@@ -1019,7 +1024,7 @@ bool split_takes(double v, double most) {
 
 bool rk4d::split_allowed(int model, const CoefD &c) {
   const double dt = c.h1;
-  if (!(dt >= 0x1p-20 && dt <= 0.125)) return false;
+  if (!(dt >= 0x1p-20 && dt <= kSplitMostDt[model == RK4_ROESSLER ? 0 : 1])) return false;
   double most[4];
   split_most(model, dt, most);
   if (model == RK4_ROESSLER)
@@ -1102,6 +1107,9 @@ SplitCoef rk4d::split_coef(int model, const CoefD &c, bool generic) {
   double most[4] = {};
   split_most(model, c.h1, most);
   for (int i = 0; i < 4; ++i) s.most[i] = high_word(most[i]);
+  s.c = c.c;
+  s.far = high_word(kSplitFar / c.h1);
+  s.big = high_word(model == RK4_ROESSLER ? kSplitBig / c.h1 : 0x1p40);
   return s;
 }
 

@@ -26,11 +26,13 @@ struct CoefD {
 
 // Coefficients of the split FP64 step (rk4_split.cuh): tau = dt / 2 (generic tableaux: dt), and the
 // products with it as float pairs (h + l).  at: Roessler a tau, harmonic w2 tau.  most: high words of the largest
-// magnitudes a site's own parameters may have (heterogeneous chains; in their order).
+// magnitudes a site's own parameters may have (heterogeneous chains; in their order); far, big: of the
+// largest |x - c| (Roessler) and of the other components of a state (split_in_range).
 struct SplitCoef {
   double w;  // tau / 3 (generic tableaux: dt)
+  double c;
   float tauh, taul, kth, ktl, k2h, k2l, ath, atl, ch, cl;
-  unsigned most[4];
+  unsigned most[4], far, big;
 };
 
 // Generic explicit Runge-Kutta tableau (strictly lower a, weights b), up to kMaxStages stages.

@@ -17,11 +17,17 @@
 //   y <- y + (tau / 3) (6 K1 + 2 D2 + 2 D3 + D4)     FP64, one rounding      (Eq. (5))
 //
 // Why this loses nothing: a pair's relative error is about 2^-49, D is dt |J| times K1, and D
-// enters the state times dt; with dt |J| at most 1/8 (split_allowed) that puts its error some
-// four bits below the rounding of the state, and the state is rounded once per component and
-// step where the FP64 form rounds it four times.  Measured against long double (N = 1024,
-// 1 .. 1000 steps, dt = 0.01, kappa = 1 and 2): 0.48 .. 0.57 of the FP64 form's error in every
-// component, Roessler and harmonic.
+// enters the state times dt; with dt |J| at most about 1/4 (split_allowed bounds the coefficients,
+// split_in_range the state: the Roessler chain's J holds x - c and z) that stays below the rounding of
+// the state, and the state is rounded once per component and step where the FP64 form rounds it four
+// times.  Error against long double in units of the FP64 form's (2-norms per component):
+//   dt = 0.01, kappa = 1 and 2, uniform[-1, 1) and 1 .. 1000 steps         0.48 .. 0.57
+//   on the attractor (c = 5.7 .. 12.5, dt c up to 1/8)                      0.50
+//   one step, uniform states, dt = 1e-4 .. 1/16, at the edge of both rules  x, y 0.5 .. 0.75, z up to 0.97
+// Where a step changes a component by more than its own size (a Roessler chain's z below 12 dt b, the
+// momenta of a harmonic chain at rest) the error of that step is up to 3 (1.25) times the FP64 form's:
+// the stages share the first slope's rounding, and a difference is no longer small.  Beyond the rules
+// (uniform states, dt = 0.01, one step) z lost a factor of 1.6 at |x|, |z| = 40 and 24 at 160.
 //
 // Every function is written over a lane type T: float (one site) or f32x2 (two sites in one
 // packed instruction), which round alike, so kernels with any number of sites per thread and
@@ -202,14 +208,16 @@ __device__ __forceinline__ void join(FPair<f32x2> v, double *out, int stride) {
 
 // ---- range ----------------------------------------------------------------------------------
 
-// Whether a state value is zero or of a magnitude the pairs represent with full relative
-// precision through a step: at least 2^-70, and below 2^16 for the Roessler chain, whose stages
-// square (z x), or 2^40 for the linear harmonic chain.  NaN and infinity are out of range.
-template <int MODEL> __device__ __forceinline__ bool split_in_range(double v) {
+// Whether component d of a site's state is zero or of a magnitude the differences' pairs are good
+// for: at least 2^-70, whose products keep their relative precision through a step, and at most what
+// keeps dt |J| where their errors stay below the state's rounding.  The Roessler chain's J holds x - c
+// and z: dt |x - c| <= 1/4, dt |y| and dt |z| <= 0.3 (c: the site's own).  The harmonic chain is linear,
+// and its limit, 2^40, only leaves room in FP32's exponents.  NaN and infinity are out of range.
+template <int MODEL> __device__ __forceinline__ bool split_in_range(double v, int d, double c, const SplitCoef &s) {
   constexpr unsigned lo = (1023u - 70u) << 20;
-  constexpr unsigned hi = (1023u + (MODEL == ROESSLER ? 16u : 40u)) << 20;
   const unsigned a = (unsigned)__double2hiint(v) & 0x7fffffffu;
-  return (a - lo < hi - lo) | ((a | (unsigned)__double2loint(v)) == 0u);
+  const bool top = MODEL == ROESSLER && d == 0 ? ((unsigned)__double2hiint(sub(v, c)) & 0x7fffffffu) <= s.far : a <= s.big;
+  return ((a >= lo) | ((a | (unsigned)__double2loint(v)) == 0u)) & top;
 }
 __device__ __forceinline__ bool is_nan(double v) {
   const unsigned a = (unsigned)__double2hiint(v) & 0x7fffffffu;

@@ -835,9 +835,11 @@ __device__ __forceinline__ bool tile_item(const R *__restrict__ in, R *__restric
     double *spd = nullptr;
     f32x2 *spf = nullptr;
 #pragma unroll
-    for (int v = 0; v < V; ++v)
+    for (int v = 0; v < V; ++v) {
+      const double c = HET && MODEL == ROESSLER ? ptl[(base + v) * P + 2] : cf.c;
 #pragma unroll
-      for (int d = 0; d < D; ++d) wide |= !split_in_range<MODEL>(y[v][d]);
+      for (int d = 0; d < D; ++d) wide |= !split_in_range<MODEL>(y[v][d], d, c, *sc);
+    }
     if constexpr (HET) {
       // the parameters move to thread-private slots (consecutive threads, consecutive addresses),
       // beside the pair coefficients of each pair of sites
@@ -904,8 +906,12 @@ __device__ __forceinline__ bool tile_item(const R *__restrict__ in, R *__restric
     for (int d = 0; d < D; ++d) {
       tl[(base + v) * D + d] = y[v][d];
       if constexpr (KAHAN) ctl[(base + v) * D + d] = cmp[v][d];
-      if constexpr (SPLIT) bad |= stored && !split_in_range<MODEL>(y[v][d]);
-      else bad |= stored && nonfinite(y[v][d]);
+      if constexpr (SPLIT) {
+        const double c = HET && MODEL == ROESSLER ? ptl[(v * P + 2) * blockDim.x + threadIdx.x] : cf.c;
+        bad |= stored && !split_in_range<MODEL>(y[v][d], d, c, *sc);
+      } else {
+        bad |= stored && nonfinite(y[v][d]);
+      }
     }
   }
   const int any_bad = __syncthreads_or(bad);
@@ -1004,7 +1010,7 @@ __device__ __forceinline__ bool packed_tile_item(const R *__restrict__ in, R *__
 #pragma unroll
     for (int v = 0; v < V; ++v)
 #pragma unroll
-      for (int d = 0; d < D; ++d) wide |= !split_in_range<MODEL>(y[v][d]);
+      for (int d = 0; d < D; ++d) wide |= !split_in_range<MODEL>(y[v][d], d, c.c, *scp);
     nan_tile = __syncthreads_or(wide);
     if (nan_tile) {
       bool live = false;
@@ -1032,7 +1038,7 @@ __device__ __forceinline__ bool packed_tile_item(const R *__restrict__ in, R *__
     for (int d = 0; d < D; ++d) {
       tl[(base + v) * D + d] = y[v][d];
       if constexpr (KAHAN) ctl[(base + v) * D + d] = cmp[v][d];
-      if constexpr (SPLIT) bad |= stored && !split_in_range<MODEL>(y[v][d]);
+      if constexpr (SPLIT) bad |= stored && !split_in_range<MODEL>(y[v][d], d, c.c, *scp);
       else bad |= stored && nonfinite(y[v][d]);
     }
   }

@@ -1,0 +1,88 @@
+"""The split FP64 step's error against long double, component by component, over the states and
+coefficients it accepts and just beyond (where the FP64 form takes over): no larger than that of the FP64
+form it replaces, whose operations (rk4_device.cuh, rk4_generic.cuh) are repeated here with one rounding each.
+
+Tolerance: the ratio of two 2-norms over 20000 sites scatters by about 0.5 % (errors of either side are
+sums of a few roundings); 1.01 is asserted.  Where the library runs the FP64 form both sides are the
+same numbers but for double roundings of the long-double products (one in 2^11)."""
+import numpy as np
+import pytest
+
+import chain_inputs as ci
+
+pytestmark = pytest.mark.gpu
+
+L = np.longdouble
+N = 20000
+
+
+def fma(a, b, c):
+    return (L(a) * b + c).astype(np.float64)
+
+
+def slope(u, p, one):
+    """Slopes of a periodic Roessler chain; one: long double throughout, else the FP64 operations."""
+    xl, xr = np.roll(u[0], 1), np.roll(u[0], -1)
+    if one:
+        return [p["kappa"] * (xl - 2 * u[0] + xr) - (u[1] + u[2]), u[0] + p["a"] * u[1], p["b"] + u[2] * (u[0] - p["c"])]
+    return [fma(p["kappa"], fma(-2.0, u[0], xl + xr), -(u[1] + u[2])), fma(p["a"], u[1], u[0]),
+            fma(u[2], u[0], fma(-p["c"], u[2], p["b"]))]
+
+
+def rk4(y, p, dt, steps):
+    """The state after `steps` steps in long double and in the FP64 form."""
+    exact, plain = [v.astype(L) for v in y], [v.copy() for v in y]
+    lp = {k: L(v) for k, v in p.items()}
+    h = L(np.float64(dt))
+    for _ in range(steps):
+        ks, u = [], exact
+        for w in (h / 2, h / 2, h, None):
+            ks.append(slope(u, lp, True))
+            if w is not None:
+                u = [v + w * k for v, k in zip(exact, ks[-1])]
+        exact = [v + h / 6 * (a + 2 * b + 2 * c + d) for v, a, b, c, d in zip(exact, *ks)]
+        acc, u = plain, plain
+        for j, w in enumerate((dt / 2, dt / 2, dt, None)):
+            k = slope(u, p, False)
+            acc = [fma(dt / 6 if j in (0, 3) else dt / 3, q, v) for q, v in zip(k, acc)]
+            if w is not None:
+                u = [fma(w, q, v) for q, v in zip(k, plain)]
+        plain = acc
+    return exact, plain
+
+
+def check(got, exact, plain, what):
+    for d in range(3):
+        ours = float(np.sqrt(np.sum((got[:, d] - exact[d]) ** 2)))
+        theirs = float(np.sqrt(np.sum((plain[d] - exact[d]) ** 2)))
+        print(f"{what}: component {d}: {ours / theirs:.3f} of the FP64 form's error")
+        assert ours <= 1.01 * theirs, (what, d)
+
+
+# dt, c, kappa, amplitude of a uniform state: ordinary ones, the edges of the state's range (dt |x - c| = 1/4)
+# and beyond, coefficients and dt at their limits and beyond
+CASES = [(0.01, 9.0, 1.0, 1.0), (0.01, 9.0, 1.0, 15.9), (0.01, 9.0, 1.0, 20.0), (0.01, 9.0, 1.0, 40.0),
+         (0.01, 9.0, 1.0, 100.0), (0.01, 9.0, 1.0, 1000.0), (0.01, 9.0, 1.0, 3e4), (0.01, 5.7, 2.0, 18.0),
+         (0.0138, 9.0, 2.0, 9.0), (0.0138, 9.0, 2.0, 12.0), (0.05, 2.4, 0.6, 2.5), (0.0625, 2.0, 0.5, 1.9),
+         (0.0625, 2.0, 0.5, 4.0), (0.07, 1.5, 0.4, 1.0), (0.125, 1.0, 0.25, 1.0), (1e-4, 1250.0, 300.0, 1200.0)]
+
+
+@pytest.mark.parametrize("dt,c,kappa,amp,steps",
+                         [(*case, steps) for case in CASES for steps in (1, 3)
+                          if steps == 1 or case[3] != 3e4])  # from 3e4 on the third step overflows
+def test_uniform_states(dt, c, kappa, amp, steps):
+    import gpu_helpers as gh
+    y0 = ci.uniform_state(N, 3, seed=1250) * amp
+    p = dict(a=0.2, b=1.0, c=c, kappa=kappa)
+    exact, plain = rk4([y0[:, d].copy() for d in range(3)], p, dt, steps)
+    for tiling in [(256, 4, 2), (128, 1, 4)]:
+        check(gh.gpu_run(y0, nsteps=steps, dt=dt, params=p, tiling=tiling), exact, plain, (dt, c, amp, steps, tiling))
+
+
+@pytest.mark.parametrize("dt,c", [(0.01, 9.0), (0.0138, 9.0), (0.01, 5.7)])
+def test_on_the_attractor(dt, c):
+    import gpu_helpers as gh
+    p = dict(a=0.2, b=1.0, c=c, kappa=1.0)
+    y0 = gh.gpu_run(ci.uniform_state(N, 3, seed=1251), nsteps=6000, dt=dt, params=p)
+    exact, plain = rk4([y0[:, d].copy() for d in range(3)], p, dt, 1)
+    check(gh.gpu_run(y0, nsteps=1, dt=dt, params=p, tiling=(256, 4, 1)), exact, plain, (dt, c))
