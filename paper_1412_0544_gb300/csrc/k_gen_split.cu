@@ -1,26 +1,30 @@
 // k_gen_split.cu -- the generic scheme (any explicit tableau of up to 7 stages, coupling range 1
-// or 2) for FP64 in the split form of rk4_split.cuh: K1 = f(y) in FP64, the later slopes' negated
-// differences n_m = K1 - k_m in float pairs,
-//   d_j = c_j K1 - sum_m a_jm n_m      (u_j = y + dt d_j, c_j the row sum; Eq. (4))
-//   y <- y + dt (B K1 - sum_m b_m n_m)  (B the sum of the weights; Eq. (5)),
-// for whatever tableau the kernel is given at run time.
+// or 2) for FP64 in the split form of rk4_split.cuh, taken one term further: K1 = f(y) and M = J(y) K1
+// (the first-order term of every later slope) in FP64, and what is left of the later slopes, the
+// remainders r_m = K1 + c_m dt M - k_m, in float pairs:
+//   u_j = y + dt (c_j K1 + e_j),  e_j = (sum_m a_jm c_m) dt M - sum_m a_jm r_m    (c_j the row sum; Eq. (4))
+//   -r_j = dt J(y) e_j + (0, 0, dt^2 (c_j K1 + e_j)_x (c_j K1 + e_j)_z)       (f's only product: Eq. (6))
+//   y <- y + dt (B K1 + (sum_m b_m c_m) dt M - sum_m b_m r_m)             (B the sum of the weights; Eq. (5)),
+// for whatever tableau the kernel is given at run time.  A first stage after K1 (no a_jm with m >= 1) has
+// e_j = 0 and needs no exchange, so a step exchanges as often as the tableau has stages.
 //
-// What bounds it: Dormand-Prince 5 with second neighbours issued 123 DFMA per site-step, now 16
-// (10 for the first slope, 6 for the update) beside some 1100 FP32 operations: FMA pipe 47 %,
-// FP64 pipe 35 % busy, 16 warps per SM (128 registers), the rest latency.  Every thread holds two
-// sites (one packed pair) whatever the tiling's sites per thread, so a tile of W sites runs on
-// W / 2 threads; the differences lie in thread-private shared-memory records, which both frees
-// their registers (five stages of three pairs, 60 registers) and lets the stage loops run over any
-// tableau's nonzero entries without a kernel per tableau.  Measured at N = 2^20, us per step, best
-// tiling: Dormand-Prince 5 + second neighbours 245 -> 78, RK4 + second neighbours 128 -> 54 (run-time
-// tableaux 345 -> 78).  With the state and the first slope in registers too (164, one block of 256
-// threads per SM) it took 89.
+// Why the extra term: the differences K1 - k_m are c_m dt |J| times K1, and with rows up to 25 in sum of
+// magnitudes (Dormand-Prince 5) their pairs' errors showed: 1.05 of the FP64 form's error after one step
+// (z 1.15, 2.2 at |x|, |z| = 20; x 1.04 with kappa = 2, kappa2 = 0.7), because the FP64 form rounds its state
+// only once a step.  The remainders are smaller again by dt |J|: 0.92 ..
+// 1.002 in each component after one and two steps (Dormand-Prince 5 and RK4, dt = 0.01 .. 0.06, kappa up to 2,
+// kappa2 up to 0.7, |x|, |z| up to 15), without normalising any pair.  M's rows in pairs left x at 1.03.
+// The weights' sum is carried to a float beyond FP64: its own rounding, times dt K1 every step, was a
+// drift of 1.2 after 20 steps.
 //
-// Error against long double, in units of the FP64 form's: 1.00 from 10 .. 20 steps on, 1.05 after
-// one Dormand-Prince step from a random state (z alone 1.15; its differences carry dt |x - c|, and
-// pairs of their own roundings), 1.01 for RK4 with second neighbours.  The tails are normalised
-// (pair_norm) where the rows multiply them by up to 11; without, 1.12.  The weights' sum is carried
-// to a float beyond FP64: its own rounding, times dt K1 every step, was a drift of 1.2.
+// What bounds it: the FP64 pipe takes 30 instructions per site-step with second neighbours (10 for K1, 11 for
+// M, 3 and 6 for the update; 123 in the FP64 form) beside some 1000 FP32
+// operations, 16 warps per SM (128 registers).  Every thread holds two sites (one packed pair) whatever the
+// tiling's sites per thread, so a tile of W sites runs on W / 2 threads; M and the remainders lie in
+// thread-private shared-memory records, which both frees their registers and lets the stage loops run over
+// any tableau's nonzero entries without a kernel per tableau.  Measured at N = 2^20, us per step, best
+// tiling, FP64 form -> now: Dormand-Prince 5 + second neighbours 245 -> 101, RK4 + second neighbours 128 -> 83
+// (78 and 54 with differences from K1 alone, 16 FP64 instructions).
 #include <algorithm>
 
 #include "rk4_generic.cuh"
@@ -29,10 +33,50 @@ namespace rk4d {
 
 constexpr int kGenSplitThreads = 512;
 
-// 8-byte words of a thread's record: the pairs of up to s - 1 differences and, when parked (blocks
-// of up to 256 threads), the state and the first slope in FP64; odd (see split_record_words).
-__host__ __device__ constexpr int gen_record_words(int s, int D, bool park) {
-  return ((s - 1 + (park ? 2 : 0)) * D * 2) | 1;
+// 8-byte words of a thread's record: -dt M and the remainders of `slots` stages as pairs and, when parked
+// (blocks of up to 256 threads), the state and the FP64 part of the update; odd (see split_record_words).
+__host__ __device__ constexpr int gen_record_words(int slots, int D, bool park) {
+  return ((slots + 1 + (park ? 2 : 0)) * D * 2) | 1;
+}
+
+// r_z = -(z dt e_x + (x - c) dt e_z + (dt dx)(dt dz)), the first two only when there is an e (EX); nde, dfe:
+// dt e_x = dfe - nde (split_linear); d: the increments c_j K1 + e of x and z.
+template <typename T, bool EX>
+__device__ __forceinline__ FPair<T> gen_remainder_z(const FPair<T> &dx, const FPair<T> &dz, const FPair<T> &ez, T nde, T dfe,
+                                                    const SplitBase<T> &b, const FPair<T> &tau) {
+  const T m1 = vset<T>(-1.f);
+  const T ntau = vmul(m1, tau.h);
+  FPair<T> u, v;
+  T np3, e3;
+  u = pair_mul(tau, ntau, dx);
+  v = pair_mul(tau, ntau, dz);
+  mul_coef(u, vmul(m1, u.h), v, np3, e3);
+  if constexpr (!EX) return {np3, vmul(m1, e3)};
+  T np1, e1, np2, e2, s, ne1, ne2;
+  mul_coef(b.z, vmul(m1, b.z.h), FPair<T>{vmul(m1, nde), dfe}, np1, e1);
+  mul_coef(b.t, vmul(m1, b.t.h), pair_mul(tau, ntau, ez), np2, e2);
+  FPair<T> r;
+  two_sum(np1, np2, s, ne1);
+  two_sum(s, np3, r.h, ne2);
+  r.l = vadd(vsub(ne1, vadd(e1, e2)), vsub(ne2, e3));
+  return r;
+}
+
+// M = J(y) K1 of one site: slope_gen's rows are linear but for the Roessler chain's z.
+template <int MODEL, int RANGE>
+__device__ __forceinline__ void gen_second_slope(const double *y, const double *k1, double l1, double r1, double l2,
+                                                 double r2, const Coef<double> &cf, double kappa2, double *M) {
+  slope_gen<double, MODEL, RANGE>(k1, l1, r1, l2, r2, cf, kappa2, M);
+  if constexpr (MODEL == ROESSLER) M[2] = fma(y[2], k1[0], mul(fma(y[0], cf.one, -cf.c), k1[2]));
+}
+// The FP64 part of the update, B K1 + (sum_m b_m c_m) dt M.
+__device__ __forceinline__ double gen_update64(double k1, double M, const SplitTableau &tb) {
+  return fma(tb.E, M, tb.unit ? k1 : mul(tb.B, k1));
+}
+// -dt M as a pair.
+template <typename T> __device__ __forceinline__ FPair<T> gen_first_order(const FPair<T> &M, const FPair<T> &tau) {
+  const T m1 = vset<T>(-1.f);
+  return pair_mul(FPair<T>{vmul(m1, tau.h), vmul(m1, tau.l)}, tau.h, M);
 }
 
 // A tile outside the split's range in the FP64 form (two sites per thread, run-time tableau).
@@ -75,7 +119,7 @@ __device__ __noinline__ void gen_wide_tile(const BlockedJob &job, ChainDesc ch, 
 }
 
 // K steps on the thread's two sites.  ex: two parities of 16 bytes per thread, a thread's two
-// coupling coordinates (FP64, or their increments as a packed pair), read by its neighbours.
+// coupling coordinates (FP64, or as a packed pair), read by its neighbours.
 template <int MODEL, int RANGE, bool MASK, bool PARK>
 __device__ __forceinline__ void gen_split_advance(double (&y)[2][Dim<MODEL>::D], uint32_t ghost, int K,
                                                   const Coef<double> &cf, double kappa2, const SplitCoef &sc,
@@ -85,7 +129,8 @@ __device__ __forceinline__ void gen_split_advance(double (&y)[2][Dim<MODEL>::D],
   const int tid = threadIdx.x, bd = blockDim.x;
   const int lt = tid > 0 ? tid - 1 : tid, rt = tid < bd - 1 ? tid + 1 : tid;
   const StageCoef<T> c = stage_coef<T>(sc);
-  double *py = reinterpret_cast<double *>(rec + (tb.s - 1) * D * 2), *pk = py + 2 * D;
+  f32x2 *rm = rec + 2 * D;  // the remainders, after -dt M
+  double *py = reinterpret_cast<double *>(rm + tb.slots * 2 * D), *ps = py + 2 * D;
   if constexpr (PARK) {
 #pragma unroll
     for (int i = 0; i < 2 * D; ++i) py[i] = y[i / D][i % D];
@@ -99,99 +144,134 @@ __device__ __forceinline__ void gen_split_advance(double (&y)[2][Dim<MODEL>::D],
     l = e[lt];
     r = e[rt];
   };
+  auto exchange64 = [&](const double (&x)[2], double (&l)[2], double (&r)[2]) {
+    ulonglong2 a, b;
+    exchange(make_ulonglong2(__double_as_longlong(x[0]), __double_as_longlong(x[1])), a, b);
+    l[1] = __longlong_as_double(a.x);
+    l[0] = __longlong_as_double(a.y);
+    r[0] = __longlong_as_double(b.x);
+    r[1] = __longlong_as_double(b.y);
+  };
 #pragma unroll 1
   for (int s = 0; s < K; ++s) {
-    double k1d[2][D];
-    FPair<T> k1[D];
+    double s64[2][D];
+    FPair<T> k1x = {}, k1z = {};  // of the first slope only these two enter a product,
+    T k1h[D];                     // and the heads B's rounding
     SplitBase<T> base = {};
     {
       if constexpr (PARK) {
 #pragma unroll
         for (int i = 0; i < 2 * D; ++i) y[i / D][i % D] = py[i];
       }
-      double x[2];
+      double x[2], l[2], r[2], k1[2][D], M[2][D];
 #pragma unroll
       for (int v = 0; v < 2; ++v) x[v] = (MASK && ((ghost >> v) & 1u)) ? 0.0 : y[v][0];
-      ulonglong2 l, r;
-      exchange(make_ulonglong2(__double_as_longlong(x[0]), __double_as_longlong(x[1])), l, r);
-      const double l2 = __longlong_as_double(l.x), l1 = __longlong_as_double(l.y);
-      const double r1 = __longlong_as_double(r.x), r2 = __longlong_as_double(r.y);
-      slope_gen<double, MODEL, RANGE>(y[0], l1, x[1], l2, r1, cf, kappa2, k1d[0]);
-      slope_gen<double, MODEL, RANGE>(y[1], x[0], r1, l1, r2, cf, kappa2, k1d[1]);
+      exchange64(x, l, r);
+      slope_gen<double, MODEL, RANGE>(y[0], l[0], x[1], l[1], r[0], cf, kappa2, k1[0]);
+      slope_gen<double, MODEL, RANGE>(y[1], x[0], r[0], l[0], r[1], cf, kappa2, k1[1]);
 #pragma unroll
-      for (int i = 0; i < D; ++i) k1[i] = Lanes<T>::split(&k1d[0][i], D);
+      for (int v = 0; v < 2; ++v) x[v] = (MASK && ((ghost >> v) & 1u)) ? 0.0 : k1[v][0];
+      exchange64(x, l, r);
+      gen_second_slope<MODEL, RANGE>(y[0], k1[0], l[0], x[1], l[1], r[0], cf, kappa2, M[0]);
+      gen_second_slope<MODEL, RANGE>(y[1], k1[1], x[0], r[0], l[0], r[1], cf, kappa2, M[1]);
+#pragma unroll
+      for (int i = 0; i < D; ++i) {
+#pragma unroll
+        for (int v = 0; v < 2; ++v) s64[v][i] = gen_update64(k1[v][i], M[v][i], tb);
+        const FPair<T> k = Lanes<T>::split(&k1[0][i], D);
+        k1h[i] = k.h;
+        if (i == 0) k1x = k;
+        if (i == 2) k1z = k;
+        const FPair<T> m = gen_first_order(Lanes<T>::split(&M[0][i], D), c.tau);
+        rec[2 * i] = m.h;
+        rec[2 * i + 1] = m.l;
+      }
       if constexpr (MODEL == ROESSLER) {
         base.z = Lanes<T>::split(&y[0][2], D);
         base.t = x_minus_c<T>(Lanes<T>::split(&y[0][0], D), {vset<T>(sc.ch), vset<T>(sc.cl)});
       }
       if constexpr (PARK) {
 #pragma unroll
-        for (int i = 0; i < 2 * D; ++i) pk[i] = k1d[i / D][i % D];
+        for (int i = 0; i < 2 * D; ++i) ps[i] = s64[i / D][i % D];
       }
     }
+    FPair<T> n[D];
 #pragma unroll 1
-    for (int j = 1; j < tb.s; ++j) {
+    for (int j = 1; j <= tb.last; ++j) {
       if (!((tb.need >> j) & 1u)) continue;
-      FPair<T> d[D], n[D];
-      {
+      FPair<T> e[D];
+#pragma unroll
+      for (int i = 0; i < D; ++i) n[i] = e[i] = {0ull, 0ull};
+      T nde = 0ull, dfe = 0ull;
+      const bool row = tb.na[j] > 0;
+      if (row) {
+        const FPair<T> g = {vset<T>(-tb.gh[j]), vset<T>(-tb.gl[j])};
+        const T ng = vset<T>(tb.gh[j]);
+#pragma unroll
+        for (int i = 0; i < D; ++i) e[i] = pair_mul(g, ng, {rec[2 * i], rec[2 * i + 1]});
+#pragma unroll 2
+        for (int q0 = 0; q0 < tb.na[j]; ++q0) {
+          const int m = tb.ma[j][q0];
+          const FPair<T> a = {vset<T>(tb.ah[j][m]), vset<T>(tb.al[j][m])};
+          const T na = vset<T>(-tb.ah[j][m]);
+          const f32x2 *q = rm + tb.slot[m] * D * 2;
+#pragma unroll
+          for (int i = 0; i < D; ++i) e[i] = pair_fnma<T>(a, na, {q[2 * i], q[2 * i + 1]}, e[i]);
+        }
+        FPair<T> X = e[0];
+        if constexpr (MASK) {
+          const bool g0 = ghost & 1u, g1 = ghost & 2u;
+          X.h = pack2(g0 ? 0.f : lane0(X.h), g1 ? 0.f : lane1(X.h));
+          X.l = pack2(g0 ? 0.f : lane0(X.l), g1 ? 0.f : lane1(X.l));
+        }
+        ulonglong2 l, r;
+        exchange(make_ulonglong2(X.h, X.l), l, r);
+        const FPair<T> xl = {pack2(lane1(l.x), lane0(X.h)), pack2(lane1(l.y), lane0(X.l))};
+        const FPair<T> xr = {pack2(lane1(X.h), lane0(r.x)), pack2(lane1(X.l), lane0(r.y))};
+        // second neighbours: the left thread's two sites, the right thread's two sites
+        split_linear<MODEL, T, RANGE>(e, xl, xr, c, n, nde, dfe, {l.x, l.y}, {r.x, r.y});
+      }
+      if constexpr (MODEL == ROESSLER) {
         const FPair<T> cj = {vset<T>(tb.ch[j]), vset<T>(tb.cl[j])};
         const T nc = vset<T>(-tb.ch[j]);
-#pragma unroll
-        for (int i = 0; i < D; ++i) d[i] = pair_mul(cj, nc, k1[i]);
+        const FPair<T> dx = pair_fma(cj, nc, k1x, e[0]), dz = pair_fma(cj, nc, k1z, e[2]);
+        n[2] = row ? gen_remainder_z<T, true>(dx, dz, e[2], nde, dfe, base, c.tau)
+                   : gen_remainder_z<T, false>(dx, dz, e[2], nde, dfe, base, c.tau);
       }
-#pragma unroll 2
-      for (int q0 = 0; q0 < tb.na[j]; ++q0) {
-        const int m = tb.ma[j][q0];
-        const FPair<T> a = {vset<T>(tb.ah[j][m]), vset<T>(tb.al[j][m])};
-        const T na = vset<T>(-tb.ah[j][m]);
-        const f32x2 *q = rec + (m - 1) * D * 2;
+      if (j != tb.last) {
+        f32x2 *o = rm + tb.slot[j] * D * 2;
 #pragma unroll
-        for (int i = 0; i < D; ++i) d[i] = pair_fnma<T>(a, na, {q[2 * i], q[2 * i + 1]}, d[i]);
-      }
-#pragma unroll
-      for (int i = 0; i < D; ++i) d[i] = pair_norm(d[i]);
-      FPair<T> X = d[0];
-      if constexpr (MASK) {
-        const bool g0 = ghost & 1u, g1 = ghost & 2u;
-        X.h = pack2(g0 ? 0.f : lane0(X.h), g1 ? 0.f : lane1(X.h));
-        X.l = pack2(g0 ? 0.f : lane0(X.l), g1 ? 0.f : lane1(X.l));
-      }
-      ulonglong2 l, r;
-      exchange(make_ulonglong2(X.h, X.l), l, r);
-      const FPair<T> xl = {pack2(lane1(l.x), lane0(X.h)), pack2(lane1(l.y), lane0(X.l))};
-      const FPair<T> xr = {pack2(lane1(X.h), lane0(r.x)), pack2(lane1(X.l), lane0(r.y))};
-      // second neighbours: the left thread's two sites, the right thread's two sites
-      split_stage<MODEL, T, RANGE, true>(d, xl, xr, base, c, n, {l.x, l.y}, {r.x, r.y});
-      f32x2 *o = rec + (j - 1) * D * 2;
-#pragma unroll
-      for (int i = 0; i < D; ++i) {
-        n[i] = pair_norm(n[i]);
-        o[2 * i] = n[i].h;
-        o[2 * i + 1] = n[i].l;
+        for (int i = 0; i < D; ++i) {
+          o[2 * i] = n[i].h;
+          o[2 * i + 1] = n[i].l;
+        }
       }
     }
     FPair<T> N[D];
 #pragma unroll
-    for (int i = 0; i < D; ++i) N[i] = {0ull, vmul(vset<T>(-tb.Bl), k1[i].h)};
+    for (int i = 0; i < D; ++i) N[i] = {0ull, vmul(vset<T>(-tb.Bl), k1h[i])};
 #pragma unroll 2
     for (int q0 = 0; q0 < tb.nb; ++q0) {
       const int m = tb.mb[q0];
       const FPair<T> b = {vset<T>(tb.bh[m]), vset<T>(tb.bl[m])};
       const T nb = vset<T>(-tb.bh[m]);
-      const f32x2 *q = rec + (m - 1) * D * 2;
+      const f32x2 *q = rm + tb.slot[m] * D * 2;
 #pragma unroll
       for (int i = 0; i < D; ++i) N[i] = pair_fma<T>(b, nb, {q[2 * i], q[2 * i + 1]}, N[i]);
     }
+    const FPair<T> bl = {vset<T>(tb.bh[tb.last]), vset<T>(tb.bl[tb.last])};
+    const T nbl = vset<T>(-tb.bh[tb.last]);
 #pragma unroll
     for (int i = 0; i < D; ++i) {
       double nd[2];
-      join(N[i], nd, 1);
-      if constexpr (PARK) {
-        py[i] = fma(sc.w, fma(tb.B, pk[i], -nd[0]), py[i]);
-        py[D + i] = fma(sc.w, fma(tb.B, pk[D + i], -nd[1]), py[D + i]);
-      } else {
-        y[0][i] = fma(sc.w, fma(tb.B, k1d[0][i], -nd[0]), y[0][i]);
-        y[1][i] = fma(sc.w, fma(tb.B, k1d[1][i], -nd[1]), y[1][i]);
+      join(pair_fma<T>(bl, nbl, n[i], N[i]), nd, 1);
+#pragma unroll
+      for (int v = 0; v < 2; ++v) {
+        if constexpr (PARK) {
+          py[v * D + i] = fma(sc.w, fma(ps[v * D + i], cf.one, -nd[v]), py[v * D + i]);
+        } else {
+          y[v][i] = fma(sc.w, fma(s64[v][i], cf.one, -nd[v]), y[v][i]);
+        }
       }
     }
   }
@@ -221,7 +301,7 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 2 : 1) k_gen_split(BlockedJob 
   const int64_t t0 = tile * (int64_t)job.G - H;
   ulonglong2 *ex = reinterpret_cast<ulonglong2 *>(smem);
   double *tl = reinterpret_cast<double *>(ex + 2 * blockDim.x);  // the tile, then the records in its place
-  f32x2 *rec = reinterpret_cast<f32x2 *>(tl) + threadIdx.x * gen_record_words(st.s, D, PARK);
+  f32x2 *rec = reinterpret_cast<f32x2 *>(tl) + threadIdx.x * gen_record_words(st.slots, D, PARK);
   tile_load<double, D, false>(tl, static_cast<const double *>(job.in), ch.off, ch.n, ch.bc, t0, W, job.total, job.hdr);
   tile_load_wait();
   __syncthreads();
@@ -275,11 +355,12 @@ static cudaError_t launch_gen_split_k(int threads, const BlockedJob &job, const 
   const cudaError_t e = set_smem_limit_once(k_gen_split<MODEL, RANGE, NT>, 200 * 1024, attr);
   if (e != cudaSuccess) return e;
   if (job.ntiles <= 0) return cudaSuccess;
+  const SplitTableau stb = split_tableau(td, dt);
   const size_t ours = (size_t)threads * (2 * sizeof(ulonglong2) +
-                                         sizeof(double) * std::max(2 * D, gen_record_words(td.s, D, NT <= 256)));
+                                         sizeof(double) * std::max(2 * D, gen_record_words(stb.slots, D, NT <= 256)));
   const size_t wide = sizeof(double) * ((size_t)gen_edge_values(2) + (size_t)threads * 2 * D);
   k_gen_split<MODEL, RANGE, NT><<<(unsigned)job.ntiles, threads, std::max(ours, wide), st>>>(
-      job, to_coef<double>(cfd, cfd.kappa), cfd.kappa2, split_coef(MODEL, cfd, true), split_tableau(td),
+      job, to_coef<double>(cfd, cfd.kappa), cfd.kappa2, split_coef(MODEL, cfd, true), stb,
       to_tableau<double>(td, dt), H);
   return cudaGetLastError();
 }
@@ -303,89 +384,132 @@ cudaError_t launch_gen_split(int model, int range, int sites, const BlockedJob &
 
 // ---- one stage per launch ---------------------------------------------------------------------
 
-// Stage state j in the split form: the increments d_j of every site (float pairs, in job.u).
-template <int MODEL>
-__global__ void __launch_bounds__(256) k_gen_split_state(GenStagedJob job, SplitTableau st, Tableau<double> tb, int j) {
+// The chain of site i; its coupling strength goes into c.
+__device__ __forceinline__ ChainDesc gen_site_chain(const GenStagedJob &job, int64_t i, Coef<double> &c) {
+  if (job.nchains == 1) return job.one;
+  int lo = 0, hi = job.nchains - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (job.chains[mid].off <= i) lo = mid; else hi = mid - 1;
+  }
+  c.kappa = job.chains[lo].kappa;
+  return job.chains[lo];
+}
+// Index of site q of a chain (boundary-resolved), or -1 beyond a fixed end.
+__device__ __forceinline__ int64_t gen_site(const GenStagedJob &job, const ChainDesc &ch, int64_t q) {
+  const int64_t g = (ch.bc == PERIODIC) ? ch.off + wrap(q, ch.n) : ((q < 0 || q >= ch.n) ? -1 : ch.off + q);
+  return g < 0 || !bounds_ok(job.hdr, in_range(g, 1, job.total)) ? -1 : g;
+}
+// M of site i from the first slopes in job.k.
+template <int MODEL, int RANGE>
+__device__ __forceinline__ void gen_staged_second(const GenStagedJob &job, const ChainDesc &ch, int64_t i,
+                                                  const Coef<double> &c, double kappa2, double *M) {
+  constexpr int D = Dim<MODEL>::D;
+  const double *Y = static_cast<const double *>(job.y), *K = static_cast<const double *>(job.k);
+  const int64_t li = i - ch.off;
+  auto xat = [&](int64_t q) {
+    const int64_t g = gen_site(job, ch, q);
+    return g < 0 ? 0.0 : K[g * D];
+  };
+  double y[D], k1[D];
+#pragma unroll
+  for (int q = 0; q < D; ++q) {
+    y[q] = Y[i * D + q];
+    k1[q] = K[i * D + q];
+  }
+  gen_second_slope<MODEL, RANGE>(y, k1, xat(li - 1), xat(li + 1), RANGE == 2 ? xat(li - 2) : 0.0,
+                                 RANGE == 2 ? xat(li + 2) : 0.0, c, kappa2, M);
+}
+
+// Stage state j in the split form: e_j of every site (float pairs, in job.u).
+template <int MODEL, int RANGE>
+__global__ void __launch_bounds__(256) k_gen_split_state(GenStagedJob job, Coef<double> cf, double kappa2, SplitCoef sc,
+                                                         SplitTableau st, Tableau<double> tb, int j) {
   constexpr int D = Dim<MODEL>::D;
   if (job.hdr->wide[job.parity]) {
     gen_state_sweep<double, D>(job, tb, j);
     return;
   }
+  if (st.na[j] == 0) return;  // e_j = 0
   const double *K = static_cast<const double *>(job.k);
   float2 *U = static_cast<float2 *>(job.u);
   const size_t plane = (size_t)job.total * D;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < (int64_t)plane; i += stride) {
-    FPair<float> d = pair_mul<float>({st.ch[j], st.cl[j]}, -st.ch[j], split1(K[i]));
-    for (int m = 1; m < j; ++m) {
-      if (!((st.anz[j] >> m) & 1u)) continue;
-      const float2 n = reinterpret_cast<const float2 *>(K + m * plane)[i];
-      d = pair_fnma<float>({st.ah[j][m], st.al[j][m]}, -st.ah[j][m], {n.x, n.y}, d);
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < job.total; i += stride) {
+    Coef<double> c = cf;
+    const ChainDesc ch = gen_site_chain(job, i, c);
+    double M[D];
+    gen_staged_second<MODEL, RANGE>(job, ch, i, c, kappa2, M);
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+      const FPair<float> nm = gen_first_order<float>(split1(M[d]), {sc.tauh, sc.taul});
+      FPair<float> e = pair_mul<float>({-st.gh[j], -st.gl[j]}, st.gh[j], nm);
+      for (int q = 0; q < st.na[j]; ++q) {
+        const int m = st.ma[j][q];
+        const float2 n = reinterpret_cast<const float2 *>(K + m * plane)[i * D + d];
+        e = pair_fnma<float>({st.ah[j][m], st.al[j][m]}, -st.ah[j][m], {n.x, n.y}, e);
+      }
+      U[i * D + d] = make_float2(e.h, e.l);
     }
-    d = pair_norm(d);
-    U[i] = make_float2(d.h, d.l);
   }
 }
 
-// Slope j: the first slope in FP64, or the negated difference of a later one as pairs.
+// Slope j: the first slope in FP64, or the remainder of a later one as pairs.
 template <int MODEL, int RANGE>
 __global__ void __launch_bounds__(256) k_gen_split_slope(GenStagedJob job, Coef<double> cf, double kappa2, SplitCoef sc,
-                                                         int j) {
+                                                         SplitTableau st, int j) {
   constexpr int D = Dim<MODEL>::D;
   if (j == 0 || job.hdr->wide[job.parity]) {
     gen_slope_sweep<double, MODEL, RANGE>(job, cf, kappa2, j);
     return;
   }
-  const double *Y = static_cast<const double *>(job.y);
+  const double *Y = static_cast<const double *>(job.y), *K = static_cast<const double *>(job.k);
   const float2 *U = static_cast<const float2 *>(job.u);
   float2 *N = reinterpret_cast<float2 *>(static_cast<double *>(job.k) + (size_t)j * job.total * D);
+  const bool row = st.na[j] > 0;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < job.total; i += stride) {
-    ChainDesc ch;
+    Coef<double> c = cf;
+    const ChainDesc ch = gen_site_chain(job, i, c);
     SplitCoef s = sc;
-    if (job.nchains == 1) {
-      ch = job.one;
-    } else {
-      int lo = 0, hi = job.nchains - 1;
-      while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (job.chains[mid].off <= i) lo = mid; else hi = mid - 1;
-      }
-      ch = job.chains[lo];
-      split_set_kappa(s, ch.kappa);
-    }
+    split_set_kappa(s, c.kappa);
     const int64_t li = i - ch.off;
-    auto xat = [&](int64_t q) -> FPair<float> {  // coupling increment of chain site q
-      const int64_t g = (ch.bc == PERIODIC) ? ch.off + wrap(q, ch.n) : ((q < 0 || q >= ch.n) ? -1 : ch.off + q);
-      if (g < 0 || !bounds_ok(job.hdr, in_range(g, 1, job.total))) return {0.f, 0.f};
+    auto xat = [&](int64_t q) -> FPair<float> {
+      const int64_t g = gen_site(job, ch, q);
+      if (g < 0) return {0.f, 0.f};
       const float2 u = U[g * D];
       return {u.x, u.y};
     };
-    FPair<float> d[D], n[D];
+    const StageCoef<float> co = stage_coef<float>(s);
+    FPair<float> e[D], n[D];
 #pragma unroll
-    for (int q = 0; q < D; ++q) {
-      const float2 u = U[i * D + q];
-      d[q] = {u.x, u.y};
+    for (int q = 0; q < D; ++q) n[q] = e[q] = {0.f, 0.f};
+    float nde = 0.f, dfe = 0.f;
+    if (row) {
+#pragma unroll
+      for (int q = 0; q < D; ++q) {
+        const float2 u = U[i * D + q];
+        e[q] = {u.x, u.y};
+      }
+      const FPair<float> none = {0.f, 0.f};
+      split_linear<MODEL, float, RANGE>(e, xat(li - 1), xat(li + 1), co, n, nde, dfe, RANGE == 2 ? xat(li - 2) : none,
+                                        RANGE == 2 ? xat(li + 2) : none);
     }
-    SplitBase<float> base = {};
     if constexpr (MODEL == ROESSLER) {
-      base.z = split1(Y[i * D + 2]);
-      base.t = x_minus_c<float>(split1(Y[i * D]), {s.ch, s.cl});
+      const FPair<float> cj = {st.ch[j], st.cl[j]};
+      const FPair<float> dx = pair_fma(cj, -cj.h, split1(K[i * D]), e[0]), dz = pair_fma(cj, -cj.h, split1(K[i * D + 2]), e[2]);
+      const SplitBase<float> base = {split1(Y[i * D + 2]), x_minus_c<float>(split1(Y[i * D]), {s.ch, s.cl})};
+      n[2] = row ? gen_remainder_z<float, true>(dx, dz, e[2], nde, dfe, base, co.tau)
+                 : gen_remainder_z<float, false>(dx, dz, e[2], nde, dfe, base, co.tau);
     }
-    const FPair<float> none = {0.f, 0.f};
-    split_stage<MODEL, float, RANGE, true>(d, xat(li - 1), xat(li + 1), base, stage_coef<float>(s), n,
-                                     RANGE == 2 ? xat(li - 2) : none, RANGE == 2 ? xat(li + 2) : none);
 #pragma unroll
-    for (int q = 0; q < D; ++q) {
-      n[q] = pair_norm(n[q]);
-      N[i * D + q] = make_float2(n[q].h, n[q].l);
-    }
+    for (int q = 0; q < D; ++q) N[i * D + q] = make_float2(n[q].h, n[q].l);
   }
 }
 
-template <int MODEL>
-__global__ void __launch_bounds__(256) k_gen_split_combine(GenStagedJob job, SplitCoef sc, SplitTableau st,
-                                                           Tableau<double> tb) {
+template <int MODEL, int RANGE>
+__global__ void __launch_bounds__(256) k_gen_split_combine(GenStagedJob job, Coef<double> cf, double kappa2, SplitCoef sc,
+                                                           SplitTableau st, Tableau<double> tb) {
   constexpr int D = Dim<MODEL>::D;
   if (job.hdr->wide[job.parity]) {
     gen_combine_sweep<double, D, false>(job, tb);
@@ -397,19 +521,26 @@ __global__ void __launch_bounds__(256) k_gen_split_combine(GenStagedJob job, Spl
   const size_t plane = (size_t)job.total * D;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   bool wide = false, bad = false;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < (int64_t)plane; i += stride) {
-    FPair<float> N = {0.f, vmul(-st.Bl, split1(K[i]).h)};
-    for (int m = 1; m < st.s; ++m) {
-      if (!((st.bnz >> m) & 1u)) continue;
-      const float2 n = reinterpret_cast<const float2 *>(K + m * plane)[i];
-      N = pair_fma<float>({st.bh[m], st.bl[m]}, -st.bh[m], {n.x, n.y}, N);
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < job.total; i += stride) {
+    Coef<double> c = cf;
+    const ChainDesc ch = gen_site_chain(job, i, c);
+    double M[D];
+    gen_staged_second<MODEL, RANGE>(job, ch, i, c, kappa2, M);
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+      FPair<float> N = {0.f, vmul(-st.Bl, split1(K[i * D + d]).h)};
+      for (int q = 0; q <= st.nb; ++q) {
+        const int m = q < st.nb ? st.mb[q] : st.last;
+        const float2 n = reinterpret_cast<const float2 *>(K + m * plane)[i * D + d];
+        N = pair_fma<float>({st.bh[m], st.bl[m]}, -st.bh[m], {n.x, n.y}, N);
+      }
+      double nd;
+      join(N, &nd, 1);
+      const double r = fma(sc.w, fma(gen_update64(K[i * D + d], M[d], st), c.one, -nd), Y[i * D + d]);
+      Y[i * D + d] = r;
+      wide |= !split_in_range<MODEL>(r, d, sc.c, sc);
+      bad |= nonfinite(r);
     }
-    double nd;
-    join(N, &nd, 1);
-    const double r = fma(sc.w, fma(st.B, K[i], -nd), Y[i]);
-    Y[i] = r;
-    wide |= !split_in_range<MODEL>(r, (int)(i % D), sc.c, sc);
-    bad |= nonfinite(r);
   }
   if (wide) job.hdr->wide[job.parity ^ 1] = 1u;
   if (bad) atomicOr(&job.hdr->status, ST_NONFINITE);
@@ -420,15 +551,15 @@ static cudaError_t gen_split_step(const GenStagedJob &job, const CoefD &cfd, con
                                   cudaStream_t st) {
   if (job.total <= 0) return cudaSuccess;
   const Tableau<double> tb = to_tableau<double>(td, dt);
-  const SplitTableau stb = split_tableau(td);
+  const SplitTableau stb = split_tableau(td, dt);
   const SplitCoef sc = split_coef(MODEL, cfd, true);
   const Coef<double> cf = to_coef<double>(cfd, cfd.kappa);
   const unsigned grid = (unsigned)staged_grid(job.total);
   for (int j = 0; j < td.s; ++j) {
-    if (j > 0) k_gen_split_state<MODEL><<<grid, 256, 0, st>>>(job, stb, tb, j);
-    k_gen_split_slope<MODEL, RANGE><<<grid, 256, 0, st>>>(job, cf, cfd.kappa2, sc, j);
+    if (j > 0) k_gen_split_state<MODEL, RANGE><<<grid, 256, 0, st>>>(job, cf, cfd.kappa2, sc, stb, tb, j);
+    k_gen_split_slope<MODEL, RANGE><<<grid, 256, 0, st>>>(job, cf, cfd.kappa2, sc, stb, j);
   }
-  k_gen_split_combine<MODEL><<<grid, 256, 0, st>>>(job, sc, stb, tb);
+  k_gen_split_combine<MODEL, RANGE><<<grid, 256, 0, st>>>(job, cf, cfd.kappa2, sc, stb, tb);
   return cudaGetLastError();
 }
 

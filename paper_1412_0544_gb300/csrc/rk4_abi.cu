@@ -432,8 +432,8 @@ const TileCost kCostHet64[] = {{64, 2, 3.4f, 1.91f, 0.46f, 0.605f}, {128, 2, 3.5
 const TileCost kCostHet32[] = {{64, 2, 3.8f, 0.30f, 0.23f, 0.036f}, {128, 2, 3.8f, 0.30f, 0.41f, 0.080f},
                                {256, 2, 4.1f, 0.39f, 0.87f, 0.169f}, {128, 4, 3.9f, 0.31f, 0.55f, 0.135f},
                                {256, 4, 5.2f, 0.39f, 1.25f, 0.276f}};
-const TileCost kCostGen64[] = {{64, 2, 2.8f, 4.50f, 0.25f, 1.51f}, {128, 2, 2.9f, 4.57f, 0.42f, 2.12f},
-                               {256, 2, 3.2f, 6.67f, 0.80f, 5.13f}};
+const TileCost kCostGen64[] = {{64, 2, 2.8f, 5.85f, 0.25f, 2.03f}, {128, 2, 2.9f, 5.94f, 0.42f, 2.88f},
+                               {256, 2, 3.2f, 8.67f, 0.80f, 6.98f}};
 const TileCost kCostGen32[] = {{128, 2, 5.3f, 0.80f, 0.55f, 0.27f}, {256, 2, 5.7f, 0.95f, 1.30f, 0.64f}};
 const TileCost kCostGen32Shape[] = {{128, 4, 7.0f, 0.47f, 0.65f, 0.28f}, {256, 4, 7.9f, 0.68f, 1.50f, 0.60f},
                                     {512, 4, 7.5f, 1.32f, 3.80f, 1.20f}};
@@ -1034,6 +1034,8 @@ bool rk4d::split_allowed(int model, const CoefD &c) {
 }
 
 bool rk4d::split_tableau_allowed(const TableauD &t) {
+  const uint32_t need = needed_mask(t);
+  if (!(need & 1u) || !(need >> 1)) return false;  // the form evaluates J K1 whether the scheme does or not
   // entries within the pairs' range, and rows small enough that the differences' pair errors,
   // multiplied by them, stay as far below the state's rounding as split_most assumes
   double b = 0.0;
@@ -1057,33 +1059,41 @@ double host_two_sum(double a, double b, double *err) {
   return s;
 }
 
-SplitTableau rk4d::split_tableau(const TableauD &t) {
+SplitTableau rk4d::split_tableau(const TableauD &t, double dt) {
   SplitTableau r{};
   r.s = t.s;
-  double b_err = 0.0;  // the weights' sum is r.B + b_err: an error of 2^-54 in it would be a drift
+  r.need = needed_mask(t);
+  for (int j = 0; j < t.s; ++j)
+    if ((r.need >> j) & 1u) r.last = j;
+  double c[kMaxStages] = {}, b_err = 0.0;  // the weights' sum is B + Bl: an error of 2^-54 in it would be a drift
   for (int j = 0; j < t.s; ++j) {
-    double row = 0.0, row_err = 0.0;
+    double row = 0.0, row_err = 0.0, g = 0.0;
     for (int m = 0; m < j; ++m) {
       row = host_two_sum(row, t.a[j][m], &row_err);
+      g += t.a[j][m] * c[m];
       const HostPair a = host_split(t.a[j][m]);
       r.ah[j][m] = a.h;
       r.al[j][m] = a.l;
-      if (t.a[j][m] != 0.0) r.anz[j] |= 1u << m;
       if (t.a[j][m] != 0.0 && m > 0) r.ma[j][r.na[j]++] = m;
     }
-    const HostPair c = host_split(row + row_err), b = host_split(t.b[j]);
-    r.ch[j] = c.h;
-    r.cl[j] = c.l;
+    c[j] = row + row_err;
+    const HostPair cj = host_split(c[j]), gj = host_split(g), b = host_split(t.b[j]);
+    r.ch[j] = cj.h;
+    r.cl[j] = cj.l;
+    r.gh[j] = gj.h;
+    r.gl[j] = gj.l;
     r.bh[j] = b.h;
     r.bl[j] = b.l;
     r.B = host_two_sum(r.B, t.b[j], &b_err);
-    if (t.b[j] != 0.0) r.bnz |= 1u << j;
-    if (t.b[j] != 0.0 && j > 0) r.mb[r.nb++] = j;
+    r.E += t.b[j] * c[j];
+    if (t.b[j] != 0.0 && j > 0 && j != r.last) r.mb[r.nb++] = j;
+    if (((r.need >> j) & 1u) && j > 0 && j != r.last) r.slot[j] = r.slots++;
   }
+  r.E *= dt;
   const double B = r.B + b_err;
   r.Bl = (float)((r.B - B) + b_err);
   r.B = B;
-  r.need = needed_mask(t);
+  r.unit = B == 1.0;
   return r;
 }
 

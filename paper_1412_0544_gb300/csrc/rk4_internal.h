@@ -137,7 +137,7 @@ struct GenStagedJob {
   const ChainDesc *chains;
   int64_t total;
   WsHeader *hdr;  // status word
-  int split;      // 1: the split form (k[0]: the first slope; the other k and u: float pairs)
+  int split;      // 1: the split form (k[0]: the first slope; the others: their remainders, and u, as float pairs)
   int parity;     // of the step (which wide flag is read)
 };
 
@@ -178,20 +178,23 @@ cudaError_t launch_split_scan(int model, const double *state, const double *sp, 
 // of its chains) may run in the split form, and the form's coefficients.
 bool split_allowed(int model, const CoefD &c);
 SplitCoef split_coef(int model, const CoefD &c, bool generic = false);
-// The generic scheme in the split form: a tableau's rows and weights for the slope differences,
-// as float pairs; a's nonzero pattern (anz, bnz), and the stages the result needs (need).
+// The generic scheme in the split form (k_gen_split.cu): a tableau's rows and weights, as float pairs
+// where they multiply the slopes' remainders, and the stages the result needs.
 struct SplitTableau {
-  int s;
-  uint32_t need, bnz, anz[kMaxStages];
-  int nb, mb[kMaxStages];                      // the stages m >= 1 of nonzero weight, in order
+  int s, last;                                 // last: the last stage needed
+  uint32_t need;
+  int nb, mb[kMaxStages];                      // the stages m >= 1 of nonzero weight but `last`, in order
   int na[kMaxStages], ma[kMaxStages][kMaxStages];  // and those with a nonzero a_jm
-  double B;                                    // sum of the weights, the first slope's factor,
-  float Bl;                                    // and what its rounding leaves
-  float ch[kMaxStages], cl[kMaxStages];        // row sums, the first slope's factors
+  int slot[kMaxStages], slots;                 // where a stage's remainders lie in a thread's record
+  double B, E;                                 // the weights' sum, and dt sum b_m c_m
+  int unit;                                    // B is 1
+  float Bl;                                    // what B's rounding leaves
+  float ch[kMaxStages], cl[kMaxStages];        // row sums c_j
+  float gh[kMaxStages], gl[kMaxStages];        // sum over m of a_jm c_m
   float ah[kMaxStages][kMaxStages], al[kMaxStages][kMaxStages], bh[kMaxStages], bl[kMaxStages];
 };
 bool split_tableau_allowed(const TableauD &t);  // whether the form takes the tableau
-SplitTableau split_tableau(const TableauD &t);
+SplitTableau split_tableau(const TableauD &t, double dt);
 cudaError_t launch_gen_split(int model, int range, int sites, const BlockedJob &job, const CoefD &cf,
                              const TableauD &tb, double dt, int H, cudaStream_t st);  // tiles of `sites` sites
 cudaError_t launch_gen_split_step(int model, int range, const GenStagedJob &job, const CoefD &cf,

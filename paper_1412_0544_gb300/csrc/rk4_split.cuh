@@ -66,7 +66,7 @@ __device__ __forceinline__ float vadd(float a, float b) { return __fadd_rn(a, b)
 __device__ __forceinline__ float vsub(float a, float b) { return __fsub_rn(a, b); }
 // Products as FMAs with a zero addend (a zero product comes out as +0): ptxas was seen to contract
 // a packed mul.rn and a later add.rn into one FMA (CUDA 13.0; the packed and the scalar forms of
-// a normalisation after a product then differed), which an FMA rules out at the same cost.
+// a sum after a product then differed), which an FMA rules out at the same cost.
 __device__ __forceinline__ float vmul(float a, float b) { return __fmaf_rn(a, b, 0.f); }
 __device__ __forceinline__ float vfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ f32x2 vadd(f32x2 a, f32x2 b) {
@@ -121,11 +121,6 @@ template <typename T> __device__ __forceinline__ void mul_coef(const FPair<T> &c
   e = vfma(c.h, v.h, np);
   e = vfma(c.h, v.l, e);
   e = vfma(c.l, v.h, e);
-}
-// The pair with its tail at most half a unit of its head (|h| >= |l| up to the head's cancellation).
-template <typename T> __device__ __forceinline__ FPair<T> pair_norm(const FPair<T> &v) {
-  const T s = vadd(v.h, v.l);
-  return {s, vsub(v.l, vsub(s, v.h))};
 }
 // a - n as a pair.
 template <typename T> __device__ __forceinline__ FPair<T> pair_sub(const FPair<T> &a, const FPair<T> &n) {
@@ -282,12 +277,12 @@ __device__ __forceinline__ FPair<T> pair_lap(const FPair<T> &x, const FPair<T> &
   return g;
 }
 
-// n = -D for the stage increments d (85 FP32 operations per site; harmonic 40; 28 more with
-// second neighbours).
-template <int MODEL, typename T, int RANGE = 1, bool NORM = false>
-__device__ __forceinline__ void split_stage(const FPair<T> *d, const FPair<T> &xl, const FPair<T> &xr,
-                                            const SplitBase<T> &b, const StageCoef<T> &c, FPair<T> *n,
-                                            const FPair<T> &xl2 = {}, const FPair<T> &xr2 = {}) {
+// The rows of n = -D that are linear in the increments d: all but the Roessler chain's z.  nd, df: tau dx
+// = df - nd (Roessler).
+template <int MODEL, typename T, int RANGE>
+__device__ __forceinline__ void split_linear(const FPair<T> *d, const FPair<T> &xl, const FPair<T> &xr,
+                                             const StageCoef<T> &c, FPair<T> *n, T &nd, T &df,
+                                             const FPair<T> &xl2 = {}, const FPair<T> &xr2 = {}) {
   const T m1 = vset<T>(-1.f);
   const FPair<T> g = pair_lap(d[0], xl, xr);
   T np, e, ne;
@@ -308,25 +303,36 @@ __device__ __forceinline__ void split_stage(const FPair<T> *d, const FPair<T> &x
     mul_coef(c.tau, ntau, w, nw, f);
     two_diff(np, nw, n[0].h, ne);
     n[0].l = vadd(vsub(ne, e), f);
-    T nd, df;  // delta = tau dx = df - nd
     mul_coef(c.tau, ntau, d[0], nd, df);
     mul_coef(c.at, vmul(m1, c.at.h), d[1], np, e);
     two_sum(nd, np, n[1].h, ne);
     n[1].l = vsub(ne, vadd(df, e));
-    T nz, q;  // zeta = tau dz = q - nz
+  } else {
+    T nq, f;  // w2 tau dq = f - nq
+    mul_coef(c.at, vmul(m1, c.at.h), d[0], nq, f);
+    two_diff(np, nq, n[1].h, ne);
+    n[1].l = vadd(vsub(ne, e), f);
+    mul_coef(c.tau, vmul(m1, c.tau.h), d[1], n[0].h, e);  // tau dp = e - n
+    n[0].l = vmul(m1, e);
+  }
+}
+
+// n = -D for the stage increments d (85 FP32 operations per site; harmonic 40).
+template <int MODEL, typename T>
+__device__ __forceinline__ void split_stage(const FPair<T> *d, const FPair<T> &xl, const FPair<T> &xr,
+                                            const SplitBase<T> &b, const StageCoef<T> &c, FPair<T> *n) {
+  T nd, df;  // delta = tau dx = df - nd
+  split_linear<MODEL, T, 1>(d, xl, xr, c, n, nd, df);
+  if constexpr (MODEL == ROESSLER) {
+    const T m1 = vset<T>(-1.f);
+    const T ntau = vmul(m1, c.tau.h);
+    T nz, q, ne;  // zeta = tau dz = q - nz
     mul_coef(c.tau, ntau, d[2], nz, q);
     T pz = vmul(c.tau.h, d[2].h);  // = -nz
-    if constexpr (NORM) {
-      const FPair<T> zn = pair_norm(FPair<T>{pz, q});
-      pz = zn.h;
-      q = zn.l;
-      nz = vmul(m1, pz);
-    }
     FPair<T> t;  // (x - c) + delta
     T te;
     two_diff(b.t.h, nd, t.h, te);
     t.l = vadd(vadd(te, b.t.l), df);
-    if constexpr (NORM) t = pair_norm(t);
     const T nzh = vmul(m1, b.z.h);
     const T p1 = vmul(nzh, nd);  // z delta = p1 - g1
     T g1 = vfma(b.z.h, nd, p1);
@@ -338,13 +344,6 @@ __device__ __forceinline__ void split_stage(const FPair<T> *d, const FPair<T> &x
     e2 = vfma(q, t.h, e2);
     two_diff(p2, p1, n[2].h, ne);
     n[2].l = vsub(vadd(ne, g1), e2);
-  } else {
-    T nq, f;  // w2 tau dq = f - nq
-    mul_coef(c.at, vmul(m1, c.at.h), d[0], nq, f);
-    two_diff(np, nq, n[1].h, ne);
-    n[1].l = vadd(vsub(ne, e), f);
-    mul_coef(c.tau, vmul(m1, c.tau.h), d[1], n[0].h, e);  // tau dp = e - n
-    n[0].l = vmul(m1, e);
   }
 }
 

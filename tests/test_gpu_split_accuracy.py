@@ -86,3 +86,80 @@ def test_on_the_attractor(dt, c):
     y0 = gh.gpu_run(ci.uniform_state(N, 3, seed=1251), nsteps=6000, dt=dt, params=p)
     exact, plain = rk4([y0[:, d].copy() for d in range(3)], p, dt, 1)
     check(gh.gpu_run(y0, nsteps=1, dt=dt, params=p, tiling=(256, 4, 1)), exact, plain, (dt, c))
+
+
+# ---- generic tableaux ---------------------------------------------------------------------------
+
+def generic(y, A, b, p, k2, dt, steps):
+    """As rk4(), any tableau, second neighbours; the FP64 form's operations as in rk4_generic.cuh."""
+    s, h = len(b), L(np.float64(dt))
+    lp = {k: L(v) for k, v in p.items()}
+
+    def f(u, one):
+        l1, l2 = np.roll(u[0], 1) + np.roll(u[0], -1), np.roll(u[0], 2) + np.roll(u[0], -2)
+        if one:
+            return [lp["kappa"] * (l1 - 2 * u[0]) + L(k2) * (l2 - 2 * u[0]) - (u[1] + u[2]), u[0] + lp["a"] * u[1],
+                    lp["b"] + u[2] * (u[0] - lp["c"])]
+        inner = -(u[1] + u[2])
+        if k2:
+            inner = fma(k2, fma(-2.0, u[0], l2), inner)
+        return [fma(p["kappa"], fma(-2.0, u[0], l1), inner), fma(p["a"], u[1], u[0]),
+                fma(u[2], u[0], fma(-p["c"], u[2], p["b"]))]
+
+    exact, plain = [v.astype(L) for v in y], [v.copy() for v in y]
+    for _ in range(steps):
+        for one in (True, False):
+            base, ks = (exact if one else plain), []
+            for j in range(s):
+                u = base
+                for m in range(j):
+                    if A[j, m]:
+                        u = [v + L(A[j, m]) * h * q for v, q in zip(u, ks[m])] if one else \
+                            [fma(A[j, m] * dt, q, v) for v, q in zip(u, ks[m])]
+                ks.append(f(u, one))
+            inc = [np.zeros_like(v) for v in base]
+            for m in range(s):
+                if b[m]:
+                    inc = [v + L(b[m]) * h * q for v, q in zip(inc, ks[m])] if one else \
+                          [fma(b[m] * dt, q, v) for v, q in zip(inc, ks[m])]
+            out = [v + i for v, i in zip(base, inc)]
+            if one:
+                exact = out
+            else:
+                plain = out
+    return exact, plain
+
+
+def generic_gpu(y0, A, b, p, k2, dt, steps, tiling):
+    import torch
+    import paper_1412_0544_gb300 as rk
+    h = rk.rk4_chain_create(rk.RK4_ROESSLER, rk.RK4_FP64, y0.shape[0], dt, rk.RK4_PERIODIC, p)
+    try:
+        rk.rk4_chain_set_tableau(h, A, b)
+        rk.rk4_chain_set_coupling2(h, k2)
+        rk.rk4_chain_set_tiling(h, *tiling)
+        st = torch.from_numpy(np.ascontiguousarray(y0)).cuda()
+        ws = torch.empty(rk.rk4_chain_workspace_bytes(h), dtype=torch.uint8, device="cuda")
+        rk.rk4_chain_integrate(h, st, None, ws, steps)
+        assert rk.rk4_chain_status(h, ws) == rk.RK4_OK
+        return st.cpu().numpy()
+    finally:
+        rk.rk4_chain_destroy(h)
+
+
+@pytest.mark.parametrize("name", ["dopri5", "rk4"])
+@pytest.mark.parametrize("dt,c,kappa,kappa2,amp", [
+    (0.01, 9.0, 1.1, 0.5, 1.0), (0.01, 9.0, 2.0, 0.7, 1.0), (0.01, 9.0, 1.0, 0.0, 1.0), (0.01, 9.0, 2.0, 0.7, 15.0),
+    (0.01, 9.0, 1.1, 0.5, 40.0), (0.0138, 9.0, 2.0, 0.25, 1.0), (0.06, 2.0, 0.5, 0.02, 0.8)])
+@pytest.mark.parametrize("steps", [1, 2])
+def test_generic_tableaux(name, dt, c, kappa, kappa2, amp, steps):
+    """Both forms round the state once a step here; the first order of the later slopes in FP64 and the
+    remainders' pairs leave the split form between 0.9 and 1."""
+    import oracle
+    import oracle_pins as P
+    A, b = (P.TABLEAUX["dopri5"][:2] if name == "dopri5" else (oracle.RK4_A, oracle.RK4_B))
+    A, b = np.asarray(A, dtype=float), np.asarray(b, dtype=float)
+    y0 = ci.uniform_state(N, 3, seed=1252) * amp
+    p = dict(a=0.2, b=1.0, c=c, kappa=kappa)
+    exact, plain = generic([y0[:, d].copy() for d in range(3)], A, b, p, kappa2, dt, steps)
+    check(generic_gpu(y0, A, b, p, kappa2, dt, steps, (128, 2, 2)), exact, plain, (name, dt, kappa, kappa2, amp, steps))
