@@ -13,7 +13,8 @@
 // (z 1.15, 2.2 at |x|, |z| = 20; x 1.04 with kappa = 2, kappa2 = 0.7), because the FP64 form rounds its state
 // only once a step.  The remainders are smaller again by dt |J|: 0.92 ..
 // 1.002 in each component after one and two steps (Dormand-Prince 5 and RK4, dt = 0.01 .. 0.06, kappa up to 2,
-// kappa2 up to 0.7, |x|, |z| up to 15), without normalising any pair.  M's rows in pairs left x at 1.03.
+// kappa2 up to 0.7, |x|, |z| up to 15).  e_z, which x - c multiplies, is normalised (z 1.004 -> 0.981 with Fehlberg's
+// tableau, dt = 0.0138).  M's rows in pairs left x at 1.03.
 // The weights' sum is carried to a float beyond FP64: its own rounding, times dt K1 every step, was a
 // drift of 1.2 after 20 steps.
 //
@@ -218,6 +219,7 @@ __device__ __forceinline__ void gen_split_advance(double (&y)[2][Dim<MODEL>::D],
 #pragma unroll
           for (int i = 0; i < D; ++i) e[i] = pair_fnma<T>(a, na, {q[2 * i], q[2 * i + 1]}, e[i]);
         }
+        if constexpr (MODEL == ROESSLER) e[2] = pair_norm(e[2]);
         FPair<T> X = e[0];
         if constexpr (MASK) {
           const bool g0 = ghost & 1u, g1 = ghost & 2u;
@@ -449,6 +451,7 @@ __global__ void __launch_bounds__(256) k_gen_split_state(GenStagedJob job, Coef<
         const float2 n = reinterpret_cast<const float2 *>(K + m * plane)[i * D + d];
         e = pair_fnma<float>({st.ah[j][m], st.al[j][m]}, -st.ah[j][m], {n.x, n.y}, e);
       }
+      if (MODEL == ROESSLER && d == 2) e = pair_norm(e);
       U[i * D + d] = make_float2(e.h, e.l);
     }
   }

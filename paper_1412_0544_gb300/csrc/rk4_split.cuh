@@ -122,6 +122,11 @@ template <typename T> __device__ __forceinline__ void mul_coef(const FPair<T> &c
   e = vfma(c.h, v.l, e);
   e = vfma(c.l, v.h, e);
 }
+// The pair with its tail at most half a unit of its head (|h| >= |l| up to the head's cancellation).
+template <typename T> __device__ __forceinline__ FPair<T> pair_norm(const FPair<T> &v) {
+  const T s = vadd(v.h, v.l);
+  return {s, vsub(v.l, vsub(s, v.h))};
+}
 // a - n as a pair.
 template <typename T> __device__ __forceinline__ FPair<T> pair_sub(const FPair<T> &a, const FPair<T> &n) {
   FPair<T> r;

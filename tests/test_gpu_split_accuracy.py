@@ -163,3 +163,29 @@ def test_generic_tableaux(name, dt, c, kappa, kappa2, amp, steps):
     p = dict(a=0.2, b=1.0, c=c, kappa=kappa)
     exact, plain = generic([y0[:, d].copy() for d in range(3)], A, b, p, kappa2, dt, steps)
     check(generic_gpu(y0, A, b, p, kappa2, dt, steps, (128, 2, 2)), exact, plain, (name, dt, kappa, kappa2, amp, steps))
+
+
+def stretched(q):
+    """A four-stage tableau whose rows cancel: sums of magnitudes 1 + 2 q and 1 + 4 q."""
+    A = np.zeros((4, 4))
+    A[1, 0], A[2, :2], A[3, :3] = 0.5, (-q, 0.5 + q), (q, -2 * q, 1 + q)
+    return A, np.array([1, 2, 2, 1]) / 6
+
+
+def fehlberg():
+    A = np.zeros((6, 6))
+    A[1, :1], A[2, :2], A[3, :3] = [1 / 4], [3 / 32, 9 / 32], [1932 / 2197, -7200 / 2197, 7296 / 2197]
+    A[4, :4], A[5, :5] = [439 / 216, -8, 3680 / 513, -845 / 4104], [-8 / 27, 2, -3544 / 2565, 1859 / 4104, -11 / 40]
+    return A, np.array([16 / 135, 0, 6656 / 12825, 28561 / 56430, -9 / 50, 2 / 55])
+
+
+@pytest.mark.parametrize("tab", [stretched(0.02), stretched(2), stretched(10), stretched(40), fehlberg()],
+                         ids=["near", "beyond", "far", "farther", "fehlberg"])
+@pytest.mark.parametrize("amp", [1.0, 9.0])
+def test_tableaux_about_the_limit(tab, amp):
+    """Tableaux that the split form takes (the first and the last) and ones whose rows would multiply its
+    pairs' errors (predicted there: 1.08, 3.9 and 8.7 in z at amplitude 9)."""
+    y0 = ci.uniform_state(N, 3, seed=1253) * amp
+    p = dict(a=0.2, b=1.0, c=9.0, kappa=1.5)
+    exact, plain = generic([y0[:, d].copy() for d in range(3)], *tab, p, 0.3, 0.0138, 1)
+    check(generic_gpu(y0, *tab, p, 0.3, 0.0138, 1, (128, 2, 1)), exact, plain, (tab[1].size, amp))
