@@ -386,22 +386,6 @@ cudaError_t launch_gen_split(int model, int range, int sites, const BlockedJob &
 
 // ---- one stage per launch ---------------------------------------------------------------------
 
-// The chain of site i; its coupling strength goes into c.
-__device__ __forceinline__ ChainDesc gen_site_chain(const GenStagedJob &job, int64_t i, Coef<double> &c) {
-  if (job.nchains == 1) return job.one;
-  int lo = 0, hi = job.nchains - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (job.chains[mid].off <= i) lo = mid; else hi = mid - 1;
-  }
-  c.kappa = job.chains[lo].kappa;
-  return job.chains[lo];
-}
-// Index of site q of a chain (boundary-resolved), or -1 beyond a fixed end.
-__device__ __forceinline__ int64_t gen_site(const GenStagedJob &job, const ChainDesc &ch, int64_t q) {
-  const int64_t g = (ch.bc == PERIODIC) ? ch.off + wrap(q, ch.n) : ((q < 0 || q >= ch.n) ? -1 : ch.off + q);
-  return g < 0 || !bounds_ok(job.hdr, in_range(g, 1, job.total)) ? -1 : g;
-}
 // M of site i from the first slopes in job.k.
 template <int MODEL, int RANGE>
 __device__ __forceinline__ void gen_staged_second(const GenStagedJob &job, const ChainDesc &ch, int64_t i,
@@ -428,18 +412,19 @@ template <int MODEL, int RANGE>
 __global__ void __launch_bounds__(256) k_gen_split_state(GenStagedJob job, Coef<double> cf, double kappa2, SplitCoef sc,
                                                          SplitTableau st, Tableau<double> tb, int j) {
   constexpr int D = Dim<MODEL>::D;
-  if (job.hdr->wide[job.parity]) {
-    gen_state_sweep<double, D>(job, tb, j);
-    return;
-  }
-  if (st.na[j] == 0) return;  // e_j = 0
   const double *K = static_cast<const double *>(job.k);
   float2 *U = static_cast<float2 *>(job.u);
   const size_t plane = (size_t)job.total * D;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < job.total; i += stride) {
     Coef<double> c = cf;
-    const ChainDesc ch = gen_site_chain(job, i, c);
+    int ci;
+    const ChainDesc ch = gen_site_chain(job, i, c, ci);
+    if (job.wide[2 * ci + job.parity]) {
+      gen_state_site<double, D>(job, tb, i, j);
+      continue;
+    }
+    if (st.na[j] == 0) continue;  // e_j = 0
     double M[D];
     gen_staged_second<MODEL, RANGE>(job, ch, i, c, kappa2, M);
 #pragma unroll
@@ -462,10 +447,6 @@ template <int MODEL, int RANGE>
 __global__ void __launch_bounds__(256) k_gen_split_slope(GenStagedJob job, Coef<double> cf, double kappa2, SplitCoef sc,
                                                          SplitTableau st, int j) {
   constexpr int D = Dim<MODEL>::D;
-  if (j == 0 || job.hdr->wide[job.parity]) {
-    gen_slope_sweep<double, MODEL, RANGE>(job, cf, kappa2, j);
-    return;
-  }
   const double *Y = static_cast<const double *>(job.y), *K = static_cast<const double *>(job.k);
   const float2 *U = static_cast<const float2 *>(job.u);
   float2 *N = reinterpret_cast<float2 *>(static_cast<double *>(job.k) + (size_t)j * job.total * D);
@@ -473,7 +454,12 @@ __global__ void __launch_bounds__(256) k_gen_split_slope(GenStagedJob job, Coef<
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < job.total; i += stride) {
     Coef<double> c = cf;
-    const ChainDesc ch = gen_site_chain(job, i, c);
+    int ci;
+    const ChainDesc ch = gen_site_chain(job, i, c, ci);
+    if (j == 0 || job.wide[2 * ci + job.parity]) {
+      gen_slope_site<double, MODEL, RANGE>(job, ch, c, kappa2, i, j);
+      continue;
+    }
     SplitCoef s = sc;
     split_set_kappa(s, c.kappa);
     const int64_t li = i - ch.off;
@@ -514,19 +500,21 @@ template <int MODEL, int RANGE>
 __global__ void __launch_bounds__(256) k_gen_split_combine(GenStagedJob job, Coef<double> cf, double kappa2, SplitCoef sc,
                                                            SplitTableau st, Tableau<double> tb) {
   constexpr int D = Dim<MODEL>::D;
-  if (job.hdr->wide[job.parity]) {
-    gen_combine_sweep<double, D, false>(job, tb);
-    if (blockIdx.x == 0 && threadIdx.x == 0) job.hdr->wide[job.parity ^ 1] = 1u;
-    return;
-  }
   double *Y = static_cast<double *>(job.y);
   const double *K = static_cast<const double *>(job.k);
   const size_t plane = (size_t)job.total * D;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  bool wide = false, bad = false;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < job.total; i += stride) {
     Coef<double> c = cf;
-    const ChainDesc ch = gen_site_chain(job, i, c);
+    int ci;
+    const ChainDesc ch = gen_site_chain(job, i, c, ci);
+    unsigned *next = job.wide + 2 * ci + (job.parity ^ 1);
+    if (job.wide[2 * ci + job.parity]) {
+      gen_combine_site<double, D, false>(job, tb, i);
+      *next = 1u;
+      continue;
+    }
+    bool wide = false, bad = false;
     double M[D];
     gen_staged_second<MODEL, RANGE>(job, ch, i, c, kappa2, M);
 #pragma unroll
@@ -544,9 +532,9 @@ __global__ void __launch_bounds__(256) k_gen_split_combine(GenStagedJob job, Coe
       wide |= !split_in_range<MODEL>(r, d, sc.c, sc);
       bad |= nonfinite(r);
     }
+    if (wide) *next = 1u;
+    if (bad) atomicOr(&job.hdr->status, ST_NONFINITE);
   }
-  if (wide) job.hdr->wide[job.parity ^ 1] = 1u;
-  if (bad) atomicOr(&job.hdr->status, ST_NONFINITE);
 }
 
 template <int MODEL, int RANGE>

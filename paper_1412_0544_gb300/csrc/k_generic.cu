@@ -26,15 +26,23 @@ namespace rk4d {
 
 template <typename R, int D>
 __global__ void __launch_bounds__(256) k_gen_state(GenStagedJob job, Tableau<R> tb, int j) {
-  gen_state_sweep<R, D>(job, tb, j);
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < job.total; i += stride) gen_state_site<R, D>(job, tb, i, j);
 }
 template <typename R, int MODEL, int RANGE>
 __global__ void __launch_bounds__(256) k_gen_slope(GenStagedJob job, Coef<R> cf, R kappa2, int j) {
-  gen_slope_sweep<R, MODEL, RANGE>(job, cf, kappa2, j);
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < job.total; i += stride) {
+    Coef<R> c = cf;
+    int ci;
+    const ChainDesc ch = gen_site_chain(job, i, c, ci);
+    gen_slope_site<R, MODEL, RANGE>(job, ch, c, kappa2, i, j);
+  }
 }
 template <typename R, int D, bool KAHAN>
 __global__ void __launch_bounds__(256) k_gen_combine(GenStagedJob job, Tableau<R> tb) {
-  gen_combine_sweep<R, D, KAHAN>(job, tb);
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < job.total; i += stride) gen_combine_site<R, D, KAHAN>(job, tb, i);
 }
 
 // ---- temporally blocked generic kernel ----------------------------------------------------

@@ -61,7 +61,7 @@ template <int MODEL, bool HET, typename R, typename F> static R split_dispatch(i
   return none;
 }
 
-// An item outside the split's range, in the FP64 form.  Not inlined: it is rare, and its
+// An item (of a packed tile, the marked segments) outside the split's range, in the FP64 form.  Not inlined: it is rare, and its
 // registers then do not add to the split's.
 template <int MODEL, int V, bool COH, bool HET, bool ALN>
 __device__ __noinline__ void wide_tile_call(const double *in, double *out, ChainDesc ch, int64_t tile, int K, int G,
@@ -74,8 +74,8 @@ template <int MODEL, int V, bool COH>
 __device__ __noinline__ void wide_packed_call(const double *in, double *out, const ChainDesc *chains,
                                               const SegDesc *segs, int s0, int s1, int K, Coef<double> cf,
                                               unsigned char *smem, int64_t sites, WsHeader *hdr) {
-  packed_tile_item<double, MODEL, V, false, COH, false>(in, out, nullptr, nullptr, chains, segs, s0, s1, K, cf, smem,
-                                                        sites, hdr);
+  packed_tile_item<double, MODEL, V, false, COH, false, false, true>(in, out, nullptr, nullptr, chains, segs, s0, s1, K,
+                                                                     cf, smem, sites, hdr);
 }
 // A packed tile of a batch; not inlined for the reason given in k_blocked.cu.
 template <int MODEL, int V, bool COH, bool PARK>

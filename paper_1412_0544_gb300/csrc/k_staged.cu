@@ -7,99 +7,100 @@
 
 namespace rk4d {
 
-// The chain of site i (its coupling strength goes into c).
-template <typename R> __device__ __forceinline__ ChainDesc staged_chain(const StagedJob &job, int64_t i, Coef<R> &c) {
+// The chain of site i, number ci (its coupling strength goes into c).
+template <typename R>
+__device__ __forceinline__ ChainDesc staged_chain(const StagedJob &job, int64_t i, Coef<R> &c, int &ci) {
+  ci = 0;
   if (job.nchains == 1) return job.one;
-  int lo = 0, hi = job.nchains - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (job.chains[mid].off <= i) lo = mid; else hi = mid - 1;
-  }
-  const ChainDesc ch = job.chains[lo];
+  ci = site_chain(job.chains, job.nchains, i);
+  const ChainDesc ch = job.chains[ci];
   c.kappa = (R)ch.kappa;
   return ch;
 }
 
+// Stage j of site i, of chain ch with coefficients c.
 template <typename R, int MODEL, bool KAHAN>
-__device__ __forceinline__ void staged_sweep(const StagedJob &job, const Coef<R> &cf, int j) {
+__device__ __forceinline__ void staged_site(const StagedJob &job, const ChainDesc &ch, Coef<R> c, int64_t i, int j) {
   constexpr int D = Dim<MODEL>::D;
   R *Y = static_cast<R *>(job.y);
   R *CMP = static_cast<R *>(job.cmp);
   const R *src = (j == 0) ? Y : static_cast<const R *>(job.uin);
   R *UOUT = static_cast<R *>(job.uout);
   R *ACC = static_cast<R *>(job.acc);
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < job.total; i += stride) {
-    Coef<R> c = cf;
-    const ChainDesc ch = staged_chain(job, i, c);
-    if (job.sp) c = site_coef<R, MODEL>(c, static_cast<const R *>(job.sp) + i * Dim<MODEL>::P);  // Eq. (1)
-    const int64_t li = i - ch.off;  // index within the chain
-    R u[D], y[D], acc[D], cmp[D], k[D];
+  if (job.sp) c = site_coef<R, MODEL>(c, static_cast<const R *>(job.sp) + i * Dim<MODEL>::P);  // Eq. (1)
+  const int64_t li = i - ch.off;  // index within the chain
+  R u[D], y[D], acc[D], cmp[D], k[D];
+#pragma unroll
+  for (int d = 0; d < D; ++d) {
+    u[d] = src[i * D + d];
+    y[d] = Y[i * D + d];
+    acc[d] = (j > 0) ? ACC[i * D + d] : R(0);
+    cmp[d] = (KAHAN && j == 3) ? CMP[i * D + d] : R(0);
+  }
+  R xl, xr;
+  if (ch.bc == PERIODIC) {
+    const int64_t il = (li == 0) ? ch.n - 1 : li - 1;
+    const int64_t ir = (li == ch.n - 1) ? 0 : li + 1;
+    if (!bounds_ok(job.hdr, in_range(ch.off + il, 1, job.total) && in_range(ch.off + ir, 1, job.total))) return;
+    xl = src[(ch.off + il) * D];
+    xr = src[(ch.off + ir) * D];
+  } else {
+    if (!bounds_ok(job.hdr, in_range(li, 1, ch.n))) return;
+    xl = (li == 0) ? R(0) : src[(i - 1) * D];
+    xr = (li == ch.n - 1) ? R(0) : src[(i + 1) * D];
+  }
+  slope<R, MODEL>(u, xl, xr, c, k);
+  stage_update<R, D, KAHAN>(j, k, y, u, acc, cmp, c);
+  if (j < 3) {
 #pragma unroll
     for (int d = 0; d < D; ++d) {
-      u[d] = src[i * D + d];
-      y[d] = Y[i * D + d];
-      acc[d] = (j > 0) ? ACC[i * D + d] : R(0);
-      cmp[d] = (KAHAN && j == 3) ? CMP[i * D + d] : R(0);
+      UOUT[i * D + d] = u[d];
+      ACC[i * D + d] = acc[d];
     }
-    R xl, xr;
-    if (ch.bc == PERIODIC) {
-      const int64_t il = (li == 0) ? ch.n - 1 : li - 1;
-      const int64_t ir = (li == ch.n - 1) ? 0 : li + 1;
-      if (!bounds_ok(job.hdr, in_range(ch.off + il, 1, job.total) && in_range(ch.off + ir, 1, job.total))) continue;
-      xl = src[(ch.off + il) * D];
-      xr = src[(ch.off + ir) * D];
-    } else {
-      if (!bounds_ok(job.hdr, in_range(li, 1, ch.n))) continue;
-      xl = (li == 0) ? R(0) : src[(i - 1) * D];
-      xr = (li == ch.n - 1) ? R(0) : src[(i + 1) * D];
-    }
-    slope<R, MODEL>(u, xl, xr, c, k);
-    stage_update<R, D, KAHAN>(j, k, y, u, acc, cmp, c);
-    if (j < 3) {
+  } else {
+    bool bad = false;
 #pragma unroll
-      for (int d = 0; d < D; ++d) {
-        UOUT[i * D + d] = u[d];
-        ACC[i * D + d] = acc[d];
-      }
-    } else {
-      bool bad = false;
-#pragma unroll
-      for (int d = 0; d < D; ++d) {
-        Y[i * D + d] = y[d];
-        if constexpr (KAHAN) CMP[i * D + d] = cmp[d];
-        bad |= nonfinite(y[d]);
-      }
-      if (bad && job.hdr) atomicOr(&job.hdr->status, ST_NONFINITE);
+    for (int d = 0; d < D; ++d) {
+      Y[i * D + d] = y[d];
+      if constexpr (KAHAN) CMP[i * D + d] = cmp[d];
+      bad |= nonfinite(y[d]);
     }
+    if (bad && job.hdr) atomicOr(&job.hdr->status, ST_NONFINITE);
   }
 }
 
 template <typename R, int MODEL, bool KAHAN>
 __global__ void __launch_bounds__(256) k_staged(StagedJob job, Coef<R> cf, int j) {
-  staged_sweep<R, MODEL, KAHAN>(job, cf, j);
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < job.total; i += stride) {
+    Coef<R> c = cf;
+    int ci;
+    const ChainDesc ch = staged_chain(job, i, c, ci);
+    staged_site<R, MODEL, KAHAN>(job, ch, c, i, j);
+  }
 }
 
 // The same in the split form (rk4_split.cuh), bit for bit what the tile kernels compute: stage 0
 // stores the first slope K1, stages 1 and 2 their negated differences, and a stage's increments
-// (the site's and its neighbours') are formed again from these.  Once a value has left the
-// split's range (the scan before the first step, or a step's result) the steps that follow run
+// (the site's and its neighbours') are formed again from these.  Once a value of a chain has left the
+// split's range (the scan before the first step, or a step's result) the chain's further steps run
 // in the FP64 form.
 template <int MODEL>
 __global__ void __launch_bounds__(256) k_staged_split(StagedJob job, Coef<double> cf, SplitCoef sc, int j) {
   constexpr int D = Dim<MODEL>::D;
-  if (job.hdr->wide[job.parity]) {
-    staged_sweep<double, MODEL, false>(job, cf, j);
-    if (j == 3 && blockIdx.x == 0 && threadIdx.x == 0) job.hdr->wide[job.parity ^ 1] = 1u;
-    return;
-  }
   double *Y = static_cast<double *>(job.y);
   double *K1 = static_cast<double *>(job.acc);
   float2 *N2 = static_cast<float2 *>(job.n2), *N3 = static_cast<float2 *>(job.n3);
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < job.total; i += stride) {
     Coef<double> c = cf;
-    const ChainDesc ch = staged_chain(job, i, c);
+    int ci;
+    const ChainDesc ch = staged_chain(job, i, c, ci);
+    if (job.wide[2 * ci + job.parity]) {
+      staged_site<double, MODEL, false>(job, ch, c, i, j);
+      if (j == 3) job.wide[2 * ci + (job.parity ^ 1)] = 1u;
+      continue;
+    }
     const int64_t li = i - ch.off;
     // the neighbours' sites, or -1 beyond a fixed end
     int64_t il = li > 0 ? i - 1 : (ch.bc == PERIODIC ? ch.off + ch.n - 1 : -1);
@@ -167,18 +168,18 @@ __global__ void __launch_bounds__(256) k_staged_split(StagedJob job, Coef<double
       wide |= !split_in_range<MODEL>(r, q, c.c, s);
       bad |= nonfinite(r);
     }
-    if (wide) job.hdr->wide[job.parity ^ 1] = 1u;
+    if (wide) job.wide[2 * ci + (job.parity ^ 1)] = 1u;
     if (bad) atomicOr(&job.hdr->status, ST_NONFINITE);
   }
 }
 
 template <int MODEL>
-__global__ void __launch_bounds__(256) k_split_scan(const double *y, const double *sp, int64_t total, SplitCoef sc,
-                                                    WsHeader *hdr) {
+__global__ void __launch_bounds__(256) k_split_scan(const double *y, const double *sp, int64_t total, int nchains,
+                                                    const ChainDesc *chains, SplitCoef sc, unsigned *flags) {
   constexpr int D = Dim<MODEL>::D, P = Dim<MODEL>::P;
-  bool wide = false;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += stride) {
+    bool wide = false;
 #pragma unroll
     for (int d = 0; d < D; ++d)
       wide |= !split_in_range<MODEL>(y[i * D + d], d, MODEL == ROESSLER && sp ? sp[i * P + 2] : sc.c, sc);
@@ -186,8 +187,8 @@ __global__ void __launch_bounds__(256) k_split_scan(const double *y, const doubl
 #pragma unroll
       for (int q = 0; q < P; ++q) wide |= !split_param_in_range(sp[i * P + q], sc.most[q]);
     }
+    if (wide) flags[2 * (nchains > 1 ? site_chain(chains, nchains, i) : 0)] = 1u;
   }
-  if (wide) hdr->wide[0] = 1u;
 }
 
 static unsigned sweep_grid(int64_t total) {
@@ -195,11 +196,14 @@ static unsigned sweep_grid(int64_t total) {
   return (unsigned)std::min<int64_t>((total + 255) / 256, cap);
 }
 
-cudaError_t launch_split_scan(int model, const double *state, const double *sp, int64_t total, const SplitCoef &sc,
-                              WsHeader *hdr, cudaStream_t st) {
-  if (total <= 0) return cudaSuccess;
-  if (model == ROESSLER) k_split_scan<ROESSLER><<<sweep_grid(total), 256, 0, st>>>(state, sp, total, sc, hdr);
-  else k_split_scan<HARMONIC><<<sweep_grid(total), 256, 0, st>>>(state, sp, total, sc, hdr);
+cudaError_t launch_split_scan(int model, const double *state, const double *sp, int64_t total, int nchains,
+                              const ChainDesc *chains, const SplitCoef &sc, unsigned *wide, cudaStream_t st) {
+  const cudaError_t e = cudaMemsetAsync(wide, 0, 2 * sizeof(unsigned) * (size_t)nchains, st);
+  if (e != cudaSuccess || total <= 0) return e;
+  if (model == ROESSLER)
+    k_split_scan<ROESSLER><<<sweep_grid(total), 256, 0, st>>>(state, sp, total, nchains, chains, sc, wide);
+  else
+    k_split_scan<HARMONIC><<<sweep_grid(total), 256, 0, st>>>(state, sp, total, nchains, chains, sc, wide);
   return cudaGetLastError();
 }
 

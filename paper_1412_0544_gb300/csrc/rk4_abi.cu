@@ -707,9 +707,10 @@ cudaError_t enqueue_integrate(rk4_chain *h, int kernel, void *state, void *comp,
     j.total = h->total;
     j.hdr = reinterpret_cast<WsHeader *>(ws + L.hdr);
     j.split = use_split(h) ? 1 : 0;
+    j.wide = reinterpret_cast<unsigned *>(ws + L.result);  // 8 bytes a chain, free while integrating
     if (j.split) {
-      e = launch_split_scan(h->model, static_cast<const double *>(state), nullptr, h->total,
-                            split_coef(h->model, cf, true), j.hdr, st);
+      e = launch_split_scan(h->model, static_cast<const double *>(state), nullptr, h->total, h->nchains, j.chains,
+                            split_coef(h->model, cf, true), j.wide, st);
       if (e != cudaSuccess) return e;
     }
     for (int64_t s = 0; s < nsteps; ++s) {
@@ -732,11 +733,12 @@ cudaError_t enqueue_integrate(rk4_chain *h, int kernel, void *state, void *comp,
     j.acc = ws + L.acc;
     void *u0 = ws + L.u0, *u1 = ws + L.u1;
     j.split = use_split(h) ? 1 : 0;
+    j.wide = reinterpret_cast<unsigned *>(ws + L.result);  // 8 bytes a chain, free while integrating
     j.n2 = u0;
     j.n3 = u1;
     if (j.split) {
       e = launch_split_scan(h->model, static_cast<const double *>(state), static_cast<const double *>(h->site_params),
-                            h->total, split_coef(h->model, cf), j.hdr, st);
+                            h->total, h->nchains, j.chains, split_coef(h->model, cf), j.wide, st);
       if (e != cudaSuccess) return e;
     }
     for (int64_t s = 0; s < nsteps; ++s) {

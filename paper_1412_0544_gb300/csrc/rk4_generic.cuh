@@ -118,93 +118,87 @@ __device__ __forceinline__ void gen_combine(const Tableau<R> &tb, const R (*k)[D
   }
 }
 
-// ---- one-stage-per-launch sweeps ----------------------------------------------------------
+// ---- one-stage-per-launch sweeps: one site i -------------------------------------------------
 
 template <typename R, int D>
-__device__ __forceinline__ void gen_state_sweep(const GenStagedJob &job, const Tableau<R> &tb, int j) {
+__device__ __forceinline__ void gen_state_site(const GenStagedJob &job, const Tableau<R> &tb, int64_t i, int j) {
   const R *Y = static_cast<const R *>(job.y);
   const R *K = static_cast<const R *>(job.k);
   R *U = static_cast<R *>(job.u);
   const size_t plane = (size_t)job.total * D;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < job.total; i += stride) {
-    R y[D], k[kMaxStages][D], u[D];
+  R y[D], k[kMaxStages][D], u[D];
 #pragma unroll
-    for (int d = 0; d < D; ++d) y[d] = Y[i * D + d];
+  for (int d = 0; d < D; ++d) y[d] = Y[i * D + d];
 #pragma unroll
-    for (int m = 0; m < kMaxStages; ++m)
+  for (int m = 0; m < kMaxStages; ++m)
 #pragma unroll
-      for (int d = 0; d < D; ++d) k[m][d] = (m < j) ? K[m * plane + i * D + d] : R(0);
-    gen_stage_state<R, D>(j, tb, y, k, u);
+    for (int d = 0; d < D; ++d) k[m][d] = (m < j) ? K[m * plane + i * D + d] : R(0);
+  gen_stage_state<R, D>(j, tb, y, k, u);
 #pragma unroll
-    for (int d = 0; d < D; ++d) U[i * D + d] = u[d];
-  }
+  for (int d = 0; d < D; ++d) U[i * D + d] = u[d];
+}
+
+// The chain of site i, number ci; its coupling strength goes into c.
+template <typename R>
+__device__ __forceinline__ ChainDesc gen_site_chain(const GenStagedJob &job, int64_t i, Coef<R> &c, int &ci) {
+  ci = 0;
+  if (job.nchains == 1) return job.one;
+  ci = site_chain(job.chains, job.nchains, i);
+  const ChainDesc ch = job.chains[ci];
+  c.kappa = (R)ch.kappa;
+  return ch;
+}
+// Index in the state of site q of a chain (boundary-resolved), or -1 beyond a fixed end.
+__device__ __forceinline__ int64_t gen_site(const GenStagedJob &job, const ChainDesc &ch, int64_t q) {
+  const int64_t g = (ch.bc == PERIODIC) ? ch.off + wrap(q, ch.n) : ((q < 0 || q >= ch.n) ? -1 : ch.off + q);
+  return g < 0 || !bounds_ok(job.hdr, in_range(g, 1, job.total)) ? -1 : g;
 }
 
 template <typename R, int MODEL, int RANGE>
-__device__ __forceinline__ void gen_slope_sweep(const GenStagedJob &job, const Coef<R> &cf, R kappa2, int j) {
+__device__ __forceinline__ void gen_slope_site(const GenStagedJob &job, const ChainDesc &ch, const Coef<R> &c, R kappa2,
+                                               int64_t i, int j) {
   constexpr int D = Dim<MODEL>::D;
   const R *src = static_cast<const R *>(j == 0 ? job.y : job.u);
   R *K = static_cast<R *>(job.k) + (size_t)j * job.total * D;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < job.total; i += stride) {
-    ChainDesc ch;
-    Coef<R> c = cf;
-    if (job.nchains == 1) {
-      ch = job.one;
-    } else {
-      int lo = 0, hi = job.nchains - 1;
-      while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (job.chains[mid].off <= i) lo = mid; else hi = mid - 1;
-      }
-      ch = job.chains[lo];
-      c.kappa = (R)ch.kappa;
-    }
-    const int64_t li = i - ch.off;
-    auto xat = [&](int64_t q) -> R {  // coupling coordinate of chain site q (boundary-resolved)
-      const int64_t g = (ch.bc == PERIODIC) ? ch.off + wrap(q, ch.n) : ((q < 0 || q >= ch.n) ? -1 : ch.off + q);
-      if (g < 0 || !bounds_ok(job.hdr, in_range(g, 1, job.total))) return R(0);
-      return src[g * D];
-    };
-    R u[D], k[D];
+  const int64_t li = i - ch.off;
+  auto xat = [&](int64_t q) -> R {  // coupling coordinate of chain site q
+    const int64_t g = gen_site(job, ch, q);
+    return g < 0 ? R(0) : src[g * D];
+  };
+  R u[D], k[D];
 #pragma unroll
-    for (int d = 0; d < D; ++d) u[d] = src[i * D + d];
-    slope_gen<R, MODEL, RANGE>(u, xat(li - 1), xat(li + 1), RANGE == 2 ? xat(li - 2) : R(0),
-                               RANGE == 2 ? xat(li + 2) : R(0), c, kappa2, k);
+  for (int d = 0; d < D; ++d) u[d] = src[i * D + d];
+  slope_gen<R, MODEL, RANGE>(u, xat(li - 1), xat(li + 1), RANGE == 2 ? xat(li - 2) : R(0),
+                             RANGE == 2 ? xat(li + 2) : R(0), c, kappa2, k);
 #pragma unroll
-    for (int d = 0; d < D; ++d) K[i * D + d] = k[d];
-  }
+  for (int d = 0; d < D; ++d) K[i * D + d] = k[d];
 }
 
 template <typename R, int D, bool KAHAN>
-__device__ __forceinline__ void gen_combine_sweep(const GenStagedJob &job, const Tableau<R> &tb) {
+__device__ __forceinline__ void gen_combine_site(const GenStagedJob &job, const Tableau<R> &tb, int64_t i) {
   R *Y = static_cast<R *>(job.y);
   R *CMP = static_cast<R *>(job.cmp);
   const R *K = static_cast<const R *>(job.k);
   const size_t plane = (size_t)job.total * D;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < job.total; i += stride) {
-    R y[D], k[kMaxStages][D], cmp[D];
+  R y[D], k[kMaxStages][D], cmp[D];
 #pragma unroll
-    for (int d = 0; d < D; ++d) {
-      y[d] = Y[i * D + d];
-      cmp[d] = KAHAN ? CMP[i * D + d] : R(0);
-    }
-#pragma unroll
-    for (int m = 0; m < kMaxStages; ++m)
-#pragma unroll
-      for (int d = 0; d < D; ++d) k[m][d] = (m < tb.s) ? K[m * plane + i * D + d] : R(0);
-    gen_combine<R, D, KAHAN>(tb, k, y, cmp);
-    bool bad = false;
-#pragma unroll
-    for (int d = 0; d < D; ++d) {
-      Y[i * D + d] = y[d];
-      if constexpr (KAHAN) CMP[i * D + d] = cmp[d];
-      bad |= nonfinite(y[d]);
-    }
-    if (bad && job.hdr) atomicOr(&job.hdr->status, ST_NONFINITE);
+  for (int d = 0; d < D; ++d) {
+    y[d] = Y[i * D + d];
+    cmp[d] = KAHAN ? CMP[i * D + d] : R(0);
   }
+#pragma unroll
+  for (int m = 0; m < kMaxStages; ++m)
+#pragma unroll
+    for (int d = 0; d < D; ++d) k[m][d] = (m < tb.s) ? K[m * plane + i * D + d] : R(0);
+  gen_combine<R, D, KAHAN>(tb, k, y, cmp);
+  bool bad = false;
+#pragma unroll
+  for (int d = 0; d < D; ++d) {
+    Y[i * D + d] = y[d];
+    if constexpr (KAHAN) CMP[i * D + d] = cmp[d];
+    bad |= nonfinite(y[d]);
+  }
+  if (bad && job.hdr) atomicOr(&job.hdr->status, ST_NONFINITE);
 }
 
 inline int64_t staged_grid(int64_t total) {

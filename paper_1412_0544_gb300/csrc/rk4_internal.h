@@ -54,8 +54,7 @@ struct WsHeader {
   unsigned bar_gen;
   int timeout_where;
   unsigned long long work[2];  // persistent kernel: next item of the current time block, by parity
-  unsigned wide[2];            // split staged scheme: the state has left the split's range, by step parity
-  unsigned char pad[216];
+  unsigned char pad[224];
 };
 
 // A piece of one batch chain placed in a shared ("packed") tile: the chain's last partial piece
@@ -123,6 +122,7 @@ struct StagedJob {
   int split;                 // 1: FP64 in the split form: acc holds K1, n2 and n3 the negated
   void *n2, *n3;             // differences of stages 2 and 3 as float pairs
   int parity;                // of the step (which wide flag is read)
+  unsigned *wide;            // per chain and step parity: its state has left the split's range
 };
 
 // One step of the generic standard scheme: stage states, slopes and the combination, each a
@@ -139,6 +139,7 @@ struct GenStagedJob {
   WsHeader *hdr;  // status word
   int split;      // 1: the split form (k[0]: the first slope; the others: their remainders, and u, as float pairs)
   int parity;     // of the step (which wide flag is read)
+  unsigned *wide;  // per chain and step parity: its state has left the split's range
 };
 
 struct PersistentJob {
@@ -171,9 +172,10 @@ template <int MODEL>
 cudaError_t launch_split_persistent(int v, int block, int grid, const PersistentJob &job, const CoefD &cf,
                                     cudaStream_t st);
 template <int MODEL> int persistent_split_max_grid(int v, int block);
-// Set hdr->wide[0] when a state value or a site's own parameter is outside the split's range.
-cudaError_t launch_split_scan(int model, const double *state, const double *sp, int64_t total, const SplitCoef &sc,
-                              WsHeader *hdr, cudaStream_t st);
+// Clear the chains' flags `wide` (two words each) and set the first of a chain's when a value of its state
+// or a site's own parameter is outside the split's range.
+cudaError_t launch_split_scan(int model, const double *state, const double *sp, int64_t total, int nchains,
+                              const ChainDesc *chains, const SplitCoef &sc, unsigned *wide, cudaStream_t st);
 // Whether every step of a handle with these coefficients (c.kappa: the largest coupling strength
 // of its chains) may run in the split form, and the form's coefficients.
 bool split_allowed(int model, const CoefD &c);

@@ -937,8 +937,12 @@ __device__ __forceinline__ bool tile_item(const R *__restrict__ in, R *__restric
 // sites are exact.  Every thread's sites lie in one segment (o and L are multiples of V), so a
 // thread takes its chain's coupling strength and, for fixed ends, its ghost mask; threads past
 // the last segment advance zeros that are never stored.
-// SPLIT, PARK and the result: as tile_item.
-template <typename R, int MODEL, int V, bool KAHAN, bool COH, bool SPLIT = false, bool PARK = false>
+// SPLIT, PARK: as tile_item, but each segment leaves the split form by itself, so that a chain's result does
+// not depend on the chains it shares a tile with: the segments that do are not stored but marked in the
+// exchange's memory (a word each: a tile has at most 2048 / 10 segments with two sites per thread, 1024 / 9
+// with one, and the exchange 256 words or more), and the result is false when there are any.  FLAGGED (the
+// FP64 form after that): only the marked segments are stored.
+template <typename R, int MODEL, int V, bool KAHAN, bool COH, bool SPLIT = false, bool PARK = false, bool FLAGGED = false>
 __device__ __forceinline__ bool packed_tile_item(const R *__restrict__ in, R *__restrict__ out,
                                                  const R *__restrict__ cin, R *__restrict__ cout,
                                                  const ChainDesc *chains, const SegDesc *segs, int s0, int s1,
@@ -950,6 +954,7 @@ __device__ __forceinline__ bool packed_tile_item(const R *__restrict__ in, R *__
   const int W = blockDim.x * V;
   R *ctl = tl + W * D;
   const int H = 4 * K;
+  int *flag = reinterpret_cast<int *>(smem);
 
   int used = 0;  // slots covered by the segments (they are in slot order)
   for (int s = s0; s < s1; ++s) {
@@ -1004,21 +1009,34 @@ __device__ __forceinline__ bool packed_tile_item(const R *__restrict__ in, R *__
       y[v][d] = tl[(base + v) * D + d];
       if constexpr (KAHAN) cmp[v][d] = ctl[(base + v) * D + d]; else cmp[v][d] = R(0);
     }
-  bool nan_tile = false;  // as in tile_item
+  bool wide = false, all_nan = false;  // SPLIT: of this thread's segment: out of range; NaN and nothing else
+  bool mine = true;                    // FLAGGED: the segment is stored
+  if constexpr (FLAGGED) {
+    mine = my >= 0 && flag[my - s0] != 0;
+    __syncthreads();  // before the exchange writes there
+  }
   if constexpr (SPLIT) {
-    bool wide = false;
-#pragma unroll
-    for (int v = 0; v < V; ++v)
-#pragma unroll
-      for (int d = 0; d < D; ++d) wide |= !split_in_range<MODEL>(y[v][d], d, c.c, *scp);
-    nan_tile = __syncthreads_or(wide);
-    if (nan_tile) {
-      bool live = false;
+    bool leaves = false, live = false;
+    if (my >= 0) {
 #pragma unroll
       for (int v = 0; v < V; ++v)
 #pragma unroll
-        for (int d = 0; d < D; ++d) live |= my >= 0 && !is_nan(y[v][d]) && !((ghost >> v) & 1u);
-      if (__syncthreads_or(live)) return false;
+        for (int d = 0; d < D; ++d) {
+          leaves |= !split_in_range<MODEL>(y[v][d], d, c.c, *scp);
+          live |= !is_nan(y[v][d]) && !((ghost >> v) & 1u);
+        }
+    }
+    if (__syncthreads_or(leaves)) {
+      for (int s = threadIdx.x; s < s1 - s0; s += blockDim.x) flag[s] = 0;
+      __syncthreads();
+      if (leaves || live) atomicOr(&flag[my - s0], (leaves ? 1 : 0) | (live ? 2 : 0));
+      __syncthreads();
+      if (my >= 0) {
+        const int f = flag[my - s0];
+        wide = f == 3;
+        all_nan = f == 1;
+      }
+      if (!__syncthreads_or(my >= 0 && !wide)) return false;  // every segment is marked (3)
     }
     SplitCoef sc = *scp;
     split_set_kappa(sc, c.kappa);
@@ -1039,25 +1057,51 @@ __device__ __forceinline__ bool packed_tile_item(const R *__restrict__ in, R *__
       tl[(base + v) * D + d] = y[v][d];
       if constexpr (KAHAN) ctl[(base + v) * D + d] = cmp[v][d];
       if constexpr (SPLIT) bad |= stored && !split_in_range<MODEL>(y[v][d], d, c.c, *scp);
-      else bad |= stored && nonfinite(y[v][d]);
+      else bad |= stored && mine && nonfinite(y[v][d]);
     }
   }
-  const int any_bad = __syncthreads_or(bad);
+  int any = __syncthreads_or(bad | wide);
+  bool marked = FLAGGED;  // the words say which segments to leave out (SPLIT) or to store (FLAGGED)
   if constexpr (SPLIT) {
-    if (any_bad && !nan_tile) return false;
-    report_nonfinite(hdr, nan_tile);
+    wide |= bad && !all_nan;
+    if (any) {
+      report_nonfinite(hdr, __syncthreads_or(all_nan));
+      any = __syncthreads_or(wide);
+    }
+    if (any) {
+      marked = true;
+      for (int s = threadIdx.x; s < s1 - s0; s += blockDim.x) flag[s] = 0;
+      __syncthreads();
+      if (wide) flag[my - s0] = 1;
+      __syncthreads();
+    }
   } else {
-    report_nonfinite(hdr, any_bad);
+    report_nonfinite(hdr, any);
+    if constexpr (FLAGGED) {
+      if (my >= 0 && base == segs[my].o) flag[my - s0] = mine;
+      __syncthreads();
+    }
   }
   for (int s = s0; s < s1; ++s) {
     const SegDesc sd = segs[s];
     if (sd.cnt <= 0 || !bounds_ok(hdr, sd.o >= 0 && sd.o + sd.L <= W && sd.cnt + 2 * H <= sd.L)) continue;
+    if (marked && (flag[s - s0] != 0) != FLAGGED) continue;
     const ChainDesc ch = chains[sd.chain];
     tile_store<R, D, COH>(out, tl, ch.off, sd.o + H, sd.g0, sd.cnt, sites, W, hdr);
     if constexpr (KAHAN) tile_store<R, D, COH>(cout, ctl, ch.off, sd.o + H, sd.g0, sd.cnt, sites, W, hdr);
   }
   __syncthreads();  // shared memory is reused by the next item
-  return true;
+  return !SPLIT || !any;
+}
+
+// The chain of site i of the state (the last one that starts at or before it).
+__device__ __forceinline__ int site_chain(const ChainDesc *chains, int nchains, int64_t i) {
+  int lo = 0, hi = nchains - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (chains[mid].off <= i) lo = mid; else hi = mid - 1;
+  }
+  return lo;
 }
 
 // Locate the chain of a tile index through the prefix array (first tile of each chain).
