@@ -311,7 +311,8 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 2 : 1) k_gen_split(BlockedJob 
   const int base = threadIdx.x * 2;
   const bool edge_tile = ch.bc == FIXED && (t0 < 0 || t0 + W > ch.n);
   uint32_t ghost = 0;
-  bool wide = false, live = false;  // as in tile_item
+  auto own_c = [](int) -> const double * { return nullptr; };
+  bool odd = false, nan_tile = false;  // as in tile_item
 #pragma unroll
   for (int v = 0; v < 2; ++v) {
     const int64_t g = t0 + base + v;
@@ -319,31 +320,40 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 2 : 1) k_gen_split(BlockedJob 
 #pragma unroll
     for (int d = 0; d < D; ++d) {
       y[v][d] = tl[(base + v) * D + d];
-      wide |= !split_in_range<MODEL>(y[v][d], d, cf.c, sc);
-      live |= !is_nan(y[v][d]) && !((ghost >> v) & 1u);
+      odd |= !((ghost >> v) & 1u) && !split_holds<MODEL>(y[v][d], d, nullptr, sc);
     }
   }
-  const bool nan_tile = __syncthreads_or(wide);
-  if (nan_tile && __syncthreads_or(live)) {
-    gen_wide_tile<MODEL, RANGE>(job, ch, t0, H, cf, kappa2, tb, smem);
-    return;
+  if (__syncthreads_or(odd)) {
+    const int last = base + 2;
+    const bool next = last < W && (!edge_tile || (t0 + last >= 0 && t0 + last < ch.n));
+    const int b = block_or(split_tile_bits<MODEL, 2>(y, ghost, sc, next ? tl + last * D : nullptr, own_c, [](int) { return true; }),
+                           reinterpret_cast<int *>(smem));
+    nan_tile = (b & kSplitWide) && !(b & kSplitLive);
+    if (!nan_tile && ((b & kSplitWide) || ((b & kSplitGap) && (b & kSplitSome)))) {
+      gen_wide_tile<MODEL, RANGE>(job, ch, t0, H, cf, kappa2, tb, smem);
+      return;
+    }
   }
   if (edge_tile) gen_split_advance<MODEL, RANGE, true, PARK>(y, ghost, job.K, cf, kappa2, sc, st, ex, rec);
   else gen_split_advance<MODEL, RANGE, false, PARK>(y, 0u, job.K, cf, kappa2, sc, st, ex, rec);
   __syncthreads();  // every record is read before the tile is written over them
   const int64_t g0 = t0 + H, rem = ch.n - g0;
   const int cnt = (int)(rem < job.G ? rem : job.G);
-  wide = false;
+  auto stored_site = [&](int v) { return base + v >= H && base + v < H + cnt; };
+  odd = false;
 #pragma unroll
   for (int v = 0; v < 2; ++v)
 #pragma unroll
     for (int d = 0; d < D; ++d) {
       tl[(base + v) * D + d] = y[v][d];
-      wide |= base + v >= H && base + v < H + cnt && !split_in_range<MODEL>(y[v][d], d, cf.c, sc);
+      odd |= stored_site(v) && !split_holds<MODEL>(y[v][d], d, nullptr, sc);
     }
-  if (__syncthreads_or(wide) && !nan_tile) {
-    gen_wide_tile<MODEL, RANGE>(job, ch, t0, H, cf, kappa2, tb, smem);
-    return;
+  if (__syncthreads_or(odd) && !nan_tile) {
+    const int b = block_or(split_tile_bits<MODEL, 2>(y, ghost, sc, nullptr, own_c, stored_site), reinterpret_cast<int *>(smem));
+    if ((b & kSplitWide) || split_has_front(b)) {
+      gen_wide_tile<MODEL, RANGE>(job, ch, t0, H, cf, kappa2, tb, smem);
+      return;
+    }
   }
   report_nonfinite(job.hdr, nan_tile);
   if (cnt > 0) tile_store<double, D>(static_cast<double *>(job.out), tl, ch.off, H, g0, cnt, job.total, W, job.hdr);
@@ -420,7 +430,7 @@ __global__ void __launch_bounds__(256) k_gen_split_state(GenStagedJob job, Coef<
     Coef<double> c = cf;
     int ci;
     const ChainDesc ch = gen_site_chain(job, i, c, ci);
-    if (job.wide[2 * ci + job.parity]) {
+    if (wide_chain(job.wide[2 * ci + job.parity])) {
       gen_state_site<double, D>(job, tb, i, j);
       continue;
     }
@@ -456,7 +466,7 @@ __global__ void __launch_bounds__(256) k_gen_split_slope(GenStagedJob job, Coef<
     Coef<double> c = cf;
     int ci;
     const ChainDesc ch = gen_site_chain(job, i, c, ci);
-    if (j == 0 || job.wide[2 * ci + job.parity]) {
+    if (j == 0 || wide_chain(job.wide[2 * ci + job.parity])) {
       gen_slope_site<double, MODEL, RANGE>(job, ch, c, kappa2, i, j);
       continue;
     }
@@ -509,9 +519,9 @@ __global__ void __launch_bounds__(256) k_gen_split_combine(GenStagedJob job, Coe
     int ci;
     const ChainDesc ch = gen_site_chain(job, i, c, ci);
     unsigned *next = job.wide + 2 * ci + (job.parity ^ 1);
-    if (job.wide[2 * ci + job.parity]) {
+    if (wide_chain(job.wide[2 * ci + job.parity])) {
       gen_combine_site<double, D, false>(job, tb, i);
-      *next = 1u;
+      *next = kWideRange;
       continue;
     }
     bool wide = false, bad = false;
@@ -529,10 +539,10 @@ __global__ void __launch_bounds__(256) k_gen_split_combine(GenStagedJob job, Coe
       join(N, &nd, 1);
       const double r = fma(sc.w, fma(gen_update64(K[i * D + d], M[d], st), c.one, -nd), Y[i * D + d]);
       Y[i * D + d] = r;
-      wide |= !split_in_range<MODEL>(r, d, sc.c, sc);
+      wide |= !split_in_range<MODEL>(r, d, nullptr, sc);
       bad |= nonfinite(r);
     }
-    if (wide) *next = 1u;
+    if (wide) *next = kWideRange;
     if (bad) atomicOr(&job.hdr->status, ST_NONFINITE);
   }
 }

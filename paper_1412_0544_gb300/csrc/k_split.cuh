@@ -165,7 +165,7 @@ static cudaError_t launch_split_k(int block, int64_t grid, const BlockedJob &job
   const size_t smem = split_smem_bytes<MODEL, V, HET>(block);
   if (grid > 0)
     k_split<MODEL, V, HET, PACKED, NT><<<(unsigned)grid, block, smem, st>>>(job, to_coef<double>(cfd, cfd.kappa),
-                                                                          split_coef(MODEL, cfd));
+                                                                          split_coef(MODEL, cfd, false, HET));
   return cudaGetLastError();
 }
 template <int MODEL>

@@ -3,7 +3,7 @@
 // blocked and persistent kernels (all three call the same per-site functions).
 #include <algorithm>
 
-#include "rk4_tile.cuh"
+#include "rk4_generic.cuh"
 
 namespace rk4d {
 
@@ -96,9 +96,9 @@ __global__ void __launch_bounds__(256) k_staged_split(StagedJob job, Coef<double
     Coef<double> c = cf;
     int ci;
     const ChainDesc ch = staged_chain(job, i, c, ci);
-    if (job.wide[2 * ci + job.parity]) {
+    if (wide_chain(job.wide[2 * ci + job.parity])) {
       staged_site<double, MODEL, false>(job, ch, c, i, j);
-      if (j == 3) job.wide[2 * ci + (job.parity ^ 1)] = 1u;
+      if (j == 3) job.wide[2 * ci + (job.parity ^ 1)] = kWideRange;
       continue;
     }
     const int64_t li = i - ch.off;
@@ -165,29 +165,50 @@ __global__ void __launch_bounds__(256) k_staged_split(StagedJob job, Coef<double
       join(N[q], &nd, 1);
       const double r = split_final(y[q], K1[i * D + q], nd, 6.0, s.w);
       Y[i * D + q] = r;
-      wide |= !split_in_range<MODEL>(r, q, c.c, s);
+      wide |= !split_in_range<MODEL>(r, q, MODEL == ROESSLER && sp ? sp + 2 : nullptr, s);
       bad |= nonfinite(r);
     }
-    if (wide) job.wide[2 * ci + (job.parity ^ 1)] = 1u;
+    if (wide) job.wide[2 * ci + (job.parity ^ 1)] = kWideRange;
     if (bad) atomicOr(&job.hdr->status, ST_NONFINITE);
   }
 }
 
-template <int MODEL>
-__global__ void __launch_bounds__(256) k_split_scan(const double *y, const double *sp, int64_t total, int nchains,
-                                                    const ChainDesc *chains, SplitCoef sc, unsigned *flags) {
+template <int MODEL, int RANGE>
+__global__ void __launch_bounds__(256) k_split_scan(StagedJob job, Coef<double> cf, double kappa2, SplitCoef sc) {
   constexpr int D = Dim<MODEL>::D, P = Dim<MODEL>::P;
+  const double *Y = static_cast<const double *>(job.y), *SP = static_cast<const double *>(job.sp);
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += stride) {
-    bool wide = false;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < job.total; i += stride) {
+    Coef<double> c = cf;
+    int ci;
+    const ChainDesc ch = staged_chain(job, i, c, ci);
+    if (SP) c = site_coef<double, MODEL>(c, SP + i * P);
+    unsigned f = 0;
+    double y[D], k[D];
 #pragma unroll
-    for (int d = 0; d < D; ++d)
-      wide |= !split_in_range<MODEL>(y[i * D + d], d, MODEL == ROESSLER && sp ? sp[i * P + 2] : sc.c, sc);
-    if (sp) {
-#pragma unroll
-      for (int q = 0; q < P; ++q) wide |= !split_param_in_range(sp[i * P + q], sc.most[q]);
+    for (int d = 0; d < D; ++d) {
+      y[d] = Y[i * D + d];
+      if (!split_in_range<MODEL>(y[d], d, MODEL == ROESSLER && SP ? SP + i * P + 2 : nullptr, sc)) f |= kWideRange;
     }
-    if (wide) flags[2 * (nchains > 1 ? site_chain(chains, nchains, i) : 0)] = 1u;
+    if (SP) {
+#pragma unroll
+      for (int q = 0; q < P; ++q)
+        if (!split_param_in_range(SP[i * P + q], sc.most[q])) f |= kWideRange;
+    }
+    auto xat = [&](int64_t q) {
+      if (ch.bc == PERIODIC) q = wrap(q, ch.n);
+      const int64_t g = ch.off + q;
+      return q < 0 || q >= ch.n || !bounds_ok(job.hdr, in_range(g, 1, job.total)) ? 0.0 : Y[g * D];
+    };
+    const int64_t li = i - ch.off;
+    slope_gen<double, MODEL, RANGE>(y, xat(li - 1), xat(li + 1), RANGE == 2 ? xat(li - 2) : 0.0,
+                                    RANGE == 2 ? xat(li + 2) : 0.0, c, kappa2, k);
+    bool rest = true;
+#pragma unroll
+    for (int d = 0; d < D; ++d) rest = rest && is_zero(k[d]);
+    f |= rest ? kWideRest : kWideMoves;
+    unsigned *flag = job.wide + 2 * ci;
+    if (f & ~*static_cast<volatile unsigned *>(flag)) atomicOr(flag, f);
   }
 }
 
@@ -196,14 +217,29 @@ static unsigned sweep_grid(int64_t total) {
   return (unsigned)std::min<int64_t>((total + 255) / 256, cap);
 }
 
-cudaError_t launch_split_scan(int model, const double *state, const double *sp, int64_t total, int nchains,
-                              const ChainDesc *chains, const SplitCoef &sc, unsigned *wide, cudaStream_t st) {
+cudaError_t launch_split_scan(int model, int range, const double *state, const double *sp, int64_t total, int nchains,
+                              const ChainDesc &one, const ChainDesc *chains, const CoefD &cfd, unsigned *wide,
+                              cudaStream_t st) {
   const cudaError_t e = cudaMemsetAsync(wide, 0, 2 * sizeof(unsigned) * (size_t)nchains, st);
   if (e != cudaSuccess || total <= 0) return e;
-  if (model == ROESSLER)
-    k_split_scan<ROESSLER><<<sweep_grid(total), 256, 0, st>>>(state, sp, total, nchains, chains, sc, wide);
-  else
-    k_split_scan<HARMONIC><<<sweep_grid(total), 256, 0, st>>>(state, sp, total, nchains, chains, sc, wide);
+  StagedJob job{};
+  job.y = const_cast<double *>(state);
+  job.sp = sp;
+  job.nchains = nchains;
+  job.one = one;
+  job.chains = chains;
+  job.total = total;
+  job.wide = wide;
+  const Coef<double> cf = to_coef<double>(cfd, cfd.kappa);
+  const SplitCoef sc = split_coef(model, cfd, false, sp != nullptr);
+  const unsigned grid = sweep_grid(total);
+  if (model == ROESSLER) {
+    if (range == 1) k_split_scan<ROESSLER, 1><<<grid, 256, 0, st>>>(job, cf, cfd.kappa2, sc);
+    else k_split_scan<ROESSLER, 2><<<grid, 256, 0, st>>>(job, cf, cfd.kappa2, sc);
+  } else {
+    if (range == 1) k_split_scan<HARMONIC, 1><<<grid, 256, 0, st>>>(job, cf, cfd.kappa2, sc);
+    else k_split_scan<HARMONIC, 2><<<grid, 256, 0, st>>>(job, cf, cfd.kappa2, sc);
+  }
   return cudaGetLastError();
 }
 
@@ -211,7 +247,7 @@ template <int MODEL>
 static cudaError_t launch_split_one(int j, const StagedJob &job, const CoefD &cfd, cudaStream_t st) {
   if (job.total <= 0) return cudaSuccess;
   k_staged_split<MODEL><<<sweep_grid(job.total), 256, 0, st>>>(job, to_coef<double>(cfd, cfd.kappa),
-                                                              split_coef(MODEL, cfd), j);
+                                                              split_coef(MODEL, cfd, false, job.sp != nullptr), j);
   return cudaGetLastError();
 }
 

@@ -709,8 +709,8 @@ cudaError_t enqueue_integrate(rk4_chain *h, int kernel, void *state, void *comp,
     j.split = use_split(h) ? 1 : 0;
     j.wide = reinterpret_cast<unsigned *>(ws + L.result);  // 8 bytes a chain, free while integrating
     if (j.split) {
-      e = launch_split_scan(h->model, static_cast<const double *>(state), nullptr, h->total, h->nchains, j.chains,
-                            split_coef(h->model, cf, true), j.wide, st);
+      e = launch_split_scan(h->model, coupling_range(h), static_cast<const double *>(state), nullptr, h->total, h->nchains,
+                            j.one, j.chains, cf, j.wide, st);
       if (e != cudaSuccess) return e;
     }
     for (int64_t s = 0; s < nsteps; ++s) {
@@ -737,8 +737,8 @@ cudaError_t enqueue_integrate(rk4_chain *h, int kernel, void *state, void *comp,
     j.n2 = u0;
     j.n3 = u1;
     if (j.split) {
-      e = launch_split_scan(h->model, static_cast<const double *>(state), static_cast<const double *>(h->site_params),
-                            h->total, h->nchains, j.chains, split_coef(h->model, cf), j.wide, st);
+      e = launch_split_scan(h->model, 1, static_cast<const double *>(state), static_cast<const double *>(h->site_params),
+                            h->total, h->nchains, j.one, j.chains, cf, j.wide, st);
       if (e != cudaSuccess) return e;
     }
     for (int64_t s = 0; s < nsteps; ++s) {
@@ -1127,7 +1127,7 @@ SplitTableau rk4d::split_tableau(const TableauD &t, double dt) {
   return r;
 }
 
-SplitCoef rk4d::split_coef(int model, const CoefD &c, bool generic) {
+SplitCoef rk4d::split_coef(int model, const CoefD &c, bool generic, bool het) {
   SplitCoef s{};
   const double tau = generic ? c.h1 : c.h2;
   s.w = generic ? c.h1 : tau / 3.0;
@@ -1147,8 +1147,10 @@ SplitCoef rk4d::split_coef(int model, const CoefD &c, bool generic) {
   double most[4] = {};
   split_most(model, c.h1, most);
   for (int i = 0; i < 4; ++i) s.most[i] = high_word(most[i]);
-  s.c = c.c;
-  s.far = high_word(kSplitFar / c.h1);
+  const double far = kSplitFar / c.h1;
+  s.far = (float)far;
+  s.most_x = high_word(het ? far + most[2] : far + c.c);
+  s.least_x = high_word(far - c.c);
   s.big = high_word(model == RK4_ROESSLER ? kSplitBig / c.h1 : 0x1p40);
   return s;
 }

@@ -26,13 +26,14 @@ struct CoefD {
 
 // Coefficients of the split FP64 step (rk4_split.cuh): tau = dt / 2 (generic tableaux: dt), and the
 // products with it as float pairs (h + l).  at: Roessler a tau, harmonic w2 tau.  most: high words of the largest
-// magnitudes a site's own parameters may have (heterogeneous chains; in their order); far, big: of the
-// largest |x - c| (Roessler) and of the other components of a state (split_in_range).
+// magnitudes a site's own parameters may have (heterogeneous chains; in their order).  The state's range
+// (split_in_range): high words of the largest x and -x (Roessler; of any site's own c for heterogeneous
+// chains, which far, the largest |x - c|, bounds then) and of the other components.
 struct SplitCoef {
   double w;  // tau / 3 (generic tableaux: dt)
-  double c;
   float tauh, taul, kth, ktl, k2h, k2l, ath, atl, ch, cl;
-  unsigned most[4], far, big;
+  unsigned most[4], most_x, least_x, big;
+  float far;
 };
 
 // Generic explicit Runge-Kutta tableau (strictly lower a, weights b), up to kMaxStages stages.
@@ -172,14 +173,19 @@ template <int MODEL>
 cudaError_t launch_split_persistent(int v, int block, int grid, const PersistentJob &job, const CoefD &cf,
                                     cudaStream_t st);
 template <int MODEL> int persistent_split_max_grid(int v, int block);
-// Clear the chains' flags `wide` (two words each) and set the first of a chain's when a value of its state
-// or a site's own parameter is outside the split's range.
-cudaError_t launch_split_scan(int model, const double *state, const double *sp, int64_t total, int nchains,
-                              const ChainDesc *chains, const SplitCoef &sc, unsigned *wide, cudaStream_t st);
+// Set the chains' flags `wide` (two words each, the first of them here) of the staged schemes' split form.
+cudaError_t launch_split_scan(int model, int range, const double *state, const double *sp, int64_t total, int nchains,
+                              const ChainDesc &one, const ChainDesc *chains, const CoefD &cf, unsigned *wide,
+                              cudaStream_t st);
+// A chain's flag: 1 when a value of its state or a site's own parameter is outside the split's range; 2 when
+// a site has a slope of zero in every component, 4 when one has not.  A chain with both (a front that runs
+// into sites at rest, whose far end the pairs do not hold: rk4_split.cuh) is advanced in the FP64 form too.
+constexpr unsigned kWideRange = 1, kWideRest = 2, kWideMoves = 4;
+__host__ __device__ constexpr bool wide_chain(unsigned f) { return (f & kWideRange) || (f & 6u) == 6u; }
 // Whether every step of a handle with these coefficients (c.kappa: the largest coupling strength
 // of its chains) may run in the split form, and the form's coefficients.
 bool split_allowed(int model, const CoefD &c);
-SplitCoef split_coef(int model, const CoefD &c, bool generic = false);
+SplitCoef split_coef(int model, const CoefD &c, bool generic = false, bool het = false);
 // The generic scheme in the split form (k_gen_split.cu): a tableau's rows and weights, as float pairs
 // where they multiply the slopes' remainders, and the stages the result needs.
 struct SplitTableau {

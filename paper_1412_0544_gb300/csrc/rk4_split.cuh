@@ -34,7 +34,13 @@
 // the one-stage-per-launch kernel agree bit for bit.
 //
 // Range: a pair needs the exponent room of FP32.  Tiles whose values leave it (split_in_range)
-// are advanced in the FP64 form instead (tile_item returns false and the caller runs it again).
+// are advanced in the FP64 form instead (tile_item returns false and the caller runs it again).  Zeros are
+// in range, but a front that runs into a chain at rest decays through every magnitude: where FP64 has 1e-60 a
+// difference underflows to an exact zero, and one of 1e-46 comes out of FP32's subnormals.  Values that
+// stay below 2^-70 send the tile to the FP64 form; zeros do (split_tile_bits) when the tile starts with two
+// neighbouring sites all zero beside one that is not, or stores a component as zero at one site and holds
+// it nonzero at another.  What is left is exact: a component that is zero throughout a tile before and after
+// has a slope of zero (a wrong zero slope elsewhere shows in the same site's other components).
 // A tile of NaN alone, what a chain that has blown up consists of, stays: its first slope and so
 // its result are NaN in either form.
 #pragma once
@@ -213,11 +219,31 @@ __device__ __forceinline__ void join(FPair<f32x2> v, double *out, int stride) {
 // keeps dt |J| where their errors stay below the state's rounding.  The Roessler chain's J holds x - c
 // and z: dt |x - c| <= 1/4, dt |y| and dt |z| <= 0.3 (c: the site's own).  The harmonic chain is linear,
 // and its limit, 2^40, only leaves room in FP32's exponents.  NaN and infinity are out of range.
-template <int MODEL> __device__ __forceinline__ bool split_in_range(double v, int d, double c, const SplitCoef &s) {
+// split_holds: the same without zero.  Integer operations on the high words: with |x - c| in FP64 the two
+// subtractions per site and launch cost 9 % at k = 1 (2^22 sites, 256 x 4 x 1, 8 steps: 1144 -> 1246 us).  own_c: a
+// heterogeneous chain's c of the site (then by the FP32 heads), else NULL.
+__device__ __forceinline__ bool is_zero(double v) {
+  return (((unsigned)__double2hiint(v) & 0x7fffffffu) | (unsigned)__double2loint(v)) == 0u;
+}
+__device__ __forceinline__ float truncated_head(double v) {  // of a magnitude in FP32's range, or 0
+  const int hi = __double2hiint(v);
+  const unsigned a = (unsigned)max((hi & 0x7fffffff) - 0x38000000, 0);
+  return __uint_as_float(__funnelshift_l((unsigned)__double2loint(v), a, 3) | ((unsigned)hi & 0x80000000u));
+}
+template <int MODEL>
+__device__ __forceinline__ bool split_holds(double v, int d, const double *own_c, const SplitCoef &s) {
   constexpr unsigned lo = (1023u - 70u) << 20;
-  const unsigned a = (unsigned)__double2hiint(v) & 0x7fffffffu;
-  const bool top = MODEL == ROESSLER && d == 0 ? ((unsigned)__double2hiint(sub(v, c)) & 0x7fffffffu) <= s.far : a <= s.big;
-  return ((a >= lo) | ((a | (unsigned)__double2loint(v)) == 0u)) & top;
+  const int hi = __double2hiint(v);
+  const unsigned a = (unsigned)hi & 0x7fffffffu;
+  if (MODEL == ROESSLER && d == 0) {
+    if (own_c) return (a >= lo) & (a <= s.most_x) & (fabsf(__fsub_rn(truncated_head(v), truncated_head(*own_c))) <= s.far);
+    return (a >= lo) & (a <= (hi < 0 ? s.least_x : s.most_x));
+  }
+  return (a >= lo) & (a <= s.big);
+}
+template <int MODEL>
+__device__ __forceinline__ bool split_in_range(double v, int d, const double *own_c, const SplitCoef &s) {
+  return is_zero(v) || split_holds<MODEL>(v, d, own_c, s);
 }
 __device__ __forceinline__ bool is_nan(double v) {
   const unsigned a = (unsigned)__double2hiint(v) & 0x7fffffffu;

@@ -759,6 +759,65 @@ template <typename R, int D> __host__ __device__ constexpr int align_sites() {
   return 16 / a;
 }
 
+// What a tile (or a packed tile's segment) holds, as far as the split form asks, in the bits of a thread's
+// sites OR-ed over it.
+enum : int {
+  kSplitWide = 1,    // a stored value that is not zero and out of range
+  kSplitLive = 2,    // a value that is not NaN
+  kSplitGap = 4,     // two neighbouring sites that are all zero
+  kSplitSome = 8,    // a value that is not zero
+  kSplitZero = 16,   // (<< d) a stored value of component d that is zero
+  kSplitValue = 128  // (<< d) one anywhere that is not
+};
+__device__ __forceinline__ bool split_has_front(int b) {  // zeros and nonzero values, of one component
+  return ((b / kSplitZero) & (b / kSplitValue) & 7) != 0;
+}
+// The bits of the thread's sites that are not ghosts.  c(v): the site's own c or NULL; stored(v): whether it is
+// stored (of the loaded tile, all are); next: the state of the site after the thread's last one, or NULL.
+template <int MODEL, int V, typename C, typename S>
+__device__ __forceinline__ int split_tile_bits(const double (&y)[V][Dim<MODEL>::D], uint32_t ghost, const SplitCoef &sc,
+                                               const double *next, C &&c, S &&stored) {
+  constexpr int D = Dim<MODEL>::D;
+  int b = 0;
+  bool before = false;  // the site before is all zero
+#pragma unroll
+  for (int v = 0; v < V; ++v) {
+    const bool real = !((ghost >> v) & 1u);
+    bool rest = real;
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+      if (is_zero(y[v][d])) {
+        if (real && stored(v)) b |= kSplitZero << d;
+      } else {
+        rest = false;
+        if (real) b |= kSplitSome | (kSplitValue << d);
+        if (real && stored(v) && !split_holds<MODEL>(y[v][d], d, c(v), sc)) b |= kSplitWide;
+      }
+      if (real && !is_nan(y[v][d])) b |= kSplitLive;
+    }
+    if (rest && before) b |= kSplitGap;
+    before = rest;
+  }
+  if (before && next) {
+    bool rest = true;
+#pragma unroll
+    for (int d = 0; d < D; ++d) rest = rest && is_zero(next[d]);
+    if (rest) b |= kSplitGap;
+  }
+  return b;
+}
+// The bits of all threads of the block; word: shared memory that nothing else uses meanwhile.
+__device__ __forceinline__ int block_or(int b, int *word) {
+  if (threadIdx.x == 0) *word = 0;
+  __syncthreads();
+  b = __reduce_or_sync(kFull, b);
+  if (b && (threadIdx.x & 31) == 0) atomicOr(word, b);
+  __syncthreads();
+  b = *word;
+  __syncthreads();
+  return b;
+}
+
 // Process one (chain, tile) item end to end: load, advance K steps, store the interior.
 // ALN (batch tiles): the window starts at the last multiple of align_sites() at or before
 // tile G - H in the state array, so it moves by whole 16-byte vectors wherever the chain
@@ -823,22 +882,28 @@ __device__ __forceinline__ bool tile_item(const R *__restrict__ in, R *__restric
   }
   bool nan_tile = false;  // SPLIT: every value is NaN already (a chain that has blown up), and stays so
   if constexpr (SPLIT) {
-    bool wide = false, live = false;  // a value outside the split's range; one that is not NaN
-    auto values_live = [&]() {
-      bool l = false;
+    double *spd = nullptr;
+    f32x2 *spf = nullptr;
+    auto own_c = [&](int v) -> const double * { return HET && MODEL == ROESSLER ? &ptl[(base + v) * P + 2] : nullptr; };
+    bool odd = false, out = false;  // a value that is zero or out of range; a parameter out of range
+#pragma unroll
+    for (int v = 0; v < V; ++v)
+#pragma unroll
+      for (int d = 0; d < D; ++d) odd |= !((ghost >> v) & 1u) && !split_holds<MODEL>(y[v][d], d, own_c(v), *sc);
+    if constexpr (HET) {
 #pragma unroll
       for (int v = 0; v < V; ++v)
 #pragma unroll
-        for (int d = 0; d < D; ++d) l |= !is_nan(y[v][d]) && !((ghost >> v) & 1u);
-      return l;
-    };
-    double *spd = nullptr;
-    f32x2 *spf = nullptr;
-#pragma unroll
-    for (int v = 0; v < V; ++v) {
-      const double c = HET && MODEL == ROESSLER ? ptl[(base + v) * P + 2] : cf.c;
-#pragma unroll
-      for (int d = 0; d < D; ++d) wide |= !split_in_range<MODEL>(y[v][d], d, c, *sc);
+        for (int i = 0; i < P; ++i) out |= !split_param_in_range(ptl[(base + v) * P + i], sc->most[i]);
+    }
+    if (__syncthreads_or(odd | out)) {
+      const int last = base + V;  // the next thread's first site, if it is the chain's
+      const bool next = last < W && (!edge_tile || (t0 + last >= 0 && t0 + last < ch.n));
+      int b = split_tile_bits<MODEL, V>(y, ghost, *sc, next ? tl + last * D : nullptr, own_c, [](int) { return true; });
+      if (out) b |= kSplitWide | kSplitLive;
+      b = block_or(b, reinterpret_cast<int *>(smem));
+      nan_tile = (b & kSplitWide) && !(b & kSplitLive);
+      if (!nan_tile && ((b & kSplitWide) || ((b & kSplitGap) && (b & kSplitSome)))) return false;
     }
     if constexpr (HET) {
       // the parameters move to thread-private slots (consecutive threads, consecutive addresses),
@@ -848,14 +913,8 @@ __device__ __forceinline__ bool tile_item(const R *__restrict__ in, R *__restric
 #pragma unroll
       for (int v = 0; v < V; ++v)
 #pragma unroll
-        for (int i = 0; i < P; ++i) {
-          p[v][i] = ptl[(base + v) * P + i];
-          const bool out = !split_param_in_range(p[v][i], sc->most[i]);
-          wide |= out;
-          live |= out;
-        }
-      nan_tile = __syncthreads_or(wide);
-      if (nan_tile && __syncthreads_or(live || values_live())) return false;
+        for (int i = 0; i < P; ++i) p[v][i] = ptl[(base + v) * P + i];
+      __syncthreads();
       spd = ptl + threadIdx.x;
       spf = reinterpret_cast<f32x2 *>(ptl + W * P) + threadIdx.x;
 #pragma unroll
@@ -877,9 +936,6 @@ __device__ __forceinline__ bool tile_item(const R *__restrict__ in, R *__restric
           o[5 * blockDim.x] = pack2(c0.l, c1.l);
         }
       }
-    } else {
-      nan_tile = __syncthreads_or(wide);
-      if (nan_tile && __syncthreads_or(live || values_live())) return false;
     }
     double *rec = nullptr;
     if constexpr (PARK) rec = tl + threadIdx.x * split_record_words<MODEL, V>();
@@ -898,17 +954,18 @@ __device__ __forceinline__ bool tile_item(const R *__restrict__ in, R *__restric
 
   const int64_t rem = ch.n - g0;
   const int cnt = (int)(rem < G ? rem : G);
-  bool bad = false;  // a stored (interior) value is NaN or infinite (SPLIT: out of range)
+  bool bad = false;  // a stored (interior) value is NaN or infinite (SPLIT: zero or out of range)
+  auto own_c = [&](int v) -> const R * { return HET && MODEL == ROESSLER ? &ptl[(v * P + 2) * blockDim.x + threadIdx.x] : nullptr; };
+  auto stored_site = [&](int v) { return base + v >= hl && base + v < hl + cnt; };
 #pragma unroll
   for (int v = 0; v < V; ++v) {
-    const bool stored = base + v >= hl && base + v < hl + cnt;
+    const bool stored = stored_site(v);
 #pragma unroll
     for (int d = 0; d < D; ++d) {
       tl[(base + v) * D + d] = y[v][d];
       if constexpr (KAHAN) ctl[(base + v) * D + d] = cmp[v][d];
       if constexpr (SPLIT) {
-        const double c = HET && MODEL == ROESSLER ? ptl[(v * P + 2) * blockDim.x + threadIdx.x] : cf.c;
-        bad |= stored && !split_in_range<MODEL>(y[v][d], d, c, *sc);
+        bad |= stored && !split_holds<MODEL>(y[v][d], d, own_c(v), *sc);
       } else {
         bad |= stored && nonfinite(y[v][d]);
       }
@@ -916,7 +973,10 @@ __device__ __forceinline__ bool tile_item(const R *__restrict__ in, R *__restric
   }
   const int any_bad = __syncthreads_or(bad);
   if constexpr (SPLIT) {
-    if (any_bad && !nan_tile) return false;
+    if (any_bad && !nan_tile) {
+      const int b = block_or(split_tile_bits<MODEL, V>(y, ghost, *sc, nullptr, own_c, stored_site), reinterpret_cast<int *>(smem));
+      if ((b & kSplitWide) || split_has_front(b)) return false;
+    }
     report_nonfinite(hdr, nan_tile);
   } else {
     report_nonfinite(hdr, any_bad);
@@ -1009,34 +1069,41 @@ __device__ __forceinline__ bool packed_tile_item(const R *__restrict__ in, R *__
       y[v][d] = tl[(base + v) * D + d];
       if constexpr (KAHAN) cmp[v][d] = ctl[(base + v) * D + d]; else cmp[v][d] = R(0);
     }
-  bool wide = false, all_nan = false;  // SPLIT: of this thread's segment: out of range; NaN and nothing else
+  bool wide = false, all_nan = false;  // SPLIT: this thread's segment leaves the form; is NaN and nothing else
+  auto own_c = [](int) -> const double * { return nullptr; };
+  auto stored_site = [&](int v) { return my >= 0 && rel + v >= H && rel + v < H + cnt; };
   bool mine = true;                    // FLAGGED: the segment is stored
   if constexpr (FLAGGED) {
     mine = my >= 0 && flag[my - s0] != 0;
     __syncthreads();  // before the exchange writes there
   }
   if constexpr (SPLIT) {
-    bool leaves = false, live = false;
-    if (my >= 0) {
+    bool odd = false;  // a value that is zero or out of range
 #pragma unroll
-      for (int v = 0; v < V; ++v)
+    for (int v = 0; v < V; ++v)
 #pragma unroll
-        for (int d = 0; d < D; ++d) {
-          leaves |= !split_in_range<MODEL>(y[v][d], d, c.c, *scp);
-          live |= !is_nan(y[v][d]) && !((ghost >> v) & 1u);
-        }
-    }
-    if (__syncthreads_or(leaves)) {
+      for (int d = 0; d < D; ++d)
+        odd |= my >= 0 && !((ghost >> v) & 1u) && !split_holds<MODEL>(y[v][d], d, nullptr, *scp);
+    if (__syncthreads_or(odd)) {
       for (int s = threadIdx.x; s < s1 - s0; s += blockDim.x) flag[s] = 0;
       __syncthreads();
-      if (leaves || live) atomicOr(&flag[my - s0], (leaves ? 1 : 0) | (live ? 2 : 0));
+      if (my >= 0) {
+        const int last = base + V;  // the next thread's first site, if it is the segment's and the chain's
+        bool next = last < segs[my].o + segs[my].L;
+        if (next && chains[segs[my].chain].bc == FIXED) {
+          const int64_t g = segs[my].g0 - H + rel + V;
+          next = g >= 0 && g < chains[segs[my].chain].n;
+        }
+        atomicOr(&flag[my - s0], split_tile_bits<MODEL, V>(y, ghost, *scp, next ? tl + last * D : nullptr, own_c,
+                                                           [](int) { return true; }));
+      }
       __syncthreads();
       if (my >= 0) {
-        const int f = flag[my - s0];
-        wide = f == 3;
-        all_nan = f == 1;
+        const int b = flag[my - s0];
+        all_nan = (b & kSplitWide) && !(b & kSplitLive);
+        wide = !all_nan && ((b & kSplitWide) || ((b & kSplitGap) && (b & kSplitSome)));
       }
-      if (!__syncthreads_or(my >= 0 && !wide)) return false;  // every segment is marked (3)
+      if (!__syncthreads_or(my >= 0 && !wide)) return false;  // every segment is marked
     }
     SplitCoef sc = *scp;
     split_set_kappa(sc, c.kappa);
@@ -1048,23 +1115,27 @@ __device__ __forceinline__ bool packed_tile_item(const R *__restrict__ in, R *__
     tile_advance<R, MODEL, V, KAHAN, true>(y, cmp, ghost, K, c, edge);
   }
 
-  bool bad = false;  // a stored (interior) value is NaN or infinite (SPLIT: out of range)
+  bool bad = false;  // a stored (interior) value is NaN or infinite (SPLIT: zero or out of range)
 #pragma unroll
   for (int v = 0; v < V; ++v) {
-    const bool stored = my >= 0 && rel + v >= H && rel + v < H + cnt;
+    const bool stored = stored_site(v);
 #pragma unroll
     for (int d = 0; d < D; ++d) {
       tl[(base + v) * D + d] = y[v][d];
       if constexpr (KAHAN) ctl[(base + v) * D + d] = cmp[v][d];
-      if constexpr (SPLIT) bad |= stored && !split_in_range<MODEL>(y[v][d], d, c.c, *scp);
+      if constexpr (SPLIT) bad |= stored && !split_holds<MODEL>(y[v][d], d, nullptr, *scp);
       else bad |= stored && mine && nonfinite(y[v][d]);
     }
   }
   int any = __syncthreads_or(bad | wide);
   bool marked = FLAGGED;  // the words say which segments to leave out (SPLIT) or to store (FLAGGED)
   if constexpr (SPLIT) {
-    wide |= bad && !all_nan;
     if (any) {
+      for (int s = threadIdx.x; s < s1 - s0; s += blockDim.x) flag[s] = 0;
+      __syncthreads();
+      if (my >= 0) atomicOr(&flag[my - s0], split_tile_bits<MODEL, V>(y, ghost, *scp, nullptr, own_c, stored_site));
+      __syncthreads();
+      if (my >= 0 && !all_nan) wide |= (flag[my - s0] & kSplitWide) || split_has_front(flag[my - s0]);
       report_nonfinite(hdr, __syncthreads_or(all_nan));
       any = __syncthreads_or(wide);
     }
