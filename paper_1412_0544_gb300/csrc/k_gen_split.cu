@@ -80,8 +80,10 @@ template <typename T> __device__ __forceinline__ FPair<T> gen_first_order(const 
   return pair_mul(FPair<T>{vmul(m1, tau.h), vmul(m1, tau.l)}, tau.h, M);
 }
 
-// A tile outside the split's range in the FP64 form (two sites per thread, run-time tableau).
-template <int MODEL, int RANGE>
+// A tile outside the split's range in the FP64 form (two sites per thread).  SHAPE: the tableau's nonzero
+// pattern where it is one of the compiled ones (Dormand-Prince 5 + second neighbours, 2^20 sites,
+// 128 x 4 x 2, a state of 1e-25: 302 -> 251 us per step, 269 as the one form of a kernel of its own).
+template <int MODEL, int RANGE, uint64_t SHAPE>
 __device__ __noinline__ void gen_wide_tile(const BlockedJob &job, ChainDesc ch, int64_t t0, int H, Coef<double> cf,
                                            double kappa2, const Tableau<double> &tb, unsigned char *smem) {
   constexpr int D = Dim<MODEL>::D, V = 2;
@@ -104,7 +106,7 @@ __device__ __noinline__ void gen_wide_tile(const BlockedJob &job, ChainDesc ch, 
       cmp[v][d] = 0.0;
     }
   }
-  gen_tile_advance<double, MODEL, V, RANGE, false, true, 0>(y, cmp, ghost, job.K, cf, kappa2, tb, edge);
+  gen_tile_advance<double, MODEL, V, RANGE, false, true, SHAPE>(y, cmp, ghost, job.K, cf, kappa2, tb, edge);
   const int64_t g0 = t0 + H, rem = ch.n - g0;
   const int cnt = (int)(rem < job.G ? rem : job.G);
   bool bad = false;
@@ -285,7 +287,7 @@ __device__ __forceinline__ void gen_split_advance(double (&y)[2][Dim<MODEL>::D],
 
 template <int MODEL, int RANGE, int NT>
 __global__ void __launch_bounds__(NT, NT <= 256 ? 2 : 1) k_gen_split(BlockedJob job, Coef<double> cf, double kappa2, SplitCoef sc,
-                                                  SplitTableau st, Tableau<double> tb, int H) {
+                                                  SplitTableau st, Tableau<double> tb, uint64_t shape, int H) {
   constexpr int D = Dim<MODEL>::D;
   constexpr bool PARK = NT <= 256;
   extern __shared__ __align__(16) unsigned char smem[];
@@ -301,6 +303,11 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 2 : 1) k_gen_split(BlockedJob 
   }
   const int W = blockDim.x * 2;
   const int64_t t0 = tile * (int64_t)job.G - H;
+  auto wide_tile = [&]() {
+    if (shape == kShapeDopri5) gen_wide_tile<MODEL, RANGE, kShapeDopri5>(job, ch, t0, H, cf, kappa2, tb, smem);
+    else if (shape == kShapeRK4) gen_wide_tile<MODEL, RANGE, kShapeRK4>(job, ch, t0, H, cf, kappa2, tb, smem);
+    else gen_wide_tile<MODEL, RANGE, 0>(job, ch, t0, H, cf, kappa2, tb, smem);
+  };
   ulonglong2 *ex = reinterpret_cast<ulonglong2 *>(smem);
   double *tl = reinterpret_cast<double *>(ex + 2 * blockDim.x);  // the tile, then the records in its place
   f32x2 *rec = reinterpret_cast<f32x2 *>(tl) + threadIdx.x * gen_record_words(st.slots, D, PARK);
@@ -330,7 +337,7 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 2 : 1) k_gen_split(BlockedJob 
                            reinterpret_cast<int *>(smem));
     nan_tile = (b & kSplitWide) && !(b & kSplitLive);
     if (!nan_tile && ((b & kSplitWide) || ((b & kSplitGap) && (b & kSplitSome)))) {
-      gen_wide_tile<MODEL, RANGE>(job, ch, t0, H, cf, kappa2, tb, smem);
+      wide_tile();
       return;
     }
   }
@@ -351,7 +358,7 @@ __global__ void __launch_bounds__(NT, NT <= 256 ? 2 : 1) k_gen_split(BlockedJob 
   if (__syncthreads_or(odd) && !nan_tile) {
     const int b = block_or(split_tile_bits<MODEL, 2>(y, ghost, sc, nullptr, own_c, stored_site), reinterpret_cast<int *>(smem));
     if ((b & kSplitWide) || split_has_front(b)) {
-      gen_wide_tile<MODEL, RANGE>(job, ch, t0, H, cf, kappa2, tb, smem);
+      wide_tile();
       return;
     }
   }
@@ -373,7 +380,7 @@ static cudaError_t launch_gen_split_k(int threads, const BlockedJob &job, const 
   const size_t wide = sizeof(double) * ((size_t)gen_edge_values(2) + (size_t)threads * 2 * D);
   k_gen_split<MODEL, RANGE, NT><<<(unsigned)job.ntiles, threads, std::max(ours, wide), st>>>(
       job, to_coef<double>(cfd, cfd.kappa), cfd.kappa2, split_coef(MODEL, cfd, true), stb,
-      to_tableau<double>(td, dt), H);
+      to_tableau<double>(td, dt), tableau_shape(td), H);
   return cudaGetLastError();
 }
 template <int MODEL, int RANGE>

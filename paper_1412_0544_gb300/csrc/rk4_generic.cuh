@@ -59,6 +59,29 @@ template <uint64_t SHAPE, typename R> __device__ __forceinline__ bool gen_b_nonz
   if constexpr (SHAPE != 0) return (SHAPE & shape_b_bit(m)) != 0; else return (tb.bnz >> m) & 1u;
 }
 
+// The nonzero pattern of a tableau (see shape_a_bit): the key of the compiled shapes.
+inline uint64_t tableau_shape(const TableauD &t) {
+  uint64_t sh = (uint64_t)t.s & 7u;
+  for (int j = 1; j < t.s; ++j)
+    for (int m = 0; m < j; ++m)
+      if (t.a[j][m] != 0.0) sh |= shape_a_bit(j, m);
+  for (int m = 0; m < t.s; ++m)
+    if (t.b[m] != 0.0) sh |= shape_b_bit(m);
+  return sh;
+}
+
+// Shapes with tile kernels compiled for them (4 sites per thread): the classical RK4 tableau
+// (the generic kernel runs it with second-neighbour coupling) and Dormand-Prince 5 (7 stages,
+// a_61 = 0, b_1 = b_6 = 0).  Other tableaux run the kernel that reads the pattern at run time.
+constexpr uint64_t kShapeRK4 = 4u | shape_a_bit(1, 0) | shape_a_bit(2, 1) | shape_a_bit(3, 2) | shape_b_bit(0) |
+                               shape_b_bit(1) | shape_b_bit(2) | shape_b_bit(3);
+constexpr uint64_t kShapeDopri5 =
+    7u | shape_a_bit(1, 0) | shape_a_bit(2, 0) | shape_a_bit(2, 1) | shape_a_bit(3, 0) | shape_a_bit(3, 1) |
+    shape_a_bit(3, 2) | shape_a_bit(4, 0) | shape_a_bit(4, 1) | shape_a_bit(4, 2) | shape_a_bit(4, 3) |
+    shape_a_bit(5, 0) | shape_a_bit(5, 1) | shape_a_bit(5, 2) | shape_a_bit(5, 3) | shape_a_bit(5, 4) |
+    shape_a_bit(6, 0) | shape_a_bit(6, 2) | shape_a_bit(6, 3) | shape_a_bit(6, 4) | shape_a_bit(6, 5) |
+    shape_b_bit(0) | shape_b_bit(2) | shape_b_bit(3) | shape_b_bit(4) | shape_b_bit(5);
+
 // Eq. (4): stage state of stage j from the step's start y and the earlier slopes.
 template <typename R, int D, uint64_t SHAPE = 0>
 __device__ __forceinline__ void gen_stage_state(int j, const Tableau<R> &tb, const R *y, const R (*k)[D], R *u) {

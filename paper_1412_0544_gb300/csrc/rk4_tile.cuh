@@ -818,6 +818,16 @@ __device__ __forceinline__ int block_or(int b, int *word) {
   return b;
 }
 
+// OR b into the word of the thread's segment (NULL: none); one access a warp where its threads share it.
+__device__ __forceinline__ void segment_or(int b, int *word) {
+  const unsigned long long w = (unsigned long long)word;
+  if (__all_sync(kFull, w == __shfl_sync(kFull, w, 0))) {
+    b = __reduce_or_sync(kFull, b);
+    if (threadIdx.x & 31) return;
+  }
+  if (word && b) atomicOr(word, b);
+}
+
 // Process one (chain, tile) item end to end: load, advance K steps, store the interior.
 // ALN (batch tiles): the window starts at the last multiple of align_sites() at or before
 // tile G - H in the state array, so it moves by whole 16-byte vectors wherever the chain
@@ -1087,6 +1097,7 @@ __device__ __forceinline__ bool packed_tile_item(const R *__restrict__ in, R *__
     if (__syncthreads_or(odd)) {
       for (int s = threadIdx.x; s < s1 - s0; s += blockDim.x) flag[s] = 0;
       __syncthreads();
+      int b = 0;
       if (my >= 0) {
         const int last = base + V;  // the next thread's first site, if it is the segment's and the chain's
         bool next = last < segs[my].o + segs[my].L;
@@ -1094,12 +1105,12 @@ __device__ __forceinline__ bool packed_tile_item(const R *__restrict__ in, R *__
           const int64_t g = segs[my].g0 - H + rel + V;
           next = g >= 0 && g < chains[segs[my].chain].n;
         }
-        atomicOr(&flag[my - s0], split_tile_bits<MODEL, V>(y, ghost, *scp, next ? tl + last * D : nullptr, own_c,
-                                                           [](int) { return true; }));
+        b = split_tile_bits<MODEL, V>(y, ghost, *scp, next ? tl + last * D : nullptr, own_c, [](int) { return true; });
       }
+      segment_or(b, my >= 0 ? &flag[my - s0] : nullptr);
       __syncthreads();
       if (my >= 0) {
-        const int b = flag[my - s0];
+        b = flag[my - s0];
         all_nan = (b & kSplitWide) && !(b & kSplitLive);
         wide = !all_nan && ((b & kSplitWide) || ((b & kSplitGap) && (b & kSplitSome)));
       }
@@ -1133,7 +1144,8 @@ __device__ __forceinline__ bool packed_tile_item(const R *__restrict__ in, R *__
     if (any) {
       for (int s = threadIdx.x; s < s1 - s0; s += blockDim.x) flag[s] = 0;
       __syncthreads();
-      if (my >= 0) atomicOr(&flag[my - s0], split_tile_bits<MODEL, V>(y, ghost, *scp, nullptr, own_c, stored_site));
+      segment_or(my >= 0 ? split_tile_bits<MODEL, V>(y, ghost, *scp, nullptr, own_c, stored_site) : 0,
+                 my >= 0 ? &flag[my - s0] : nullptr);
       __syncthreads();
       if (my >= 0 && !all_nan) wide |= (flag[my - s0] & kSplitWide) || split_has_front(flag[my - s0]);
       report_nonfinite(hdr, __syncthreads_or(all_nan));
