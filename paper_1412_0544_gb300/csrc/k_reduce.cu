@@ -54,9 +54,15 @@ __device__ __forceinline__ double site_energy(const R *y, const R *c, const Chai
 // and the right neighbour's value comes from the next lane, already converted (conversions of an
 // FP32 state issue on the FP64 pipe too).  The sites' terms one by one, as site_energy weights
 // them, where a sum leaves the range in which a square can neither overflow nor lose bits that
-// its weight might bring back.  The call for 2^22 sites: harmonic FP64 173 -> 98 us, FP32 232 -> 170,
-// Roessler FP64 91 -> 60 (32 of it launches, copies and the wait).
-__device__ __forceinline__ bool sum_in_range(double s) { return s >= 0x1p-800 && s <= 0x1p800; }
+// its weight might bring back.  A sum of zero is in range when every value in it was zero (seen: their
+// bits OR-ed), as the momenta of a chain released at rest are.  The call for 2^22 sites: harmonic FP64
+// 173 -> 98 us, FP32 232 -> 170, Roessler FP64 91 -> 60 (32 of it launches, copies and the wait).
+__device__ __forceinline__ unsigned seen(double v) {
+  return ((unsigned)__double2hiint(v) & 0x7fffffffu) | (unsigned)__double2loint(v);
+}
+__device__ __forceinline__ bool sum_in_range(double s, unsigned seen) {
+  return (s >= 0x1p-800 && s <= 0x1p800) || seen == 0u;
+}
 
 template <int MODEL, typename R>
 __device__ __forceinline__ double sum_energy(const R *y, const R *c, const ChainDesc &ch, int64_t first, int64_t stride,
@@ -64,6 +70,7 @@ __device__ __forceinline__ double sum_energy(const R *y, const R *c, const Chain
   constexpr int D = Dim<MODEL>::D;
   const int lane = threadIdx.x & 31;
   double s[4] = {0.0, 0.0, 0.0, 0.0};
+  unsigned z[4] = {0, 0, 0, 0};  // what the sums' values had of bits
 #pragma unroll 4
   for (int64_t i = first; i - lane < hi; i += stride) {  // warp-uniform
     double v[D];
@@ -71,7 +78,10 @@ __device__ __forceinline__ double sum_energy(const R *y, const R *c, const Chain
     for (int d = 0; d < D; ++d) v[d] = i < hi ? site_value<MODEL>(y, c, (ch.off + i) * D + d) : 0.0;
     if constexpr (MODEL == ROESSLER) {
 #pragma unroll
-      for (int d = 0; d < D; ++d) s[d] = fma(v[d], v[d], s[d]);
+      for (int d = 0; d < D; ++d) {
+        s[d] = fma(v[d], v[d], s[d]);
+        z[d] |= seen(v[d]);
+      }
     } else {
       double qr = __shfl_down_sync(kFull, v[0], 1);
       if (i < hi && (lane == 31 || i + 1 == hi)) {
@@ -83,20 +93,30 @@ __device__ __forceinline__ double sum_energy(const R *y, const R *c, const Chain
         s[0] = fma(v[1], v[1], s[0]);
         s[1] = fma(q, q, s[1]);
         s[2] = fma(dq, dq, s[2]);
-        if (i == 0 && ch.bc == FIXED) s[2] = fma(q, q, s[2]);
+        z[0] |= seen(v[1]);
+        z[1] |= seen(q);
+        z[2] |= seen(dq);
+        if (i == 0 && ch.bc == FIXED) {
+          s[2] = fma(q, q, s[2]);
+          z[2] |= seen(q);
+        }
         if (kappa2 != 0.0) {
           double q2;
           if (i + 2 < ch.n) q2 = site_value<MODEL>(y, c, (ch.off + i + 2) * D);
           else q2 = (ch.bc == PERIODIC) ? site_value<MODEL>(y, c, (ch.off + (i + 2) % ch.n) * D) : 0.0;
           const double d2 = q2 - q;
           s[3] = fma(d2, d2, s[3]);
-          if (i < 2 && ch.bc == FIXED) s[3] = fma(q, q, s[3]);
+          z[3] |= seen(d2);
+          if (i < 2 && ch.bc == FIXED) {
+            s[3] = fma(q, q, s[3]);
+            z[3] |= seen(q);
+          }
         }
       }
     }
   }
-  bool plain = sum_in_range(s[0]) && sum_in_range(s[1]) && sum_in_range(s[2]);
-  if (MODEL == HARMONIC && kappa2 != 0.0) plain = plain && sum_in_range(s[3]);
+  bool plain = sum_in_range(s[0], z[0]) && sum_in_range(s[1], z[1]) && sum_in_range(s[2], z[2]);
+  if (MODEL == HARMONIC && kappa2 != 0.0) plain = plain && sum_in_range(s[3], z[3]);
   if (plain) {  // every value is finite
     if constexpr (MODEL == ROESSLER) return 0.5 * (s[0] + s[1] + s[2]);
     else return 0.5 * (s[0] + w2 * s[1] + ch.kappa * s[2] + kappa2 * s[3]);
