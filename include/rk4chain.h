@@ -142,7 +142,8 @@ int rk4_chain_get_kernel(const rk4_chain *h, int *kernel);
 
 /* Sets the tiling (block, v, k; G is computed).  block = 0 restores the automatic choice, which
  * each integration makes from the sites and its steps (from the sites alone for a batch);
- * rk4_chain_get_tiling then reports its seed.
+ * rk4_chain_get_tiling then reports what the last integration ran with, before the first one (and
+ * after any other change of the handle) the choice's seed.
  * The largest block depends on the kernel the handle runs (its register budget): 1024
  * threads for v = 1, 512 for v = 2 and 4, 256 for v = 8, the generic scheme and the
  * heterogeneous FP32 Roessler chain with v = 4.  Errors: RK4_EINVAL when block, v or k is out

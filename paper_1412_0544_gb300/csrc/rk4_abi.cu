@@ -85,6 +85,7 @@ struct rk4_chain {
   bool tiling_auto = true;
   rk4_tiling tiling{};
   rk4_tiling run{};  // what the current integration runs with (run_tiling)
+  unsigned run_version = 0;  // config_version + 1 of the last integration with the automatic tiling
   // its last few automatic choices, by the number of steps, under one configuration
   struct {
     int64_t steps = -1;
@@ -455,13 +456,13 @@ double tiles_estimate(const rk4_chain *h, int W, int v, int k) {
 }
 
 // The tiling an integration of nsteps runs with.  One that was set or tuned is taken as it is.
-// The automatic choice (whose seed rk4_chain_get_tiling reports) depends on the sites and the
-// steps: a short chain needs small tiles to reach every SM and many steps per launch to pay for
-// the launch, a long one wide tiles.  Measured against the seed, us per step: FP64 1000 sites 8.9
-// -> 1.6 (128 x 1, k = 8), 65537 sites 8.9 -> 2.9 (512 x 1, k = 11), 2^22 sites 144 -> 115 (128 x 4,
-// k = 4); FP32 65537 sites 2.3 -> 0.5 (128 x 4, k = 16), 2^22 sites 12.7 -> 8.9 (256 x 8, k = 16).  Over
-// 300 .. 2^24 sites of both models and precisions the choice is within 3 % of the best tiling in the
-// median, 10 % at worst.
+// The automatic choice (rk4_chain_get_tiling: its seed, then what the last integration ran with)
+// depends on the sites and the steps: a short chain needs small tiles to reach every SM and many
+// steps per launch to pay for the launch, a long one wide tiles.  Measured against the seed, us per
+// step: FP64 1000 sites 8.9 -> 1.6 (128 x 1, k = 8), 65537 sites 8.9 -> 2.9 (512 x 1, k = 11), 2^22 sites
+// 144 -> 117 (128 x 4, k = 4); FP32 65537 sites 2.3 -> 0.5 (128 x 4, k = 16), 2^22 sites 12.7 -> 8.9
+// (256 x 8, k = 16).  Over 300 .. 2^24 sites of both models and precisions the choice is within 3 % of
+// the best tiling in the median, 10 % at worst.
 // The FP64 form (coefficients outside split_allowed) keeps the seed.
 rk4_tiling run_tiling(rk4_chain *h, int64_t nsteps) {
   if (!h->tiling_auto) return h->tiling;
@@ -865,6 +866,7 @@ int integrate_impl(rk4_chain *h, void *state, void *comp, void *ws, size_t ws_by
   if (nsteps == 0) return RK4_OK;
   if (ensure_pinned(h) != cudaSuccess) return RK4_ECUDA;
   h->run = run_tiling(h, nsteps);
+  if (h->tiling_auto && kernel != RK4_KERNEL_STAGED) h->run_version = h->config_version + 1;
   const Plan P = make_plan(h, nsteps, kernel == RK4_KERNEL_STAGED ? 1 : h->run.k);
   if (kernel != RK4_KERNEL_STAGED) {
     // tile counts must fit a 1-D grid and the int32 prefix tables
@@ -1324,7 +1326,7 @@ int rk4_chain_set_tiling(rk4_chain *h, int block, int v, int k) {
 
 int rk4_chain_get_tiling(const rk4_chain *h, rk4_tiling *out) {
   if (!h || !out) return RK4_EINVAL;
-  *out = h->tiling;
+  *out = h->tiling_auto && h->run_version == h->config_version + 1 ? h->run : h->tiling;
   return RK4_OK;
 }
 
