@@ -533,12 +533,6 @@ __device__ __forceinline__ void split_advance(double (&y)[V][Dim<MODEL>::D], uin
   }
 }
 
-// Global loads: the read-only path for one-shot launches; L2-coherent loads (bypassing L1)
-// inside the persistent kernel, whose buffers are rewritten by other blocks between barriers.
-template <bool COH, typename T> __device__ __forceinline__ T gld(const T *p) {
-  if constexpr (COH) return __ldcg(p); else return __ldg(p);
-}
-
 // Block-cooperative copies of `count` values between global and shared memory.
 //
 // copy_in_vec / copy_out_vec access global memory by 16-byte vectors wherever whole vectors
@@ -586,28 +580,28 @@ __device__ __forceinline__ void copy_out_matched(R *__restrict__ dst, const R *s
   for (int e = head + nv * kPer + threadIdx.x; e < count; e += blockDim.x) dst[e] = src[e];
 }
 
-template <bool COH, typename R>
+template <typename R>
 __device__ __forceinline__ void copy_in_vec(R *dst, const R *__restrict__ src, int count) {
   constexpr int kPer = 16 / (int)sizeof(R);
   const unsigned ms = (unsigned)(reinterpret_cast<uintptr_t>(src) & 15u);
   int head = (int)(((16u - ms) & 15u) / sizeof(R));  // values before the first whole vector
   if (head > count) head = count;
   const int nv = (count - head) / kPer;
-  for (int e = threadIdx.x; e < head; e += blockDim.x) dst[e] = gld<COH>(src + e);
+  for (int e = threadIdx.x; e < head; e += blockDim.x) dst[e] = __ldcg(src + e);
   const int4 *s4 = reinterpret_cast<const int4 *>(src + head);
   if (ms == (unsigned)(reinterpret_cast<uintptr_t>(dst) & 15u)) {
     int4 *d4 = reinterpret_cast<int4 *>(dst + head);
-    for (int e = threadIdx.x; e < nv; e += blockDim.x) d4[e] = gld<COH>(s4 + e);
+    for (int e = threadIdx.x; e < nv; e += blockDim.x) d4[e] = __ldcg(s4 + e);
   } else {
     for (int e = threadIdx.x; e < nv; e += blockDim.x) {
-      const int4 w = gld<COH>(s4 + e);
+      const int4 w = __ldcg(s4 + e);
       const R *p = reinterpret_cast<const R *>(&w);
       R *d = dst + head + e * kPer;
 #pragma unroll
       for (int q = 0; q < kPer; ++q) d[q] = p[q];
     }
   }
-  for (int e = head + nv * kPer + threadIdx.x; e < count; e += blockDim.x) dst[e] = gld<COH>(src + e);
+  for (int e = head + nv * kPer + threadIdx.x; e < count; e += blockDim.x) dst[e] = __ldcg(src + e);
 }
 template <typename R>
 __device__ __forceinline__ void copy_out_vec(R *__restrict__ dst, const R *src, int count) {
@@ -662,14 +656,14 @@ __device__ __forceinline__ void copy_in_async(R *dst, const R *__restrict__ src,
   const unsigned ms = (unsigned)(reinterpret_cast<uintptr_t>(src) & 15u);
   if (ms != (unsigned)(reinterpret_cast<uintptr_t>(dst) & 15u)) {
     if constexpr (COH) {
-      copy_in_vec<COH>(dst, src, count);
+      copy_in_vec(dst, src, count);
     } else {
       for (int e = threadIdx.x; e < count; e += blockDim.x) cp_async(dst + e, src + e, (int)sizeof(R));
     }
     return;
   }
   auto one = [&](int e) {
-    if constexpr (COH) dst[e] = gld<COH>(src + e); else cp_async(dst + e, src + e, (int)sizeof(R));
+    if constexpr (COH) dst[e] = __ldcg(src + e); else cp_async(dst + e, src + e, (int)sizeof(R));
   };
   int head = (int)(((16u - ms) & 15u) / sizeof(R));
   if (head > count) head = count;
