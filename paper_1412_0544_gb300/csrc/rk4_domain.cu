@@ -52,7 +52,9 @@ struct rk4_domain {
 namespace {
 
 constexpr size_t kAlign = 256;
-constexpr int64_t kWideTileSites = (int64_t)1 << 20;  // from here on 2048-site tiles: see rk4_domain_create
+// FP32 chains from here on take eight sites per thread, and from the second on 2048-site tiles: see
+// rk4_domain_create
+constexpr int64_t kEightSites = (int64_t)1 << 19, kWideTileSites = (int64_t)1 << 22;
 size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
 bool any_ghost(const rk4_domain *d) { return d->bc == RK4_PERIODIC || d->nparts > 1; }
@@ -212,14 +214,17 @@ int rk4_domain_create(rk4_domain **out, int model, int precision, int64_t n, dou
   }
   // few long parts: one blocked launch over all of them is the natural scheme.  FP32 runs
   // several steps per launch (bandwidth-bound at k = 1): an exchange period of up to 16 steps is one
-  // launch (run_period), a longer one several of at most 16.  Eight sites per thread where the
-  // parts fill the chip with such tiles (2^24 sites, k = 16: 5.16e11 site-steps/s against 4.66e11 with
-  // four, 256 x 4 x 8 4.38e11).
+  // launch (run_periods), a longer one several of at most 16.  128 steps in 4 parts, us at 256 x 4, 128 x 8
+  // and 256 x 8, Roessler (the harmonic chain's order is the same): periods of 16 steps 2^18 sites 254, 252,
+  // 284; 2^19 335, 324, 329; 2^21 786, 761, 765; 2^22 1362, 1332, 1297; 2^24 4842, 4701, 4433; periods of 8, whose
+  // halo is half as wide, 2^17 403, 427, 427; 2^18 426, 427, 496; 2^19 512, 493, 545; 2^22 1646, 1613, 1718; 2^24
+  // 5387, 5207, 5664.
   rk4_chain_set_kernel(d->h, RK4_KERNEL_BLOCKED);
   if (d->fp32 && ghosts) {
     const int k = (int)std::min<int64_t>(16, std::max<int64_t>(1, ghost / 4));
+    const int block = k == 16 && n >= kWideTileSites ? 256 : 128;
     // keeps what it has if a shape is not valid
-    if (n < kWideTileSites || k < 8 || rk4_chain_set_tiling(d->h, 256, 8, k) != RK4_OK)
+    if (n < kEightSites || k < 8 || rk4_chain_set_tiling(d->h, block, 8, k) != RK4_OK)
       rk4_chain_set_tiling(d->h, 256, 4, k);
   }
   *out = d;
