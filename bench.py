@@ -52,8 +52,8 @@ HBM_GBS_FALLBACK = 6800.0
 # fallback when the probe cannot run).  The classical RK4 Roessler step issues 49 DFMA per
 # site-step in FP64 (4 x 7 slope, whose two additions are issued as exact FMAs a*1+b, 9 stage
 # states, 12 update) in its FP64 form and 13 (7 first slope, 6 update) in the split form that the
-# kernels run (the dopri5 scheme 16: 10 and 6), whose other operations are FP32; the roof is the DFMA
-# rate either way.  FP32: the larger of the scalar and packed (f32x2) FMA lane rates.
+# kernels run (the generic scheme with second neighbours 30), whose other operations are FP32; the roof is
+# the DFMA rate either way.  FP32: the larger of the scalar and packed (f32x2) FMA lane rates.
 FP64_INST_PEAK = 0.6272e12
 FP32_INST_PEAK = 40.12e12
 PEAK_SOURCE = "fallback constants from an earlier pipe_probe run"
@@ -77,7 +77,7 @@ def probe_peaks():
 
 FP64_INST_PER_SITE_STEP = 49     # DFMA of the FP64 form (the slope's 8 additions issued as a * 1 + b)
 SPLIT_FP64_INST = 13             # DFMA of the split form: first slope 7, update 6
-SPLIT_FP64_INST_GENERIC = 16     # the same with second neighbours: first slope 10, update 6
+SPLIT_FP64_INST_GENERIC = 30     # of the generic one with second neighbours: first slope 10, its derivative 11, update 9
 FP32K_INST_PER_SITE_STEP = 58    # the update: 4 operations per component instead of 1 FMA
 # DRAM traffic (read + write bytes) per launch of the FP64 blocked kernel from one ncu capture,
 # with the chain length it was taken at: valid only for the kernel code (kernel_hash) and the
@@ -102,7 +102,7 @@ def code_only(src: str) -> str:
 
 
 BLOCKED_SOURCES = ("rk4_device.cuh", "rk4_split.cuh", "rk4_tile.cuh", "k_split.cuh", "k_blocked.cu")
-GENERIC_SOURCES = ("rk4_device.cuh", "rk4_tile.cuh", "rk4_generic.cuh", "k_generic.cu")
+GENERIC_SOURCES = ("rk4_device.cuh", "rk4_split.cuh", "rk4_tile.cuh", "rk4_generic.cuh", "k_generic.cu", "k_gen_split.cu")
 
 
 def kernel_hash(read=None, files=BLOCKED_SOURCES) -> str:
@@ -797,6 +797,13 @@ def main():
                 "hbm_frac_effective_state": sps_k * 2 * D * 8 / 1e9 / hbm_peak,
                 # DRAM bandwidth the kernel draws: ncu's bytes per launch over this run's launch time
                 "dram_GBs": traffic / launch_s / 1e9 if traffic else None}
+    # what the FP64 form's 49-instruction stream reaches on register-resident sites: alone, and with a tile
+    # kernel's exchange and barrier per stage
+    for key, rate in (("arithmetic_only", "rk4_fp64_regs_inst_per_s"),
+                      ("arithmetic_with_exchange", "rk4_fp64_regs_smem_roundtrip_inst_per_s")):
+        if probe and rate in probe:
+            roofline[f"{key}_rate"] = float(probe[rate]) / 1e9
+            roofline[f"frac_of_{key}"] = achieved_inst * 1e9 / float(probe[rate])
     # --- end to end through the C ABI with host buffers ------------------------------
     host = torch.empty((n, D), dtype=torch.float64).pin_memory()
     host.copy_(st.cpu())
