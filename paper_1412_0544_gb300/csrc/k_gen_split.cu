@@ -11,15 +11,15 @@
 // Why the extra term: the differences K1 - k_m are c_m dt |J| times K1, and with rows up to 25 in sum of
 // magnitudes (Dormand-Prince 5) their pairs' errors showed: 1.05 of the FP64 form's error after one step
 // (z 1.15, 2.2 at |x|, |z| = 20; x 1.04 with kappa = 2, kappa2 = 0.7), because the FP64 form rounds its state
-// only once a step.  The remainders are smaller again by dt |J|: 0.92 ..
-// 1.002 in each component after one and two steps (Dormand-Prince 5 and RK4, dt = 0.01 .. 0.06, kappa up to 2,
-// kappa2 up to 0.7, |x|, |z| up to 15).  e_z, which x - c multiplies, is normalised (z 1.004 -> 0.981 with Fehlberg's
-// tableau, dt = 0.0138).  M's rows in pairs left x at 1.03.
+// only once a step.  The remainders are smaller again by dt |J|: 0.87 .. 1.002 in each component after
+// one and two steps (Dormand-Prince 5 and RK4, dt = 0.01 .. 0.06, kappa up to 2, kappa2 up to 0.7, |x|, |z| up
+// to 15).  e_z, which x - c multiplies, is normalised (z 1.004 -> 0.981 with Fehlberg's tableau, dt = 0.0138).
+// M's rows in pairs left x at 1.03.
 // The weights' sum is carried to a float beyond FP64: its own rounding, times dt K1 every step, was a
 // drift of 1.2 after 20 steps.
 //
 // What bounds it: the FP64 pipe takes 30 instructions per site-step with second neighbours (10 for K1, 11 for
-// M, 3 and 6 for the update; 123 in the FP64 form) beside some 1000 FP32
+// M, 3 and 6 for the update; 123 in the FP64 form) beside about 1300 FP32
 // operations, 16 warps per SM (128 registers).  Every thread holds two sites (one packed pair) whatever the
 // tiling's sites per thread, so a tile of W sites runs on W / 2 threads; M and the remainders lie in
 // thread-private shared-memory records, which both frees their registers and lets the stage loops run over

@@ -3,9 +3,10 @@
 // (k_split_roessler.cu, k_split_harmonic.cu), so that they compile side by side.
 //
 // What bounds it: 13 FP64 instructions per site-step (Roessler: 7 for the first slope, 6 for the
-// update; harmonic 8) at 0.6 T/s allow 4.6e10 site-steps/s; beside them about 300 FP32
-// operations (packed two sites per instruction, 40 T lane-operations/s) and 110 integer ones.
-// Measured at N = 2^24 against the FP64 form (49 instructions, 1.23e10 site-steps/s): 3.68e10 at
+// update; harmonic 8) at 0.6 T/s allow 4.6e10 site-steps/s; beside them about 400 FP32
+// operations (three later stages at 85, 102 for the sums and increments, 33 to convert; packed two
+// sites per instruction, 40 T lane-operations/s) and 110 integer ones.
+// Measured at N = 2^24 against the FP64 form (49 instructions, 1.23e10 site-steps/s): 3.67e10 at
 // 256 x 2 x 4 and 128 x 4 x 4; harmonic 6.4e10 (128 x 4 x 4) against 1.90e10.
 #pragma once
 #include "k_grid_barrier.cuh"

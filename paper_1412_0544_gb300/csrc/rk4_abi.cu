@@ -1013,10 +1013,10 @@ void split_most(int model, double dt, double *most) {
     most[1] = 1.0 / (512.0 * dt * dt);
   }
 }
-// The largest |x - c| and |y|, |z| of a Roessler state (split_in_range).  One step of uniform states, dt =
-// 0.01, a, c and kappa at their limits, error of z in units of the FP64 form's: 0.86 with these, 1.1
-// with dt |x - c| up to 0.3, 1.6 with 0.4; the attractor reaches dt |x - c| = 0.21, dt z = 0.24 for c = 9 and
-// 0.29, 0.49 for c at its limit.
+// The largest |x - c| and |y|, |z| of a Roessler state (split_in_range), times dt.  One step of uniform
+// states of amplitude A, dt = 0.01, error of z in units of the FP64 form's: 0.73 at dt A = 0.2, 0.89 at 0.25,
+// 1.18 at 0.3, 1.56 at 0.4; x alone up to dt |x - c| = 0.25 0.81, 0.3 0.99.  The attractor reaches dt |x - c| = 0.21,
+// dt z = 0.24 for c = 9 and 0.29, 0.49 for c at its limit.
 constexpr double kSplitFar = 0.25, kSplitBig = 0.3;
 constexpr double kSplitMostDt[] = {1.0 / 16, 1.0 / 8};  // Roessler (1.05 .. 1.3 from 1/12 on), harmonic
 bool split_takes(double v, double most) {

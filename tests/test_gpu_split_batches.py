@@ -16,13 +16,10 @@ LENGTHS = np.array([3000, 40, 7, 2100, 33, 64, 1, 500, 12, 90], dtype=np.int64)
 
 
 @pytest.mark.parametrize("kernel,tiling", SCHEMES)
-@pytest.mark.parametrize("model", [ROE, HAR])
-@pytest.mark.parametrize("value", [1e-120, 1e4, 1e14, np.nan])
+@pytest.mark.parametrize("model,value", [(ROE, 1e-120), (ROE, 1e4), (ROE, np.nan), (HAR, 1e-120), (HAR, 1e14), (HAR, np.nan)])
 def test_other_chains_keep_their_bits(kernel, tiling, model, value):
     import torch
     import paper_1412_0544_gb300 as rk
-    if value == (1e14 if model == ROE else 1e4):
-        pytest.skip("beyond FP64 in a few steps, or within the range")
     m = len(LENGTHS)
     off = np.concatenate(([0], np.cumsum(LENGTHS)))
     D = 3 if model == ROE else 2
