@@ -85,18 +85,18 @@ FP32K_INST_PER_SITE_STEP = 58    # the update: 4 operations per component instea
 # proportional to the sites it advances (one read and one write of each tile), so a capture at
 # N = 2^24 scales to the N = 2^27 workload by the site count.
 TRAFFIC = {
-    ("90381b6f0dfc25ff", "128,4,2"): (402730496 + 358060800, 1 << 24),
-    ("90381b6f0dfc25ff", "128,4,4"): (402899456 + 358327808, 1 << 24),
-    ("90381b6f0dfc25ff", "128,4,8"): (402785280 + 358649856, 1 << 24),
-    ("90381b6f0dfc25ff", "128,8,4"): (402804992 + 355816704, 1 << 24),
-    ("90381b6f0dfc25ff", "128,8,8"): (402787328 + 355889408, 1 << 24),
-    ("90381b6f0dfc25ff", "256,2,2"): (402800640 + 358162176, 1 << 24),
-    ("90381b6f0dfc25ff", "256,2,4"): (402846720 + 358069248, 1 << 24),
-    ("90381b6f0dfc25ff", "256,2,8"): (402856448 + 358657792, 1 << 24),
-    ("90381b6f0dfc25ff", "256,4,4"): (402824704 + 355953664, 1 << 24),
-    ("90381b6f0dfc25ff", "256,4,8"): (402806272 + 356186880, 1 << 24),
-    ("90381b6f0dfc25ff", "512,2,4"): (403021824 + 357889024, 1 << 24),
-    ("90381b6f0dfc25ff", "512,2,8"): (403138048 + 358125312, 1 << 24),
+    ("33881277ea58e1d8", "128,4,2"): (402732800 + 357960960, 1 << 24),
+    ("33881277ea58e1d8", "128,4,4"): (403709440 + 357963264, 1 << 24),
+    ("33881277ea58e1d8", "128,4,8"): (403094784 + 358764032, 1 << 24),
+    ("33881277ea58e1d8", "128,8,4"): (402825728 + 355761408, 1 << 24),
+    ("33881277ea58e1d8", "128,8,8"): (402899712 + 356287744, 1 << 24),
+    ("33881277ea58e1d8", "256,2,2"): (402732032 + 357962752, 1 << 24),
+    ("33881277ea58e1d8", "256,2,4"): (403470592 + 358254592, 1 << 24),
+    ("33881277ea58e1d8", "256,2,8"): (402822400 + 358872576, 1 << 24),
+    ("33881277ea58e1d8", "256,4,4"): (402746880 + 355839744, 1 << 24),
+    ("33881277ea58e1d8", "256,4,8"): (403842816 + 356381952, 1 << 24),
+    ("33881277ea58e1d8", "512,2,4"): (402732288 + 357843456, 1 << 24),
+    ("33881277ea58e1d8", "512,2,8"): (402940416 + 358331648, 1 << 24),
 }
 
 

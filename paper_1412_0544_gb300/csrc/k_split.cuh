@@ -64,11 +64,11 @@ template <int MODEL, bool HET, typename R, typename F> static R split_dispatch(i
 
 // An item (of a packed tile, the marked segments) outside the split's range, in the FP64 form.  Not inlined: it is rare, and its
 // registers then do not add to the split's.
-template <int MODEL, int V, bool COH, bool HET, bool ALN>
+template <int MODEL, int V, bool HET, bool ALN>
 __device__ __noinline__ void wide_tile_call(const double *in, double *out, ChainDesc ch, int64_t tile, int K, int G,
                                             Coef<double> cf, unsigned char *smem, int64_t sites, WsHeader *hdr,
                                             const double *sp) {
-  tile_item<double, MODEL, V, false, COH, HET, ALN, false>(in, out, nullptr, nullptr, ch, tile, K, G, cf, smem, sites,
+  tile_item<double, MODEL, V, false, false, HET, ALN, false>(in, out, nullptr, nullptr, ch, tile, K, G, cf, smem, sites,
                                                            hdr, sp);
 }
 template <int MODEL, int V, bool COH>
@@ -119,12 +119,16 @@ __global__ void __launch_bounds__(NT, split_min_blocks(MODEL, V, HET)) k_split(B
   const double *sp = static_cast<const double *>(job.sp);
   if (!tile_item<double, MODEL, V, false, false, HET, PACKED, true, PARK>(in, out, nullptr, nullptr, ch, tile, job.K, job.G,
                                                                     cf, smem, job.total, job.hdr, sp, &sc))
-    wide_tile_call<MODEL, V, false, HET, PACKED>(in, out, ch, tile, job.K, job.G, cf, smem, job.total, job.hdr, sp);
+    wide_tile_call<MODEL, V, HET, PACKED>(in, out, ch, tile, job.K, job.G, cf, smem, job.total, job.hdr, sp);
 }
 
-// One full tile of the persistent kernel as a call of its own (as persistent_tile_call).
-template <int MODEL, int V, bool BATCH, bool PARK>
-__device__ __noinline__ void persistent_split_call(const PersistentJob &job, int ki, const double *in, double *out,
+// One full tile of the persistent kernel as a call of its own (as persistent_tile_call), in the split form
+// or (WIDE) in the FP64 form; false when it is outside the split's range.  The FP64 form is called from the
+// kernel's loop: from within the split form's call ptxas gave it registers that cost 13 % (64 chains of 64000
+// sites, a state of 1e-25, 8 steps: 3308 -> 2938 us; 4096 of 1000 sites in range 1052 -> 1041).  Packed tiles,
+// a few per launch, keep theirs inside (outside: 1041 -> 1054).
+template <int MODEL, int V, bool BATCH, bool PARK, bool WIDE>
+__device__ __noinline__ bool persistent_split_call(const PersistentJob &job, int ki, const double *in, double *out,
                                                    int64_t item, int K, int G, Coef<double> cf, SplitCoef sc,
                                                    unsigned char *smem) {
   ChainDesc ch;
@@ -133,13 +137,12 @@ __device__ __noinline__ void persistent_split_call(const PersistentJob &job, int
     const int ci = batch_chain(job.bt[ki], job.nchains, item - job.bt[ki].npacked, smem, tile);
     ch = job.chains[ci];
     cf.kappa = ch.kappa;
-    split_set_kappa(sc, ch.kappa);
+    if constexpr (!WIDE) split_set_kappa(sc, ch.kappa);
   } else {
     ch = job.one;
   }
-  if (!tile_item<double, MODEL, V, false, true, false, BATCH, true, PARK>(in, out, nullptr, nullptr, ch, tile, K, G, cf,
-                                                                    smem, job.total, job.hdr, nullptr, &sc))
-    wide_tile_call<MODEL, V, true, false, BATCH>(in, out, ch, tile, K, G, cf, smem, job.total, job.hdr, nullptr);
+  return tile_item<double, MODEL, V, false, true, false, BATCH, !WIDE, PARK && !WIDE>(
+      in, out, nullptr, nullptr, ch, tile, K, G, cf, smem, job.total, job.hdr, nullptr, &sc);
 }
 
 // The split form of k_persistent.
@@ -153,8 +156,8 @@ __global__ void __launch_bounds__(NT, split_min_blocks(MODEL, V, false)) k_persi
     if (BATCH && item < job.bt[ki].npacked)
       split_packed_call<MODEL, V, true, PARK>(i, o, job.chains, job.bt[ki].segs, job.bt[ki].pack_prefix, item, K, cf, &sc,
                                         smem, job.total, job.hdr);
-    else
-      persistent_split_call<MODEL, V, BATCH, PARK>(job, ki, i, o, item, K, G, cf, sc, smem);
+    else if (!persistent_split_call<MODEL, V, BATCH, PARK, false>(job, ki, i, o, item, K, G, cf, sc, smem))
+      persistent_split_call<MODEL, V, BATCH, PARK, true>(job, ki, i, o, item, K, G, cf, sc, smem);
   });
 }
 
